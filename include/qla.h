@@ -85,9 +85,9 @@ typedef struct {
     int potential;       /* QLA_POT_PAPER (default) or QLA_POT_UNITARY */
     int steps_per_pass;  /* full time steps fused per HBM pass: 0 = automatic (2; FP32 with chunk_rows
                             set: 2 from 2^25 sites up, else 4), else 1, 2 or 4 */
-    int chunk_rows;      /* rows of one sweep tile, else 0 = automatic: each family's rows are
-                            split into one share of equal estimated cost per resident CTA
-                            (see qla_sweep_split) */
+    int chunk_rows;      /* rows swept by one warp of a strip (0 = automatic); with the shared-memory
+                            sweep (the persistent launch form, planes of 2^32 bytes or more), rows of
+                            one tile, 0 = the balanced split (see qla_sweep_split) */
     int device;          /* CUDA device ordinal; -1 = the calling thread's current device */
     void *stream;        /* cudaStream_t to run on; NULL = a non-blocking stream owned by the context */
     int families;        /* QLA_FAMILIES_BOTH (default), or QLA_FAMILY_TM / QLA_FAMILY_TE: only that
@@ -103,7 +103,8 @@ void qla_default_options(qla_options *opt);
 /* Device memory one context needs (bytes; each buffer 256-byte aligned). */
 typedef struct {
     size_t state_bytes;    /* one state buffer (6 planes); two are needed (ping-pong) */
-    size_t coeff_bytes;    /* rotation and potential coefficient planes */
+    size_t coeff_bytes;    /* rotation and potential coefficients, in the layout of the sweep that the
+                              options select (query with the options given to qla_create) */
     size_t index_bytes;    /* n_x, n_y, n_z (double) */
     size_t scratch_bytes;  /* reduction scratch for the diagnostics */
 } qla_buffer_sizes;
@@ -324,8 +325,10 @@ qla_status qla_sweep_split(int Nx, int Ny, int precision, int steps_per_pass, in
 qla_status qla_sweep_dependencies(int Nx, int Ny, int steps_per_pass, int ctas, int family, int share, int *deps,
                                   int capacity, int *count);
 
-/* The split the context's passes of steps_per_pass steps use for `family`
- * (with the persistent launch form, one layer's split per family):
+/* The balanced split of a pass of steps_per_pass steps over `family` on the
+ * context's device, as its shared-memory sweep would use it (with the persistent
+ * launch form, one layer's split per family; passes of the marching sweep
+ * cut strips of their own into equal row ranges instead):
  * *ctas = CTAs of the family's layer (0 when the context sweeps tiles of
  * chunk_rows rows instead, or does not advance the family), and, if bounds is
  * not NULL and *ctas > 0, the share bounds as qla_sweep_split writes them

@@ -39,16 +39,18 @@ def save_cache(cache: dict, path: Optional[str] = None) -> None:
 
 
 def kernel_version() -> str:
-    """sha256 prefix of the sweep kernel's source: cached choices of an older
+    """sha256 prefix of the sweep kernels' sources: cached choices of an older
     kernel are not reused."""
     import hashlib
 
-    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", "qla_sweep.cuh")
+    h = hashlib.sha256()
     try:
-        with open(src, "rb") as f:
-            return hashlib.sha256(f.read()).hexdigest()[:12]
+        for name in ("qla_sweep.cuh", "qla_march.cuh"):
+            with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", name), "rb") as f:
+                h.update(f.read())
     except OSError:
         return "unknown"
+    return h.hexdigest()[:12]
 
 
 def single_key(Nx: int, Ny: int, precision: str, sequence: str, potential: str, gpu: str) -> str:

@@ -41,6 +41,9 @@ struct qla_ctx {
     int K = 4;
     int chunk = 0;
     int ctas[5] = {0, 0, 0, 0, 0};  // balanced split (chunk == 0): CTAs per family of a pass of K steps
+    bool march = false;             // the marching form (launch_march) serves the context's passes
+    qla::MarchGeo geo{};
+    int nfam = 2, fam0 = 0;         // families advanced (TM = 0, TE = 1)
     bool persistent = false;        // passes of K steps in one cooperative launch per qla_step (QLA_LAUNCH_*)
     unsigned *pass_done = nullptr;  // device [2][kPersistMaxCtas]: passes completed per share (persistent form)
     unsigned pass_epoch = 0;        // passes the persistent launches have completed (the counters' base)
@@ -137,9 +140,20 @@ int balanced_ctas(int Nx, int Ny, int K, int prec, int interleaved, int sms) {
 // FP32, the balanced split, K instantiated for it, the seam layout (Nx a
 // multiple of 8, at least 256 columns) and at most kPersistMaxCtas shares.
 bool persistent_applies(const qla_ctx *c) {
-    return c->opt.precision == QLA_FP32 && c->chunk == 0 && qla::sweep_persistent_supported(0, c->K) &&
+    return !c->march && c->opt.precision == QLA_FP32 && c->chunk == 0 && qla::sweep_persistent_supported(0, c->K) &&
            c->Nx % 8 == 0 && c->Nx >= qla::sweep_strip_width() && c->ctas[c->K] >= 1 &&
            c->ctas[c->K] <= qla::kPersistMaxCtas;
+}
+
+// Whether the marching form serves a context: every lattice whose planes it can
+// address, unless the persistent launch form (on the shared-memory sweep and
+// its pair planes) was asked for and applies.
+bool march_applies(const qla_options &o, int Nx, int Ny, qla::MarchGeo *g) {
+    if (!qla::march_geometry(o.precision == QLA_FP64 ? 1 : 0, Nx, Ny, g) || g->strips > 65535) return false;
+    const int K = o.steps_per_pass > 0 ? o.steps_per_pass
+                                       : default_steps_per_pass(o.precision, Nx, Ny, o.chunk_rows);
+    return !(o.launch == QLA_LAUNCH_PERSISTENT && o.precision == QLA_FP32 && o.chunk_rows == 0 &&
+             qla::sweep_persistent_supported(0, K) && Nx % 8 == 0 && Nx >= qla::sweep_strip_width());
 }
 
 // Whether component `comp` (Eq. 15 order) belongs to a family the context
@@ -151,6 +165,19 @@ bool family_has(const qla_ctx *c, int comp) {
 }
 
 qla_status launch_pass(qla_ctx *c, int K) {
+    if (c->march) {
+        // K = 4 (and FP64's K = 2) as passes of two steps (of one): the same values, in less time
+        const int per = std::min(K, c->opt.precision == QLA_FP64 ? 1 : 2);
+        for (int k = 0; k < K; k += per) {
+            const cudaError_t e = qla::launch_march(
+                c->geo, per, c->state[c->cur], c->state[c->cur ^ 1], c->coef, c->nfam, c->fam0,
+                c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, c->opt.potential == QLA_POT_UNITARY ? 1 : 0,
+                c->stream);
+            if (e != cudaSuccess) return fail(c, QLA_ECUDA, "sweep launch (K=%d): %s", K, cudaGetErrorString(e));
+            c->cur ^= 1;
+        }
+        return QLA_OK;
+    }
     qla::SweepArgs a{};
     a.q_in = c->state[c->cur];
     a.q_out = c->state[c->cur ^ 1];
@@ -257,7 +284,10 @@ qla_status qla_query_buffer_sizes(int Nx, int Ny, const qla_options *opt, qla_bu
     const size_t P = size_t(Nx) * size_t(Ny);
     const size_t es = elem_size(o);
     out->state_bytes = round_up(6 * P * es, kAlign);
-    out->coeff_bytes = round_up(size_t(qla::NCOEF) * P * es, kAlign);
+    qla::MarchGeo g;
+    const int nfam = o.families == QLA_FAMILIES_BOTH ? 2 : 1;
+    out->coeff_bytes = round_up(march_applies(o, Nx, Ny, &g) ? qla::march_bytes(g, nfam)
+                                                             : size_t(qla::NCOEF) * P * es, kAlign);
     out->index_bytes = round_up(3 * P * sizeof(double), kAlign);
     out->scratch_bytes = round_up(qla::diag_scratch_bytes(Nx, Ny), kAlign) + round_up(sizeof(qla::DiagResult), kAlign) +
                          kAlign +  // sweep error flag, share-order counter
@@ -351,9 +381,14 @@ qla_status qla_create(int Nx, int Ny, const double *n_x, const double *n_y, cons
         if (cudaMemcpyAsync(c->index + size_t(k) * P, nn[k], P * sizeof(double), cudaMemcpyHostToDevice,
                             c->stream) != cudaSuccess)
             return bail(QLA_ECUDA);
-    if (qla::launch_coefficients(c->index, c->coef, Nx, Ny, delta, o.precision,
-                                 o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, o.potential == QLA_POT_UNITARY ? 1 : 0,
-                                 c->stream) != cudaSuccess)
+    c->march = march_applies(o, Nx, Ny, &c->geo);
+    c->nfam = o.families == QLA_FAMILIES_BOTH ? 2 : 1;
+    c->fam0 = o.families == QLA_FAMILY_TE ? 1 : 0;
+    const int inter = o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, unit = o.potential == QLA_POT_UNITARY ? 1 : 0;
+    if ((c->march ? qla::launch_march_records(c->geo, c->index, c->coef, c->nfam, c->fam0, delta,
+                                              o.precision == QLA_FP64 ? 1 : 0, inter, unit, c->stream)
+                  : qla::launch_coefficients(c->index, c->coef, Nx, Ny, delta, o.precision, inter, unit, c->stream)) !=
+        cudaSuccess)
         return bail(QLA_ECUDA);
     if (cudaMemsetAsync(c->state[0], 0, bs.state_bytes, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->state[1], 0, bs.state_bytes, c->stream) != cudaSuccess)
@@ -366,6 +401,7 @@ qla_status qla_create(int Nx, int Ny, const double *n_x, const double *n_y, cons
             if (qla::sweep_supported(o.precision, k))
                 c->ctas[k] = balanced_ctas(Nx, Ny, k, o.precision == QLA_FP64 ? 1 : 0,
                                            o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, sm_count(c->dev));
+    if (c->march) qla::march_plan(&c->geo, c->nfam, c->chunk, sm_count(c->dev));
     // QLA_LAUNCH_AUTO: one launch per pass, measured the faster form (the persistent one on GB300, 8192^2,
     // 2 steps per pass, site-updates/s: both families 62.1 G with the families alternating per pass against
     // 83.5 G; TM alone 161.2 against 164.6 G; TE alone 166.2 against 163.5 G)
@@ -568,7 +604,7 @@ qla_status qla_debug_apply(qla_ctx *c, int op, int count) {
     for (int k = 0; k < count; ++k) {
         bool swapped = false;
         const cudaError_t e = qla::debug_apply(op, c->opt.precision, c->state[c->cur], c->state[c->cur ^ 1], c->coef,
-                                               c->Nx, c->Ny, c->opt.potential == QLA_POT_UNITARY ? 1 : 0, c->stream,
+                                               c->march ? &c->geo : nullptr, c->nfam, c->fam0, c->Nx, c->Ny, c->opt.potential == QLA_POT_UNITARY ? 1 : 0, c->stream,
                                                &swapped);
         if (e != cudaSuccess) return fail(c, QLA_ECUDA, "qla_debug_apply: %s", cudaGetErrorString(e));
         if (swapped) c->cur ^= 1;

@@ -63,26 +63,41 @@ __device__ void tuned_pair_f32(double ang, float &mf, float &sf) {
 enum PairKind { PK_SHEAR, PK_ROTATION, PK_PRINTED_V };
 
 template <typename T>
-__device__ void store_pair(T *coef, size_t P, int pair, size_t i, double ang, PairKind kind) {
-    T *dst = coef + 2 * (size_t(pair) * P + i);
+__device__ void make_pair_of(double ang, PairKind kind, T &x, T &y) {
     if constexpr (sizeof(T) == 4) {
-        float xf, sf;
         if (kind == PK_SHEAR) {
-            shear_pair_f32(ang, xf, sf);
+            shear_pair_f32(ang, x, y);
         } else if (kind == PK_ROTATION) {
-            tuned_pair_f32(ang, xf, sf);
+            tuned_pair_f32(ang, x, y);
         } else {
             const double sh = sin(0.5 * ang);
-            xf = (float)(-2.0 * sh * sh);
-            sf = (float)sin(ang);
+            x = (float)(-2.0 * sh * sh);
+            y = (float)sin(ang);
         }
-        dst[0] = xf;
-        dst[1] = sf;
     } else {
         const double sh = sin(0.5 * ang);
-        dst[0] = -2.0 * sh * sh;
-        dst[1] = sin(ang);
+        x = -2.0 * sh * sh;
+        y = sin(ang);
     }
+}
+
+template <typename T>
+__device__ void store_pair(T *coef, size_t P, int pair, size_t i, double ang, PairKind kind) {
+    T *dst = coef + 2 * (size_t(pair) * P + i);
+    make_pair_of<T>(ang, kind, dst[0], dst[1]);
+}
+
+// Eq. 25 at site (x, y), central differences over lattice spacing delta:
+// delta^2 (dn/dx) / n^2 along x (axis 0) or y (axis 1).
+__device__ __forceinline__ double potential_angle(const double *__restrict__ n, int x, int y, int Nx, int Ny, int axis,
+                                                  double delta) {
+    const int xp = x + 1 == Nx ? 0 : x + 1, xm = x == 0 ? Nx - 1 : x - 1;
+    const int yp = y + 1 == Ny ? 0 : y + 1, ym = y == 0 ? Ny - 1 : y - 1;
+    const size_t r = size_t(y) * Nx;
+    const double v = n[r + x];
+    const double d = axis == 0 ? (n[r + xp] - n[r + xm]) / (2.0 * delta)
+                               : (n[size_t(yp) * Nx + x] - n[size_t(ym) * Nx + x]) / (2.0 * delta);
+    return delta * delta * d / (v * v);
 }
 
 // One thread per site. n: [3][Ny][Nx] double (n_x, n_y, n_z).
@@ -96,21 +111,12 @@ __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, 
     const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < P; i += size_t(gridDim.x) * blockDim.x) {
         const int y = int(i / Nx), x = int(i % Nx);
-        const int xp = x + 1 == Nx ? 0 : x + 1, xm = x == 0 ? Nx - 1 : x - 1;
-        const int yp = y + 1 == Ny ? 0 : y + 1, ym = y == 0 ? Ny - 1 : y - 1;
-        const size_t r = size_t(y) * Nx;
-        const double vnx = nx[i], vny = ny[i], vnz = nz[i];
         // Eq. 24
-        const double th0 = delta / (4.0 * vnx), th1 = delta / (4.0 * vny), th2 = delta / (4.0 * vnz);
-        // Eq. 25 with central differences over lattice spacing delta
-        const double dny_dx = (ny[r + xp] - ny[r + xm]) / (2.0 * delta);
-        const double dnx_dy = (nx[size_t(yp) * Nx + x] - nx[size_t(ym) * Nx + x]) / (2.0 * delta);
-        const double dnz_dx = (nz[r + xp] - nz[r + xm]) / (2.0 * delta);
-        const double dnz_dy = (nz[size_t(yp) * Nx + x] - nz[size_t(ym) * Nx + x]) / (2.0 * delta);
-        const double b0 = delta * delta * dny_dx / (vny * vny);
-        const double b1 = delta * delta * dnx_dy / (vnx * vnx);
-        const double b2 = delta * delta * dnz_dx / (vnz * vnz);
-        const double b3 = delta * delta * dnz_dy / (vnz * vnz);
+        const double th0 = delta / (4.0 * nx[i]), th1 = delta / (4.0 * ny[i]), th2 = delta / (4.0 * nz[i]);
+        const double b0 = potential_angle(ny, x, y, Nx, Ny, 0, delta);
+        const double b1 = potential_angle(nx, x, y, Nx, Ny, 1, delta);
+        const double b2 = potential_angle(nz, x, y, Nx, Ny, 0, delta);
+        const double b3 = potential_angle(nz, x, y, Nx, Ny, 1, delta);
         const PairKind ck = unitary ? PK_ROTATION : PK_SHEAR;
         const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
         store_pair<T>(coef, P, P_TM_C, i, th2, ck);
@@ -120,6 +126,74 @@ __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, 
         store_pair<T>(coef, P, P_TM_VY, i, b3 * vscale, vk);
         store_pair<T>(coef, P, P_TE_VX, i, b0 * vscale, vk);
         store_pair<T>(coef, P, P_TE_VY, i, b1 * vscale, vk);
+    }
+}
+
+// The same pairs as the marching form's records (one block per row of a strip).
+template <typename T>
+__global__ void march_records_kernel(const double *__restrict__ n, T *__restrict__ rec, int fam, MarchGeo g,
+                                     double delta, int interleaved, int unitary) {
+    const size_t P = size_t(g.Nx) * size_t(g.Ny);
+    const double *nx = n, *ny = n + P, *nz = n + 2 * P;
+    const double *ncx = fam ? ny : nz, *ncy = fam ? nx : nz;  // indices of C_X and V_X, of C_Y and V_Y
+    const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
+    const PairKind ck = unitary ? PK_ROTATION : PK_SHEAR;
+    const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
+    const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW, strip = blockIdx.y;
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+        int y = (r - MARCH_ABOVE) % g.Ny;
+        y = y < 0 ? y + g.Ny : y;
+        for (int c = threadIdx.x; c < g.W; c += blockDim.x) {
+            int x = (strip * g.w_valid - g.halo + c) % g.Nx;
+            x = x < 0 ? x + g.Nx : x;
+            const size_t i = size_t(y) * g.Nx + x;
+            T *const d = rec + (size_t(strip) * rows + r) * MARCH_FIELDS * g.W + c;
+            make_pair_of<T>(delta / (4.0 * ncx[i]), ck, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
+            if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), ck, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
+            for (int axis = 0; axis < 2; ++axis) {
+                const double b = potential_angle(axis ? ncy : ncx, x, y, g.Nx, g.Ny, axis, delta) * vscale;
+                T *const v = d + (axis ? F_VY : F_VX) * g.W;
+                if (b == 0.0) {  // the pair of a zero angle, without its sines
+                    v[0] = T(-0.0);
+                    v[g.W] = T(b);
+                } else {
+                    make_pair_of<T>(b, vk, v[0], v[g.W]);
+                }
+            }
+        }
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ bool nonzero_value(T v) {
+    return v != T(0);
+}
+
+// flags[strip][r]: whether any V pair of the strip's columns is nonzero in rows
+// [r - march_flag_back(2), r + MARCH_GROUP - 1] (periodic).
+constexpr int FLAG_ROWS = 64;
+template <typename T>
+__global__ void __launch_bounds__(256) march_flags_kernel(const T *__restrict__ rec, unsigned char *__restrict__ flags,
+                                                          MarchGeo g) {
+    constexpr int BACK = march_flag_back(2);
+    __shared__ unsigned char rf[FLAG_ROWS + BACK + MARCH_GROUP];
+    const int strip = blockIdx.y, r0 = blockIdx.x * FLAG_ROWS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
+    const int n = min(FLAG_ROWS, g.Ny - r0);
+    static_assert(BACK <= MARCH_ABOVE && MARCH_GROUP <= MARCH_BELOW, "rows of the window have records");
+    for (int k = warp; k < n + BACK + MARCH_GROUP - 1; k += 8) {
+        const T *v = rec + ((size_t(strip) * rows + MARCH_ABOVE + r0 - BACK + k) * MARCH_FIELDS + F_VX) * g.W;
+        bool nz = false;
+        for (int c = lane; c < 4 * g.W; c += 32) nz = nz || nonzero_value(v[c]);
+        nz = __any_sync(0xffffffffu, nz);
+        if (lane == 0) rf[k] = nz ? 1 : 0;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += 256) {
+        unsigned char f = 0;
+        for (int i = 0; i < BACK + MARCH_GROUP; ++i) f |= rf[k + i];
+        flags[size_t(strip) * g.Ny + r0 + k] = f;
     }
 }
 
@@ -172,6 +246,31 @@ cudaError_t launch_coefficients(const double *n, void *coef, int Nx, int Ny, dou
         coef_kernel<double><<<grid_for(P, B), B, 0, st>>>(n, static_cast<double *>(coef), Nx, Ny, delta,
                                                            interleaved, unitary);
     return cudaGetLastError();
+}
+
+cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, int nfam, int fam0, double delta,
+                                 int precision, int interleaved, int unitary, cudaStream_t st) {
+    char *m = static_cast<char *>(mem);
+    const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
+    const dim3 grid(unsigned(rows < 4096 ? rows : 4096), unsigned(g.strips));
+    const dim3 fgrid(unsigned((g.Ny + FLAG_ROWS - 1) / FLAG_ROWS), unsigned(g.strips));
+    if (g.strips > 65535) return cudaErrorInvalidValue;
+    for (int z = 0; z < nfam; ++z) {
+        void *rec = m + z * g.record_bytes;
+        unsigned char *flags = reinterpret_cast<unsigned char *>(m + nfam * g.record_bytes + z * g.flag_bytes);
+        if (precision == 0) {
+            march_records_kernel<float><<<grid, g.W, 0, st>>>(n, static_cast<float *>(rec), fam0 + z, g, delta,
+                                                              interleaved, unitary);
+            march_flags_kernel<float><<<fgrid, 256, 0, st>>>(static_cast<const float *>(rec), flags, g);
+        } else {
+            march_records_kernel<double><<<grid, g.W, 0, st>>>(n, static_cast<double *>(rec), fam0 + z, g, delta,
+                                                               interleaved, unitary);
+            march_flags_kernel<double><<<fgrid, 256, 0, st>>>(static_cast<const double *>(rec), flags, g);
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_init_pulse(void *q, int Nx, int Ny, int precision, int pol, double x0, double sigma,

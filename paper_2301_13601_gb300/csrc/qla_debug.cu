@@ -13,10 +13,34 @@ namespace {
 
 constexpr int DBG_THREADS = 256;
 
+// Where a context keeps its coefficients: pair planes, or the marching form's
+// records (null for a family that is not advanced; its state is zero).
+template <typename T>
+struct CoefView {
+    const typename Ar<T>::T2 *pairs;
+    const T *rec[2];
+    MarchGeo g;
+
+    __device__ __forceinline__ bool has(int plane) const { return pairs || rec[plane >= P_TE_VX]; }
+    __device__ __forceinline__ typename Ar<T>::T2 at(int plane, long long P, long long i) const {
+        if (pairs) return pairs[plane * P + i];
+        const int fields[NPAIR] = {F_VX, F_CX, F_VY, F_VX, F_CX, F_CY, F_VY};
+        const int y = int(i / g.Nx), x = int(i - (long long)y * g.Nx), strip = x / g.w_valid;
+        const T *r = rec[plane >= P_TE_VX] +
+                     ((size_t(strip) * (MARCH_ABOVE + g.Ny + MARCH_BELOW) + MARCH_ABOVE + y) * MARCH_FIELDS +
+                      fields[plane]) * g.W + (x - strip * g.w_valid + g.halo);
+        typename Ar<T>::T2 v;
+        v.x = r[0];
+        v.y = r[g.W];
+        return v;
+    }
+};
+
 template <bool DAG, int SG, bool SHR, typename T>
-__device__ __forceinline__ void rot_pair(T *q, const typename Ar<T>::T2 *cp, long long P, long long i, int hub,
+__device__ __forceinline__ void rot_pair(T *q, const CoefView<T> &cp, long long P, long long i, int hub,
                                          int partner, int plane) {
-    const typename Ar<T>::T2 c = cp[plane * P + i];
+    if (!cp.has(plane)) return;
+    const typename Ar<T>::T2 c = cp.at(plane, P, i);
     T h = q[hub * P + i], p = q[partner * P + i];
     rot<DAG, SG, SHR>(h, p, c.x, c.y);
     q[hub * P + i] = h;
@@ -25,7 +49,7 @@ __device__ __forceinline__ void rot_pair(T *q, const typename Ar<T>::T2 *cp, lon
 
 // C_X (axis 0) or C_Y (axis 1) on both families, or their transposes.
 template <int AXIS, bool DAG, bool SHR, typename T>
-__global__ void __launch_bounds__(DBG_THREADS) collide_kernel(T *q, const typename Ar<T>::T2 *cp, long long P) {
+__global__ void __launch_bounds__(DBG_THREADS) collide_kernel(T *q, const CoefView<T> cp, long long P) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
         if (AXIS == 0) {
             rot_pair<DAG, Fam<0>::SGX, SHR>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::CX);
@@ -38,9 +62,10 @@ __global__ void __launch_bounds__(DBG_THREADS) collide_kernel(T *q, const typena
 }
 
 template <int TAU, bool HUB, bool UNIT, typename T>
-__device__ __forceinline__ void pot_pair(T *q, const typename Ar<T>::T2 *cp, long long P, long long i, int hub,
+__device__ __forceinline__ void pot_pair(T *q, const CoefView<T> &cp, long long P, long long i, int hub,
                                          int partner, int plane) {
-    const typename Ar<T>::T2 c = cp[plane * P + i];  // (cos b - 1, sin b)
+    if (!cp.has(plane)) return;
+    const typename Ar<T>::T2 c = cp.at(plane, P, i);  // (cos b - 1, sin b)
     T h = q[hub * P + i], p = q[partner * P + i];
     vop_pair<TAU, HUB, UNIT>(h, p, c.y, c.x);
     q[hub * P + i] = h;
@@ -50,7 +75,7 @@ __device__ __forceinline__ void pot_pair(T *q, const typename Ar<T>::T2 *cp, lon
 // V_X (axis 0) or V_Y (axis 1) on both families, as one application in the
 // context's step (its pair planes hold that application's angles).
 template <int AXIS, bool UNIT, typename T>
-__global__ void __launch_bounds__(DBG_THREADS) potential_kernel(T *q, const typename Ar<T>::T2 *cp, long long P) {
+__global__ void __launch_bounds__(DBG_THREADS) potential_kernel(T *q, const CoefView<T> cp, long long P) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
         if (AXIS == 0) {
             pot_pair<Fam<0>::TX, Fam<0>::VX_HUB, UNIT>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::VX);
@@ -83,11 +108,17 @@ __global__ void __launch_bounds__(DBG_THREADS) stream_kernel(const T *__restrict
 }
 
 template <typename T>
-cudaError_t apply_t(int op, void *state, void *spare, const void *coef, int Nx, int Ny, int unitary, cudaStream_t st,
-                    bool *swapped) {
-    using T2 = typename Ar<T>::T2;
+cudaError_t apply_t(int op, void *state, void *spare, const void *coef, const MarchGeo *geo, int nfam, int fam0, int Nx,
+                    int Ny, int unitary, cudaStream_t st, bool *swapped) {
     T *q = static_cast<T *>(state);
-    const T2 *cp = static_cast<const T2 *>(coef);
+    CoefView<T> cp{};
+    if (geo) {
+        cp.g = *geo;
+        for (int z = 0; z < nfam; ++z)
+            cp.rec[fam0 + z] = reinterpret_cast<const T *>(static_cast<const char *>(coef) + z * geo->record_bytes);
+    } else {
+        cp.pairs = static_cast<const typename Ar<T>::T2 *>(coef);
+    }
     const long long P = (long long)Nx * Ny;
     const int blocks = int(std::min<long long>((P + DBG_THREADS - 1) / DBG_THREADS, 152LL * 16));
     *swapped = false;
@@ -134,10 +165,11 @@ cudaError_t apply_t(int op, void *state, void *spare, const void *coef, int Nx, 
 
 }  // namespace
 
-cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, int Nx, int Ny, int unitary,
-                        cudaStream_t st, bool *swapped) {
-    return precision == QLA_FP64 ? apply_t<double>(op, state, spare, coef, Nx, Ny, unitary, st, swapped)
-                                 : apply_t<float>(op, state, spare, coef, Nx, Ny, unitary, st, swapped);
+cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, const MarchGeo *geo,
+                        int nfam, int fam0, int Nx, int Ny, int unitary, cudaStream_t st, bool *swapped) {
+    return precision == QLA_FP64
+               ? apply_t<double>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, unitary, st, swapped)
+               : apply_t<float>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, unitary, st, swapped);
 }
 
 }  // namespace qla

@@ -230,6 +230,44 @@ int sweep_strip_width();  // input columns per strip (halo included)
 int sweep_occupancy_f32(int K, int interleaved);  // resident CTAs per SM
 int sweep_occupancy_f64(int K, int interleaved);
 
+// ---------------------------------------------------------------------------
+// Marching form of the sweep (qla_march.cuh): strips and coefficient records.
+// ---------------------------------------------------------------------------
+// Records of a family: [strips][MARCH_ABOVE + Ny + MARCH_BELOW] rows of fields
+// x, y of C_X, C_Y, V_X, V_Y (see CoefPair; TM: C_Y unused, its C_X serves
+// both), each W values: the strip's columns with their halo. Rows repeat
+// periodically above row 0 and below row Ny - 1, as far as the shares at either
+// end copy. Flags of a family: [strips][Ny] bytes, see launch_march_records.
+constexpr int MARCH_FIELDS = 8;
+constexpr int F_CX = 0, F_CY = 2, F_VX = 4, F_VY = 6;
+constexpr int MARCH_ABOVE = 20, MARCH_BELOW = 24;
+constexpr int MARCH_GROUP = 4;  // rows covered by a flag
+constexpr __host__ __device__ int march_flag_back(int K) { return 5 * (K - 1) + 4; }
+struct MarchGeo {
+    int Nx, Ny;
+    int W, halo;     // columns of a strip, of its halo on each side
+    int w_valid;     // columns written: W - 2 halo
+    int strips;
+    int es;          // element size
+    int chunks[3];   // row ranges per strip of a pass of K steps (march_plan)
+    size_t record_bytes;  // of one family
+    size_t flag_bytes;    // of one family (a multiple of 256)
+};
+// The marching form serves the lattice (a plane below 2^32 bytes) and its
+// geometry: FP32 128 columns with a halo of 8 (two steps), FP64 64 with 4 (one).
+bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g);
+// Chooses the row ranges of a pass over nfam families on a device of sms SMs.
+// chunk: rows per range (0: automatic).
+void march_plan(MarchGeo *g, int nfam, int chunk, int sms);
+// One pass of K steps (FP32: 1, 2; FP64: 1) over the families f0 .. f0 + nfam - 1.
+// mem: the advanced families' records, then their flags (march_bytes).
+size_t march_bytes(const MarchGeo &g, int nfam);
+cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out, const void *mem, int nfam, int fam0,
+                         int interleaved, int unitary, cudaStream_t st);
+// Records and flags from the device index planes n[3][Ny][Nx] (double).
+cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, int nfam, int fam0, double delta,
+                                 int precision, int interleaved, int unitary, cudaStream_t st);
+
 // Coefficients (Eq. 24-25) from the device index planes n[3][Ny][Nx] (double).
 cudaError_t launch_coefficients(const double *n, void *coef, int Nx, int Ny, double delta,
                                 int precision, int interleaved, int unitary, cudaStream_t st);
@@ -303,8 +341,11 @@ cudaError_t launch_pack_weights(const float *w, int nout, int cin, int nout_pad,
 
 // One operator of the step (qla_debug_apply), in place on `state` or, for a
 // streaming op, from `state` into `spare` (*swapped set).
-cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, int Nx, int Ny, int unitary,
-                        cudaStream_t st, bool *swapped);
+// The coefficients are the pair planes `coef`, or (geo not null) the marching
+// records of families fam0 .. fam0 + nfam - 1 (a family without records is zero
+// and stays so).
+cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, const MarchGeo *geo,
+                        int nfam, int fam0, int Nx, int Ny, int unitary, cudaStream_t st, bool *swapped);
 
 }  // namespace qla
 

@@ -1,0 +1,674 @@
+// Marching form of the fused sweep: K full QLA time steps per HBM pass with
+// the state held in registers.
+//
+// The operators of a step (Eq. 18, 20, 22, 23, 28) and their per-site
+// arithmetic are those of qla_sweep.cuh (rot, vop_pair; families as there), in
+// the same order, so both forms give the same values. What differs is where a
+// row lives between its operators:
+//  * A warp owns a strip of 32 C columns (C consecutive columns per lane) and
+//    marches down its rows alone. The x operators of a row act on the lane's C
+//    registers (shifts are register renames plus one warp shuffle); the y
+//    operators follow on the same registers, each y-shift a saved register per
+//    column, the output trailing the input by 4 rows. The K time levels are
+//    chained in the warp: level j's output row is level j+1's input row one
+//    iteration later (one row of lag, so that the levels of an iteration do not
+//    depend on each other and their operations interleave). No state passes
+//    through shared memory and no block barrier is needed.
+//  * The strip carries a halo of at least 4K columns on each side; the columns
+//    between are written. A share of rows [y0, y1) is fed from y0 - 4K.
+//  * FP32 arithmetic is packed: two adjacent columns per fma.rn.f32x2 (the
+//    same roundings as two scalar FMAs). Measured on GB300 with independent
+//    rotations in registers: 28 T FMA/s scalar, 36 packed, in half the issue
+//    slots.
+//  * Input rows (three state planes and the collision coefficients of level 0)
+//    are copied by cp.async into a ring of D rows private to the warp, D - 1
+//    rows ahead; the collision coefficients of the later levels, which the L2
+//    still holds, one row ahead. Every lane copies exactly what it reads.
+//  * V_X' and V_Y' are the identity where their angles vanish. A flag per strip
+//    and row (march_flags, computed with the coefficients) says whether any
+//    angle is nonzero in the rows that a group of iterations starting there
+//    applies; groups without one neither load the V planes nor apply them.
+// Coefficients lie in records, one per strip and row: MARCH_FIELDS rows of the
+// strip's 32 C columns (halo included), periodic rows repeated above and below,
+// so that every coefficient copy of an iteration, whatever its level and lag, is
+// one address register plus a constant, aligned for any Nx.
+// Measured on GB300 against the shared-memory sweep (us per step, both
+// families, three-cylinder-like media): 8192^2 874 -> 538 (124.7 G site-updates/s,
+// 5.6 TB/s of HBM traffic), 4096^2 240 -> 155, 2048^2 83 -> 52, 1024^2 43.6 ->
+// 21.7, 256^2 29 -> 10. That sweep was bound by instruction issue (half of its
+// instructions index and control work) and its two block barriers per row
+// block; this one by the fixed latencies of its chains with the 8 warps per SM
+// that 255 registers leave (two steps; issue slots 47% busy, FMA pipe 38%) and,
+// on the largest lattices, by HBM. On the way there (8192^2): one body per family
+// and with and without potentials, scalar FMAs 925 us (instruction cache); one
+// body for both families 731; packed FMAs 628; planes by 32-bit offsets 591.
+#pragma once
+
+#include "qla_sweep.cuh"
+
+namespace qla {
+
+constexpr int MARCH_LAG = 1;    // rows between a level's output and the next level's input
+
+// Iterations of a share before its first output row leaves: level j works on
+// row F0 + it - (4 + MARCH_LAG) j in iteration it, F0 = y0 - 4K.
+constexpr int march_delay(int K) { return 8 * K + MARCH_LAG * (K - 1); }
+static_assert(march_flag_back(2) >= (4 + MARCH_LAG) + 4, "V rows of a group");
+
+// A family's planes and what distinguishes the families at run time (one code
+// serves both, so that the warps of an SM share its instruction cache whatever
+// their family). The TE hub is carried with its sign flipped, which turns the
+// orientations of all of its operators into the TM ones (IEEE arithmetic is
+// symmetric under it, so the values are unchanged); what remains is which
+// member the printed potential rows write.
+struct MarchFam {
+    const char *h, *px, *py;        // input planes
+    const char *rec;                // coefficient records
+    char *oh, *opx, *opy;           // output planes
+    const unsigned char *flags;     // [strips][Ny]
+    int te;
+};
+
+struct MarchArgs {
+    MarchFam fam[2];  // the advanced families, in grid order
+    int Nx, Ny;
+    int w_valid, halo, strips;  // strip geometry (MarchGeo)
+    int chunks;                 // row ranges per strip, one warp each
+    int ctas_fam;               // CTAs per family
+};
+
+template <typename T, int C, int K, int D, bool INTER>
+struct MarchLayout {
+    static_assert(D == 2 || D == 3, "copy groups in flight");
+    static constexpr int W = 32 * C;
+    static constexpr int RB = W * int(sizeof(T));  // one row of a plane
+    static constexpr int REC = 7 * RB;             // a level-0 row: h, x-partner, y-partner, C_X (2), C_Y (2)
+    static constexpr int CREC = 4 * RB;            // a later level's C_X, C_Y
+    static constexpr int VYS = INTER ? 4 : 2;      // rows of V_Y kept (Eq. 28 applies it at lags 2 and 4)
+    static constexpr int VREC = (2 + VYS) * 2 * RB;  // per level: V_X (two rows), V_Y
+    static constexpr int C_OFF = D * REC;
+    static constexpr int V_OFF = C_OFF + (K - 1) * 2 * CREC;
+    static constexpr int WARP = V_OFF + K * VREC;
+};
+
+// ---- vectors of a lane's columns --------------------------------------------
+// FP32: packed pairs; FP64: scalars. NV vectors hold the lane's C columns.
+struct F32x2 {
+    unsigned long long v;
+};
+template <typename T>
+struct MarchVec;
+template <>
+struct MarchVec<float> {
+    using V = F32x2;
+    static constexpr int N = 2;
+    static __device__ __forceinline__ V pack(float a, float b) {
+        V r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+        return r;
+    }
+    static __device__ __forceinline__ void unpack(V v, float &a, float &b) {
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v.v));
+    }
+    static __device__ __forceinline__ V neg(V a) {
+        float x, y;
+        unpack(a, x, y);
+        return pack(-x, -y);
+    }
+    static __device__ __forceinline__ V fma(V a, V b, V c) {
+        V r;
+        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+        return r;
+    }
+    static __device__ __forceinline__ V mul(V a, V b) {
+        V r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+        return r;
+    }
+    static __device__ __forceinline__ V add(V a, V b) {
+        V r;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+        return r;
+    }
+    static __device__ __forceinline__ V zero() { return V{0ull}; }
+    static __device__ __forceinline__ V flip(V a, unsigned mask) {
+        return V{a.v ^ ((unsigned long long)(mask) << 32 | mask)};
+    }
+};
+template <>
+struct MarchVec<double> {
+    using V = double;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ V neg(V a) { return -a; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return __fma_rn(a, b, c); }
+    static __device__ __forceinline__ V mul(V a, V b) { return __dmul_rn(a, b); }
+    static __device__ __forceinline__ V add(V a, V b) { return __dadd_rn(a, b); }
+    static __device__ __forceinline__ V zero() { return 0.0; }
+    static __device__ __forceinline__ V flip(V a, unsigned mask) {
+        return __hiloint2double(__double2hiint(a) ^ int(mask), __double2loint(a));
+    }
+};
+
+// rot and vop_pair of qla_sweep.cuh on vectors.
+template <bool DAG, int SG, bool SHEAR, typename T, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_rot(V &h, V &p, V m, V s) {
+    using A = MarchVec<T>;
+    constexpr bool pos = (SG > 0) != DAG;
+    if constexpr (SHEAR) {
+        h = A::fma(pos ? m : A::neg(m), p, h);
+        p = A::fma(pos ? A::neg(s) : s, h, p);
+        h = A::fma(pos ? m : A::neg(m), p, h);
+    } else {
+        const V sp = A::mul(s, p);
+        const V sh = A::mul(s, h);
+        const V u = A::fma(m, h, pos ? sp : A::neg(sp));
+        const V v = A::fma(m, p, pos ? A::neg(sh) : sh);
+        h = A::add(h, u);
+        p = A::add(p, v);
+    }
+}
+template <int TAU, bool HUB, bool UNIT, typename T, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_vop(V &h, V &p, V s, V c) {
+    using A = MarchVec<T>;
+    V &t = HUB ? h : p;
+    V &src = HUB ? p : h;
+    const V ss = A::mul(s, src);
+    const V t2 = A::add(t, A::fma(c, t, TAU > 0 ? ss : A::neg(ss)));
+    if (UNIT) {
+        const V st = A::mul(s, t);
+        src = A::add(src, A::fma(c, src, TAU > 0 ? A::neg(st) : st));
+    }
+    t = t2;
+}
+
+// a(x) <- a(x-1), a(x) <- a(x+1) across the warp's 32 C columns
+template <typename T, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_from_left(V (&a)[NV]) {
+    if constexpr (MarchVec<T>::N == 2) {
+        float x[NV], y[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(a[k], x[k], y[k]);
+        const float e = __shfl_up_sync(0xffffffffu, y[NV - 1], 1);
+        a[0] = MarchVec<T>::pack(e, x[0]);
+#pragma unroll
+        for (int k = 1; k < NV; ++k) a[k] = MarchVec<T>::pack(y[k - 1], x[k]);
+    } else {
+        const V e = __shfl_up_sync(0xffffffffu, a[NV - 1], 1);
+#pragma unroll
+        for (int k = NV - 1; k > 0; --k) a[k] = a[k - 1];
+        a[0] = e;
+    }
+}
+template <typename T, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_from_right(V (&a)[NV]) {
+    if constexpr (MarchVec<T>::N == 2) {
+        float x[NV], y[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(a[k], x[k], y[k]);
+        const float e = __shfl_down_sync(0xffffffffu, x[0], 1);
+#pragma unroll
+        for (int k = 0; k + 1 < NV; ++k) a[k] = MarchVec<T>::pack(y[k], x[k + 1]);
+        a[NV - 1] = MarchVec<T>::pack(y[NV - 1], e);
+    } else {
+        const V e = __shfl_down_sync(0xffffffffu, a[0], 1);
+#pragma unroll
+        for (int k = 0; k + 1 < NV; ++k) a[k] = a[k + 1];
+        a[NV - 1] = e;
+    }
+}
+
+// The lane's NV vectors of a staged row (p: its first byte), and their store.
+template <typename T, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_lds(V (&v)[NV], const unsigned char *p) {
+    if constexpr (sizeof(V) * NV == 16) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(p);
+        memcpy(&v[0], &a.x, 8);
+        memcpy(&v[1], &a.y, 8);
+    } else {
+        static_assert(sizeof(V) * NV == 8, "8 or 16 bytes per lane");
+        v[0] = *reinterpret_cast<const V *>(p);
+    }
+}
+template <typename T, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_stg(T *dst, const V (&v)[NV]) {
+    if constexpr (sizeof(V) * NV == 16) {
+        ulonglong2 a;
+        memcpy(&a.x, &v[0], 8);
+        memcpy(&a.y, &v[1], 8);
+        *reinterpret_cast<ulonglong2 *>(dst) = a;
+    } else {
+        *reinterpret_cast<V *>(dst) = v[0];
+    }
+}
+template <typename T, int C, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_stg_some(T *dst, const V (&v)[NV], const bool (&ok)[C]) {
+    T x[C];
+    if constexpr (MarchVec<T>::N == 2) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(v[k], x[2 * k], x[2 * k + 1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < C; ++k) x[k] = v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < C; ++k)
+        if (ok[k]) dst[k] = x[k];
+}
+
+template <int BYTES>
+__device__ __forceinline__ void march_cp(unsigned dst, const void *src) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
+}
+
+// One time level's y pipeline: a saved value per y-shift, the collision
+// coefficients of the last three rows and the x-partner's last four rows.
+template <typename V, int NV>
+struct MarchPipe {
+    V S[8][NV];
+    V m[3][NV], s[3][NV];
+    V d[4][NV];
+};
+
+static_assert(Fam<1>::SGX == -Fam<0>::SGX && Fam<1>::SGY == -Fam<0>::SGY && Fam<1>::TX == -Fam<0>::TX &&
+                  Fam<1>::TY == -Fam<0>::TY,
+              "a sign flip of the hub maps the TE orientations to the TM ones");
+static_assert(!Fam<0>::VX_HUB && !Fam<0>::VY_HUB && Fam<1>::VX_HUB && Fam<1>::VY_HUB, "potential targets");
+
+// V' on the lane's columns of all levels (ld loads level j's coefficients).
+template <int TAU, bool UNIT, typename T, int K, int NV, typename V, class LD>
+__device__ __forceinline__ void march_v(bool te, V (&h)[K][NV], V (&p)[K][NV], LD &&ld) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        V m[NV], s[NV];
+        ld(j, m, s);
+        if (te) {
+#pragma unroll
+            for (int c = 0; c < NV; ++c) march_vop<TAU, true, UNIT, T>(h[j][c], p[j][c], s[c], m[c]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NV; ++c) march_vop<TAU, false, UNIT, T>(h[j][c], p[j][c], s[c], m[c]);
+        }
+    }
+}
+
+// One row of every level: level j's h, p (y-partner), px (x-partner) enter as
+// row R_j of its input and leave as row R_j - 4 of its output. vx, vy2, vy4
+// load the V coefficients (V_X of row R, or of R - 4 with Eq. 23; V_Y of rows
+// R - 2 and R - 4).
+template <bool INTER, bool UNIT, typename T, int K, int NV, typename V, class VX, class VY2, class VY4>
+__device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][NV], V (&p)[K][NV], V (&px)[K][NV],
+                                           const V (&cxm)[K][NV], const V (&cxs)[K][NV], const V (&cym)[K][NV],
+                                           const V (&cys)[K][NV], bool von, bool te, VX &&vx, VY2 &&vy2, VY4 &&vy4) {
+    using Fm = Fam<0>;
+    constexpr bool SHR = shear_collisions<T, UNIT>();
+    constexpr int SX = Fm::SGX, SY = Fm::SGY;
+#define MARCH_ALL(expr)               \
+    _Pragma("unroll") for (int j = 0; j < K; ++j) { expr; }
+#define MARCH_ROT(DAG, SG, H, PP, M, S) \
+    _Pragma("unroll") for (int j = 0; j < K; ++j) _Pragma("unroll") for (int c = 0; c < NV; ++c) \
+        march_rot<DAG, SG, SHR, T>(H[j][c], PP[j][c], M[c], S[c]);
+#define MARCH_X(DAG) MARCH_ROT(DAG, SX, h, px, cxm[j], cxs[j])
+#define MARCH_Y(DAG, M, S) MARCH_ROT(DAG, SY, h, p, M, S)
+    MARCH_X(true)
+    MARCH_ALL((march_from_left<T, NV>(px[j])))
+    MARCH_X(false)
+    MARCH_ALL((march_from_right<T, NV>(px[j])))
+    MARCH_X(true)
+    MARCH_ALL((march_from_right<T, NV>(h[j])))
+    MARCH_X(false)
+    MARCH_ALL((march_from_left<T, NV>(h[j])))
+    if constexpr (INTER) {
+        if (von) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);
+    }
+    MARCH_X(false)
+    MARCH_ALL((march_from_right<T, NV>(px[j])))
+    MARCH_X(true)
+    MARCH_ALL((march_from_left<T, NV>(px[j])))
+    MARCH_X(false)
+    MARCH_ALL((march_from_left<T, NV>(h[j])))
+    MARCH_X(true)
+    MARCH_ALL((march_from_right<T, NV>(h[j])))
+    if constexpr (INTER) {
+        if (von) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);
+    }
+    auto swap = [&](V (&a)[NV], V (&b)[NV]) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+            const V t = a[c];
+            a[c] = b[c];
+            b[c] = t;
+        }
+    };
+    MARCH_Y(true, cym[j], cys[j])         // C+   (row R)
+    MARCH_ALL(swap(Y[j].S[0], p[j]))      // p <- p(r-1)
+    MARCH_Y(false, cym[j], cys[j])        // C    (row R)
+    MARCH_ALL(swap(Y[j].S[1], h[j]))      // p <- p(r+1): now row R-1
+    MARCH_Y(true, Y[j].m[0], Y[j].s[0])   // C+   (row R-1)
+    MARCH_ALL(swap(Y[j].S[2], p[j]))      // h <- h(r+1): now row R-2
+    MARCH_Y(false, Y[j].m[1], Y[j].s[1])  // C    (row R-2)
+    MARCH_ALL(swap(Y[j].S[3], h[j]))      // h <- h(r-1)
+    if constexpr (INTER) {
+        if (von) march_v<Fm::TY, UNIT, T, K, NV, V>(te, h, p, vy2);  // V_Y' (row R-2)
+    }
+    MARCH_Y(false, Y[j].m[1], Y[j].s[1])  // C    (row R-2)
+    MARCH_ALL(swap(Y[j].S[4], h[j]))      // p <- p(r+1): now row R-3
+    MARCH_Y(true, Y[j].m[2], Y[j].s[2])   // C+   (row R-3)
+    MARCH_ALL(swap(Y[j].S[5], p[j]))      // p <- p(r-1)
+    MARCH_Y(false, Y[j].m[2], Y[j].s[2])  // C    (row R-3)
+    MARCH_ALL(swap(Y[j].S[6], h[j]))      // h <- h(r-1)
+    MARCH_Y(true, Y[j].m[2], Y[j].s[2])   // C+   (row R-3)
+    MARCH_ALL(swap(Y[j].S[7], p[j]))      // h <- h(r+1): now row R-4
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+            const V t = Y[j].d[3][c];  // the x-partner's row R-4
+            Y[j].d[3][c] = Y[j].d[2][c];
+            Y[j].d[2][c] = Y[j].d[1][c];
+            Y[j].d[1][c] = Y[j].d[0][c];
+            Y[j].d[0][c] = px[j][c];
+            px[j][c] = t;
+            Y[j].m[2][c] = Y[j].m[1][c];
+            Y[j].s[2][c] = Y[j].s[1][c];
+            Y[j].m[1][c] = Y[j].m[0][c];
+            Y[j].s[1][c] = Y[j].s[0][c];
+            Y[j].m[0][c] = cym[j][c];
+            Y[j].s[0][c] = cys[j][c];
+        }
+    if (von) {
+        if constexpr (!INTER) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);  // V_X (row R-4)
+        march_v<Fm::TY, UNIT, T, K, NV, V>(te, h, p, vy4);                        // V_Y (row R-4)
+    }
+#undef MARCH_ALL
+#undef MARCH_ROT
+#undef MARCH_X
+#undef MARCH_Y
+}
+
+// One warp's share: rows [y0, y1) of strip `strip` of a family. sm: the
+// warp's shared memory. VEC: rows and strips keep the alignment of the lane's
+// vectors (Nx a multiple of C); else the copies and stores go element by element.
+template <typename T, int C, int K, int D, int U, bool INTER, bool UNIT, bool VEC>
+__device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &F, int strip, int y0, int y1, unsigned char *sm,
+                                            int lane) {
+    using L = MarchLayout<T, C, K, D, INTER>;
+    using MV = MarchVec<T>;
+    using V = typename MV::V;
+    constexpr int NV = C / MV::N;
+    static_assert(NV * MV::N == C, "whole vectors");
+    constexpr int LB = C * int(sizeof(T));  // a lane's bytes of a row
+    constexpr int RB = L::RB;
+    const int Nx = A.Nx, Ny = A.Ny;
+    // Places in a plane as 32-bit byte offsets (a plane holds less than 2^32
+    // bytes, checked on the host) from plane addresses that lie in the
+    // kernel's parameters: an access then takes one address register and no
+    // 64-bit arithmetic.
+    const unsigned pitch = unsigned(Nx) * unsigned(sizeof(T)), plane_bytes = pitch * unsigned(Ny);
+    const bool te = F.te != 0;
+    const unsigned hsign = te ? 0x80000000u : 0u;
+    const int cy_off = te ? 2 * RB : 0;  // TM: C_X and C_Y are one plane
+
+    const int o_lo = strip * A.w_valid;
+    const int o_hi = min(o_lo + A.w_valid, Nx);
+    const int xbase = o_lo - A.halo;
+    constexpr int NGC = VEC ? 1 : C;  // global columns of the lane (VEC: of its first column)
+    unsigned gc[NGC];
+#pragma unroll
+    for (int k = 0; k < NGC; ++k) gc[k] = unsigned(wrapi(xbase + C * lane + k, Nx)) * unsigned(sizeof(T));
+    const unsigned sbase = tc::smem_addr(sm) + unsigned(lane) * LB;
+    sm += lane * LB;
+
+    const int F0 = y0 - 4 * K;
+    // ro: byte offset of the row (VEC: of the lane's first column in it)
+    auto row = [&](unsigned dst, const char *plane, unsigned ro) {
+        if constexpr (VEC) {
+            march_cp<LB>(dst, plane + ro);
+        } else {
+#pragma unroll
+            for (int k = 0; k < C; ++k) march_cp<sizeof(T)>(dst + k * unsigned(sizeof(T)), plane + (ro + gc[k]));
+        }
+    };
+    // coefficient copies: two fields (x, y) of the record `dr` rows from the
+    // level-0 row that cp points to
+    constexpr int RECB = MARCH_FIELDS * RB;
+    const char *cp = F.rec + (size_t(strip) * (MARCH_ABOVE + Ny + MARCH_BELOW) + size_t(MARCH_ABOVE + F0)) * RECB +
+                     lane * LB;
+    auto field2 = [&](unsigned dst, int dr, int field) {
+        march_cp<LB>(dst, cp + (dr * RECB + field * RB));
+        march_cp<LB>(dst + RB, cp + (dr * RECB + (field + 1) * RB));
+    };
+    auto copy0 = [&](unsigned slot_off, unsigned ro, int dr) {
+        const unsigned b = sbase + slot_off;
+        row(b, F.h, ro);
+        row(b + RB, F.px, ro);
+        row(b + 2 * RB, F.py, ro);
+        field2(b + 3 * RB, dr, F_CX);
+        if (te) field2(b + 5 * RB, dr, F_CY);
+    };
+    auto copyc = [&](int j, int slot, int dr) {
+        const unsigned b = sbase + L::C_OFF + ((j - 1) * 2 + slot) * L::CREC;
+        field2(b, dr, F_CX);
+        if (te) field2(b + 2 * RB, dr, F_CY);
+    };
+    // V rows that level j applies in iteration i (dr: its level row from cp)
+    auto copyv = [&](int j, int i, int dr) {
+        const unsigned b = sbase + L::V_OFF + j * L::VREC;
+        if constexpr (INTER) {
+            field2(b + (i & 1) * 2 * RB, dr, F_VX);
+            field2(b + (2 + ((i + 2) & 3)) * 2 * RB, dr - 2, F_VY);
+        } else {
+            field2(b + (i & 1) * 2 * RB, dr - 4, F_VX);
+            field2(b + (2 + (i & 1)) * 2 * RB, dr - 4, F_VY);
+        }
+    };
+
+    MarchPipe<V, NV> pipe[K];
+    V hh[K][NV], hp[K][NV], hx[K][NV];  // the rows entering each level (level 0: from the ring)
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) pipe[j].S[k][c] = MV::zero();
+#pragma unroll
+            for (int k = 0; k < 3; ++k) pipe[j].m[k][c] = pipe[j].s[k][c] = MV::zero();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) pipe[j].d[k][c] = MV::zero();
+            hh[j][c] = hp[j][c] = hx[j][c] = MV::zero();
+        }
+
+    const unsigned char *const flags = F.flags + size_t(strip) * Ny;
+    const int nit = y1 - y0 + march_delay(K);
+    const int ngroups = (nit + U - 1) / U;
+    int rg = wrapi(F0, Ny);  // wrapped level-0 row of the group's first iteration
+    auto step_row = [&](int &r, unsigned &off) {  // next row, wrapped (r counts up to 0 at the wrap)
+        off += pitch;
+        if (++r == 0) {
+            r = -Ny;
+            off -= plane_bytes;
+        }
+    };
+    // prologue: level-0 rows F0 .. F0 + D - 2, the later levels' first collision rows, the first V rows
+    unsigned von = flags[rg], von1 = flags[wrapi(rg + U, Ny)], von2 = flags[wrapi(rg + 2 * U, Ny)];
+    int row_c = rg - Ny;  // level-0 copies
+    unsigned off_c = unsigned(rg) * pitch + (VEC ? gc[0] : 0u);
+#pragma unroll
+    for (int j = 1; j < K; ++j) copyc(j, 0, -(4 + MARCH_LAG) * j);
+    if (von)
+        for (int j = 0; j < K; ++j) copyv(j, 0, -(4 + MARCH_LAG) * j);
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k) {
+        copy0(k * L::REC, off_c, k);
+        step_row(row_c, off_c);
+        cp_async_commit();
+    }
+    unsigned rd_off = 0, wr_off = (D - 1) * L::REC;
+
+    // output: row y0 + it - march_delay(K)
+    bool ok[NGC];
+#pragma unroll
+    for (int k = 0; k < NGC; ++k) {
+        const int c = C * lane + k;
+        ok[k] = c >= A.halo && xbase + c < o_hi;
+    }
+    const int n_out = y1 - y0;
+    // (offsets of rows and columns that are not written wrap around harmlessly)
+    unsigned out_off = unsigned(y0 - march_delay(K)) * pitch + unsigned((xbase + C * lane) * int(sizeof(T)));
+
+    for (int g = 0, it0 = 0; g < ngroups; ++g, it0 += U) {
+        const unsigned von3 = flags[wrap_down(rg + 3 * U, Ny)];  // read three groups ahead
+        // V_Y rows are copied up to four iterations before their last use
+        const bool on = von != 0, vcopy = (von | von1 | (U < 4 ? von2 : 0u)) != 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = U == 4 ? u : it0 + u;  // iteration index mod 4 (compile time when U = 4)
+            // all copies but the newest level-0 row's have landed (a lane reads only what it copied)
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 2) : "memory");
+#pragma unroll
+            for (int j = 1; j < K; ++j) copyc(j, (i + 1) & 1, 1 - (4 + MARCH_LAG) * j);
+            if (vcopy) {
+#pragma unroll
+                for (int j = 0; j < K; ++j) copyv(j, i + 1, 1 - (4 + MARCH_LAG) * j);
+            }
+            if constexpr (D > 2) cp_async_commit();
+            copy0(wr_off, off_c, D - 1);
+            step_row(row_c, off_c);
+            cp_async_commit();
+            cp += RECB;
+            wr_off = wr_off == (D - 1) * L::REC ? 0u : wr_off + L::REC;
+
+            V cxm[K][NV], cxs[K][NV], cym[K][NV], cys[K][NV];
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+                const unsigned char *cb = sm + L::C_OFF + ((j - 1) * 2 + (i & 1)) * L::CREC;
+                if (j == 0) {
+                    const unsigned char *rec = sm + rd_off;
+                    march_lds<T, NV>(hh[0], rec);
+                    march_lds<T, NV>(hx[0], rec + RB);
+                    march_lds<T, NV>(hp[0], rec + 2 * RB);
+#pragma unroll
+                    for (int c = 0; c < NV; ++c) hh[0][c] = MV::flip(hh[0][c], hsign);
+                    cb = rec + 3 * RB;
+                }
+                march_lds<T, NV>(cxm[j], cb);
+                march_lds<T, NV>(cxs[j], cb + RB);
+                march_lds<T, NV>(cym[j], cb + cy_off);
+                march_lds<T, NV>(cys[j], cb + cy_off + RB);
+            }
+            rd_off = rd_off == (D - 1) * L::REC ? 0u : rd_off + L::REC;
+            auto vrow = [&](int slot) {
+                return [&, slot](int j, V(&m)[NV], V(&s)[NV]) {
+                    const unsigned char *vb = sm + L::V_OFF + j * L::VREC + slot * 2 * RB;
+                    march_lds<T, NV>(m, vb);
+                    march_lds<T, NV>(s, vb + RB);
+                };
+            };
+            march_rows<INTER, UNIT, T, K, NV, V>(pipe, hh, hp, hx, cxm, cxs, cym, cys, on, te, vrow(i & 1),
+                                                 vrow(2 + ((i + 2) & 3)), vrow(INTER ? 2 + (i & 3) : 2 + (i & 1)));
+            const int ro = it0 + u - march_delay(K);
+            if (ro >= 0 && ro < n_out) {
+                V h[NV];
+#pragma unroll
+                for (int c = 0; c < NV; ++c) h[c] = MV::flip(hh[K - 1][c], hsign);
+                T *const oh = reinterpret_cast<T *>(F.oh + out_off), *const ox = reinterpret_cast<T *>(F.opx + out_off),
+                         *const oy = reinterpret_cast<T *>(F.opy + out_off);
+                if constexpr (VEC) {
+                    if (ok[0]) {
+                        march_stg<T, NV>(oh, h);
+                        march_stg<T, NV>(ox, hx[K - 1]);
+                        march_stg<T, NV>(oy, hp[K - 1]);
+                    }
+                } else {
+                    march_stg_some<T, C, NV>(oh, h, ok);
+                    march_stg_some<T, C, NV>(ox, hx[K - 1], ok);
+                    march_stg_some<T, C, NV>(oy, hp[K - 1], ok);
+                }
+            }
+            out_off += pitch;
+#pragma unroll
+            for (int j = K - 1; j > 0; --j)
+#pragma unroll
+                for (int c = 0; c < NV; ++c) {
+                    hh[j][c] = hh[j - 1][c];
+                    hp[j][c] = hp[j - 1][c];
+                    hx[j][c] = hx[j - 1][c];
+                }
+        }
+        von = von1;
+        von1 = von2;
+        von2 = von3;
+        rg = wrap_down(rg + U, Ny);
+    }
+    cp_async_wait_all();
+}
+
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, bool UNIT, bool VEC>
+__global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_constant__ MarchArgs A) {
+    using L = MarchLayout<T, C, K, D, INTER>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0);
+    const int layer = int(blockIdx.x) >= A.ctas_fam ? 1 : 0;
+    const int w = (int(blockIdx.x) - layer * A.ctas_fam) * WPC + warp;
+    if (w >= A.strips * A.chunks) return;
+    const int strip = w % A.strips, chunk = w / A.strips;
+    const int y0 = int((long long)A.Ny * chunk / A.chunks);
+    const int y1 = int((long long)A.Ny * (chunk + 1) / A.chunks);
+    march_share<T, C, K, D, U, INTER, UNIT, VEC>(A, A.fam[layer], strip, y0, y1, smem_raw + warp * L::WARP, lane);
+}
+
+// Host: a family's entry (fam: 0 = TM, 1 = TE).
+template <typename T>
+MarchFam march_fam(const void *q_in, void *q_out, const void *rec, const unsigned char *flags, int fam, int Nx,
+                          int Ny) {
+    const size_t PB = size_t(Nx) * Ny * sizeof(T);
+    const char *q = static_cast<const char *>(q_in);
+    char *o = static_cast<char *>(q_out);
+    MarchFam f;
+    const bool te = fam != 0;
+    const int h = te ? Fam<1>::H : Fam<0>::H, px = te ? Fam<1>::PX : Fam<0>::PX, py = te ? Fam<1>::PY : Fam<0>::PY;
+    f.h = q + h * PB;
+    f.px = q + px * PB;
+    f.py = q + py * PB;
+    f.oh = o + h * PB;
+    f.opx = o + px * PB;
+    f.opy = o + py * PB;
+    f.rec = static_cast<const char *>(rec);
+    f.flags = flags;
+    f.te = te ? 1 : 0;
+    return f;
+}
+
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, bool UNIT, bool VEC>
+cudaError_t launch_march_t(const MarchArgs &a, int nfam, cudaStream_t st) {
+    using L = MarchLayout<T, C, K, D, INTER>;
+    auto kern = march_kernel<T, C, K, D, U, WPC, MINB, INTER, UNIT, VEC>;
+    // set on every launch: the attribute belongs to the device, a process may use several
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::WARP * WPC);
+    if (e != cudaSuccess) return e;
+    MarchArgs m = a;
+    m.ctas_fam = (a.strips * a.chunks + WPC - 1) / WPC;
+    kern<<<unsigned(m.ctas_fam) * unsigned(nfam), 32 * WPC, L::WARP * WPC, st>>>(m);
+    return cudaGetLastError();
+}
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool VEC>
+cudaError_t launch_march_modes(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st) {
+    if (interleaved)
+        return unitary ? launch_march_t<T, C, K, D, U, WPC, MINB, true, true, VEC>(a, nfam, st)
+                       : launch_march_t<T, C, K, D, U, WPC, MINB, true, false, VEC>(a, nfam, st);
+    return unitary ? launch_march_t<T, C, K, D, U, WPC, MINB, false, true, VEC>(a, nfam, st)
+                   : launch_march_t<T, C, K, D, U, WPC, MINB, false, false, VEC>(a, nfam, st);
+}
+
+// The instantiated forms, one translation unit each (qla_march_*.cu).
+cudaError_t launch_march_f32_k1(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f32_k2(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f32_k2_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f64_k1(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f64_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+
+}  // namespace qla

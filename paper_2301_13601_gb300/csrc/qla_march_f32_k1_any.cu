@@ -1,0 +1,8 @@
+// Marching sweep, FP32, one step per pass: 12 warps per SM (168 registers); rows of any length (element copies).
+#include "qla_march.cuh"
+
+namespace qla {
+cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st) {
+    return launch_march_modes<float, 4, 1, 2, 2, 4, 3, false>(a, nfam, interleaved, unitary, st);
+}
+}  // namespace qla

@@ -1,0 +1,8 @@
+// Marching sweep, FP32, two steps per pass: 8 warps per SM (255 registers); rows of any length (element copies).
+#include "qla_march.cuh"
+
+namespace qla {
+cudaError_t launch_march_f32_k2_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st) {
+    return launch_march_modes<float, 4, 2, 3, 4, 4, 2, false>(a, nfam, interleaved, unitary, st);
+}
+}  // namespace qla
