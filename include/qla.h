@@ -128,9 +128,10 @@ typedef struct {
  * delta: the perturbation parameter (Eq. 24-25), 0 < delta <= 0.5.
  * The collision angles theta_i = delta/(4 n_i) (Eq. 24) and potential angles
  * beta from central differences of n (Eq. 25, lattice spacing delta) are
- * computed once on the device in FP64 and stored as (cos-1, sin) pairs in the
- * state precision; in FP32 each rotation pair is rounded so that
- * (1 + m)^2 + s^2 is as close to 1 as FP32 allows.
+ * computed once on the device in FP64 and stored as pairs in the state
+ * precision: (tan(a/2), sin a) of a rotation, (cos b - 1, sin b) of a printed
+ * potential row; in FP32 the rotation pairs are rounded so that the operator
+ * keeps the norm as closely as FP32 allows.
  * buffers: NULL = the library allocates with cudaMalloc and frees on destroy.
  * The state is zero after creation. Errors: QLA_EINVAL (n <= 0, non-finite n or
  * delta, bad sizes), QLA_ENOMEM, QLA_ECUDA. On error *out is NULL. */

@@ -166,8 +166,15 @@ bool family_has(const qla_ctx *c, int comp) {
 
 qla_status launch_pass(qla_ctx *c, int K) {
     if (c->march) {
-        // K = 4 (and FP64's K = 2) as passes of two steps (of one): the same values, in less time
-        const int per = std::min(K, c->opt.precision == QLA_FP64 ? 1 : 2);
+        // K = 4 in passes of two steps; FP64 and, without an explicit choice,
+        // small FP32 lattices in passes of one: the same values in less time (us
+        // per step with one and two steps per pass, three contexts in turn / one
+        // alone: 256^2 4.1/10.3 and 4.8/13.4, 512^2 6.2/12.3 and 7.1/15.0, 1024^2
+        // 18.5/26.6 and 13.7/24.9; FP64, bound by its pipe, pays two steps'
+        // halos once more)
+        const bool one = c->opt.precision == QLA_FP64 ||
+                         (c->opt.steps_per_pass == 0 && (long long)c->Nx * c->Ny <= (1LL << 19));
+        const int per = std::min(K, one ? 1 : 2);
         for (int k = 0; k < K; k += per) {
             const cudaError_t e = qla::launch_march(
                 c->geo, per, c->state[c->cur], c->state[c->cur ^ 1], c->coef, c->nfam, c->fam0,

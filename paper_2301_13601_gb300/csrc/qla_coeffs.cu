@@ -19,64 +19,55 @@ __device__ void shear_pair_f32(double ang, float &tf, float &sf) {
     sf = (float)(2.0 * t / (1.0 + t * t));
 }
 
-// FP32 (cos(a) - 1, sin(a)) pair chosen among FP32 values within a few ulps of
-// the correctly rounded ones so that (1 + m)^2 + s^2 - 1 (evaluated exactly in
-// FP64: every term is a product of two FP32 values) is as small as possible:
-// each rotation then keeps the energy (Eq. 27) to ~1e-13, with the angle
-// changed by a few ulps of m and s at most.
-__device__ void tuned_pair_f32(double ang, float &mf, float &sf) {
-    const double sh = sin(0.5 * ang);
-    const double m = -2.0 * sh * sh;  // cos(ang) - 1 without cancellation
-    const double s = sin(ang);
-    const float m0 = (float)m, s0 = (float)s;
-    if (!(fabsf(m0) >= 1e-30f) || !(fabsf(s0) >= 1e-30f)) {  // zero or denormal: keep the rounded values
-        mf = m0;
+// FP32 pair (t, s) near (tan(a / 2), sin(a)) for the four-FMA rotation of the
+// sweep, whose matrix is [1 - s t, s; -s, 1 - s t]: among FP32 values within a
+// few ulps of the correctly rounded ones, the pair that brings
+// (1 - s t)^2 + s^2 - 1 = s (s (1 + t^2) - 2 t) (evaluated in FP64) closest to
+// zero, so that each rotation keeps the energy (Eq. 27) to ~1e-12, with the
+// angle changed by a few ulps at most.
+__device__ void tuned_pair_f32(double ang, float &tf, float &sf) {
+    const float t0 = (float)tan(0.5 * ang), s0 = (float)sin(ang);
+    if (!(fabsf(t0) >= 1e-30f) || !(fabsf(s0) >= 1e-30f)) {  // zero or denormal: keep the rounded values
+        tf = t0;
         sf = s0;
         return;
     }
-    const int mi = __float_as_int(m0), si = __float_as_int(s0);
+    // for each t the best s is the FP32 value nearest to 2 t / (1 + t^2)
     double best = 1e300;
-    int bdm = 0, bds = 0;
-    for (int dm = -4; dm <= 4; ++dm) {
-        const float mc = __int_as_float(mi + dm);
-        for (int ds = -2; ds <= 2; ++ds) {
-            const float sc = __int_as_float(si + ds);
-            const double dmc = (double)mc, dsc = (double)sc;
-            const double e = fabs(2.0 * dmc + dmc * dmc + dsc * dsc);
-            const int cost = abs(dm) + abs(ds);
-            if (e < best || (e == best && cost < abs(bdm) + abs(bds))) {
-                best = e;
-                bdm = dm;
-                bds = ds;
-            }
+    tf = t0;
+    sf = s0;
+    for (int k = 0; k <= 8; ++k) {
+        const int dt = (k + 1) / 2 * (k & 1 ? 1 : -1);  // 0, 1, -1, .. 4, -4: the nearest of equals stays
+        const float tc = __int_as_float(__float_as_int(t0) + dt);
+        const double t = (double)tc, q = 1.0 + t * t;
+        const float sc = (float)(2.0 * t / q);
+        const double s = (double)sc;
+        const double e = fabs(s * (s * q - 2.0 * t));
+        if (e < best) {
+            best = e;
+            tf = tc;
+            sf = sc;
         }
     }
-    mf = __int_as_float(mi + bdm);
-    sf = __int_as_float(si + bds);
 }
 
 // How a pair is stored (see CoefPair and rot in the sweep): a collision of the
-// three-shear form (FP32 with the printed potentials: (tan(a/2), sin a)), a
-// rotation of the (cos - 1, sin) form (FP32: tuned for orthogonality) or a
-// printed potential row (cos a - 1, sin a). FP64 stores (cos a - 1, sin a)
-// for all.
+// three-shear form (FP32 with the printed potentials), a rotation of the
+// four-FMA form (FP32: tuned for orthogonality), both (tan(a/2), sin a), or a
+// printed potential row (cos a - 1, sin a).
 enum PairKind { PK_SHEAR, PK_ROTATION, PK_PRINTED_V };
 
 template <typename T>
 __device__ void make_pair_of(double ang, PairKind kind, T &x, T &y) {
-    if constexpr (sizeof(T) == 4) {
-        if (kind == PK_SHEAR) {
-            shear_pair_f32(ang, x, y);
-        } else if (kind == PK_ROTATION) {
-            tuned_pair_f32(ang, x, y);
-        } else {
-            const double sh = sin(0.5 * ang);
-            x = (float)(-2.0 * sh * sh);
-            y = (float)sin(ang);
-        }
-    } else {
+    if (kind == PK_PRINTED_V) {
         const double sh = sin(0.5 * ang);
-        x = -2.0 * sh * sh;
+        x = (T)(-2.0 * sh * sh);  // cos(ang) - 1 without cancellation
+        y = (T)sin(ang);
+    } else if constexpr (sizeof(T) == 4) {
+        if (kind == PK_SHEAR) shear_pair_f32(ang, x, y);
+        else tuned_pair_f32(ang, x, y);
+    } else {
+        x = tan(0.5 * ang);
         y = sin(ang);
     }
 }

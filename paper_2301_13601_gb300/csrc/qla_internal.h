@@ -12,11 +12,11 @@ namespace qla {
 // state precision. The angle a is a collision angle (Eq. 24) or an effective
 // potential angle b (Eq. 25, scaled by 1/2 when interleaved (Eq. 28) and by
 // 1/2 again for the unitary potentials).
-// A collision pair is (x = tan(a/2), y = sin(a)) in FP32 with the printed
-// potentials (three-shear form) and (x = cos(a) - 1, y = sin(a)) otherwise; a
-// potential pair is (cos(b) - 1, sin(b)). FP32 pairs of the (cos - 1, sin)
-// form that are rotations (collisions and the unitary potentials) are tuned
-// for orthogonality. Signs of the operators are applied by the kernels.
+// A collision pair, and a potential pair of the unitary potentials, is
+// (x = tan(a/2), y = sin(a)); a printed potential pair is (cos(b) - 1, sin(b)).
+// FP32 pairs of the three-shear collisions (printed potentials) take y nearest
+// to 2x / (1 + x^2), the others are tuned for orthogonality. Signs of the
+// operators are applied by the kernels.
 // The order puts the two planes that the sweep copies together next to each
 // other: (V_X, C_X) for the x-pass and (C_Y, V_Y) for the y-pass of a family.
 enum CoefPair {

@@ -24,25 +24,44 @@ size_t march_bytes(const MarchGeo &g, int nfam) { return size_t(nfam) * (g.recor
 
 namespace {
 
-// Row ranges per strip. One warp each, `slots` resident at a time over the
-// families together. A single wave ends with its slowest warp (the rows whose
-// V angles are nonzero cost more, measured up to a quarter over the mean);
-// several waves even that out at the price of march_delay(K) more rows per
-// share. FP32, two steps, GB300 (us per step): 8192^2 8 row ranges (one wave)
-// 739, 16 678, 32 628, 64 639; 4096^2 16 (one wave) 160, 32 155, 64 165.
-int march_chunks(const MarchGeo &g, int nfam, int delay, int slots) {
-    const double strips = double(g.strips) * nfam;
+// Row ranges per strip (one warp each). An iteration of a warp takes `lat`
+// alone on its scheduler and `busy` of the scheduler's time (us, measured on
+// GB300: FP32 from runs at 256^2 to 8192^2, FP64 from its pipe, which takes a
+// warp instruction in 64 cycles). A pass alone on the GPU lasts as long as its
+// most loaded SM; with others it costs the scheduler time it uses. Few ranges
+// leave schedulers idle, many pay the march_delay(K) iterations before a
+// range's first output row once more each: the sum of the two is minimised.
+// CTAs of four warps load an SM's four schedulers evenly. A pass of one wave
+// ends with its slowest warp (rows with nonzero V angles cost more): 1.35 times
+// the mean at worst; more waves even out. us per step, three contexts in turn /
+// one alone: 256^2 rows 1, 4, 16: 7.1/12.3, 4.1/10.3, 6.0/16.4; 2048^2 rows 32,
+// 64, 128: 49.7/59.9, 39.8/52.0, 36.3/64.6; 8192^2 rows 128, 256, 1024:
+// 532/565, 501/552, 483/620; FP64 256^2 rows 2, 8, 16: 150/221, 78/129, 64/192.
+struct MarchCost {
+    int resident;  // CTAs per SM
+    double lat, busy;
+};
+constexpr MarchCost kMarchCost[3] = {{3, 5.2, 5.2}, {3, 0.55, 0.32}, {2, 0.89, 0.62}};  // FP64, FP32 K = 1, K = 2
+constexpr double kLaunchUs = 3.0;
+
+int march_chunks(const MarchGeo &g, int nfam, int K, int sms) {
+    const MarchCost m = kMarchCost[g.es == 8 ? 0 : K];
     int best = 1;
     double cost = 1e300;
     for (int n = 1; n <= g.Ny; ++n) {
-        const double share = double((g.Ny + n - 1) / n + delay);
-        const double waves = strips * n / slots;
-        const double c = waves <= 1.0 ? 1.25 * share : waves * share + 0.6 * share;
+        const double its = double((g.Ny + n - 1) / n + march_delay(K));
+        const long long ctas = (long long)nfam * (((long long)g.strips * n + 3) / 4);
+        const long long per_sm = (ctas + sms - 1) / sms;
+        const double busy = double(g.strips) * nfam * n * its * m.busy / (4.0 * sms);
+        const double alone = per_sm <= m.resident
+                                 ? 1.35 * its * (m.lat > per_sm * m.busy ? m.lat : per_sm * m.busy)
+                                 : busy + 0.6 * its * m.resident * m.busy;
+        const double c = kLaunchUs + alone + busy;
         if (c < cost) {
             cost = c;
             best = n;
         }
-        if (waves > 32.0) break;
+        if (per_sm > 32LL * m.resident) break;
     }
     return best;
 }
@@ -51,8 +70,7 @@ int march_chunks(const MarchGeo &g, int nfam, int delay, int slots) {
 
 void march_plan(MarchGeo *g, int nfam, int chunk, int sms) {
     for (int K = 1; K <= 2; ++K)
-        g->chunks[K] = chunk > 0 ? (g->Ny + chunk - 1) / chunk
-                                 : march_chunks(*g, nfam, march_delay(K), sms * (K == 2 ? 8 : 12));
+        g->chunks[K] = chunk > 0 ? (g->Ny + chunk - 1) / chunk : march_chunks(*g, nfam, K, sms);
     g->chunks[0] = 0;
 }
 

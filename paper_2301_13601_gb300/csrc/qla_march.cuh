@@ -159,12 +159,10 @@ __device__ __forceinline__ void march_rot(V &h, V &p, V m, V s) {
         p = A::fma(pos ? A::neg(s) : s, h, p);
         h = A::fma(pos ? m : A::neg(m), p, h);
     } else {
-        const V sp = A::mul(s, p);
-        const V sh = A::mul(s, h);
-        const V u = A::fma(m, h, pos ? sp : A::neg(sp));
-        const V v = A::fma(m, p, pos ? A::neg(sh) : sh);
-        h = A::add(h, u);
-        p = A::add(p, v);
+        const V u = A::fma(pos ? A::neg(m) : m, h, p);
+        const V v = A::fma(pos ? m : A::neg(m), p, h);
+        h = A::fma(pos ? s : A::neg(s), u, h);
+        p = A::fma(pos ? A::neg(s) : s, v, p);
     }
 }
 template <int TAU, bool HUB, bool UNIT, typename T, typename V = typename MarchVec<T>::V>
@@ -172,13 +170,12 @@ __device__ __forceinline__ void march_vop(V &h, V &p, V s, V c) {
     using A = MarchVec<T>;
     V &t = HUB ? h : p;
     V &src = HUB ? p : h;
-    const V ss = A::mul(s, src);
-    const V t2 = A::add(t, A::fma(c, t, TAU > 0 ? ss : A::neg(ss)));
-    if (UNIT) {
-        const V st = A::mul(s, t);
-        src = A::add(src, A::fma(c, src, TAU > 0 ? A::neg(st) : st));
+    if constexpr (UNIT) {
+        march_rot<false, TAU, false, T>(t, src, c, s);
+    } else {
+        const V ss = A::mul(s, src);
+        t = A::add(t, A::fma(c, t, TAU > 0 ? ss : A::neg(ss)));
     }
-    t = t2;
 }
 
 // a(x) <- a(x-1), a(x) <- a(x+1) across the warp's 32 C columns

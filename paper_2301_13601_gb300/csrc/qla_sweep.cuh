@@ -35,10 +35,10 @@
 //    not used.)
 //  * In FP32 with the printed potentials a collision is three shears
 //    (h += t p, p -= s h, h += t p with t = tan(theta/2): three FMAs, the
-//    determinant exactly 1); otherwise the (cos-1, sin) form
-//    h' = h + (m h + s p), one rounding at the scale of each output, with FP32
-//    pairs tuned at creation for orthogonality. Coefficients are stored as
-//    pairs of the form the kernel uses (see rot).
+//    determinant exactly 1); otherwise each output is its input plus sin(theta)
+//    times a combination formed first, one rounding at the scale of the output,
+//    with FP32 pairs tuned at creation for orthogonality. Coefficients are stored
+//    as pairs of the form the kernel uses (see rot).
 #pragma once
 
 #include <cuda.h>
@@ -167,9 +167,13 @@ struct Fam<1> {
 // Collision C (DAG = false) or its transpose (DAG = true) on (h, p) with
 // orientation SG: the rotation h' = c h + SG s p, p' = -SG s h + c p by the
 // angle theta (c = cos theta, s = sin theta).
-//  * SHEAR = false: pair (m, s) with m = cos(theta) - 1:
-//      h' = h + (m h + SG s p),   p' = p + (m p - SG s h)
-//    (one rounding at the scale of each output; six instructions).
+//  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t,
+//    so
+//      h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p)
+//    (four FMAs; one rounding at the scale of each output, those of the inner
+//    combinations enter scaled by s). The form h' = h + (m h + s p) with m =
+//    cos theta - 1 took six operations for the same errors: FP64 256^2, whose
+//    pipe is the bound, 64 -> 43 us per step.
 //  * SHEAR = true (FP32 with the printed potentials): pair (t, s) with
 //    t = tan(theta / 2), as three shears
 //      h1 = h + SG t p,  p' = p - SG s h1,  h' = h1 + SG t p'
@@ -189,17 +193,16 @@ __device__ __forceinline__ void rot(T &h, T &p, T m, T s) {
         p = pos ? A::fma(-s, h, p) : A::fma(s, h, p);
         h = pos ? A::fma(t, p, h) : A::fma(-t, p, h);
     } else {
-        const T sp = A::mul(s, p);
-        const T sh = A::mul(s, h);
-        const T u = pos ? A::fma(m, h, sp) : A::fma(m, h, -sp);
-        const T v = pos ? A::fma(m, p, -sh) : A::fma(m, p, sh);
-        h = A::add(h, u);
-        p = A::add(p, v);
+        const T t = m;
+        const T u = A::fma(pos ? -t : t, h, p);
+        const T v = A::fma(pos ? t : -t, p, h);
+        h = A::fma(pos ? s : -s, u, h);
+        p = A::fma(pos ? -s : s, v, p);
     }
 }
 
 // Collision form of a configuration: three shears in FP32 with the printed
-// potentials; the (cos - 1, sin) form in FP64, and in FP32 with the unitary
+// potentials; the four-FMA form in FP64, and in FP32 with the unitary
 // potentials, where every operator is an exact rotation and the tuned pairs
 // keep the energy (Eq. 27) to FP32 rounding over 1e4 steps.
 template <typename T, bool UNIT>
@@ -207,18 +210,18 @@ constexpr bool shear_collisions() {
     return std::is_same<T, float>::value && !UNIT;
 }
 
-// Potential row: target' = target + (c target + TAU s source), c = cos(b) - 1,
-// s = sin(b); the unitary variant also rotates the source:
-// source' = source + (c source - TAU s target).
+// Potential row as printed: target' = target + (c target + TAU s source),
+// c = cos(b) - 1, s = sin(b). The unitary variant rotates the pair (target,
+// source) by b with orientation TAU (rot, pair (tan(b / 2), sin(b))).
 template <int TAU, bool UNIT, typename T>
 __device__ __forceinline__ void vop(T &target, T &source, T s, T c) {
     using A = Ar<T>;
+    if constexpr (UNIT) {
+        rot<false, TAU, false>(target, source, c, s);
+        return;
+    }
     const T ss = A::mul(s, source);
     const T t2 = A::add(target, TAU > 0 ? A::fma(c, target, ss) : A::fma(c, target, -ss));
-    if (UNIT) {
-        const T st = A::mul(s, target);
-        source = A::add(source, TAU > 0 ? A::fma(c, source, -st) : A::fma(c, source, st));
-    }
     target = t2;
 }
 
