@@ -351,7 +351,7 @@ void qla_destroy(qla_ctx *ctx);
  * periodic lattice, medium, delta and pulse, Sec. 4 setting) advanced by one
  * persistent kernel launch that is captured once into a CUDA graph and
  * replayed by every qla_batch_run. The kernel takes work items
- * (instance, pass of steps_per_pass fused steps, family, tile) from a queue
+ * (instance, pass of two fused steps, family, tile) from a queue
  * ordered by pass; before a pass it waits, with a time limit, for the
  * previous pass of the same lattice to complete. FP32 only.
  * ------------------------------------------------------------------------- */
@@ -364,7 +364,7 @@ typedef struct {
     long long nsteps;                /* steps per qla_batch_run; a multiple of steps_per_pass */
     int pulse_polarization;          /* QLA_POL_EZ or QLA_POL_EY: initial pulse as qla_init_pulse; -1: zero state */
     double pulse_x0, pulse_sigma, pulse_amplitude;
-    int chunk_rows;                  /* rows per tile; 0 = automatic */
+    int chunk_rows;                  /* rows swept by one warp of a strip; 0 = automatic */
 } qla_instance_desc;
 
 /* Create a batch of `count` lattices (descs copied; the host arrays are only
@@ -376,9 +376,8 @@ typedef struct {
 qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla_options *opt, qla_batch **out);
 
 /* Advance every lattice by its nsteps (one graph launch; blocks until done).
- * QLA_ETIMEOUT if a dependency wait or a tile's wait for its TMA copies
- * exceeded its limit (the states are then partially advanced and should be
- * discarded). */
+ * QLA_ETIMEOUT if a dependency wait exceeded its limit (the states are then
+ * partially advanced and should be discarded). */
 qla_status qla_batch_run(qla_batch *b);
 
 /* State of lattice i (creation order) as a host float array [6][Ny][Nx]. */

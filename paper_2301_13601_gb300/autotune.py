@@ -124,7 +124,7 @@ def tune_single(n_x, n_y, n_z, delta: float, precision: str = "fp32", sequence: 
     return entry
 
 
-def tune_batch(instances: List[dict], ks: Sequence[int] = (2, 4), chunks: Sequence[int] = (256, 512, 768, 1024),
+def tune_batch(instances: List[dict], ks: Sequence[int] = (2, 4), chunks: Sequence[int] = (0, 32, 64, 128, 256),
                step_scale: int = 8, use_cache: bool = True, sequence: str = "interleaved",
                potential: str = "paper") -> dict:
     """Pick steps per pass and one rows-per-tile value for a batch by timing a

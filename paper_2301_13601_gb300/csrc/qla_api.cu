@@ -145,11 +145,14 @@ bool persistent_applies(const qla_ctx *c) {
            c->ctas[c->K] <= qla::kPersistMaxCtas;
 }
 
-// Whether the marching form serves a context: every lattice whose planes it can
-// address, unless the persistent launch form (on the shared-memory sweep and
-// its pair planes) was asked for and applies.
+// Whether the marching form serves a context: unless the persistent launch form
+// (on the shared-memory sweep and its pair planes) was asked for and applies,
+// every lattice but a tall one much narrower than a strip, whose records (a
+// whole strip wide) would take many times the memory of the pair planes.
 bool march_applies(const qla_options &o, int Nx, int Ny, qla::MarchGeo *g) {
-    if (!qla::march_geometry(o.precision == QLA_FP64 ? 1 : 0, Nx, Ny, g) || g->strips > 65535) return false;
+    if (!qla::march_geometry(o.precision == QLA_FP64 ? 1 : 0, Nx, Ny, g)) return false;
+    const size_t pairs = size_t(qla::NCOEF) * size_t(Nx) * Ny * g->es;
+    if (qla::march_bytes(*g, 2) > std::max(size_t(1) << 30, 4 * pairs)) return false;
     const int K = o.steps_per_pass > 0 ? o.steps_per_pass
                                        : default_steps_per_pass(o.precision, Nx, Ny, o.chunk_rows);
     return !(o.launch == QLA_LAUNCH_PERSISTENT && o.precision == QLA_FP32 && o.chunk_rows == 0 &&

@@ -1,15 +1,20 @@
 // Batched QLA: many independent lattices (of uneven sizes) advanced by one
 // persistent kernel, replayed as a CUDA graph.
 //
-// Work items are (instance, pass, family, tile) with a tile one strip x chunk
-// of one family (see qla_sweep.cuh). Items are numbered pass-major: every item
-// of pass p precedes every item of pass p + 1, so a CTA that takes an item of
-// pass p + 1 can rely on all items of pass p having been taken by running
-// CTAs, which never wait on later passes: the queue cannot deadlock. Before
-// starting an item of pass p > 0 a CTA waits until all tiles of pass p - 1 of
-// the same (instance, family) are complete (a counter per pair, incremented
-// after a fence). The wait is bounded by a time limit after which the kernel
-// records QLA_ETIMEOUT, stops taking items and returns.
+// Work items are (instance, pass of two steps, family, tile) with a tile the
+// shares of four warps of the marching sweep (qla_march.cuh). Items are numbered
+// pass-major: every item of pass p precedes every item of pass p + 1, so a CTA
+// that takes an item of pass p + 1 can rely on all items of pass p having been
+// taken by running CTAs, which never wait on later passes: the queue cannot
+// deadlock. Before starting an item of pass p > 0 a CTA waits until all tiles
+// of pass p - 1 of the same (instance, family) are complete (a counter per pair,
+// incremented after a fence). The wait is bounded by a time limit after which
+// the kernel records QLA_ETIMEOUT, stops taking items and returns.
+//
+// A lattice offers only its own tiles until its pass completes, so the tiles
+// are low enough for the batch together to fill the GPU (batch_rows). Ten lattices
+// of sides 256 to 1024, 400 steps: 110 ms with tiles of up to 768 rows of the
+// shared-memory sweep (15 G site-updates/s, most SMs idle), 21 ms now (78 G).
 #include <math.h>
 #include <string.h>
 
@@ -19,27 +24,21 @@
 #include <vector>
 
 #include "../../include/qla.h"
-#include "qla_sweep.cuh"
+#include "qla_march.cuh"
 
 namespace qla {
 
 struct BatchInst {
-    void *q[2];
-    const void *coef;
-    int Nx, Ny, w_valid, chunk, nsx, ncy, tiles, passes, vec;
-    int tma, merged;  // tensor maps encoded (see BatchMaps); merged-level coefficient map encoded
-    int seam;         // the seam strip layout (SweepArgs::seam)
-};
-
-// TMA tensor maps of one instance (as SweepParams, for both state buffers),
-// kept in device memory and read by the TMA unit from there.
-struct BatchMaps {
-    SweepMaps m[2];  // per state buffer holding the input
+    char *q[2];
+    const char *rec[2];             // per family
+    const unsigned char *flags[2];
+    int Nx, Ny, w_valid, halo, strips, chunks;
+    int tiles;                      // per pass and family
+    int passes;                     // of kBatchSteps steps
 };
 
 struct BatchSched {
     const BatchInst *inst;           // sorted by passes, descending
-    const BatchMaps *maps;           // [ninst], same order
     int ninst;
     int maxpass;
     const long long *pass_start;     // [maxpass + 1]
@@ -53,104 +52,101 @@ struct BatchSched {
     unsigned int withhold;           // test hook: extra completions a dependency waits for (0 normally)
 };
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
-__global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, NY>::MINB)
-    batch_kernel(const BatchSched S) {
+// The marching configuration of the batch: two steps per pass.
+constexpr int kBatchSteps = 2;
+constexpr int BC = 4, BD = 3, BU = 4, BWPC = 4, BMINB = 2;
+
+// Largest k in [0, n) with a[k] <= v (a ascending, a[0] <= v): 32 candidates
+// per round, one dependent load each, by a whole warp.
+__device__ __forceinline__ int warp_search(const long long *a, int n, long long v, int lane) {
+    int lo = 0;
+    while (n > 1) {
+        const int step = (n + 31) / 32;
+        const int k = lane * step;
+        const bool le = k < n && a[lo + k] <= v;
+        const int last = 31 - __clz(int(__ballot_sync(0xffffffffu, le) | 1u));
+        lo += last * step;
+        n = min(step, n - last * step);
+    }
+    return lo;
+}
+
+template <bool INTER, bool UNIT, bool VEC>
+__global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSched S) {
+    using L = MarchLayout<float, BC, kBatchSteps, BD, INTER>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // stop, instance, pass, family, strip, chunk: after the sweep's layout in
-    // the dynamic allocation (a static array would shift the 1024-byte aligned
-    // dynamic base by a whole kilobyte)
-    using L = SweepLayout<T, K, R, INTER>;
-    int *const sh = reinterpret_cast<int *>(smem_raw + L::SMEM);
+    __shared__ MarchArgs args;  // the item's lattice and family (entry 0)
+    __shared__ int item[4];     // stop, instance, family, tile
+    const int lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0);
     for (;;) {
-        if (threadIdx.x == 0) {
-            int stop = 0, inst = 0, pass = 0, fam = 0, tile = 0;
-            const unsigned long long g = atomicAdd(S.next, 1ull);
-            const unsigned long long total = (unsigned long long)S.pass_start[S.maxpass];
-            if (g >= total || *(volatile int *)S.error) {
-                stop = 1;
-            } else {
-                int lo = 0, hi = S.maxpass;
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if ((unsigned long long)S.pass_start[mid] <= g) lo = mid;
-                    else hi = mid;
-                }
-                pass = lo;
+        if (warp == 0) {
+            unsigned long long g = 0;
+            if (lane == 0) g = atomicAdd(S.next, 1ull);
+            g = __shfl_sync(0xffffffffu, g, 0);
+            int stop = g >= (unsigned long long)S.pass_start[S.maxpass] || *(volatile int *)S.error ? 1 : 0;
+            int inst = 0, fam = 0, tile = 0;
+            if (!stop) {
+                const int pass = warp_search(S.pass_start, S.maxpass, (long long)g, lane);
                 const long long r = (long long)g - S.pass_start[pass];
-                lo = 0;
-                hi = S.active_count[pass];
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (S.tile_prefix[mid] <= r) lo = mid;
-                    else hi = mid;
-                }
-                inst = lo;
+                inst = warp_search(S.tile_prefix, S.active_count[pass], r, lane);
+                const BatchInst &I = S.inst[inst];
                 const int rr = int(r - S.tile_prefix[inst]);
-                const int tiles = S.inst[inst].tiles;
+                const int tiles = I.tiles;
                 fam = rr / tiles;
                 tile = rr % tiles;
-                if (pass > 0) {
-                    const unsigned int target = (unsigned int)pass * (unsigned int)tiles + S.withhold;
-                    const unsigned long long t0 = global_ns();
-                    while (ld_acquire_u32(&S.done[2 * inst + fam]) < target) {
-                        if (*(volatile int *)S.error) {  // another CTA gave up: stop as well
-                            stop = 1;
-                            break;
+                if (lane == 0) {
+                    const int par = (S.cur[inst] + pass) & 1;
+                    args.fam[0] = march_fam<float>(I.q[par], I.q[par ^ 1], I.rec[fam], I.flags[fam], fam, I.Nx, I.Ny);
+                    args.Nx = I.Nx;
+                    args.Ny = I.Ny;
+                    args.w_valid = I.w_valid;
+                    args.halo = I.halo;
+                    args.strips = I.strips;
+                    args.chunks = I.chunks;
+                    if (pass > 0) {
+                        const unsigned int target = (unsigned int)pass * (unsigned int)tiles + S.withhold;
+                        const unsigned long long t0 = global_ns();
+                        while (int(ld_acquire_u32(&S.done[2 * inst + fam]) - target) < 0) {
+                            if (*(volatile int *)S.error) {  // another CTA gave up: stop as well
+                                stop = 1;
+                                break;
+                            }
+                            if ((long long)(global_ns() - t0) > S.timeout_ns) {
+                                atomicExch(S.error, 1);
+                                stop = 1;
+                                break;
+                            }
+                            __nanosleep(64);
                         }
-                        if ((long long)(global_ns() - t0) > S.timeout_ns) {
-                            atomicExch(S.error, 1);
-                            stop = 1;
-                            break;
-                        }
-                        __nanosleep(256);
                     }
                 }
+                stop = __shfl_sync(0xffffffffu, stop, 0);
             }
-            sh[0] = stop;
-            sh[1] = inst;
-            sh[2] = pass;
-            sh[3] = fam;
-            sh[4] = tile % S.inst[inst].nsx;
-            sh[5] = tile / S.inst[inst].nsx;
+            if (lane == 0) {
+                item[0] = stop;
+                item[1] = inst;
+                item[2] = fam;
+                item[3] = tile;
+            }
         }
         __syncthreads();
-        if (sh[0]) break;
-        const int inst = sh[1], pass = sh[2], fam = sh[3], strip = sh[4], chunk = sh[5];
-        const BatchInst &I = S.inst[inst];
-        const int par = (S.cur[inst] + pass) & 1;
-        SweepArgs a;
-        a.q_in = I.q[par];
-        a.q_out = I.q[par ^ 1];
-        a.coef = I.coef;
-        a.Nx = I.Nx;
-        a.Ny = I.Ny;
-        a.w_valid = I.w_valid;
-        a.chunk = I.chunk;
-        a.ctas = 0;
-        a.seam = I.seam;
-        a.interleaved = INTER ? 1 : 0;
-        a.unitary = UNIT ? 1 : 0;
-        a.vec = I.vec;
-        a.fam0 = 0;
-        a.error = S.error;  // a TMA wait that runs out stops the batch like a dependency timeout
-        const BatchMaps *M = I.tma ? &S.maps[inst] : nullptr;
-        // the input rows were written by other CTAs (generic proxy) and are
-        // read here by TMA loads (async proxy)
-        asm volatile("fence.proxy.async;\n" ::: "memory");
-        const int yb = chunk * I.chunk, ye = min(yb + I.chunk, I.Ny);
-        const bool failed =
-            fam == 0 ? sweep_body<T, K, R, NY, INTER, UNIT, 0>(a, strip, yb, ye, smem_raw, M ? &M->m[par] : nullptr,
-                                                               I.merged != 0)
-                     : sweep_body<T, K, R, NY, INTER, UNIT, 1>(a, strip, yb, ye, smem_raw, M ? &M->m[par] : nullptr,
-                                                               I.merged != 0);
-        if (failed) break;  // the error flag is set: every CTA stops at its next work item
+        if (item[0]) break;
+        const int w = item[3] * BWPC + warp;
+        if (w < args.strips * args.chunks) {
+            const int strip = w % args.strips, chunk = w / args.strips;
+            const int y0 = int((long long)args.Ny * chunk / args.chunks);
+            const int y1 = int((long long)args.Ny * (chunk + 1) / args.chunks);
+            march_share<float, BC, kBatchSteps, BD, BU, INTER, UNIT, VEC>(args, args.fam[0], strip, y0, y1,
+                                                                           smem_raw + warp * L::WARP, lane);
+        }
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
-            atomicAdd(&S.done[2 * inst + fam], 1u);
+            atomicAdd(&S.done[2 * item[1] + item[2]], 1u);
         }
+        __syncthreads();  // the item's words are read before the next item overwrites them
     }
 }
 
@@ -160,55 +156,35 @@ __global__ void batch_flip(const BatchInst *inst, int *cur, int n) {
     if (i < n) cur[i] ^= (inst[i].passes & 1);
 }
 
-constexpr int kBatchRows = 4;  // rows per iteration of the batch's sweep configurations (K = 2 and 4)
-
-// dynamic shared memory of the batch kernel: the sweep's layout + 6 scheduler words
-template <int K, int R, bool INTER>
-constexpr size_t batch_smem() {
-    return SweepLayout<float, K, R, INTER>::SMEM + 32;
-}
-
-// Sets the shared-memory attribute and returns the persistent grid size
-// (SMs x resident CTAs); called before stream capture.
-template <int K, int R, int NY, bool INTER, bool UNIT>
-cudaError_t prepare_batch_t(int sms, int *grid) {
-    using Cfg = SweepCfg<float, K, R, NY>;
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel<float, K, R, NY, INTER, UNIT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(batch_smem<K, R, INTER>()));
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, batch_kernel<float, K, R, NY, INTER, UNIT>, Cfg::NT,
-                                                      batch_smem<K, R, INTER>());
-    if (e != cudaSuccess) return e;
-    *grid = sms * (occ < 1 ? 1 : occ);
-    return cudaSuccess;
-}
-
-template <int K, int R, int NY, bool INTER, bool UNIT>
-cudaError_t launch_batch_t(const BatchSched &S, int grid, cudaStream_t st) {
-    using Cfg = SweepCfg<float, K, R, NY>;
-    batch_kernel<float, K, R, NY, INTER, UNIT><<<grid, Cfg::NT, batch_smem<K, R, INTER>(), st>>>(S);
+// Sets the shared-memory attribute and returns the persistent grid size (SMs x
+// resident CTAs); called before stream capture. With S: launches *grid CTAs.
+template <bool INTER, bool UNIT, bool VEC>
+cudaError_t batch_t(int sms, int *grid, const BatchSched *S, cudaStream_t st) {
+    using L = MarchLayout<float, BC, kBatchSteps, BD, INTER>;
+    constexpr int smem = L::WARP * BWPC;
+    auto kern = batch_kernel<INTER, UNIT, VEC>;
+    if (S == nullptr) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        int occ = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * BWPC, smem);
+        if (e != cudaSuccess) return e;
+        *grid = sms * (occ < 1 ? 1 : occ);
+        return cudaSuccess;
+    }
+    kern<<<*grid, 32 * BWPC, smem, st>>>(*S);
     return cudaGetLastError();
 }
 
-// mode dispatch: op(integral constants) for the four (interleaved, unitary) variants
-template <int K, int R, int NY>
-cudaError_t batch_modes(bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
-    if (S == nullptr) {
-        if (inter) return unit ? prepare_batch_t<K, R, NY, true, true>(sms, grid) : prepare_batch_t<K, R, NY, true, false>(sms, grid);
-        return unit ? prepare_batch_t<K, R, NY, false, true>(sms, grid) : prepare_batch_t<K, R, NY, false, false>(sms, grid);
-    }
-    if (inter) return unit ? launch_batch_t<K, R, NY, true, true>(*S, *grid, st) : launch_batch_t<K, R, NY, true, false>(*S, *grid, st);
-    return unit ? launch_batch_t<K, R, NY, false, true>(*S, *grid, st) : launch_batch_t<K, R, NY, false, false>(*S, *grid, st);
-}
-
 // S == nullptr: prepare (attribute + grid size); otherwise launch with *grid CTAs.
-cudaError_t batch_dispatch(int K, bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
-    switch (K) {
-        case 2: return batch_modes<2, kBatchRows, 2>(inter, unit, sms, grid, S, st);
-        case 4: return batch_modes<4, kBatchRows, 2>(inter, unit, sms, grid, S, st);
-        default: return cudaErrorInvalidValue;
-    }
+// vec: every lattice's rows copy in vectors (march_vectors).
+template <bool VEC>
+cudaError_t batch_modes(bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
+    if (inter) return unit ? batch_t<true, true, VEC>(sms, grid, S, st) : batch_t<true, false, VEC>(sms, grid, S, st);
+    return unit ? batch_t<false, true, VEC>(sms, grid, S, st) : batch_t<false, false, VEC>(sms, grid, S, st);
+}
+cudaError_t batch_dispatch(bool vec, bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
+    return vec ? batch_modes<true>(inter, unit, sms, grid, S, st) : batch_modes<false>(inter, unit, sms, grid, S, st);
 }
 
 }  // namespace qla
@@ -222,7 +198,7 @@ struct qla_batch {
     int K = 4;
     int dev = 0;
     int sms = 152;
-    bool inter = true, unit = false;
+    bool inter = true, unit = false, vec = true;
     cudaStream_t stream = nullptr;
     std::vector<qla::BatchInst> inst;  // sorted order
     std::vector<int> order;            // order[k] = user index of sorted instance k
@@ -230,7 +206,6 @@ struct qla_batch {
     std::vector<int> cur;              // host copy of the parities
     std::vector<void *> allocs;
     qla::BatchInst *d_inst = nullptr;
-    qla::BatchMaps *d_maps = nullptr;
     long long *d_pass_start = nullptr;
     int *d_active = nullptr;
     long long *d_tile_prefix = nullptr;
@@ -264,12 +239,16 @@ cudaError_t dalloc(qla_batch *b, P **p, size_t bytes) {
     return e;
 }
 
-// Rows per tile in the batch. Measured on the 64-lattice workload (sides
-// 256-2048, 4 steps per pass), site-updates/s: 512 rows 52.5 G, 768 and 1024
-// rows 53.3 G, 2048 rows 50.1 G.
-int auto_batch_chunk(int Ny) {
-    int ch = std::min(Ny, 768);
-    return std::max(1, ch);
+// Rows per share of the lattices that set none: as many as let the batch's
+// warps fill the GPU's slots (8 per SM) a little more than once (a lattice's
+// pass ends with its last tile; more, lower shares pay the march_delay(2) = 17
+// warm-up rows more often), and at least 8. Ten lattices of sides 256 to 1024,
+// 400 steps: 16 rows 34.8 ms, 28 (filled twice) 23.9, 48 21.2, 64 22.2, 96 28.5;
+// the three largest of them: 15 rows 16.5 ms, 32 14.1, 64 20.4.
+int batch_rows(const std::vector<qla::MarchGeo> &geo, int sms) {
+    double units = 0.0;
+    for (const qla::MarchGeo &g : geo) units += 2.0 * g.strips * g.Ny;
+    return std::max(8, int(units / (1.15 * 8.0 * sms) + 0.5));
 }
 
 }  // namespace
@@ -323,34 +302,47 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     for (int k = 0; k < count; ++k) b->slot[b->order[k]] = k;
     b->inst.resize(count);
     b->cur.assign(count, 0);
-    const int W = qla::sweep_strip_width();
     size_t scratch_max = 0;
+    std::vector<qla::MarchGeo> geo(count);
+    for (int k = 0; k < count; ++k) {
+        const qla_instance_desc &d = descs[b->order[k]];
+        if (!qla::march_geometry(0, d.Nx, d.Ny, &geo[k])) return bail(QLA_EUNSUPPORTED);
+        b->vec = b->vec && qla::march_vectors(geo[k]);
+    }
+    const int rows = batch_rows(geo, b->sms);
     for (int k = 0; k < count; ++k) {
         const qla_instance_desc &d = descs[b->order[k]];
         qla::BatchInst &I = b->inst[k];
+        const qla::MarchGeo &g = geo[k];
         const size_t P = size_t(d.Nx) * d.Ny;
         I.Nx = d.Nx;
         I.Ny = d.Ny;
-        I.w_valid = W - 8 * K;
-        I.chunk = d.chunk_rows > 0 ? std::min(d.chunk_rows, d.Ny) : auto_batch_chunk(d.Ny);
-        I.ncy = (d.Ny + I.chunk - 1) / I.chunk;
-        I.passes = int(d.nsteps / K);
-        I.vec = 1;
-        float *q0, *q1, *coef;
+        I.w_valid = g.w_valid;
+        I.halo = g.halo;
+        I.strips = g.strips;
+        const int ch = std::min(d.chunk_rows > 0 ? d.chunk_rows : rows, d.Ny);
+        I.chunks = (d.Ny + ch - 1) / ch;
+        I.tiles = (I.strips * I.chunks + qla::BWPC - 1) / qla::BWPC;
+        I.passes = int(d.nsteps / qla::kBatchSteps);
+        float *q0, *q1;
+        char *mem;
         double *idx;
         if (dalloc(b, &q0, 6 * P * 4) != cudaSuccess || dalloc(b, &q1, 6 * P * 4) != cudaSuccess ||
-            dalloc(b, &coef, size_t(qla::NCOEF) * P * 4) != cudaSuccess || dalloc(b, &idx, 3 * P * 8) != cudaSuccess) {
+            dalloc(b, &mem, qla::march_bytes(g, 2)) != cudaSuccess || dalloc(b, &idx, 3 * P * 8) != cudaSuccess) {
             cudaGetLastError();
             return bail(QLA_ENOMEM);
         }
-        I.q[0] = q0;
-        I.q[1] = q1;
-        I.coef = coef;
+        I.q[0] = reinterpret_cast<char *>(q0);
+        I.q[1] = reinterpret_cast<char *>(q1);
+        for (int f = 0; f < 2; ++f) {
+            I.rec[f] = mem + f * g.record_bytes;
+            I.flags[f] = reinterpret_cast<const unsigned char *>(mem + 2 * g.record_bytes + f * g.flag_bytes);
+        }
         const double *nn[3] = {d.n_x, d.n_y, d.n_z};
         for (int c = 0; c < 3; ++c)
             if (cudaMemcpyAsync(idx + c * P, nn[c], P * 8, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
                 return bail(QLA_ECUDA);
-        if (qla::launch_coefficients(idx, coef, d.Nx, d.Ny, d.delta, 0, b->inter ? 1 : 0, b->unit ? 1 : 0, b->stream) !=
+        if (qla::launch_march_records(g, idx, mem, 2, 0, d.delta, 0, b->inter ? 1 : 0, b->unit ? 1 : 0, b->stream) !=
             cudaSuccess)
             return bail(QLA_ECUDA);
         if (cudaMemsetAsync(q0, 0, 6 * P * 4, b->stream) != cudaSuccess ||
@@ -368,36 +360,6 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         cudaFree(idx);
         b->allocs.pop_back();
     }
-    // TMA tensor maps of every instance (both state buffers) and its strips:
-    // the seam layout where TMA applies (every strip copies with TMA); an
-    // instance whose maps cannot be encoded copies with cp.async in the plain
-    // layout
-    std::vector<qla::BatchMaps> maps(count);
-    for (int k = 0; k < count; ++k) {
-        qla::BatchInst &I = b->inst[k];
-        I.seam = qla::make_sweep_split(I.Nx, I.Ny, K, qla::kBatchRows, 1).seam;
-        bool ok = true;
-        for (int par = 0; par < 2 && ok; ++par) {
-            qla::SweepArgs a;
-            memset(&a, 0, sizeof(a));
-            a.q_in = I.q[par];
-            a.coef = I.coef;
-            a.Nx = I.Nx;
-            a.Ny = I.Ny;
-            a.w_valid = I.w_valid;
-            a.chunk = I.chunk;
-            a.seam = I.seam;
-            int merged = 0;
-            memset(&maps[k].m[par], 0, sizeof(qla::SweepMaps));
-            ok = qla::make_sweep_maps(a, K, qla::kBatchRows, maps[k].m[par], &merged);
-            if (par == 0) I.merged = merged;
-        }
-        I.tma = ok ? 1 : 0;
-        const qla::SweepSplit sp = qla::make_sweep_split(I.Nx, I.Ny, K, qla::kBatchRows, I.tma);
-        I.seam = sp.seam;
-        I.nsx = sp.nsx;
-        I.tiles = I.nsx * I.ncy;
-    }
     // schedule tables
     b->maxpass = b->inst[0].passes;
     std::vector<long long> tile_prefix(count + 1, 0);
@@ -412,7 +374,6 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     }
     b->total_items = pass_start[b->maxpass];
     if (dalloc(b, &b->d_inst, sizeof(qla::BatchInst) * count) != cudaSuccess ||
-        dalloc(b, &b->d_maps, sizeof(qla::BatchMaps) * count) != cudaSuccess ||
         dalloc(b, &b->d_pass_start, sizeof(long long) * (b->maxpass + 1)) != cudaSuccess ||
         dalloc(b, &b->d_active, sizeof(int) * active.size()) != cudaSuccess ||
         dalloc(b, &b->d_tile_prefix, sizeof(long long) * (count + 1)) != cudaSuccess ||
@@ -424,7 +385,6 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     if (cudaMallocHost(reinterpret_cast<void **>(&b->h_diag), sizeof(qla::DiagResult)) != cudaSuccess)
         return bail(QLA_ENOMEM);
     if (cudaMemcpy(b->d_inst, b->inst.data(), sizeof(qla::BatchInst) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_maps, maps.data(), sizeof(qla::BatchMaps) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_pass_start, pass_start.data(), sizeof(long long) * pass_start.size(), cudaMemcpyHostToDevice) !=
             cudaSuccess ||
         cudaMemcpy(b->d_active, active.data(), sizeof(int) * active.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -432,7 +392,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(b->d_cur, 0, sizeof(int) * count) != cudaSuccess)
         return bail(QLA_ECUDA);
-    if (qla::batch_dispatch(b->K, b->inter, b->unit, b->sms, &b->grid, nullptr, nullptr) != cudaSuccess)
+    if (qla::batch_dispatch(b->vec, b->inter, b->unit, b->sms, &b->grid, nullptr, nullptr) != cudaSuccess)
         return bail(QLA_ECUDA);
     *out = b;
     return QLA_OK;
@@ -444,7 +404,6 @@ qla_status qla_batch_run(qla_batch *b) {
     if (!b->exec) {
         qla::BatchSched S;
         S.inst = b->d_inst;
-        S.maps = b->d_maps;
         S.ninst = b->n;
         S.maxpass = b->maxpass;
         S.pass_start = b->d_pass_start;
@@ -461,7 +420,7 @@ qla_status qla_batch_run(qla_batch *b) {
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned) * 2 * b->n, b->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_error, 0, 64, b->stream);
         if (e == cudaSuccess && b->maxpass > 0)
-            e = qla::batch_dispatch(b->K, b->inter, b->unit, b->sms, &b->grid, &S, b->stream);
+            e = qla::batch_dispatch(b->vec, b->inter, b->unit, b->sms, &b->grid, &S, b->stream);
         if (e == cudaSuccess) {
             qla::batch_flip<<<(b->n + 127) / 128, 128, 0, b->stream>>>(b->d_inst, b->d_cur, b->n);
             e = cudaGetLastError();
@@ -486,7 +445,7 @@ qla_status qla_batch_run(qla_batch *b) {
         return QLA_ECUDA;
     for (int k = 0; k < b->n; ++k) b->cur[k] ^= (b->inst[k].passes & 1);
     if (err) {
-        b->msg = "a dependency wait or a TMA copy wait timed out";
+        b->msg = "a dependency wait timed out";
         return QLA_ETIMEOUT;
     }
     return QLA_OK;
@@ -528,7 +487,7 @@ qla_status qla_batch_info(const qla_batch *b, long long *total_items, int *steps
     if (steps_per_pass) *steps_per_pass = b->K;
     if (site_updates) {
         long long s = 0;
-        for (const auto &I : b->inst) s += (long long)I.Nx * I.Ny * I.passes * b->K;
+        for (const auto &I : b->inst) s += (long long)I.Nx * I.Ny * I.passes * qla::kBatchSteps;
         *site_updates = s;
     }
     return QLA_OK;

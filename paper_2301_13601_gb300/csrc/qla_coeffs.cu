@@ -130,8 +130,8 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
     const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
     const PairKind ck = unitary ? PK_ROTATION : PK_SHEAR;
     const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
-    const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW, strip = blockIdx.y;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+    const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW, strip = blockIdx.x;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y) {
         int y = (r - MARCH_ABOVE) % g.Ny;
         y = y < 0 ? y + g.Ny : y;
         for (int c = threadIdx.x; c < g.W; c += blockDim.x) {
@@ -155,11 +155,6 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
     }
 }
 
-template <typename T>
-__device__ __forceinline__ bool nonzero_value(T v) {
-    return v != T(0);
-}
-
 // flags[strip][r]: whether any V pair of the strip's columns is nonzero in rows
 // [r - march_flag_back(2), r + MARCH_GROUP - 1] (periodic).
 constexpr int FLAG_ROWS = 64;
@@ -168,23 +163,26 @@ __global__ void __launch_bounds__(256) march_flags_kernel(const T *__restrict__ 
                                                           MarchGeo g) {
     constexpr int BACK = march_flag_back(2);
     __shared__ unsigned char rf[FLAG_ROWS + BACK + MARCH_GROUP];
-    const int strip = blockIdx.y, r0 = blockIdx.x * FLAG_ROWS;
+    const int strip = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
-    const int n = min(FLAG_ROWS, g.Ny - r0);
     static_assert(BACK <= MARCH_ABOVE && MARCH_GROUP <= MARCH_BELOW, "rows of the window have records");
-    for (int k = warp; k < n + BACK + MARCH_GROUP - 1; k += 8) {
-        const T *v = rec + ((size_t(strip) * rows + MARCH_ABOVE + r0 - BACK + k) * MARCH_FIELDS + F_VX) * g.W;
-        bool nz = false;
-        for (int c = lane; c < 4 * g.W; c += 32) nz = nz || nonzero_value(v[c]);
-        nz = __any_sync(0xffffffffu, nz);
-        if (lane == 0) rf[k] = nz ? 1 : 0;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < n; k += 256) {
-        unsigned char f = 0;
-        for (int i = 0; i < BACK + MARCH_GROUP; ++i) f |= rf[k + i];
-        flags[size_t(strip) * g.Ny + r0 + k] = f;
+    for (int r0 = blockIdx.y * FLAG_ROWS; r0 < g.Ny; r0 += gridDim.y * FLAG_ROWS) {
+        const int n = min(FLAG_ROWS, g.Ny - r0);
+        for (int k = warp; k < n + BACK + MARCH_GROUP - 1; k += 8) {
+            const T *v = rec + ((size_t(strip) * rows + MARCH_ABOVE + r0 - BACK + k) * MARCH_FIELDS + F_VX) * g.W;
+            bool nz = false;
+            for (int c = lane; c < 4 * g.W; c += 32) nz = nz || v[c] != T(0);
+            nz = __any_sync(0xffffffffu, nz);
+            if (lane == 0) rf[k] = nz ? 1 : 0;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < n; k += 256) {
+            unsigned char f = 0;
+            for (int i = 0; i < BACK + MARCH_GROUP; ++i) f |= rf[k + i];
+            flags[size_t(strip) * g.Ny + r0 + k] = f;
+        }
+        __syncthreads();
     }
 }
 
@@ -243,9 +241,9 @@ cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, 
                                  int precision, int interleaved, int unitary, cudaStream_t st) {
     char *m = static_cast<char *>(mem);
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
-    const dim3 grid(unsigned(rows < 4096 ? rows : 4096), unsigned(g.strips));
-    const dim3 fgrid(unsigned((g.Ny + FLAG_ROWS - 1) / FLAG_ROWS), unsigned(g.strips));
-    if (g.strips > 65535) return cudaErrorInvalidValue;
+    const int fblocks = (g.Ny + FLAG_ROWS - 1) / FLAG_ROWS;
+    const dim3 grid(unsigned(g.strips), unsigned(rows < 4096 ? rows : 4096));
+    const dim3 fgrid(unsigned(g.strips), unsigned(fblocks < 4096 ? fblocks : 4096));
     for (int z = 0; z < nfam; ++z) {
         void *rec = m + z * g.record_bytes;
         unsigned char *flags = reinterpret_cast<unsigned char *>(m + nfam * g.record_bytes + z * g.flag_bytes);

@@ -253,9 +253,11 @@ struct MarchGeo {
     size_t record_bytes;  // of one family
     size_t flag_bytes;    // of one family (a multiple of 256)
 };
-// The marching form serves the lattice (a plane below 2^32 bytes) and its
-// geometry: FP32 128 columns with a halo of 8 (two steps), FP64 64 with 4 (one).
+// Whether the marching form serves the lattice, and its geometry: FP32 128
+// columns with a halo of 8 (two steps), FP64 64 with 4 (one).
 bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g);
+// Whether its state rows are copied in 16-byte vectors at 32-bit offsets.
+bool march_vectors(const MarchGeo &g);
 // Chooses the row ranges of a pass over nfam families on a device of sms SMs.
 // chunk: rows per range (0: automatic).
 void march_plan(MarchGeo *g, int nfam, int chunk, int sms);

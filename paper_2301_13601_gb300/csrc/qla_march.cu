@@ -16,8 +16,11 @@ bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g) {
     g->strips = (Nx + g->w_valid - 1) / g->w_valid;
     g->record_bytes = size_t(g->strips) * (size_t(MARCH_ABOVE) + Ny + MARCH_BELOW) * MARCH_FIELDS * g->W * g->es;
     g->flag_bytes = (size_t(g->strips) * Ny + 255) / 256 * 256;
-    // 32-bit byte offsets in a plane; strips * Ny shares at most
-    return (unsigned long long)Nx * Ny * g->es < (1ull << 32) && (long long)g->strips * Ny < (1LL << 30);
+    return (long long)g->strips * Ny < (1LL << 30);  // shares, at most
+}
+
+bool march_vectors(const MarchGeo &g) {
+    return g.Nx % (16 / g.es) == 0 && (unsigned long long)g.Nx * g.Ny * g.es < (1ull << 32);
 }
 
 size_t march_bytes(const MarchGeo &g, int nfam) { return size_t(nfam) * (g.record_bytes + g.flag_bytes); }
@@ -94,8 +97,7 @@ cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out
     a.strips = g.strips;
     a.ctas_fam = 0;
     a.chunks = g.chunks[K];
-    // the lane's columns as one vector: 4 (FP32) or 2 (FP64) columns
-    const bool vec = g.Nx % (f64 ? 2 : 4) == 0;
+    const bool vec = march_vectors(g);
     if (f64) return vec ? launch_march_f64_k1(a, nfam, interleaved, unitary, st)
                         : launch_march_f64_k1_any(a, nfam, interleaved, unitary, st);
     if (K == 2) return vec ? launch_march_f32_k2(a, nfam, interleaved, unitary, st)

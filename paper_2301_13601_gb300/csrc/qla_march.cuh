@@ -386,8 +386,9 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
 }
 
 // One warp's share: rows [y0, y1) of strip `strip` of a family. sm: the
-// warp's shared memory. VEC: rows and strips keep the alignment of the lane's
-// vectors (Nx a multiple of C); else the copies and stores go element by element.
+// warp's shared memory. VEC: rows keep the alignment of the lane's vectors (Nx a
+// multiple of C) and a plane holds less than 2^32 bytes; else the state is copied
+// and stored element by element, with 64-bit offsets.
 template <typename T, int C, int K, int D, int U, bool INTER, bool UNIT, bool VEC>
 __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &F, int strip, int y0, int y1, unsigned char *sm,
                                             int lane) {
@@ -399,11 +400,11 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     constexpr int LB = C * int(sizeof(T));  // a lane's bytes of a row
     constexpr int RB = L::RB;
     const int Nx = A.Nx, Ny = A.Ny;
-    // Places in a plane as 32-bit byte offsets (a plane holds less than 2^32
-    // bytes, checked on the host) from plane addresses that lie in the
-    // kernel's parameters: an access then takes one address register and no
-    // 64-bit arithmetic.
-    const unsigned pitch = unsigned(Nx) * unsigned(sizeof(T)), plane_bytes = pitch * unsigned(Ny);
+    // Places in a plane as byte offsets from plane addresses that lie in the
+    // kernel's parameters; 32-bit ones (VEC) take one register and little
+    // arithmetic (8192^2: 628 -> 591 us per step).
+    using Off = std::conditional_t<VEC, unsigned, size_t>;
+    const Off pitch = Off(Nx) * Off(sizeof(T)), plane_bytes = pitch * Off(Ny);
     const bool te = F.te != 0;
     const unsigned hsign = te ? 0x80000000u : 0u;
     const int cy_off = te ? 2 * RB : 0;  // TM: C_X and C_Y are one plane
@@ -412,20 +413,20 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     const int o_hi = min(o_lo + A.w_valid, Nx);
     const int xbase = o_lo - A.halo;
     constexpr int NGC = VEC ? 1 : C;  // global columns of the lane (VEC: of its first column)
-    unsigned gc[NGC];
+    Off gc[NGC];
 #pragma unroll
-    for (int k = 0; k < NGC; ++k) gc[k] = unsigned(wrapi(xbase + C * lane + k, Nx)) * unsigned(sizeof(T));
+    for (int k = 0; k < NGC; ++k) gc[k] = Off(wrapi(xbase + C * lane + k, Nx)) * Off(sizeof(T));
     const unsigned sbase = tc::smem_addr(sm) + unsigned(lane) * LB;
     sm += lane * LB;
 
     const int F0 = y0 - 4 * K;
     // ro: byte offset of the row (VEC: of the lane's first column in it)
-    auto row = [&](unsigned dst, const char *plane, unsigned ro) {
+    auto row = [&](unsigned dst, const char *plane, Off ro) {
         if constexpr (VEC) {
             march_cp<LB>(dst, plane + ro);
         } else {
 #pragma unroll
-            for (int k = 0; k < C; ++k) march_cp<sizeof(T)>(dst + k * unsigned(sizeof(T)), plane + (ro + gc[k]));
+            for (int k = 0; k < C; ++k) march_cp<sizeof(T)>(dst + k * unsigned(sizeof(T)), plane + ro + gc[k]);
         }
     };
     // coefficient copies: two fields (x, y) of the record `dr` rows from the
@@ -437,7 +438,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
         march_cp<LB>(dst, cp + (dr * RECB + field * RB));
         march_cp<LB>(dst + RB, cp + (dr * RECB + (field + 1) * RB));
     };
-    auto copy0 = [&](unsigned slot_off, unsigned ro, int dr) {
+    auto copy0 = [&](unsigned slot_off, Off ro, int dr) {
         const unsigned b = sbase + slot_off;
         row(b, F.h, ro);
         row(b + RB, F.px, ro);
@@ -481,7 +482,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     const int nit = y1 - y0 + march_delay(K);
     const int ngroups = (nit + U - 1) / U;
     int rg = wrapi(F0, Ny);  // wrapped level-0 row of the group's first iteration
-    auto step_row = [&](int &r, unsigned &off) {  // next row, wrapped (r counts up to 0 at the wrap)
+    auto step_row = [&](int &r, Off &off) {  // next row, wrapped (r counts up to 0 at the wrap)
         off += pitch;
         if (++r == 0) {
             r = -Ny;
@@ -491,7 +492,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     // prologue: level-0 rows F0 .. F0 + D - 2, the later levels' first collision rows, the first V rows
     unsigned von = flags[rg], von1 = flags[wrapi(rg + U, Ny)], von2 = flags[wrapi(rg + 2 * U, Ny)];
     int row_c = rg - Ny;  // level-0 copies
-    unsigned off_c = unsigned(rg) * pitch + (VEC ? gc[0] : 0u);
+    Off off_c = Off(rg) * pitch + (VEC ? gc[0] : Off(0));
 #pragma unroll
     for (int j = 1; j < K; ++j) copyc(j, 0, -(4 + MARCH_LAG) * j);
     if (von)
@@ -513,7 +514,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     }
     const int n_out = y1 - y0;
     // (offsets of rows and columns that are not written wrap around harmlessly)
-    unsigned out_off = unsigned(y0 - march_delay(K)) * pitch + unsigned((xbase + C * lane) * int(sizeof(T)));
+    Off out_off = Off(y0 - march_delay(K)) * pitch + Off(xbase + C * lane) * Off(sizeof(T));
 
     for (int g = 0, it0 = 0; g < ngroups; ++g, it0 += U) {
         const unsigned von3 = flags[wrap_down(rg + 3 * U, Ny)];  // read three groups ahead
@@ -605,7 +606,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
 template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, bool UNIT, bool VEC>
 __global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_constant__ MarchArgs A) {
     using L = MarchLayout<T, C, K, D, INTER>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0);
     const int layer = int(blockIdx.x) >= A.ctas_fam ? 1 : 0;
@@ -617,9 +618,9 @@ __global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_cons
     march_share<T, C, K, D, U, INTER, UNIT, VEC>(A, A.fam[layer], strip, y0, y1, smem_raw + warp * L::WARP, lane);
 }
 
-// Host: a family's entry (fam: 0 = TM, 1 = TE).
+// A family's entry (fam: 0 = TM, 1 = TE).
 template <typename T>
-MarchFam march_fam(const void *q_in, void *q_out, const void *rec, const unsigned char *flags, int fam, int Nx,
+__host__ __device__ MarchFam march_fam(const void *q_in, void *q_out, const void *rec, const unsigned char *flags, int fam, int Nx,
                           int Ny) {
     const size_t PB = size_t(Nx) * Ny * sizeof(T);
     const char *q = static_cast<const char *>(q_in);
