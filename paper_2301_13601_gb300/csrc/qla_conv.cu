@@ -4,9 +4,11 @@
 // Activations hold nimg images of H x W stacked ([nimg][H][W][C]); each image
 // is periodic on its own. One tile = 128 consecutive pixels of one image row
 // (M = 128), all output channels, K = 9 taps x input channels. Input rows
-// (130 pixels with the x halo, CIN channels) are staged once each in the
-// interleaved K-major layout, so the three x taps are shifted windows of the
-// same row (no swizzle: any 16-byte aligned start is a valid operand). Each
+// (130 pixels with the x halo, CIN channels) are staged once each, so the three
+// x taps are shifted windows of the same row. 64 channels: a pixel is one
+// 128-byte line of the 128-byte swizzled K-major layout, loaded by TMA, and a
+// window starts on any line. 16 channels: the interleaved K-major layout
+// without swizzle (any 16-byte aligned start is a valid operand). Each
 // staged input row is multiplied once per (x tap, 16-channel slice) against
 // the weights of all three y taps at once (N = 3 NOUT), accumulating into the
 // TMEM accumulators of the three output rows it feeds. All 9 taps of the
@@ -19,10 +21,12 @@
 // GELU is the tanh form 0.5 x (1 + tanh(sqrt(2/pi) (x + 0.044715 x^3))).
 #include <cuda_bf16.h>
 #include <math.h>
+#include <string.h>
 
 #include "../../include/qla_surrogate.h"
 #include "qla_internal.h"
 #include "qla_tc.cuh"
+#include "qla_tma.h"
 
 namespace qla {
 
@@ -59,6 +63,43 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// Two channels per operation (the same roundings as one by one): the epilogues
+// are bound by their instruction issue.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_get(F2 a, float &x, float &y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 gelu_f2(F2 x) {  // gelu_f of both
+    const float k0 = 0.7978845608028654f, k1 = 0.7978845608028654f * 0.044715f;
+    const F2 arg = f2_mul(x, f2_fma(f2(k1, k1), f2_mul(x, x), f2(k0, k0)));
+    float a, b;
+    f2_get(arg, a, b);
+    const F2 t = f2(tanh_fast(a), tanh_fast(b)), hx = f2_mul(x, f2(0.5f, 0.5f));
+    return f2_fma(hx, t, hx);
+}
+
 __device__ __forceinline__ uint32_t bf2(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t *>(&h);
@@ -74,6 +115,13 @@ struct ConvLayout {
     // Ring depth; even, so that a slot is always released by the same epilogue group.
     static constexpr int NS = CCH >= 8 && NOUT >= 64 ? 8 : (CCH >= 8 ? 6 : 8);
     static_assert(NS % 2 == 0, "ring slots alternate between the two epilogue groups");
+    // SWZ: the ring is NS * 130 lines of 128 bytes, line = slot * 130 + pixel;
+    // the swizzle (16-byte chunk ^ line mod 8) goes by absolute line, for TMA and
+    // MMA alike, so slots need no alignment of their own. One lane loads a row
+    // in three boxes where a warp's cp.async took about 35 instructions per lane.
+    // Last layer at 1024^2 94 -> 72 us, hidden layers 96 -> 95 (bound by the MMA
+    // issue, see mma_bf16_leader, and their stores).
+    static constexpr bool SWZ = CCH == 8;
     static constexpr int A_BYTES = CCH * NS * HALO_PX * 16;
     static constexpr int B_BYTES = 9 * CCH * NOUT * 16;
     static constexpr int A_OFF = 0;
@@ -87,6 +135,23 @@ struct ConvLayout {
     static constexpr int TMEM_COLS = 512;
     static constexpr int NB = TMEM_COLS / NOUT;  // output-row accumulators (NOUT columns each)
 };
+
+// 16-byte chunk c of the pixel at `line` in the swizzled ring (byte offset).
+__device__ __forceinline__ int conv_swz(int line, int c) { return line * 128 + ((c ^ (line & 7)) << 4); }
+
+// Tensor maps of the swizzled form's input [nimg * H][W][64]: boxes of 128
+// pixels and of one (the halo pixels, which wrap around the image).
+struct ConvMaps {
+    CUtensorMap px128, px1;
+};
+
+__device__ __forceinline__ void conv_tma(uint32_t dst, const CUtensorMap *map, int x, int row, uint64_t *bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(x), "r"(row), "r"(tc::smem_addr(bar))
+        : "memory");
+}
 
 constexpr int CONV_EPI_WARPS = 8;
 constexpr int CONV_MMA_WARP = 8;
@@ -167,9 +232,27 @@ __host__ __device__ __forceinline__ void conv_row_mmas(int j, int len, int b0, F
     const int k_lo = j - len + 1 > 0 ? j - len + 1 : 0;
     const int k_hi = j < 2 ? j : 2;
     const int wrap = NB - b0;  // first ky whose block wraps to 0
+    if (k_lo == 0 && k_hi == 2 && wrap > 2) {
+        // a row inside the run whose three blocks do not wrap (most of them): a
+        // list of constants
 #pragma unroll
+        for (int kx = 0; kx < 3; ++kx) {
+#pragma unroll
+            for (int k2 = 0; k2 < CCH / 2; ++k2) {
+                const uint32_t ao = uint32_t((2 * k2) * NS * HP + kx), bo = uint32_t((kx * CCH + 2 * k2) * 3 * NOUT);
+                if (kx == 0 && k2 == 0) {
+                    emit(ConvMma{kx, k2, 0, 0, b0, 0, ao, bo});
+                    emit(ConvMma{kx, k2, 1, 2, b0 + 1, 1, ao, bo + NOUT});
+                } else {
+                    emit(ConvMma{kx, k2, 0, 2, b0, 1, ao, bo});
+                }
+            }
+        }
+        return;
+    }
+#pragma unroll 1
     for (int kx = 0; kx < 3; ++kx) {
-#pragma unroll
+#pragma unroll 1
         for (int k2 = 0; k2 < CCH / 2; ++k2) {
             const bool first = kx == 0 && k2 == 0;
             for (int ka = k_lo; ka <= k_hi;) {
@@ -219,8 +302,9 @@ __host__ __device__ __forceinline__ void conv_walk_rows(long long u_begin, long 
 // rows of 128-pixel column blocks, ordered (image, column block, row); each CTA
 // takes a contiguous range and walks down its column blocks with a ring of
 // halo rows in shared memory, so every input row is loaded once per block.
-//   warp 9 (loader)   cp.async of each halo row into the ring; arrival on
-//                     full[slot] when its copies land; waits on empty[slot]
+//   warp 9 (loader)   copies each halo row into the ring (64 channels: three TMA
+//                     boxes by one lane; 16: cp.async), which complete on
+//                     full[slot]; waits on empty[slot]
 //   warp 8 (MMA)      per input row, one lane issues the 3 x CCH/2 MMAs (x tap,
 //                     16-channel slice) whose N = 3 NOUT columns are the
 //                     accumulators of the three output rows the row feeds,
@@ -239,7 +323,7 @@ __host__ __device__ __forceinline__ void conv_walk_rows(long long u_begin, long 
 // flag and the role stops, and the others time out in turn, so the kernel
 // always ends.
 template <int CCH, int NOUT>
-__global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvArgs a) {
+__global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvArgs a, const __grid_constant__ ConvMaps maps) {
     using L = ConvLayout<CCH, NOUT>;
     constexpr int CIN = 8 * CCH;
     constexpr int NS = L::NS;
@@ -248,8 +332,8 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
     constexpr int NB = L::NB;
     __shared__ uint64_t full_bar[NS], empty_bar[NS], accf_bar[NB], acce_bar[NB], done_bar;
     __shared__ uint32_t tmem_base_s;
-    __shared__ float bias_s[64];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ __align__(16) float bias_s[64];
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int H = a.H, W = a.W;
     const int TPR = W / 128;
     const long long T = (long long)a.nimg * TPR * H;
@@ -271,7 +355,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
     if (warp == CONV_MMA_WARP) tc::tmem_alloc(&tmem_base_s, L::TMEM_COLS);
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            tc::mbar_init(&full_bar[s], 32);
+            tc::mbar_init(&full_bar[s], L::SWZ ? 1 : 32);
             tc::mbar_init(&empty_bar[s], 1 + CONV_EPI_WARPS / 2);
         }
         for (int b = 0; b < NB; ++b) {
@@ -304,6 +388,18 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                 }
                 int yy = (sg.y_s - 1 + j) % H;
                 yy = yy < 0 ? yy + H : yy;
+                if constexpr (L::SWZ) {
+                    if (lane == 0) {
+                        const int row = sg.img * H + yy;
+                        const uint32_t dst = tc::smem_addr(As) + uint32_t(slot * HP * 128);
+                        tc::mbar_arrive_expect_tx(&full_bar[slot], HP * 128);
+                        conv_tma(dst, &maps.px1, sg.x0 == 0 ? W - 1 : sg.x0 - 1, row, &full_bar[slot]);
+                        conv_tma(dst + 128, &maps.px128, sg.x0, row, &full_bar[slot]);
+                        conv_tma(dst + 129 * 128, &maps.px1, sg.x0 + 128 == W ? 0 : sg.x0 + 128, row, &full_bar[slot]);
+                    }
+                    __syncwarp();
+                    continue;
+                }
                 const __nv_bfloat16 *row = ximg + (size_t)yy * W * CIN;
                 for (int i = lane; i < CCH * HP; i += 32) {
                     const int c = i % CCH, px = i / CCH;
@@ -316,6 +412,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
             u0 += sg.len;
         }
         cp_async_wait_0();
+        if constexpr (L::SWZ) {  // no copy outlives the CTA, also when a role gave up
+            for (long long r = g > NS ? g - NS : 0; r < g; ++r)
+                if (!tc::mbar_wait(&full_bar[r % NS], uint32_t((r / NS) & 1), CONV_WAIT_TRIES)) ok = false;
+        }
         if (!ok && lane == 0) atomicExch(a.error, 1);
     } else if (warp == CONV_MMA_WARP) {
         // ---------------- MMA issuer ----------------
@@ -329,10 +429,12 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
         constexpr uint32_t IDESC3 = tc::make_idesc_bf16(128, 3 * NOUT);
         constexpr uint32_t A_LBO = NS * HP * 16, A_SBO = 128;
         constexpr uint32_t B_LBO = 3 * NOUT * 16, B_SBO = 128;
-        const uint64_t ad0 = tc::make_desc(tc::smem_addr(As), A_LBO, A_SBO);
+        const uint64_t ad0 = L::SWZ ? tc::make_desc_sw128(tc::smem_addr(As), 1024)
+                                    : tc::make_desc(tc::smem_addr(As), A_LBO, A_SBO);
         const uint64_t bd0 = tc::make_desc(tc::smem_addr(Bs), B_LBO, B_SBO);
         const uint32_t a_lo0 = uint32_t(ad0), a_hi = uint32_t(ad0 >> 32);
         const uint32_t b_lo0 = uint32_t(bd0), b_hi = uint32_t(bd0 >> 32);
+        const uint32_t leader = tc::elect_one();
         bool ok = true;
         conv_walk_rows(u_begin, u_end, H, TPR, [&](const ConvSeg &sg, int j, long long r, long long on) {
             const int b0 = conv_block(on, NB);
@@ -342,25 +444,24 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                 ok = false;
             if (!ok) return false;
             tc::fence_after_sync();
-            if (lane == 0) {
-                const uint32_t a_row = a_lo0 + uint32_t(int(r % NS) * HP);  // (slot * HP * 16) >> 4
+            {
+                // (slot * HP * line bytes) >> 4
+                const uint32_t a_row = a_lo0 + uint32_t(int(r % NS) * HP * (L::SWZ ? 8 : 1));
                 conv_row_mmas<CCH, NOUT, NS, HP>(j, sg.len, b0, [&](const ConvMma &m) {
                     const uint32_t idesc = m.kb == m.ka ? IDESC1 : (m.kb == m.ka + 1 ? IDESC2 : IDESC3);
-                    tc::mma_bf16_lohi(tmem + uint32_t(m.blk * NOUT), a_row + m.a_off, a_hi, b_lo0 + m.b_off, b_hi,
-                                      idesc, uint32_t(m.acc));
+                    // swizzled: a pixel is 8 units of 16 bytes, a 16-channel slice 2
+                    const uint32_t a_off = L::SWZ ? uint32_t(8 * m.kx + 2 * m.k2) : m.a_off;
+                    tc::mma_bf16_leader(leader, tmem + uint32_t(m.blk * NOUT), a_row + a_off, a_hi, b_lo0 + m.b_off,
+                                        b_hi, idesc, uint32_t(m.acc));
                 });
-                tc::mma_commit(&empty_bar[r % NS]);  // the tensor cores are done with row r
+                tc::mma_commit_leader(leader, &empty_bar[r % NS]);  // the tensor cores are done with row r
                 const int bd = conv_row_done_block(j, on, NB);
-                if (bd >= 0) tc::mma_commit(&accf_bar[bd]);  // output row on - 2
+                if (bd >= 0) tc::mma_commit_leader(leader, &accf_bar[bd]);  // output row on - 2
             }
-            __syncwarp();
             return true;
         });
-        if (lane == 0) {
-            tc::mma_commit(&done_bar);  // tracks every MMA issued above
-            if (!tc::mbar_wait(&done_bar, 0u, CONV_WAIT_TRIES)) ok = false;
-        }
-        __syncwarp();
+        tc::mma_commit_leader(leader, &done_bar);  // tracks every MMA issued above
+        if (!tc::mbar_wait(&done_bar, 0u, CONV_WAIT_TRIES)) ok = false;
         if (!ok && lane == 0) atomicExch(a.error, 1);
     } else {
         // ---------------- epilogue ----------------
@@ -421,58 +522,76 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                     break;
                 }
                 tc::fence_after_sync();
+                if constexpr (L::SWZ) {
+                    // the centre row, which TMA wrote and this warp may read as the
+                    // residual, is released only below, so this phase is the row's
+                    if (res_smem && !tc::mbar_wait(&full_bar[(g + i + 1) % NS], uint32_t(((g + i + 1) / NS) & 1),
+                                                   CONV_WAIT_TRIES)) {
+                        ok = false;
+                        break;
+                    }
+                }
 #pragma unroll 1
                 for (int cbi = 0; cbi < NCB; ++cbi) {
                     const int cb0 = 32 * cbi;
                     const int y = sg.y_s + i;
                     const size_t p = ((size_t)sg.img * H + y) * W + sg.x0 + m;
+                    const size_t tile = ((size_t)sg.img * H + y) * TPR + (sg.x0 >> 7);  // ConvArgs::tiled
                     float v[32];
                     const uint32_t ta = tmem + uint32_t(b * NOUT + cb0) + (uint32_t(32 * q) << 16);
                     if constexpr (NC == 32) tc::tmem_ld32(ta, v);
                     else tc::tmem_ld16(ta, v);
+                    if (a.epi != EPI_DGRAD) {
 #pragma unroll
-                    for (int k = 0; k < NC; ++k) v[k] += bias_s[cb0 + k];
+                        for (int k = 0; k < NC; k += 4) {
+                            const float4 bb = *reinterpret_cast<const float4 *>(bias_s + cb0 + k);
+                            f2_get(f2_add(f2(v[k], v[k + 1]), f2(bb.x, bb.y)), v[k], v[k + 1]);
+                            f2_get(f2_add(f2(v[k + 2], v[k + 3]), f2(bb.z, bb.w)), v[k + 2], v[k + 3]);
+                        }
+                    }
                     if (a.epi == EPI_GELU) {
-                        const uint4 *rp =
-                            res_smem ? reinterpret_cast<const uint4 *>(
-                                           As + (((cb0 / 8) * NS + int((g + i + 1) % NS)) * HP + m + 1) * 16)
-                            : a.aux0 ? reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.aux0) +
-                                                                       p * NOUT + cb0)
-                                     : nullptr;
-                        const int rstride = res_smem ? NS * HP : 1;  // uint4 steps between 8-channel chunks
+                        const bool res = a.aux0 != nullptr;
+                        const uint4 *const rp =
+                            reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.aux0) + p * NOUT + cb0);
+                        const int line = int((g + i + 1) % NS) * HP + m + 1;  // the centre pixel in the ring
                         uint4 av[NC / 8], zv[NC / 8];
 #pragma unroll
                         for (int c4 = 0; c4 < NC / 8; ++c4) {
                             float g8[8];
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) g8[k] = gelu_f(v[8 * c4 + k]);
-                            if (rp) {
-                                const uint4 w4 = rp[c4 * rstride];
+                            for (int k = 0; k < 8; k += 2)
+                                f2_get(gelu_f2(f2(v[8 * c4 + k], v[8 * c4 + k + 1])), g8[k], g8[k + 1]);
+                            if (res) {
+                                const uint4 w4 =
+                                    res_smem ? *reinterpret_cast<const uint4 *>(
+                                                   L::SWZ ? As + conv_swz(line, cb0 / 8 + c4)
+                                                          : As + (((cb0 / 8 + c4) * NS + int((g + i + 1) % NS)) * HP +
+                                                                  m + 1) * 16)
+                                             : rp[c4];
                                 const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    g8[2 * k] += __uint_as_float(ww[k] << 16);
-                                    g8[2 * k + 1] += __uint_as_float(ww[k] & 0xffff0000u);
-                                }
+                                for (int k = 0; k < 4; ++k)
+                                    f2_get(f2_add(f2(g8[2 * k], g8[2 * k + 1]),
+                                                  f2(__uint_as_float(ww[k] << 16),
+                                                     __uint_as_float(ww[k] & 0xffff0000u))),
+                                           g8[2 * k], g8[2 * k + 1]);
                             }
                             av[c4] = make_uint4(bf2(g8[0], g8[1]), bf2(g8[2], g8[3]), bf2(g8[4], g8[5]),
                                                 bf2(g8[6], g8[7]));
                             const float *z = v + 8 * c4;
                             zv[c4] = make_uint4(bf2(z[0], z[1]), bf2(z[2], z[3]), bf2(z[4], z[5]), bf2(z[6], z[7]));
                         }
-                        // Staged stores measured faster for the first layer (59.6 vs 63.8 us at
-                        // 1024^2) and with z also stored (73.9 vs 141 us), slower for a hidden
-                        // layer storing only the activation (99.0 vs 96.1 us).
-                        if (CCH < 8 || a.out0) {
-                            store_half_bf16<NC, NOUT, L::STG_STRIDE>(stg, av, static_cast<__nv_bfloat16 *>(a.out1),
-                                                                     p - lane, cb0, lane);
-                            if (a.out0)
-                                store_half_bf16<NC, NOUT, L::STG_STRIDE>(
-                                    stg, zv, static_cast<__nv_bfloat16 *>(a.out0), p - lane, cb0, lane);
-                        } else {
-                            uint4 *ao = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.out1) + p * NOUT + cb0);
+                        // Staged stores: hidden layer at 1024^2 69.3 us against 75.3 with a
+                        // lane storing its own pixel's 16-byte pieces.
+                        store_half_bf16<NC, NOUT, L::STG_STRIDE>(stg, av, static_cast<__nv_bfloat16 *>(a.out1),
+                                                                 p - lane, cb0, lane);
+                        if (a.out0 && a.tiled) {
+                            uint4 *const zo = static_cast<uint4 *>(a.out0) + tile * (NOUT / 8 * 128) + cb0 / 8 * 128 + m;
 #pragma unroll
-                            for (int c4 = 0; c4 < NC / 8; ++c4) ao[c4] = av[c4];
+                            for (int c4 = 0; c4 < NC / 8; ++c4) zo[c4 * 128] = zv[c4];
+                        } else if (a.out0) {
+                            store_half_bf16<NC, NOUT, L::STG_STRIDE>(stg, zv, static_cast<__nv_bfloat16 *>(a.out0),
+                                                                     p - lane, cb0, lane);
                         }
                     } else if (a.epi == EPI_LINEAR) {
                         float4 *op = reinterpret_cast<float4 *>(static_cast<float *>(a.out0) + p * NOUT + cb0);
@@ -480,12 +599,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                         for (int k = 0; k < NC / 4; ++k)
                             op[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
                     } else if (a.epi == EPI_DGRAD) {
-                        const float4 *gin = a.aux0 ? reinterpret_cast<const float4 *>(
-                                                         static_cast<const float *>(a.aux0) + p * NOUT + cb0)
-                                                   : nullptr;
-                        float4 *go = reinterpret_cast<float4 *>(static_cast<float *>(a.out0) + p * NOUT + cb0);
-                        const uint4 *zp = reinterpret_cast<const uint4 *>(
-                            static_cast<const __nv_bfloat16 *>(a.zprev) + p * NOUT + cb0);
+                        // this lane's pixel: 16-byte pieces, `step` apart
+                        const size_t g0 = a.tiled ? tile * (NOUT / 4 * 128) + cb0 / 4 * 128 + m : (p * NOUT + cb0) / 4;
+                        const size_t z0 = a.tiled ? tile * (NOUT / 8 * 128) + cb0 / 8 * 128 + m : (p * NOUT + cb0) / 8;
+                        const int step = a.tiled ? 128 : 1;
+                        const float4 *const gin = a.aux0 ? static_cast<const float4 *>(a.aux0) + g0 : nullptr;
+                        float4 *const go = static_cast<float4 *>(a.out0) + g0;
+                        const uint4 *const zp = static_cast<const uint4 *>(a.zprev) + z0;
                         uint4 dzv[NC / 8];
 #pragma unroll
                         for (int c4 = 0; c4 < NC / 8; ++c4) {
@@ -493,13 +613,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
 #pragma unroll
                             for (int k = 0; k < 8; ++k) g8[k] = v[8 * c4 + k];
                             if (gin) {
-                                const float4 g0 = gin[2 * c4], g1 = gin[2 * c4 + 1];
-                                g8[0] += g0.x; g8[1] += g0.y; g8[2] += g0.z; g8[3] += g0.w;
-                                g8[4] += g1.x; g8[5] += g1.y; g8[6] += g1.z; g8[7] += g1.w;
+                                const float4 ga = gin[2 * c4 * step], gb = gin[(2 * c4 + 1) * step];
+                                g8[0] += ga.x; g8[1] += ga.y; g8[2] += ga.z; g8[3] += ga.w;
+                                g8[4] += gb.x; g8[5] += gb.y; g8[6] += gb.z; g8[7] += gb.w;
                             }
-                            go[2 * c4] = make_float4(g8[0], g8[1], g8[2], g8[3]);
-                            go[2 * c4 + 1] = make_float4(g8[4], g8[5], g8[6], g8[7]);
-                            const uint4 z4 = zp[c4];
+                            go[2 * c4 * step] = make_float4(g8[0], g8[1], g8[2], g8[3]);
+                            go[(2 * c4 + 1) * step] = make_float4(g8[4], g8[5], g8[6], g8[7]);
+                            const uint4 z4 = zp[c4 * step];
                             const uint32_t zz[4] = {z4.x, z4.y, z4.z, z4.w};
                             float d[8];
 #pragma unroll
@@ -561,7 +681,23 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long rows = (long long)a.nimg * a.H * (a.W / 128);
     const int grid = rows < sms ? int(rows) : sms;
-    conv3x3_tc_kernel<CCH, NOUT><<<grid, CONV_THREADS, L::SMEM_LAUNCH, st>>>(a);
+    ConvMaps maps;
+    memset(&maps, 0, sizeof(maps));
+    if (L::SWZ) {
+        const EncodeTiledFn fn = encode_tiled_fn();
+        if (!fn) return cudaErrorNotSupported;
+        const cuuint64_t dim[3] = {64, cuuint64_t(a.W), cuuint64_t(a.nimg) * cuuint64_t(a.H)};
+        const cuuint64_t str[2] = {128, cuuint64_t(a.W) * 128};
+        const cuuint32_t one[3] = {1, 1, 1};
+        for (int k = 0; k < 2; ++k) {
+            const cuuint32_t box[3] = {64, k ? 1u : 128u, 1};
+            if (fn(k ? &maps.px1 : &maps.px128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(a.x), dim, str,
+                   box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return cudaErrorInvalidValue;
+        }
+    }
+    conv3x3_tc_kernel<CCH, NOUT><<<grid, CONV_THREADS, L::SMEM_LAUNCH, st>>>(a, maps);
     return cudaGetLastError();
 }
 
@@ -831,6 +967,7 @@ extern "C" qla_status qla_conv3x3_bf16(const void *x, int nimg, int H, int W, in
     a.out1 = out1;
     a.scale = scale;
     a.error = error_flag;
+    a.tiled = 0;
     const cudaError_t e = qla::launch_conv(cin, nout, a, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? QLA_OK : QLA_ECUDA;
 }

@@ -314,6 +314,13 @@ struct ConvArgs {
     void *out1;           // GELU: BF16 activation; DGRAD: BF16 dz
     float scale;          // QUPDATE
     int *error;           // set to 1 when a bounded wait runs out
+    // z (GELU out0, zprev) and g (DGRAD aux0, out0) in pixel tiles instead of NHWC
+    // (nout = 64): per 128 pixels of a row, 16-byte channel groups of all 128
+    // pixels one after another ([tile][64 * element size / 16][128][16 bytes]).
+    // Only these epilogues read them, one pixel per lane, so every access is
+    // 512 contiguous bytes of a warp; in NHWC a warp's 16-byte accesses lie 128
+    // or 256 bytes apart.
+    int tiled;
 };
 // Supported (cin, nout): (16, 64), (64, 64), (64, 16).
 bool conv_supported(int cin, int nout);

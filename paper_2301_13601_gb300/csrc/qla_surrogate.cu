@@ -308,6 +308,7 @@ qla_status conv(qla_surrogate *s, int cin, int nout, const void *x, const void *
     a.out1 = out1;
     a.scale = scale;
     a.error = s->err;
+    a.tiled = 1;  // z and the input gradients are only passed from epilogue to epilogue
     SG_CUDA(s, launch_conv(cin, nout, a, st));
     return QLA_OK;
 }

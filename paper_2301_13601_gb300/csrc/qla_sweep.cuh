@@ -48,6 +48,7 @@
 
 #include "qla_internal.h"
 #include "qla_tc.cuh"
+#include "qla_tma.h"
 
 namespace qla {
 
@@ -373,11 +374,6 @@ __device__ __forceinline__ void tma_box5(void *dst, const CUtensorMap *map, int 
         "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(tc::smem_addr(bar))
         : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(tc::smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-
 // Copies the strip's 256 columns of one global row into a (swizzled) shared
 // row: lane l copies strip columns 8l .. 8l+7. xb: wrapped global column of
 // strip column 0; nowrap: the strip lies inside [0, Nx).
@@ -645,7 +641,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
     auto tma_group_x = [&](int it, bool with_state, int half) {
         // every level's blocks are loaded (an inactive level's are not read)
         const uint32_t row_bytes = uint32_t(K * NXS) * CROW + (with_state ? 3u * SROW : 0u);
-        if (tid == 0) mbar_arrive_expect_tx(&tbar[0], uint32_t(R) * row_bytes);
+        if (tid == 0) tc::mbar_arrive_expect_tx(&tbar[0], uint32_t(R) * row_bytes);
         const int ntask = 1 + (with_state ? NSB : 0);
         for (int t = warp + NWARP * lane; t < ntask; t += 32 * NWARP) {
             if (t == 0) {
@@ -659,7 +655,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
         }
     };
     auto tma_group_y = [&](int it) {
-        if (tid == 0) mbar_arrive_expect_tx(&tbar[1], uint32_t(R * K * NYS) * CROW);
+        if (tid == 0) tc::mbar_arrive_expect_tx(&tbar[1], uint32_t(R * K * NYS) * CROW);
         constexpr int ntask = INTER ? 1 : 2;
         for (int t = warp + NWARP * lane; t < ntask; t += 32 * NWARP) {
             if (t == 0) tma_planes(true, 0, 2, it, Fm::CY, &tbar[1]);  // C_Y, V_Y
@@ -994,26 +990,6 @@ __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, N
         if (failed) break;
         u += y1 - y0;
     }
-}
-
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no link
-// against the driver library); null if unavailable.
-using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-inline EncodeTiledFn encode_tiled_fn() {
-    static EncodeTiledFn fn = [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            return EncodeTiledFn(nullptr);
-        }
-        return reinterpret_cast<EncodeTiledFn>(p);
-    }();
-    return fn;
 }
 
 // Tensor maps of one FP32 pass (see SweepMaps); false when TMA cannot be used

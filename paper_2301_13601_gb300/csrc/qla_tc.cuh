@@ -32,6 +32,15 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;                // layout type (bits 61-63) 0: no swizzle
 }
 
+// K-major operand in the 128-byte swizzled layout: rows of 128 bytes (64 BF16
+// values), 16-byte chunk c of the row at absolute 128-byte line l stored at
+// chunk c ^ (l & 7); sbo_bytes between groups of eight rows. The start address
+// may lie on any 128-byte line (the swizzle goes by absolute address), plus 32
+// bytes per 16-value step along K.
+__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr, uint32_t sbo_bytes) {
+    return make_desc(saddr, 16, sbo_bytes) | uint64_t(2) << 61;
+}
+
 // Instruction descriptor for kind::f16 with BF16 A and B, FP32 accumulator,
 // both operands K-major, shape M x N.
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
@@ -50,6 +59,11 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
 // pending on it); a later mbar_init may then set it up afresh.
 __device__ __forceinline__ void mbar_inval(uint64_t *bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes)
+                 : "memory");
 }
 
 __device__ __forceinline__ void fence_mbar_init() {
@@ -148,6 +162,39 @@ __device__ __forceinline__ void mma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo, ui
         "setp.ne.b32 p, %6, 0;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n}\n" ::"r"(d_tmem),
         "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// True in one lane of a converged warp.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p;
+}
+
+// The same issued by the lane whose `leader` is set, with the whole warp in
+// uniform control flow: the operands are then computed in uniform registers,
+// where the instruction takes them, instead of being moved there one by one in
+// a branch that one lane takes. That branch cost 190 cycles per MMA whatever its
+// width: 1024^2 hidden layer without its epilogue 78 -> 56 us, last layer with it
+// 72 -> 42 us.
+__device__ __forceinline__ void mma_bf16_leader(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
+                                                uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p, q;\n.reg .b64 ad, bd;\n"
+        "mov.b64 ad, {%1, %2};\n"
+        "mov.b64 bd, {%3, %4};\n"
+        "setp.ne.b32 p, %6, 0;\n"
+        "setp.ne.b32 q, %7, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(leader)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_leader(uint32_t leader, uint64_t *bar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_addr(bar)),
+        "r"(leader)
         : "memory");
 }
 
