@@ -25,6 +25,7 @@
 
 #include "../../include/qla_surrogate.h"
 #include "qla_internal.h"
+#include "qla_pack.cuh"
 #include "qla_tc.cuh"
 #include "qla_tma.h"
 
@@ -710,11 +711,15 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
 // tile; ky = 2 and an unused half in the other); kx is a 16-byte shift of the
 // start address along K. Six accumulator tiles (2 row pairs x 3 kx) of N = NT
 // columns stay in TMEM for all of a CTA's rows; at the end each CTA writes its
-// partial sums [9][NT][64] (FP32), reduced over CTAs in a fixed order later.
+// partial sums [9][NT][64] (FP32), reduced over CTAs in a fixed order later,
+// and those of the bias gradient [NT], summed by warps that the tensor cores
+// leave idle (a kernel of its own read g once more, 22 us per layer).
 // The x ring has one mirror slot after the last, a copy of slot 0, so that two
 // consecutive rows are always adjacent in memory. Source x may have 16 or 64
 // channels (16: the other chunks stay zero).
 // ---------------------------------------------------------------------------
+constexpr int WG_SUM_WARPS = 4;  // warps that sum the bias gradient
+
 template <int NT>
 struct WgradLayout {
     static constexpr int HP = 130;
@@ -736,7 +741,8 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint64_t xf_bar[NSX], xe_bar[NSX], gf_bar[NSG], ge_bar[NSG], done_bar;
     __shared__ uint32_t tmem_base_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ float bias_s[WG_SUM_WARPS][NT];
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int H = a.H, W = a.W;
     const int TPR = W / 128;
     const long long T = (long long)a.nimg * TPR * H;
@@ -754,7 +760,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
         }
         for (int s = 0; s < NSG; ++s) {
             tc::mbar_init(&gf_bar[s], 32);
-            tc::mbar_init(&ge_bar[s], 1);
+            tc::mbar_init(&ge_bar[s], 1 + WG_SUM_WARPS);
         }
         tc::mbar_init(&done_bar, 1);
         tc::fence_mbar_init();
@@ -819,6 +825,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
         const uint64_t ad0 = tc::make_desc(x_base, A_LBO, A_SBO), bd0 = tc::make_desc(g_base, B_LBO, B_SBO);
         const uint32_t a_lo0 = uint32_t(ad0), a_hi = uint32_t(ad0 >> 32);
         const uint32_t b_lo0 = uint32_t(bd0), b_hi = uint32_t(bd0 >> 32);
+        const uint32_t leader = tc::elect_one();
         long long gx = 0, gn = 0;
         bool ok = true, first = true;
         for (long long u0 = u_begin; u0 < u_end && ok;) {
@@ -831,37 +838,72 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
                 if (!tc::mbar_wait(&gf_bar[gn % NSG], uint32_t((gn / NSG) & 1), CONV_WAIT_TRIES)) ok = false;
                 if (!ok) break;
                 tc::fence_after_sync();
-                if (lane == 0) {
-                    const uint32_t s0 = uint32_t((gx + i) % NSX), s2 = uint32_t((gx + i + 2) % NSX);
-                    const uint32_t g_lo = b_lo0 + uint32_t(gn % NSG) * (L::GSLOT >> 4);
-                    const uint32_t a0_lo = a_lo0 + s0 * 8 * HP, a1_lo = a_lo0 + s2 * 8 * HP;
+                const uint32_t s0 = uint32_t((gx + i) % NSX), s2 = uint32_t((gx + i + 2) % NSX);
+                const uint32_t g_lo = b_lo0 + uint32_t(gn % NSG) * (L::GSLOT >> 4);
+                const uint32_t a0_lo = a_lo0 + s0 * 8 * HP, a1_lo = a_lo0 + s2 * 8 * HP;
+                const uint32_t acc0 = first ? 0u : 1u;
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
+                for (int kk = 0; kk < 8; ++kk) {
 #pragma unroll
-                        for (int kx = 0; kx < 3; ++kx) {
-                            const uint32_t acc = (first && kk == 0) ? 0u : 1u;
-                            tc::mma_bf16_lohi(tmem + kx * NT, a0_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk, b_hi, IDESC,
-                                              acc);
-                            tc::mma_bf16_lohi(tmem + (3 + kx) * NT, a1_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk, b_hi,
-                                              IDESC, acc);
-                        }
-                    }
-                    tc::mma_commit(&ge_bar[gn % NSG]);
-                    tc::mma_commit(&xe_bar[(gx + i) % NSX]);
-                    if (i == sg.len - 1) {
-                        tc::mma_commit(&xe_bar[(gx + i + 1) % NSX]);
-                        tc::mma_commit(&xe_bar[(gx + i + 2) % NSX]);
+                    for (int kx = 0; kx < 3; ++kx) {
+                        const uint32_t acc = kk == 0 ? acc0 : 1u;
+                        tc::mma_bf16_leader(leader, tmem + kx * NT, a0_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk, b_hi,
+                                            IDESC, acc);
+                        tc::mma_bf16_leader(leader, tmem + (3 + kx) * NT, a1_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk,
+                                            b_hi, IDESC, acc);
                     }
                 }
+                tc::mma_commit_leader(leader, &ge_bar[gn % NSG]);
+                tc::mma_commit_leader(leader, &xe_bar[(gx + i) % NSX]);
+                if (i == sg.len - 1) {
+                    tc::mma_commit_leader(leader, &xe_bar[(gx + i + 1) % NSX]);
+                    tc::mma_commit_leader(leader, &xe_bar[(gx + i + 2) % NSX]);
+                }
                 first = false;
-                __syncwarp();
             }
             gx += sg.len + 2;
             u0 += sg.len;
         }
-        if (lane == 0) tc::mma_commit(&done_bar);
-        __syncwarp();
+        tc::mma_commit_leader(leader, &done_bar);
         if (!ok && lane == 0) atomicExch(a.error, 1);
+    }
+    if (warp < WG_SUM_WARPS) {
+        // bias gradient: the column sums of g, from the staged rows, while the
+        // tensor cores work. Lane = pixel (32 of the row's 128 per warp); its sums
+        // of all NT channels stay in registers until the CTA's rows are done.
+        float sum[NT];
+#pragma unroll
+        for (int k = 0; k < NT; ++k) sum[k] = 0.0f;
+        const long long rows = u_end - u_begin;
+        bool ok = true;
+        for (long long r = 0; r < rows; ++r) {
+            const int slot = int(r % NSG);
+            if (!tc::mbar_wait(&gf_bar[slot], uint32_t((r / NSG) & 1), CONV_WAIT_TRIES)) {
+                ok = false;
+                break;
+            }
+            const uint4 *const row = reinterpret_cast<const uint4 *>(Gs + slot * L::GSLOT) + 32 * warp + lane;
+#pragma unroll
+            for (int c = 0; c < NT / 8; ++c) {
+                const uint4 v = row[c * 128];
+                const uint32_t vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    f2_get(f2_add(f2(sum[8 * c + 2 * k], sum[8 * c + 2 * k + 1]),
+                                  f2(__uint_as_float(vv[k] << 16), __uint_as_float(vv[k] & 0xffff0000u))),
+                           sum[8 * c + 2 * k], sum[8 * c + 2 * k + 1]);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ge_bar[slot]);
+        }
+        if (!ok && lane == 0) atomicExch(a.error, 1);
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            float v = sum[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == k % 32) bias_s[warp][k] = v;
+        }
     }
     if (warp < CONV_EPI_WARPS) {
         // epilogue: partial sums of this CTA
@@ -899,6 +941,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    if (tid < NT) {
+        float v = bias_s[0][tid];
+        for (int w = 1; w < WG_SUM_WARPS; ++w) v += bias_s[w][tid];
+        a.bpart[(size_t)blockIdx.x * NT + tid] = v;
+    }
     if (warp == CONV_MMA_WARP) tc::tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
@@ -972,38 +1019,11 @@ extern "C" qla_status qla_conv3x3_bf16(const void *x, int nimg, int H, int W, in
     return e == cudaSuccess ? QLA_OK : QLA_ECUDA;
 }
 
-// ---------------------------------------------------------------------------
-// Weight packing: FP32 w[nout][cin][3][3] -> BF16 [9][cin_pad/8][nout_pad][8]
-// (the B operand layout of conv3x3_tc_kernel), zero-padded.
-//   PACK_PLAIN       packed[t][c][n] = w[n][c][t]
-//   PACK_ADJOINT     the input-gradient convolution of w: w'[c][n][ky][kx] =
-//                    w[n][c][2-ky][2-kx] (packed outputs = w's inputs)
-//   PACK_TIED_INPUT  as PLAIN, but packed input channels 0-5 and 6-11 both
-//                    read logical 0-5 (high and low BF16 parts of the same
-//                    field) and 12-14 read logical 6-8
-// ---------------------------------------------------------------------------
 namespace qla {
 
 __global__ void pack_conv_weights_kernel(const float *__restrict__ w, int nout, int cin, int nout_pad, int cin_pad,
                                          int mode, __nv_bfloat16 *__restrict__ out) {
-    const int total = 9 * cin_pad * nout_pad;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int j = i % 8;
-        const int n = (i / 8) % nout_pad;
-        const int chunk = (i / (8 * nout_pad)) % (cin_pad / 8);
-        const int t = i / (8 * nout_pad * (cin_pad / 8));
-        int c = chunk * 8 + j;
-        const int ky = t / 3, kx = t % 3;
-        float v = 0.0f;
-        if (mode == PACK_ADJOINT) {
-            // packed output channel n ranges over the original inputs, packed input c over the original outputs
-            if (n < cin && c < nout) v = w[((size_t(c) * cin + n) * 3 + (2 - ky)) * 3 + (2 - kx)];
-        } else {
-            if (mode == PACK_TIED_INPUT) c = c < 6 ? c : (c < 15 ? c - 6 : cin);
-            if (n < nout && c < cin) v = w[((size_t(n) * cin + c) * 3 + ky) * 3 + kx];
-        }
-        out[i] = __float2bfloat16_rn(v);
-    }
+    pack_conv_weights_elements(w, nout, cin, nout_pad, cin_pad, mode, out);
 }
 
 cudaError_t launch_pack_weights(const float *w, int nout, int cin, int nout_pad, int cin_pad, int mode,

@@ -336,6 +336,7 @@ struct WgradArgs {
     int nt;
     int nimg, H, W;
     float *part;
+    float *bpart;  // per-CTA partial sums [cta][nt] of sum_p g[p][n]
     int *error;
 };
 int wgrad_grid(const WgradArgs &a);

@@ -25,6 +25,7 @@
 
 #include "../../include/qla_surrogate.h"
 #include "qla_internal.h"
+#include "qla_pack.cuh"
 
 namespace qla {
 namespace sg {
@@ -36,7 +37,6 @@ constexpr int CINP[NL] = {16, 64, 64, 64, 64, 64};  // packed input channels
 constexpr int NOUT[NL] = {64, 64, 64, 64, 64, 6};   // logical output channels
 constexpr int NOUTP[NL] = {64, 64, 64, 64, 64, 16};
 constexpr int X0C = 16;                              // x0 channels: Q hi (6), Q lo (6), n (3), 0
-constexpr int BIAS_BLOCKS = 256;                     // pixel splits of the bias-gradient reduction
 constexpr int RED_BLOCKS = 512;                      // partial sums of the loss reductions
 
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
@@ -149,59 +149,43 @@ __global__ void loss_grad_kernel(const float *__restrict__ f, const float *__res
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// ---- bias gradient: partial sums of g over pixel ranges -------------------
-// 16-byte loads: NT/8 threads per pixel, 256 / (NT/8) pixels per pass.
-template <int NT>
-__global__ void bias_grad_kernel(const __nv_bfloat16 *__restrict__ g, long long NP, float *__restrict__ bpart) {
-    constexpr int TPP = NT / 8;       // threads per pixel
-    constexpr int PPB = 256 / TPP;    // pixels per pass
-    __shared__ float sh[PPB][NT + 1];
-    const int c8 = threadIdx.x % TPP, pl = threadIdx.x / TPP;
-    const long long per = (NP + gridDim.x - 1) / gridDim.x;
-    const long long b = blockIdx.x * per, e = b + per < NP ? b + per : NP;
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long p = b + pl; p < e; p += PPB) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(g + p * NT + 8 * c8);
-        acc[0] += bf_lo(v.x); acc[1] += bf_hi(v.x); acc[2] += bf_lo(v.y); acc[3] += bf_hi(v.y);
-        acc[4] += bf_lo(v.z); acc[5] += bf_hi(v.z); acc[6] += bf_lo(v.w); acc[7] += bf_hi(v.w);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) sh[pl][8 * c8 + k] = acc[k];
-    __syncthreads();
-    if (threadIdx.x < NT) {
-        float t = 0.0f;
-        for (int k = 0; k < PPB; ++k) t += sh[k][threadIdx.x];
-        bpart[size_t(blockIdx.x) * NT + threadIdx.x] = t;
-    }
-}
-
-// Sum the per-CTA partials part[S][9][NT][CT] and bias partials bpart[SB][NT]
+// Sum the per-CTA partials part[S][9][NT][CT] and bias partials bpart[S][NT]
 // in a fixed order into the logical gradient layout gw[n][c][ky][kx], gb[n];
 // tied: packed input channels c and c+6 (c < 6) both belong to logical c,
-// packed 12-14 to logical 6-8.
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int S, const float *__restrict__ bpart, int SB,
-                                    int NT, int CT, int nout, int cin, int tied, float *__restrict__ gw,
-                                    float *__restrict__ gb) {
+// packed 12-14 to logical 6-8. A block sums 32 outputs, eight threads each over
+// every eighth CTA (one thread over all 152: 25 us per layer, few loads in
+// flight).
+constexpr int RED_SPLIT = 8;
+__global__ void __launch_bounds__(32 * RED_SPLIT) wgrad_reduce_kernel(const float *__restrict__ part,
+                                                                      const float *__restrict__ bpart, int S, int NT,
+                                                                      int CT, int nout, int cin, int tied,
+                                                                      float *__restrict__ gw, float *__restrict__ gb) {
+    __shared__ float sh[RED_SPLIT][32];
     const int total = nout * cin * 9;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = threadIdx.x & 31, sp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + o;
+    // c fastest: consecutive threads read consecutive partials
+    const int c = i % cin, n = (i / cin) % nout, t = i / (cin * nout);
+    float acc = 0.0f;
     if (i < total) {
-        // c fastest: consecutive threads read consecutive partials
-        const int c = i % cin, n = (i / cin) % nout, t = i / (cin * nout);
         const int c1 = tied ? (c < 6 ? c : c + 6) : c;
         const int c2 = (tied && c < 6) ? c + 6 : -1;
-        float acc = 0.0f;
-        for (int s = 0; s < S; ++s) {
-            const float *o = part + ((size_t(s) * 9 + t) * NT + n) * CT;
-            acc += o[c1];
-            if (c2 >= 0) acc += o[c2];
+        for (int s = sp; s < S; s += RED_SPLIT) {
+            const float *p = part + ((size_t(s) * 9 + t) * NT + n) * CT;
+            acc += p[c1];
+            if (c2 >= 0) acc += p[c2];
         }
-        gw[(n * cin + c) * 9 + t] = acc;
     } else if (i < total + nout) {
-        const int n = i - total;
-        float acc = 0.0f;
-        for (int s = 0; s < SB; ++s) acc += bpart[size_t(s) * NT + n];
-        gb[n] = acc;
+        for (int s = sp; s < S; s += RED_SPLIT) acc += bpart[size_t(s) * NT + (i - total)];
     }
+    sh[sp][o] = acc;
+    __syncthreads();
+    if (sp != 0) return;
+    float v = sh[0][o];
+#pragma unroll
+    for (int k = 1; k < RED_SPLIT; ++k) v += sh[k][o];
+    if (i < total) gw[(n * cin + c) * 9 + t] = v;
+    else if (i < total + nout) gb[i - total] = v;
 }
 
 // ---- Adam on the flat FP32 parameter vector --------------------------------
@@ -217,9 +201,30 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
     }
 }
 
-__global__ void pad_bias_kernel(const float *__restrict__ b, int n, int npad, float *__restrict__ out) {
-    const int i = threadIdx.x;
-    if (i < npad) out[i] = i < n ? b[i] : 0.0f;
+// Every layer's packed operands after an update, one launch: block (x, l) for
+// the forward weights and biases of layer l, block (x, NL + l) for its adjoint
+// weights (eleven packing and six bias kernels took about 50 us per training step).
+struct PackAll {
+    const float *params;
+    long long off_w[NL], off_b[NL];
+    void *wf[NL], *wb[NL];
+    float *bpad[NL];
+    int nout[NL], cin[NL], noutp[NL], cinp[NL];
+};
+__global__ void pack_all_kernel(const PackAll a) {
+    const int l = blockIdx.y % NL;
+    const bool adjoint = int(blockIdx.y) >= NL;
+    if (adjoint && (l == 0 || !a.wb[l])) return;
+    const float *w = a.params + a.off_w[l];
+    const int nout = a.nout[l], cin = a.cin[l], noutp = a.noutp[l], cinp = a.cinp[l];
+    if (adjoint) {
+        pack_conv_weights_elements(w, nout, cin, cinp, noutp, PACK_ADJOINT, static_cast<__nv_bfloat16 *>(a.wb[l]));
+    } else {
+        pack_conv_weights_elements(w, nout, cin, noutp, cinp, l == 0 ? PACK_TIED_INPUT : PACK_PLAIN,
+                                   static_cast<__nv_bfloat16 *>(a.wf[l]));
+        if (blockIdx.x == 0 && int(threadIdx.x) < noutp)
+            a.bpad[l][threadIdx.x] = int(threadIdx.x) < nout ? a.params[a.off_b[l] + threadIdx.x] : 0.0f;
+    }
 }
 
 }  // namespace sg
@@ -314,15 +319,21 @@ qla_status conv(qla_surrogate *s, int cin, int nout, const void *x, const void *
 }
 
 qla_status repack(qla_surrogate *s, cudaStream_t st) {
+    PackAll a;
+    a.params = s->params;
     for (int l = 0; l < NL; ++l) {
-        const float *w = s->params + s->off_w[l];
-        SG_CUDA(s, launch_pack_weights(w, NOUT[l], CIN[l], NOUTP[l], CINP[l], l == 0 ? PACK_TIED_INPUT : PACK_PLAIN,
-                                       s->wf[l], st));
-        if (l > 0 && s->wb[l])
-            SG_CUDA(s, launch_pack_weights(w, NOUT[l], CIN[l], CINP[l], NOUTP[l], PACK_ADJOINT, s->wb[l], st));
-        pad_bias_kernel<<<1, 64, 0, st>>>(s->params + s->off_b[l], NOUT[l], NOUTP[l], s->bpad[l]);
-        SG_CUDA(s, cudaGetLastError());
+        a.off_w[l] = s->off_w[l];
+        a.off_b[l] = s->off_b[l];
+        a.wf[l] = s->wf[l];
+        a.wb[l] = s->wb[l];
+        a.bpad[l] = s->bpad[l];
+        a.nout[l] = NOUT[l];
+        a.cin[l] = CIN[l];
+        a.noutp[l] = NOUTP[l];
+        a.cinp[l] = CINP[l];
     }
+    pack_all_kernel<<<dim3(36, 2 * NL), 256, 0, st>>>(a);
+    SG_CUDA(s, cudaGetLastError());
     s->packed = true;
     return QLA_OK;
 }
@@ -375,18 +386,14 @@ qla_status wgrad(qla_surrogate *s, int l, const void *x, int cs, const void *g, 
     w.H = s->cfg.H;
     w.W = s->cfg.W;
     w.part = s->wpart;
+    w.bpart = s->bpart;
     w.error = s->err;
     int S = 0;
     SG_CUDA(s, launch_wgrad_tc(w, &S, st));
-    if (nt == 64)
-        bias_grad_kernel<64><<<BIAS_BLOCKS, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(g), s->NP, s->bpart);
-    else
-        bias_grad_kernel<16><<<BIAS_BLOCKS, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(g), s->NP, s->bpart);
-    SG_CUDA(s, cudaGetLastError());
     const int total = NOUT[l] * CIN[l] * 9 + NOUT[l];
-    wgrad_reduce_kernel<<<(total + 255) / 256, 256, 0, st>>>(s->wpart, S, s->bpart, BIAS_BLOCKS, nt, 64, NOUT[l],
-                                                             CIN[l], l == 0 ? 1 : 0, s->grads + s->off_w[l],
-                                                             s->grads + s->off_b[l]);
+    wgrad_reduce_kernel<<<(total + 31) / 32, 32 * RED_SPLIT, 0, st>>>(s->wpart, s->bpart, S, nt, 64, NOUT[l], CIN[l],
+                                                                      l == 0 ? 1 : 0, s->grads + s->off_w[l],
+                                                                      s->grads + s->off_b[l]);
     SG_CUDA(s, cudaGetLastError());
     return QLA_OK;
 }
@@ -502,7 +509,7 @@ qla_status qla_surrogate_create(const qla_surrogate_config *cfg, qla_surrogate *
     add(train ? NP * 16 * 4 : 0);                                                                // fout
     for (int k = 0; k < 2; ++k) add(train ? NP * HID * 4 : 0);                                   // da
     add(train ? size_t(s->sms) * 9 * HID * HID * 4 : 0);                                         // wpart (per CTA)
-    add(train ? size_t(BIAS_BLOCKS) * HID * 4 : 0);                                              // bpart
+    add(train ? size_t(s->sms) * HID * 4 : 0);                                                   // bpart (per CTA)
     add(RED_BLOCKS * 8);                                                                         // red
     add(4 * 8);                                                                                  // scal
     add(sizeof(int));                                                                            // err
