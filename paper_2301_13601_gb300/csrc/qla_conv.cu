@@ -323,7 +323,9 @@ __host__ __device__ __forceinline__ void conv_walk_rows(long long u_begin, long 
 // two where the ring wraps). Every wait is bounded; a timeout sets the error
 // flag and the role stops, and the others time out in turn, so the kernel
 // always ends.
-template <int CCH, int NOUT>
+// DG: the input-gradient epilogue (a kernel of its own: the registers of its
+// prefetched rows cost the others 10%).
+template <int CCH, int NOUT, bool DG>
 __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvArgs a, const __grid_constant__ ConvMaps maps) {
     using L = ConvLayout<CCH, NOUT>;
     constexpr int CIN = 8 * CCH;
@@ -509,6 +511,36 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                     if (i_first < sg.len) qload(i_first, qv);
                 }
             }
+            // input gradient (64 channels out): the incoming gradient and the
+            // pre-activation of the next 32 channels are loaded as soon as the last
+            // ones are used, before their accumulator is waited for
+            constexpr bool DPRE = DG && NOUT == 64;
+            constexpr int NGQ = DPRE ? 8 : 1, NZQ = DPRE ? 4 : 1;
+            float4 gq[NGQ];
+            uint4 zq[NZQ];
+            const size_t dstep = a.tiled ? 128 : 1;  // 16-byte pieces of a pixel
+            auto dpix = [&](int i, int cb0, int per) {  // in units of `per` channels (16 bytes)
+                const size_t row = (size_t)sg.img * H + sg.y_s + i;
+                return a.tiled ? (row * TPR + (sg.x0 >> 7)) * (NOUT / per * 128) + cb0 / per * 128 + m
+                               : ((row * W + sg.x0 + m) * NOUT + cb0) / per;
+            };
+            auto dload = [&](int i, int cb0) {
+                if (a.aux0) {
+                    const float4 *const gin = static_cast<const float4 *>(a.aux0) + dpix(i, cb0, 4);
+#pragma unroll
+                    for (int k = 0; k < NGQ; ++k) gq[k] = gin[k * dstep];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < NGQ; ++k) gq[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                const uint4 *const zp = static_cast<const uint4 *>(a.zprev) + dpix(i, cb0, 8);
+#pragma unroll
+                for (int k = 0; k < NZQ; ++k) zq[k] = zp[k * dstep];
+            };
+            if constexpr (DPRE) {
+                const int i_first = int(((long long)grp - o_seg) & 1);
+                if (i_first < sg.len) dload(i_first, 0);
+            }
             for (int i = 0; i < sg.len; ++i, ++o) {
                 if (int(o & 1) != grp) continue;
                 float qn[NQ];
@@ -542,7 +574,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                     const uint32_t ta = tmem + uint32_t(b * NOUT + cb0) + (uint32_t(32 * q) << 16);
                     if constexpr (NC == 32) tc::tmem_ld32(ta, v);
                     else tc::tmem_ld16(ta, v);
-                    if (a.epi != EPI_DGRAD) {
+                    if constexpr (!DG) {
 #pragma unroll
                         for (int k = 0; k < NC; k += 4) {
                             const float4 bb = *reinterpret_cast<const float4 *>(bias_s + cb0 + k);
@@ -550,7 +582,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                             f2_get(f2_add(f2(v[k + 2], v[k + 3]), f2(bb.z, bb.w)), v[k + 2], v[k + 3]);
                         }
                     }
-                    if (a.epi == EPI_GELU) {
+                    if (!DG && a.epi == EPI_GELU) {
                         const bool res = a.aux0 != nullptr;
                         const uint4 *const rp =
                             reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.aux0) + p * NOUT + cb0);
@@ -594,44 +626,72 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
                             store_half_bf16<NC, NOUT, L::STG_STRIDE>(stg, zv, static_cast<__nv_bfloat16 *>(a.out0),
                                                                      p - lane, cb0, lane);
                         }
-                    } else if (a.epi == EPI_LINEAR) {
+                    } else if (!DG && a.epi == EPI_LINEAR) {
                         float4 *op = reinterpret_cast<float4 *>(static_cast<float *>(a.out0) + p * NOUT + cb0);
 #pragma unroll
                         for (int k = 0; k < NC / 4; ++k)
                             op[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-                    } else if (a.epi == EPI_DGRAD) {
-                        // this lane's pixel: 16-byte pieces, `step` apart
-                        const size_t g0 = a.tiled ? tile * (NOUT / 4 * 128) + cb0 / 4 * 128 + m : (p * NOUT + cb0) / 4;
-                        const size_t z0 = a.tiled ? tile * (NOUT / 8 * 128) + cb0 / 8 * 128 + m : (p * NOUT + cb0) / 8;
-                        const int step = a.tiled ? 128 : 1;
-                        const float4 *const gin = a.aux0 ? static_cast<const float4 *>(a.aux0) + g0 : nullptr;
-                        float4 *const go = static_cast<float4 *>(a.out0) + g0;
-                        const uint4 *const zp = static_cast<const uint4 *>(a.zprev) + z0;
-                        uint4 dzv[NC / 8];
+                    } else if constexpr (DG) {
+                        if constexpr (DPRE) {
+                            float4 *const go = static_cast<float4 *>(a.out0) + dpix(i, cb0, 4);
+                            uint4 dzv[NC / 8], zc[NC / 8];
 #pragma unroll
-                        for (int c4 = 0; c4 < NC / 8; ++c4) {
-                            float g8[8];
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) g8[k] = v[8 * c4 + k];
-                            if (gin) {
-                                const float4 ga = gin[2 * c4 * step], gb = gin[(2 * c4 + 1) * step];
-                                g8[0] += ga.x; g8[1] += ga.y; g8[2] += ga.z; g8[3] += ga.w;
-                                g8[4] += gb.x; g8[5] += gb.y; g8[6] += gb.z; g8[7] += gb.w;
+                            for (int c4 = 0; c4 < NC / 8; ++c4) {
+                                const float4 ga = gq[2 * c4], gb = gq[2 * c4 + 1];
+                                float *const g8 = v + 8 * c4;
+                                if (a.aux0) {
+                                    g8[0] += ga.x; g8[1] += ga.y; g8[2] += ga.z; g8[3] += ga.w;
+                                    g8[4] += gb.x; g8[5] += gb.y; g8[6] += gb.z; g8[7] += gb.w;
+                                }
+                                zc[c4] = zq[c4];
                             }
-                            go[2 * c4 * step] = make_float4(g8[0], g8[1], g8[2], g8[3]);
-                            go[(2 * c4 + 1) * step] = make_float4(g8[4], g8[5], g8[6], g8[7]);
-                            const uint4 z4 = zp[c4 * step];
-                            const uint32_t zz[4] = {z4.x, z4.y, z4.z, z4.w};
-                            float d[8];
+                            if (cb0 == 0) dload(i, 32);
+                            else if (i + 2 < sg.len) dload(i + 2, 0);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                d[2 * k] = g8[2 * k] * gelu_grad(__uint_as_float(zz[k] << 16));
-                                d[2 * k + 1] = g8[2 * k + 1] * gelu_grad(__uint_as_float(zz[k] & 0xffff0000u));
+                            for (int c4 = 0; c4 < NC / 8; ++c4) {
+                                const float *const g8 = v + 8 * c4;
+                                go[2 * c4 * dstep] = make_float4(g8[0], g8[1], g8[2], g8[3]);
+                                go[(2 * c4 + 1) * dstep] = make_float4(g8[4], g8[5], g8[6], g8[7]);
+                                const uint32_t zz[4] = {zc[c4].x, zc[c4].y, zc[c4].z, zc[c4].w};
+                                float d[8];
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    d[2 * k] = g8[2 * k] * gelu_grad(__uint_as_float(zz[k] << 16));
+                                    d[2 * k + 1] = g8[2 * k + 1] * gelu_grad(__uint_as_float(zz[k] & 0xffff0000u));
+                                }
+                                dzv[c4] = make_uint4(bf2(d[0], d[1]), bf2(d[2], d[3]), bf2(d[4], d[5]), bf2(d[6], d[7]));
                             }
-                            dzv[c4] = make_uint4(bf2(d[0], d[1]), bf2(d[2], d[3]), bf2(d[4], d[5]), bf2(d[6], d[7]));
+                            store_half_bf16<NC, NOUT, L::STG_STRIDE>(
+                                stg, dzv, static_cast<__nv_bfloat16 *>(a.out1), p - lane, cb0, lane);
+                        } else {
+                            const float4 *const gin =
+                                a.aux0 ? static_cast<const float4 *>(a.aux0) + p * NOUT / 4 : nullptr;
+                            float4 *const go = static_cast<float4 *>(a.out0) + p * NOUT / 4;
+                            const uint4 *const zp = static_cast<const uint4 *>(a.zprev) + p * NOUT / 8;
+                            uint4 dzv[NC / 8];
+#pragma unroll
+                            for (int c4 = 0; c4 < NC / 8; ++c4) {
+                                float *const g8 = v + 8 * c4;
+                                if (gin) {
+                                    const float4 ga = gin[2 * c4], gb = gin[2 * c4 + 1];
+                                    g8[0] += ga.x; g8[1] += ga.y; g8[2] += ga.z; g8[3] += ga.w;
+                                    g8[4] += gb.x; g8[5] += gb.y; g8[6] += gb.z; g8[7] += gb.w;
+                                }
+                                go[2 * c4] = make_float4(g8[0], g8[1], g8[2], g8[3]);
+                                go[2 * c4 + 1] = make_float4(g8[4], g8[5], g8[6], g8[7]);
+                                const uint4 z4 = zp[c4];
+                                const uint32_t zz[4] = {z4.x, z4.y, z4.z, z4.w};
+                                float d[8];
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    d[2 * k] = g8[2 * k] * gelu_grad(__uint_as_float(zz[k] << 16));
+                                    d[2 * k + 1] = g8[2 * k + 1] * gelu_grad(__uint_as_float(zz[k] & 0xffff0000u));
+                                }
+                                dzv[c4] = make_uint4(bf2(d[0], d[1]), bf2(d[2], d[3]), bf2(d[4], d[5]), bf2(d[6], d[7]));
+                            }
+                            store_half_bf16<NC, NOUT, L::STG_STRIDE>(
+                                stg, dzv, static_cast<__nv_bfloat16 *>(a.out1), p - lane, cb0, lane);
                         }
-                        store_half_bf16<NC, NOUT, L::STG_STRIDE>(stg, dzv, static_cast<__nv_bfloat16 *>(a.out1),
-                                                                 p - lane, cb0, lane);
                     } else if (cb0 == 0) {  // EPI_QUPDATE: channels 0..5
                         const size_t pix = (size_t)y * W + sg.x0 + m;
                         float *qo = static_cast<float *>(a.out0) + (size_t)sg.img * 6 * qP;
@@ -671,10 +731,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
     if (warp == CONV_MMA_WARP) tc::tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
-template <int CCH, int NOUT>
+template <int CCH, int NOUT, bool DG>
 cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
     using L = ConvLayout<CCH, NOUT>;
-    cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel<CCH, NOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(conv3x3_tc_kernel<CCH, NOUT, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          L::SMEM_LAUNCH);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 148;
@@ -698,7 +758,7 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
                 return cudaErrorInvalidValue;
         }
     }
-    conv3x3_tc_kernel<CCH, NOUT><<<grid, CONV_THREADS, L::SMEM_LAUNCH, st>>>(a, maps);
+    conv3x3_tc_kernel<CCH, NOUT, DG><<<grid, CONV_THREADS, L::SMEM_LAUNCH, st>>>(a, maps);
     return cudaGetLastError();
 }
 
@@ -981,9 +1041,10 @@ bool conv_supported(int cin, int nout) {
 }
 
 cudaError_t launch_conv(int cin, int nout, const ConvArgs &a, cudaStream_t st) {
-    if (cin == 16 && nout == 64) return launch_conv_t<2, 64>(a, st);
-    if (cin == 64 && nout == 64) return launch_conv_t<8, 64>(a, st);
-    if (cin == 64 && nout == 16) return launch_conv_t<8, 16>(a, st);
+    const bool dg = a.epi == EPI_DGRAD;
+    if (cin == 16 && nout == 64) return dg ? launch_conv_t<2, 64, true>(a, st) : launch_conv_t<2, 64, false>(a, st);
+    if (cin == 64 && nout == 64) return dg ? launch_conv_t<8, 64, true>(a, st) : launch_conv_t<8, 64, false>(a, st);
+    if (cin == 64 && nout == 16) return dg ? launch_conv_t<8, 16, true>(a, st) : launch_conv_t<8, 16, false>(a, st);
     return cudaErrorInvalidValue;
 }
 
