@@ -125,164 +125,328 @@ __device__ __forceinline__ double f2d_exact(float v) {
     return double(v);
 }
 
-// FP32 state: the same sums and maxima as the generic kernel below, with the
-// FP64 pipe doing only what needs FP64: a site's squares are summed as an
-// exact-product float pair and enter the FP64 row sum by two additions (sites
-// with values beyond 2^+-60, where FP32 squares could overflow or lose their
-// error term, take FP64 squares instead), the divergence is formed in FP64
-// as (q3(x+1) - q3(x-1)) + (q4(y+1) - q4(y-1)) with the factors 1/2 and 1/4
-// applied to the reduced max and sum (exact scalings), and the site norms |B|^2
-// are screened in FP32: a site's FP64 norm is computed only when its FP32 norm
-// (relative error below 2^-22) reaches the running maximum lowered by 2^-20,
-// so no site whose FP64 norm exceeds the maximum is skipped. max |div| is kept
-// as the bit pattern of a non-negative double (integer order = numeric order;
-// NaN excluded, as fmax would).
-__global__ void __launch_bounds__(DIAG_THREADS) diag_partial_f32(const float *__restrict__ q, int Nx, int Ny,
+// Unevaluated FP32 pair hi + lo (|lo| about 2^-24 |hi|). The rounding intrinsics
+// keep the compiler from contracting the error terms away.
+struct FPair {
+    float hi, lo;
+    // adds the pair (p, e): the high parts by TwoSum, the low parts in FP32
+    __device__ __forceinline__ void add(float p, float e) {
+        const float s = __fadd_rn(hi, p);
+        const float bb = __fsub_rn(s, hi);
+        const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+        lo = __fadd_rn(lo, __fadd_rn(t, e));
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return f2d_exact(hi) + f2d_exact(lo); }
+};
+
+// Screening of a maximum by FP32 approximations f >= 0 of the FP64 values
+// (relative error below 2^-20): a site above the pending one by more than
+// 2^-18 replaces it, a site below it by more is dropped, and only one in
+// between has its FP64 value computed at once; the pending site's is at the
+// end. (Computing it whenever a running maximum rose did so at a third of the
+// sites of a smooth field, for some lane of the warp.)
+struct Screen {
+    float best = 0.0f;
+    __device__ __forceinline__ bool replaces(float f) const { return f > best * (1.0f + 0x1p-18f); }
+    __device__ __forceinline__ bool close(float f) const { return f >= best * (1.0f - 0x1p-18f) && f > 0.0f; }
+};
+
+// |v| in [2^-50, 2^60): a square and its FMA error are then normal FP32 numbers
+// or the error is zero, and sums of squares do not overflow.
+__device__ __forceinline__ bool pair_range(float v) {
+    return (__float_as_uint(v) & 0x7fffffffu) - 0x26800000u < 0x37000000u;
+}
+__device__ __forceinline__ bool is_zero(float v) { return (__float_as_uint(v) << 1) == 0u; }
+
+// FP32 state. GB300's FP64 pipe takes a warp instruction in 64 cycles of a
+// scheduler (the generic kernel below is bound by it, and so was this one with
+// six FP64 operations per site: 305 us at 4096^2), so a site costs none:
+//  * its sum of squares and its squared divergence are FP32 pairs (products
+//    with their FMA errors, sums by TwoSum), added to pairs that enter the FP64
+//    sums after PAIR_SITES sites: relative error about 2^-46 of such a partial
+//    sum, unbiased, over many of them below FP64's own rounding;
+//  * the divergence (q3(x+1) - q3(x-1)) + (q4(y+1) - q4(y-1)) is formed as a pair
+//    from exact differences; the factors 1/2 and 1/4 are applied to the reduced
+//    max and sum;
+//  * the maxima are screened in FP32 (Screen below); max |div| is kept as the bit
+//    pattern of a non-negative double (integer order = numeric order; NaN
+//    excluded, as fmax would).
+// Sites with values outside [2^-50, 2^60) take FP64 throughout.
+constexpr int PAIR_SITES = 32;
+// (four blocks per SM: all of the grid's 608 resident at once)
+__global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float *__restrict__ q, int Nx, int Ny,
                                                                  Partial *__restrict__ part) {
     const size_t P = size_t(Nx) * size_t(Ny);
-    const float *q3 = q + 3 * P, *q4 = q + 4 * P;
+    const float *q4 = q + 4 * P;
     CSum e{0.0, 0.0}, d{0.0, 0.0};
     unsigned long long dmax_bits = 0;
     double b2max = 0.0;
-    float b2thr = 0.0f;
+    Screen sb, sd;
+    float pb[3] = {0.0f, 0.0f, 0.0f}, pd[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // the pending sites' values
+    auto exact_b2 = [&](float v3, float v4, float v5) {
+        const double d3 = f2d_exact(v3), d4 = f2d_exact(v4), d5 = f2d_exact(v5);
+        const double b2 = (d3 * d3 + d4 * d4) + d5 * d5;
+        if (b2 > b2max) b2max = b2;
+    };
+    auto exact_div = [&](float rr, float l, float up, float dn) {
+        const double dv = (f2d_exact(rr) - f2d_exact(l)) + (f2d_exact(up) - f2d_exact(dn));
+        const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) & 0x7fffffffffffffffull;
+        if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
+        return dv;
+    };
     unsigned long long nf = 0;
+    FPair ep{0.0f, 0.0f}, dp{0.0f, 0.0f};
+    int pending = 0;
+    const unsigned W = unsigned(Nx);
     for (int y = blockIdx.x; y < Ny; y += gridDim.x) {
         const int yp = y + 1 == Ny ? 0 : y + 1, ym = y == 0 ? Ny - 1 : y - 1;
-        const size_t r = size_t(y) * Nx;
-        double erow = 0.0, drow = 0.0;
-        for (int x = threadIdx.x; x < Nx; x += blockDim.x) {
-            const size_t i = r + x;
+        const float *row[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) row[c] = q + c * P + size_t(y) * W;
+        const float *const q4p = q4 + size_t(yp) * W, *const q4m = q4 + size_t(ym) * W;
+        double e64 = 0.0, d64 = 0.0;  // sites outside the pair range
+        for (unsigned x = threadIdx.x; x < W; x += DIAG_THREADS) {
+            const unsigned xp = x + 1 == W ? 0 : x + 1, xm = x == 0 ? W - 1 : x - 1;
             float v[6];
-            bool ff = true;  // every |v| zero or in [2^-60, 2^60): FP32 squares and their errors are exact
+            unsigned big = 0u, small = 0xffffffffu;
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
-                v[c] = q[size_t(c) * P + i];
-                if (!isfinite(v[c])) ++nf;
+                v[c] = row[c][x];
                 const unsigned ua = __float_as_uint(v[c]) & 0x7fffffffu;
-                ff = ff && (ua == 0u || ua - 0x21800000u < 0x3c000000u);
+                big = max(big, ua);
+                small = min(small, ua - 1u);  // zero counts as large
             }
+            const bool ff = big < 0x5d800000u && small >= 0x267fffffu;  // every |v| zero or in [2^-50, 2^60)
+            const float l = row[3][xm], rr = row[3][xp], dn = q4m[x], up = q4p[x];
             if (ff) {
-                // the site's sum of squares as an unevaluated float pair: each
-                // square is p + e exactly (e by FMA), the p are added by TwoSum,
-                // the low parts in FP32 (relative error ~2^-47 of the site value,
-                // unbiased); two FP64 additions enter it into the row sum
-                // (intrinsics: no contraction of a product into the TwoSum)
-                float hi = __fmul_rn(v[0], v[0]), lo = __fmaf_rn(v[0], v[0], -hi);
+                FPair s;
+                s.hi = __fmul_rn(v[0], v[0]);
+                s.lo = __fmaf_rn(v[0], v[0], -s.hi);
 #pragma unroll
                 for (int c = 1; c < 6; ++c) {
-                    const float pc = __fmul_rn(v[c], v[c]);
-                    const float ec = __fmaf_rn(v[c], v[c], -pc);
-                    const float sc = __fadd_rn(hi, pc);
-                    const float bb = __fsub_rn(sc, hi);
-                    const float tc = __fadd_rn(__fsub_rn(hi, __fsub_rn(sc, bb)), __fsub_rn(pc, bb));
-                    lo = __fadd_rn(lo, __fadd_rn(tc, ec));
-                    hi = sc;
+                    const float p = __fmul_rn(v[c], v[c]);
+                    s.add(p, __fmaf_rn(v[c], v[c], -p));
                 }
-                erow = (erow + f2d_exact(hi)) + f2d_exact(lo);
+                ep.add(s.hi, s.lo);
             } else {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
+                    if (!isfinite(v[c])) ++nf;
                     const double dv = f2d_exact(v[c]);
-                    erow = fma(dv, dv, erow);
+                    e64 = fma(dv, dv, e64);
                 }
             }
             const float b2f = fmaf(v[3], v[3], fmaf(v[4], v[4], v[5] * v[5]));
-            if (!(b2f < b2thr)) {  // candidate for the maximum (also when b2f is inf or NaN)
-                const double d3 = f2d_exact(v[3]), d4 = f2d_exact(v[4]), d5 = f2d_exact(v[5]);
-                const double b2 = (d3 * d3 + d4 * d4) + d5 * d5;
-                if (b2 > b2max) {
-                    b2max = b2;
-                    b2thr = __double2float_rd(b2 * (1.0 - 0x1p-20));
-                }
+            if (!ff) {
+                exact_b2(v[3], v[4], v[5]);
+            } else if (sb.replaces(b2f)) {
+                sb.best = b2f;
+                pb[0] = v[3]; pb[1] = v[4]; pb[2] = v[5];
+            } else if (sb.close(b2f) && !(v[3] == pb[0] && v[4] == pb[1] && v[5] == pb[2])) {
+                exact_b2(v[3], v[4], v[5]);
             }
-            const int xp = x + 1 == Nx ? 0 : x + 1, xm = x == 0 ? Nx - 1 : x - 1;
-            const double dv = (f2d_exact(q3[r + xp]) - f2d_exact(q3[r + xm])) +
-                              (f2d_exact(q4[size_t(yp) * Nx + x]) - f2d_exact(q4[size_t(ym) * Nx + x]));
-            drow = fma(dv, dv, drow);
-            const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) &
-                                          0x7fffffffffffffffull;
-            if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
+            // the divergence as a pair: exact differences, their sum by TwoSum
+            FPair g{__fsub_rn(rr, l), 0.0f};
+            {
+                const float bb = __fsub_rn(g.hi, rr);
+                g.lo = __fsub_rn(__fsub_rn(rr, __fsub_rn(g.hi, bb)), __fadd_rn(l, bb));
+                const float s2 = __fsub_rn(up, dn);
+                const float b2 = __fsub_rn(s2, up);
+                g.add(s2, __fsub_rn(__fsub_rn(up, __fsub_rn(s2, b2)), __fadd_rn(dn, b2)));
+                const float h = __fadd_rn(g.hi, g.lo);  // renormalised
+                g.lo = __fsub_rn(g.lo, __fsub_rn(h, g.hi));
+                g.hi = h;
+            }
+            const float ga = fabsf(g.hi);
+            if (pair_range(g.hi)) {
+                const float p = __fmul_rn(g.hi, g.hi);
+                dp.add(p, __fmaf_rn(2.0f * g.hi, g.lo, __fmaf_rn(g.hi, g.hi, -p)));
+                if (sd.replaces(ga)) {
+                    sd.best = ga;
+                    pd[0] = rr; pd[1] = l; pd[2] = up; pd[3] = dn;
+                } else if (sd.close(ga) && !(rr == pd[0] && l == pd[1] && up == pd[2] && dn == pd[3])) {
+                    exact_div(rr, l, up, dn);
+                }
+            } else if (!is_zero(g.hi)) {
+                const double dv = exact_div(rr, l, up, dn);
+                d64 = fma(dv, dv, d64);
+            }
+            if (++pending == PAIR_SITES) {
+                e.add(ep.value());
+                d.add(0.25 * dp.value());
+                ep = FPair{0.0f, 0.0f};
+                dp = FPair{0.0f, 0.0f};
+                pending = 0;
+            }
         }
-        e.add(erow);
-        d.add(0.25 * drow);
+        if (e64 != 0.0) e.add(e64);  // (a NaN is not zero)
+        if (d64 != 0.0) d.add(0.25 * d64);
     }
+    e.add(ep.value());
+    d.add(0.25 * dp.value());
+    exact_b2(pb[0], pb[1], pb[2]);
+    exact_div(pd[0], pd[1], pd[2], pd[3]);
     const double dmax = 0.5 * __longlong_as_double(static_cast<long long>(dmax_bits));
     block_reduce_write(Partial{e.s, e.c, d.s, d.c, dmax, sqrt(b2max), nf, 0ull}, part);
 }
 
 // Divergence of D (Sec. 4.2): D = (n_x q0, n_y q1, n_z q2) for the diagonal
 // dielectric eps_i = n_i^2 (Eq. 15: q_i = n_i E_i), central differences in
-// lattice units; the same partition and trees as diag_partial. The record's
-// div fields hold sum div^2 and max |div|, its B field max |D|; the energy
-// fields are zero.
+// lattice units. The record's div fields hold sum div^2 and max |div|, its B
+// field max |D|; the energy fields are zero.
+//
+// The FP64 pipe is the bound, so each product is formed once: a warp covers 30
+// columns with one more on either side (D_x of the neighbours by shuffle) and
+// walks down a tile's rows (D_y of the rows above and below in registers); six
+// FP64 operations per site, where a thread per site that formed its four
+// neighbours' products and |D|^2 itself took about thirty (4096^2: 760 us).
+// max |D|^2 is screened in FP32 (Screen), FP32 states are widened
+// on the integer pipe, and the factors 1/2 and 1/4 are applied to the reduced
+// values.
+constexpr int DIVD_COLS = 30 * (DIAG_THREADS / 32);
+constexpr int DIVD_MAX_ROWS = 32;
+
+__device__ __forceinline__ bool same_bits(double a, double b) {
+    return __double_as_longlong(a) == __double_as_longlong(b);
+}
+__device__ __forceinline__ double widen(float v) { return f2d_exact(v); }
+__device__ __forceinline__ double widen(double v) { return v; }
+// v truncated to FP32 on the integer pipe; *ok is cleared unless v is zero or
+// |v| in [2^-50, 2^60) (then the result is within 2^-22 of v, relatively).
+__device__ __forceinline__ float narrow_for_screen(double v, bool *ok) {
+    const unsigned hi = unsigned(__double2hiint(v)), lo = unsigned(__double2loint(v));
+    const unsigned ex = (hi >> 20) & 0x7ffu;
+    const bool zero = ((hi << 1) | lo) == 0u;
+    *ok = *ok && (zero || ex - (1023u - 50u) < 110u);
+    return zero ? 0.0f : __uint_as_float((hi & 0x80000000u) | ((ex - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+}
+
 template <typename T>
-__global__ void __launch_bounds__(DIAG_THREADS) divD_partial(const T *__restrict__ q, const double *__restrict__ idx,
-                                                             int Nx, int Ny, Partial *__restrict__ part) {
+__global__ void __launch_bounds__(DIAG_THREADS, 4) divD_partial(const T *__restrict__ q, const double *__restrict__ idx,
+                                                             int Nx, int Ny, int tile_rows,
+                                                             Partial *__restrict__ part) {
     const size_t P = size_t(Nx) * size_t(Ny);
     const T *q0 = q, *q1 = q + P, *q2 = q + 2 * P;
     const double *nx = idx, *ny = idx + P, *nz = idx + 2 * P;
     CSum d{0.0, 0.0};
-    double dmax = 0.0, d2max = 0.0;
+    unsigned long long dmax_bits = 0;
+    double d2max = 0.0;
+    Screen sc;
+    double pdx = 0.0, pdy = 0.0, pnz = 0.0;  // the pending site's D_x, D_y, n_z
+    T pv2 = T(0);
+    auto exact_d2 = [&](double dx, double dy, double n, T v) {
+        const double dz = n * widen(v);
+        const double d2 = dx * dx + dy * dy + dz * dz;
+        if (d2 > d2max) d2max = d2;
+    };
     unsigned long long nf = 0;
-    for (int y = blockIdx.x; y < Ny; y += gridDim.x) {
-        const int yp = y + 1 == Ny ? 0 : y + 1, ym = y == 0 ? Ny - 1 : y - 1;
-        const size_t r = size_t(y) * Nx;
-        double drow = 0.0;
-        for (int x = threadIdx.x; x < Nx; x += blockDim.x) {
-            const size_t i = r + x;
-            const int xp = x + 1 == Nx ? 0 : x + 1, xm = x == 0 ? Nx - 1 : x - 1;
-            const size_t ixp = r + xp, ixm = r + xm, iyp = size_t(yp) * Nx + x, iym = size_t(ym) * Nx + x;
-            const double dv = 0.5 * (nx[ixp] * double(q0[ixp]) - nx[ixm] * double(q0[ixm])) +
-                              0.5 * (ny[iyp] * double(q1[iyp]) - ny[iym] * double(q1[iym]));
-            drow = fma(dv, dv, drow);
-            dmax = fmax(dmax, fabs(dv));
-            const double dx = nx[i] * double(q0[i]), dy = ny[i] * double(q1[i]), dz = nz[i] * double(q2[i]);
-            d2max = fmax(d2max, dx * dx + dy * dy + dz * dz);
-            if (!finite_val(q0[i]) || !finite_val(q1[i]) || !finite_val(q2[i])) ++nf;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ctiles = (Nx + DIVD_COLS - 1) / DIVD_COLS, rtiles = (Ny + tile_rows - 1) / tile_rows;
+    for (long long t = blockIdx.x; t < (long long)ctiles * rtiles; t += gridDim.x) {
+        const int xc = int(t % ctiles) * DIVD_COLS + warp * 30 + lane - 1;
+        const int y0 = int(t / ctiles) * tile_rows, y1 = min(y0 + tile_rows, Ny);
+        const bool mine = lane >= 1 && lane <= 30 && xc < Nx;
+        int x = xc % Nx;  // halo columns wrap around; columns past them are not used
+        x = x < 0 ? x + Nx : x;
+        auto dy_of = [&](int y) {
+            const int w = y < 0 ? y + Ny : (y >= Ny ? y - Ny : y);
+            const size_t i = size_t(w) * Nx + x;
+            return ny[i] * widen(q1[i]);
+        };
+        double below = dy_of(y0 - 1), here = dy_of(y0), sum = 0.0;
+        for (int y = y0; y < y1; ++y) {
+            const size_t i = size_t(y) * Nx + x;
+            const T v0 = q0[i], v1 = q1[i], v2 = q2[i];
+            const double above = dy_of(y + 1);
+            const double dx = nx[i] * widen(v0);
+            const double left = __shfl_up_sync(0xffffffffu, dx, 1), right = __shfl_down_sync(0xffffffffu, dx, 1);
+            const double dv = (right - left) + (above - below);
+            sum = fma(dv, dv, sum);  // (lanes whose column is another warp's do not add theirs)
+            const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) &
+                                          0x7fffffffffffffffull;
+            if (mine) {
+                if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
+                if (!finite_val(v0) || !finite_val(v1) || !finite_val(v2)) ++nf;
+            }
+            bool ok = true;
+            const double dnz = nz[i];
+            const float fx = narrow_for_screen(dx, &ok), fy = narrow_for_screen(here, &ok);
+            const float fz = narrow_for_screen(dnz, &ok) * narrow_for_screen(widen(v2), &ok);
+            const float f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+            if (mine) {
+                if (!ok) {
+                    exact_d2(dx, here, dnz, v2);
+                } else if (sc.replaces(f)) {
+                    sc.best = f;
+                    pdx = dx;
+                    pdy = here;
+                    pnz = dnz;
+                    pv2 = v2;
+                } else if (sc.close(f) && !(same_bits(dx, pdx) && same_bits(here, pdy) && same_bits(dnz, pnz) &&
+                                            v2 == pv2)) {
+                    exact_d2(dx, here, dnz, v2);
+                }
+            }
+            below = here;
+            here = above;
         }
-        d.add(drow);
+        if (mine) d.add(0.25 * sum);
     }
+    exact_d2(pdx, pdy, pnz, pv2);
+    const double dmax = 0.5 * __longlong_as_double(static_cast<long long>(dmax_bits));
     block_reduce_write(Partial{0.0, 0.0, d.s, d.c, dmax, sqrt(d2max), nf, 0ull}, part);
 }
 
+// One block combines the partial records in a fixed tree: half of its warps the
+// energy sums (and max |div|, the non-finite count), the other half the
+// divergence sums (and max |B|), lanes by shuffle. Latency is all it costs, a
+// chain of FP64 additions per level (both sums in every thread, through shared
+// memory: 13 us).
 __global__ void __launch_bounds__(DIAG_THREADS) diag_final(const Partial *__restrict__ part, int n,
                                                            DiagResult *__restrict__ out) {
-    CSum e{0.0, 0.0}, d{0.0, 0.0};
-    double dmax = 0.0, bmax = 0.0;
+    constexpr int HALF = DIAG_THREADS / 2, WARPS = HALF / 32;
+    const bool first = threadIdx.x < HALF;
+    CSum s{0.0, 0.0};
+    double mx = 0.0;
     unsigned long long nf = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = int(threadIdx.x % HALF); i < n; i += HALF) {
         const Partial p = part[i];
-        e.merge(CSum{p.e_s, p.e_c});
-        d.merge(CSum{p.d_s, p.d_c});
-        dmax = fmax(dmax, p.dmax);
-        bmax = fmax(bmax, p.bmax);
+        s.merge(first ? CSum{p.e_s, p.e_c} : CSum{p.d_s, p.d_c});
+        const double m = first ? p.dmax : p.bmax;  // non-negative or NaN: the larger number
+        mx = m > mx ? m : mx;
         nf += p.nonfinite;
     }
-    __shared__ Partial sh[DIAG_THREADS];
-    sh[threadIdx.x] = Partial{e.s, e.c, d.s, d.c, dmax, bmax, nf, 0ull};
-    __syncthreads();
-    for (int w = DIAG_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            Partial a = sh[threadIdx.x];
-            const Partial b = sh[threadIdx.x + w];
-            CSum es{a.e_s, a.e_c}, ds{a.d_s, a.d_c};
-            es.merge(CSum{b.e_s, b.e_c});
-            ds.merge(CSum{b.d_s, b.d_c});
-            a.e_s = es.s; a.e_c = es.c; a.d_s = ds.s; a.d_c = ds.c;
-            a.dmax = fmax(a.dmax, b.dmax);
-            a.bmax = fmax(a.bmax, b.bmax);
-            a.nonfinite += b.nonfinite;
-            sh[threadIdx.x] = a;
-        }
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        s.merge(CSum{__shfl_down_sync(0xffffffffu, s.s, o), __shfl_down_sync(0xffffffffu, s.c, o)});
+        const double m = __shfl_down_sync(0xffffffffu, mx, o);
+        mx = m > mx ? m : mx;
+        nf += __shfl_down_sync(0xffffffffu, nf, o);
     }
-    if (threadIdx.x == 0) {
-        const Partial a = sh[0];
-        out->energy_sum = a.e_s + a.e_c;
-        out->div_sq_sum = a.d_s + a.d_c;
-        out->div_max = a.dmax;
-        out->b_max = a.bmax;
-        out->nonfinite = a.nonfinite;
+    __shared__ CSum ss[2 * WARPS];
+    __shared__ double sm[2 * WARPS];
+    __shared__ unsigned long long sn[2 * WARPS];
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) {
+        ss[w] = s;
+        sm[w] = mx;
+        sn[w] = nf;
+    }
+    __syncthreads();
+    if (threadIdx.x % HALF == 0) {
+        for (int k = 1; k < WARPS; ++k) {
+            s.merge(ss[w + k]);
+            mx = sm[w + k] > mx ? sm[w + k] : mx;
+            nf += sn[w + k];
+        }
+        if (first) {
+            out->energy_sum = s.s + s.c;
+            out->div_max = mx;
+            out->nonfinite = nf;
+        } else {
+            out->div_sq_sum = s.s + s.c;
+            out->b_max = mx;
+        }
     }
 }
 
@@ -313,12 +477,17 @@ cudaError_t launch_diagnostics(const void *q, int precision, int Nx, int Ny, voi
 
 cudaError_t launch_divD(const void *q, int precision, const double *index, int Nx, int Ny, void *scratch,
                         DiagResult *out_dev, cudaStream_t st) {
-    const int G = diag_blocks(Nx, Ny);
+    // tiles of at most 32 rows, lower where that would leave blocks idle
+    const int ctiles = (Nx + DIVD_COLS - 1) / DIVD_COLS;
+    int rows = int((long long)ctiles * Ny / diag_blocks(Nx, Ny));
+    rows = rows < 4 ? 4 : (rows > DIVD_MAX_ROWS ? DIVD_MAX_ROWS : rows);
+    const long long tiles = (long long)ctiles * ((Ny + rows - 1) / rows);
+    const int G = tiles < diag_blocks(Nx, Ny) ? int(tiles) : diag_blocks(Nx, Ny);
     Partial *part = static_cast<Partial *>(scratch);
     if (precision == 0)
-        divD_partial<float><<<G, DIAG_THREADS, 0, st>>>(static_cast<const float *>(q), index, Nx, Ny, part);
+        divD_partial<float><<<G, DIAG_THREADS, 0, st>>>(static_cast<const float *>(q), index, Nx, Ny, rows, part);
     else
-        divD_partial<double><<<G, DIAG_THREADS, 0, st>>>(static_cast<const double *>(q), index, Nx, Ny, part);
+        divD_partial<double><<<G, DIAG_THREADS, 0, st>>>(static_cast<const double *>(q), index, Nx, Ny, rows, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     diag_final<<<1, DIAG_THREADS, 0, st>>>(part, G, out_dev);
