@@ -20,11 +20,10 @@ __device__ void shear_pair_f32(double ang, float &tf, float &sf) {
 }
 
 // FP32 pair (t, s) near (tan(a / 2), sin(a)) for the four-FMA rotation of the
-// sweep, whose matrix is [1 - s t, s; -s, 1 - s t]: among FP32 values within a
-// few ulps of the correctly rounded ones, the pair that brings
+// sweep, whose matrix is [1 - s t, s; -s, 1 - s t]: among FP32 values next to the
+// correctly rounded ones, the pair that brings
 // (1 - s t)^2 + s^2 - 1 = s (s (1 + t^2) - 2 t) (evaluated in FP64) closest to
-// zero, so that each rotation keeps the energy (Eq. 27) to ~1e-12, with the
-// angle changed by a few ulps at most.
+// zero, so that each rotation keeps the energy (Eq. 27) to ~1e-12.
 __device__ void tuned_pair_f32(double ang, float &tf, float &sf) {
     const float t0 = (float)tan(0.5 * ang), s0 = (float)sin(ang);
     if (!(fabsf(t0) >= 1e-30f) || !(fabsf(s0) >= 1e-30f)) {  // zero or denormal: keep the rounded values
@@ -32,12 +31,13 @@ __device__ void tuned_pair_f32(double ang, float &tf, float &sf) {
         sf = s0;
         return;
     }
-    // for each t the best s is the FP32 value nearest to 2 t / (1 + t^2)
+    // for each t the best s is the FP32 value nearest to 2 t / (1 + t^2); t moves
+    // by one ulp at most (four brought the norm no closer than the arithmetic's own
+    // rounding and put 1e-7 of angle error, 4% in a 48-step run, in its place)
     double best = 1e300;
     tf = t0;
     sf = s0;
-    for (int k = 0; k <= 8; ++k) {
-        const int dt = (k + 1) / 2 * (k & 1 ? 1 : -1);  // 0, 1, -1, .. 4, -4: the nearest of equals stays
+    for (int dt = -1; dt <= 1; ++dt) {
         const float tc = __int_as_float(__float_as_int(t0) + dt);
         const double t = (double)tc, q = 1.0 + t * t;
         const float sc = (float)(2.0 * t / q);
