@@ -155,32 +155,40 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
     }
 }
 
-// flags[strip][r]: whether any V pair of the strip's columns is nonzero in rows
-// [r - march_flag_back(2), r + MARCH_GROUP - 1] (periodic).
+// flags[strip][r] (MARCH_V, MARCH_C): whether any V pair of the strip's columns
+// is nonzero in rows [r - march_flag_back(2), r + MARCH_GROUP - 1], and whether
+// any C pair of rows [r - MARCH_SAME_BACK, r + MARCH_SAME_AHEAD] differs from the
+// row above it.
 constexpr int FLAG_ROWS = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) march_flags_kernel(const T *__restrict__ rec, unsigned char *__restrict__ flags,
-                                                          MarchGeo g) {
-    constexpr int BACK = march_flag_back(2);
-    __shared__ unsigned char rf[FLAG_ROWS + BACK + MARCH_GROUP];
+                                                          int fam, MarchGeo g) {
+    constexpr int BACK = march_flag_back(2) > MARCH_SAME_BACK ? march_flag_back(2) : MARCH_SAME_BACK;
+    constexpr int AHEAD = MARCH_GROUP - 1 > MARCH_SAME_AHEAD ? MARCH_GROUP - 1 : MARCH_SAME_AHEAD;
+    __shared__ unsigned char rf[FLAG_ROWS + BACK + AHEAD];
     const int strip = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
-    static_assert(BACK <= MARCH_ABOVE && MARCH_GROUP <= MARCH_BELOW, "rows of the window have records");
+    const int cfields = fam ? 4 : 2;  // TM: C_Y is not stored
+    static_assert(BACK < MARCH_ABOVE && AHEAD < MARCH_BELOW && F_CX == 0 && F_CY == 2, "rows and fields compared");
     for (int r0 = blockIdx.y * FLAG_ROWS; r0 < g.Ny; r0 += gridDim.y * FLAG_ROWS) {
         const int n = min(FLAG_ROWS, g.Ny - r0);
-        for (int k = warp; k < n + BACK + MARCH_GROUP - 1; k += 8) {
-            const T *v = rec + ((size_t(strip) * rows + MARCH_ABOVE + r0 - BACK + k) * MARCH_FIELDS + F_VX) * g.W;
-            bool nz = false;
-            for (int c = lane; c < 4 * g.W; c += 32) nz = nz || v[c] != T(0);
+        for (int k = warp; k < n + BACK + AHEAD; k += 8) {
+            const T *const r = rec + (size_t(strip) * rows + MARCH_ABOVE + r0 - BACK + k) * MARCH_FIELDS * g.W;
+            const T *const above = r - MARCH_FIELDS * g.W;
+            bool nz = false, differs = false;
+            for (int c = lane; c < 4 * g.W; c += 32) nz = nz || r[F_VX * g.W + c] != T(0);
+            for (int c = lane; c < cfields * g.W; c += 32) differs = differs || r[c] != above[c];
             nz = __any_sync(0xffffffffu, nz);
-            if (lane == 0) rf[k] = nz ? 1 : 0;
+            differs = __any_sync(0xffffffffu, differs);
+            if (lane == 0) rf[k] = (unsigned char)((nz ? MARCH_V : 0) | (differs ? MARCH_C : 0));
         }
         __syncthreads();
         for (int k = threadIdx.x; k < n; k += 256) {
-            unsigned char f = 0;
-            for (int i = 0; i < BACK + MARCH_GROUP; ++i) f |= rf[k + i];
-            flags[size_t(strip) * g.Ny + r0 + k] = f;
+            unsigned f = 0;
+            for (int i = -march_flag_back(2); i < MARCH_GROUP; ++i) f |= rf[k + BACK + i] & MARCH_V;
+            for (int i = -MARCH_SAME_BACK; i <= MARCH_SAME_AHEAD; ++i) f |= rf[k + BACK + i] & MARCH_C;
+            flags[size_t(strip) * g.Ny + r0 + k] = (unsigned char)f;
         }
         __syncthreads();
     }
@@ -250,11 +258,11 @@ cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, 
         if (precision == 0) {
             march_records_kernel<float><<<grid, g.W, 0, st>>>(n, static_cast<float *>(rec), fam0 + z, g, delta,
                                                               interleaved, unitary);
-            march_flags_kernel<float><<<fgrid, 256, 0, st>>>(static_cast<const float *>(rec), flags, g);
+            march_flags_kernel<float><<<fgrid, 256, 0, st>>>(static_cast<const float *>(rec), flags, fam0 + z, g);
         } else {
             march_records_kernel<double><<<grid, g.W, 0, st>>>(n, static_cast<double *>(rec), fam0 + z, g, delta,
                                                                interleaved, unitary);
-            march_flags_kernel<double><<<fgrid, 256, 0, st>>>(static_cast<const double *>(rec), flags, g);
+            march_flags_kernel<double><<<fgrid, 256, 0, st>>>(static_cast<const double *>(rec), flags, fam0 + z, g);
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -242,6 +242,13 @@ constexpr int MARCH_FIELDS = 8;
 constexpr int F_CX = 0, F_CY = 2, F_VX = 4, F_VY = 6;
 constexpr int MARCH_ABOVE = 20, MARCH_BELOW = 24;
 constexpr int MARCH_GROUP = 4;  // rows covered by a flag
+// Flag bits of (strip, row r), for a group of iterations whose first level-0
+// row is r: some V angle applied in it is nonzero; the C fields of rows
+// [r - 6, r + 5] are not all the same (the rows that it copies and those whose
+// places they take: level 0 rows up to r + 5 over ones three before, later
+// levels rows from r - 4 over ones two before).
+constexpr unsigned MARCH_V = 1, MARCH_C = 2;
+constexpr int MARCH_SAME_BACK = 5, MARCH_SAME_AHEAD = 5;
 constexpr __host__ __device__ int march_flag_back(int K) { return 5 * (K - 1) + 4; }
 struct MarchGeo {
     int Nx, Ny;
