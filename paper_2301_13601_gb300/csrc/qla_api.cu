@@ -167,7 +167,8 @@ bool family_has(const qla_ctx *c, int comp) {
     return c->opt.families == QLA_FAMILY_TM ? tm : !tm;
 }
 
-qla_status launch_pass(qla_ctx *c, int K) {
+// chained: the last launch on the stream was a pass of this context.
+qla_status launch_pass(qla_ctx *c, int K, bool chained) {
     if (c->march) {
         // K = 4 in passes of two steps; FP64 and, without an explicit choice,
         // small FP32 lattices in passes of one: the same values in less time (us
@@ -182,7 +183,8 @@ qla_status launch_pass(qla_ctx *c, int K) {
             const cudaError_t e = qla::launch_march(
                 c->geo, per, c->state[c->cur], c->state[c->cur ^ 1], c->coef, c->nfam, c->fam0,
                 c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, c->opt.potential == QLA_POT_UNITARY ? 1 : 0,
-                c->stream);
+                chained, c->stream);
+            chained = true;
             if (e != cudaSuccess) return fail(c, QLA_ECUDA, "sweep launch (K=%d): %s", K, cudaGetErrorString(e));
             c->cur ^= 1;
         }
@@ -514,7 +516,7 @@ qla_status qla_step(qla_ctx *c, long long nsteps) {
     while (left > 0) {
         int k = c->K;
         while (k > 1 && (k > left || !qla::sweep_supported(c->opt.precision, k))) --k;
-        s = launch_pass(c, k);
+        s = launch_pass(c, k, left < nsteps);
         if (s != QLA_OK) return s;
         left -= k;
         c->steps += k;

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSche
             const int strip = w % args.strips, chunk = w / args.strips;
             const int y0 = int((long long)args.Ny * chunk / args.chunks);
             const int y1 = int((long long)args.Ny * (chunk + 1) / args.chunks);
-            march_share<float, BC, kBatchSteps, BD, BU, INTER, UNIT, VEC>(args, args.fam[0], strip, y0, y1,
+            march_share<float, BC, kBatchSteps, BD, BU, INTER, UNIT, VEC, false>(args, args.fam[0], strip, y0, y1,
                                                                            smem_raw + warp * L::WARP, lane);
         }
         __threadfence();

@@ -269,10 +269,11 @@ bool march_vectors(const MarchGeo &g);
 // chunk: rows per range (0: automatic).
 void march_plan(MarchGeo *g, int nfam, int chunk, int sms);
 // One pass of K steps (FP32: 1, 2; FP64: 1) over the families f0 .. f0 + nfam - 1.
-// mem: the advanced families' records, then their flags (march_bytes).
+// mem: the advanced families' records, then their flags (march_bytes). chained:
+// the last launch on the stream was such a pass, over the same records.
 size_t march_bytes(const MarchGeo &g, int nfam);
 cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out, const void *mem, int nfam, int fam0,
-                         int interleaved, int unitary, cudaStream_t st);
+                         int interleaved, int unitary, bool chained, cudaStream_t st);
 // Records and flags from the device index planes n[3][Ny][Nx] (double).
 cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, int nfam, int fam0, double delta,
                                  int precision, int interleaved, int unitary, cudaStream_t st);

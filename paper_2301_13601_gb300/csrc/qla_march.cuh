@@ -80,6 +80,7 @@ struct MarchArgs {
     int w_valid, halo, strips;  // strip geometry (MarchGeo)
     int chunks;                 // row ranges per strip, one warp each
     int ctas_fam;               // CTAs per family
+    int chained;                // the launch before it on the stream is a pass over the same records
 };
 
 template <typename T, int C, int K, int D, bool INTER>
@@ -394,7 +395,19 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
 // warp's shared memory. VEC: rows keep the alignment of the lane's vectors (Nx a
 // multiple of C) and a plane holds less than 2^32 bytes; else the state is copied
 // and stored element by element, with 64-bit offsets.
-template <typename T, int C, int K, int D, int U, bool INTER, bool UNIT, bool VEC>
+// Passes of one FP32 step are chained: each may be launched while the one before
+// it finishes its last group of rows, and waits for its end before it reads the
+// state (griddepcontrol). Such a pass, on a small lattice, is about as long as a
+// launch takes: 16 steps of 256^2 76 -> 64 us. Passes of two FP32 steps are not:
+// they are longer, and the two instructions cost the fullest register file 3%
+// (2048^2 4.02 -> 4.14 ms, 8192^2 9.85 -> 10.15); nor are FP64's, whose waiting
+// CTAs keep other streams' CTAs off the pipe (256^2 1.23 -> 1.26 ms).
+template <typename T>
+constexpr bool march_chains(int K) {
+    return sizeof(T) == 4 && K == 1;
+}
+
+template <typename T, int C, int K, int D, int U, bool INTER, bool UNIT, bool VEC, bool CHAIN>
 __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &F, int strip, int y0, int y1, unsigned char *sm,
                                             int lane) {
     using L = MarchLayout<T, C, K, D, INTER>;
@@ -504,6 +517,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     for (int j = 1; j < K; ++j) copyc(j, 0, -(4 + MARCH_LAG) * j);
     if (von & MARCH_V)
         for (int j = 0; j < K; ++j) copyv(j, 0, -(4 + MARCH_LAG) * j);
+    if constexpr (CHAIN) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 #pragma unroll
     for (int k = 0; k < D - 1; ++k) {
         copy0(k * L::REC, off_c, k, true);
@@ -529,6 +543,8 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
         const bool on = (von & MARCH_V) != 0, vcopy = ((von | von1 | (U < 4 ? von2 : 0u)) & MARCH_V) != 0;
         // (the first D - 1 rows came with the prologue, the ring is full after iteration 0)
         const bool ccopy = it0 == 0 || (von & MARCH_C) != 0;
+        if constexpr (CHAIN)
+            if (g == ngroups - 1) asm volatile("griddepcontrol.launch_dependents;\n");
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int i = U == 4 ? u : it0 + u;  // iteration index mod 4 (compile time when U = 4)
@@ -626,7 +642,8 @@ __global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_cons
     const int strip = w % A.strips, chunk = w / A.strips;
     const int y0 = int((long long)A.Ny * chunk / A.chunks);
     const int y1 = int((long long)A.Ny * (chunk + 1) / A.chunks);
-    march_share<T, C, K, D, U, INTER, UNIT, VEC>(A, A.fam[layer], strip, y0, y1, smem_raw + warp * L::WARP, lane);
+    march_share<T, C, K, D, U, INTER, UNIT, VEC, march_chains<T>(K)>(A, A.fam[layer], strip, y0, y1,
+                                                                     smem_raw + warp * L::WARP, lane);
 }
 
 // A family's entry (fam: 0 = TM, 1 = TE).
@@ -660,7 +677,17 @@ cudaError_t launch_march_t(const MarchArgs &a, int nfam, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     MarchArgs m = a;
     m.ctas_fam = (a.strips * a.chunks + WPC - 1) / WPC;
-    kern<<<unsigned(m.ctas_fam) * unsigned(nfam), 32 * WPC, L::WARP * WPC, st>>>(m);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(m.ctas_fam) * unsigned(nfam));
+    cfg.blockDim = dim3(32 * WPC);
+    cfg.dynamicSmemBytes = L::WARP * WPC;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = march_chains<T>(K) && a.chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kern, m);
     return cudaGetLastError();
 }
 template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool VEC>

@@ -83,3 +83,25 @@ def test_single_operators_read_the_records():
                 sim.debug_apply(op)
                 out.append(sim.get_fields(np.float32))
         assert np.array_equal(*out), op
+
+
+# one row range, several warps and CTAs, more CTAs than the device takes at once
+@pytest.mark.parametrize("Nx, Ny, chunk_rows", [(64, 8, 0), (256, 256, 0), (301, 207, 0), (1024, 256, 1)])
+def test_chained_passes_match_single_ones(Nx, Ny, chunk_rows):
+    """Passes of one call are launched before the one before them has ended; a
+    call of one step has nothing to overlap with. The same operations: the same
+    bits, also when another context's passes run between them."""
+    n = medium(Nx, Ny)
+    q = np.random.default_rng(3).standard_normal((6, Ny, Nx))
+    steps = 41
+    kw = dict(chunk_rows=chunk_rows, steps_per_pass=1)
+    with Simulation(*n, 0.2, **kw) as one, Simulation(*n, 0.2, **kw) as many, Simulation(*n, 0.2, **kw) as beside:
+        for sim in (one, many, beside):
+            sim.set_fields(q)
+        for _ in range(steps):
+            one.step(1)
+        many.step(steps)
+        beside.step(steps)
+        ref = one.get_fields()
+        assert np.array_equal(many.get_fields(), ref)
+        assert np.array_equal(beside.get_fields(), ref)
