@@ -731,6 +731,20 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
     if (warp == CONV_MMA_WARP) tc::tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
+// Tensor map of rows of W 64-channel pixels, boxes of n pixels in swizzled lines.
+cudaError_t pixel_map(CUtensorMap *map, const void *base, int W, long long rows, unsigned n) {
+    const EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint64_t dim[3] = {64, cuuint64_t(W), cuuint64_t(rows)};
+    const cuuint64_t str[2] = {128, cuuint64_t(W) * 128};
+    const cuuint32_t one[3] = {1, 1, 1}, box[3] = {64, n, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dim, str, box, one,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? cudaSuccess
+               : cudaErrorInvalidValue;
+}
+
 template <int CCH, int NOUT, bool DG>
 cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
     using L = ConvLayout<CCH, NOUT>;
@@ -745,18 +759,9 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
     ConvMaps maps;
     memset(&maps, 0, sizeof(maps));
     if (L::SWZ) {
-        const EncodeTiledFn fn = encode_tiled_fn();
-        if (!fn) return cudaErrorNotSupported;
-        const cuuint64_t dim[3] = {64, cuuint64_t(a.W), cuuint64_t(a.nimg) * cuuint64_t(a.H)};
-        const cuuint64_t str[2] = {128, cuuint64_t(a.W) * 128};
-        const cuuint32_t one[3] = {1, 1, 1};
-        for (int k = 0; k < 2; ++k) {
-            const cuuint32_t box[3] = {64, k ? 1u : 128u, 1};
-            if (fn(k ? &maps.px1 : &maps.px128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(a.x), dim, str,
-                   box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                return cudaErrorInvalidValue;
-        }
+        const long long img_rows = (long long)a.nimg * a.H;
+        if ((e = pixel_map(&maps.px128, a.x, a.W, img_rows, 128)) != cudaSuccess) return e;
+        if ((e = pixel_map(&maps.px1, a.x, a.W, img_rows, 1)) != cudaSuccess) return e;
     }
     conv3x3_tc_kernel<CCH, NOUT, DG><<<grid, CONV_THREADS, L::SMEM_LAUNCH, st>>>(a, maps);
     return cudaGetLastError();
@@ -765,39 +770,59 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // Weight gradient on the tensor cores:
 //   dW[n][c][ky][kx] = sum_p g[p][n] x[p + (ky-1, kx-1)][c]
-// as D[m][n] = sum_k A[m][k] B[n][k] with K = pixels and both operands
-// MN-major (NHWC rows give 8 consecutive channels per 16 bytes). A rows are
-// (ky, c) for two consecutive halo rows stacked in M = 128 (ky = 0, 1 in one
-// tile; ky = 2 and an unused half in the other); kx is a 16-byte shift of the
-// start address along K. Six accumulator tiles (2 row pairs x 3 kx) of N = NT
-// columns stay in TMEM for all of a CTA's rows; at the end each CTA writes its
-// partial sums [9][NT][64] (FP32), reduced over CTAs in a fixed order later,
-// and those of the bias gradient [NT], summed by warps that the tensor cores
-// leave idle (a kernel of its own read g once more, 22 us per layer).
+// as D[m][n] = sum_k A[m][k] B[n][k] with K = the 128 pixels of a tile of x and
+// both operands MN-major. A rows are (ky, c) for two consecutive rows of x stacked
+// in M = 128 (ky = 0, 1 in one tile; ky = 2 and an unused half in the other); B
+// columns are (kx, n): g[p + (0, 1 - kx)] for the three kx side by side, N = 3 NT,
+// so that an A tile is read from shared memory once for the three of them (one
+// MMA of N = 64 per kx read 6 KB for 32 cycles of arithmetic, and, with kx as a
+// shift of A, across lines: 80 cycles each). The tile's edges need g's halo pixels,
+// not x's. With 64 channels a pixel of g is a swizzled line, and the next kx is
+// the operand that starts one line earlier: no copies. At 4 x 256 x 512 the
+// 64 -> 64 layers take 36 us (54 before), of which 20 are their DRAM traffic
+// (134 MB) and 22 their MMAs; 16 -> 64 35 (48), 64 -> 16 25 (42).
+// Two accumulator tiles (the row pairs) stay in TMEM for all of a CTA's rows; at
+// the end each CTA writes its partial sums [9][NT][64] (FP32), reduced over CTAs
+// in a fixed order later, and those of the bias gradient [NT], summed by warps
+// that the tensor cores leave idle (a kernel of its own read g once more, 22 us
+// per layer).
 // The x ring has one mirror slot after the last, a copy of slot 0, so that two
 // consecutive rows are always adjacent in memory. Source x may have 16 or 64
 // channels (16: the other chunks stay zero).
 // ---------------------------------------------------------------------------
 constexpr int WG_SUM_WARPS = 4;  // warps that sum the bias gradient
+// The load warp and the epilogue warps that sum nothing copy 16-channel rows.
+constexpr int WG_LOADERS = 1 + CONV_EPI_WARPS - WG_SUM_WARPS;
 
-template <int NT>
+template <int CS, int NT>
 struct WgradLayout {
-    static constexpr int HP = 130;
+    // 64-channel operands lie in swizzled lines of one pixel each, brought by TMA;
+    // 16-channel ones in planes of 8-channel chunks, copied by WG_LOADERS warps.
+    static constexpr bool SWX = CS == 64, SWG = NT == 64;
     static constexpr int NSX = 6;
-    static constexpr int XSLOT = 8 * HP * 16;
+    static constexpr int XSLOT = 128 * 128;
     static constexpr int X_BYTES = (NSX + 1) * XSLOT;
     static constexpr int NSG = 4;
-    static constexpr int GSLOT = (NT / 8) * 128 * 16;
-    static constexpr int G_OFF = ((X_BYTES + 1023) / 1024) * 1024;
+    static constexpr int GSLOT = SWG ? 130 * 128 : 3 * NT * 128 * 2;  // halo pixels, or three shifted copies
+    static constexpr int G_OFF = X_BYTES;
     static constexpr int SMEM = G_OFF + NSG * GSLOT;
-    static constexpr int TMEM_COLS = NT == 64 ? 512 : 128;  // 6 tiles x NT columns
+    static constexpr int TMEM_COLS = NT == 64 ? 512 : 128;  // 2 tiles x 3 NT columns
+};
+
+struct WgradMaps {
+    CUtensorMap x128, g128, g1;
 };
 
 template <int CS, int NT>
-__global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradArgs a) {
-    using L = WgradLayout<NT>;
-    constexpr int NSX = L::NSX, NSG = L::NSG, HP = L::HP;
-    constexpr int CCS = CS / 8;  // source chunks per pixel
+__global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradArgs a,
+                                                                   const __grid_constant__ WgradMaps maps) {
+    using L = WgradLayout<CS, NT>;
+    constexpr int NSX = L::NSX, NSG = L::NSG;
+    constexpr bool SWX = L::SWX, SWG = L::SWG;
+    constexpr int CCS = CS / 8, CCT = NT / 8;  // chunks per pixel
+    // A warp copies 4 (or 2) chunks of 8 (or 16) pixels at a time: whole lines of
+    // shared memory, half lines of global memory.
+    constexpr int XB = CCS < 4 ? CCS : 4, GB = CCT < 4 ? CCT : 4;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint64_t xf_bar[NSX], xe_bar[NSX], gf_bar[NSG], ge_bar[NSG], done_bar;
     __shared__ uint32_t tmem_base_s;
@@ -811,15 +836,17 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
     uint8_t *Xs = smem;
     uint8_t *Gs = smem + L::G_OFF;
 
-    for (int i = tid; i < L::X_BYTES / 16; i += CONV_THREADS) reinterpret_cast<uint4 *>(Xs)[i] = make_uint4(0, 0, 0, 0);
+    if constexpr (!SWX)  // the other chunks stay zero
+        for (int i = tid; i < L::X_BYTES / 16; i += CONV_THREADS)
+            reinterpret_cast<uint4 *>(Xs)[i] = make_uint4(0, 0, 0, 0);
     if (warp == CONV_MMA_WARP) tc::tmem_alloc(&tmem_base_s, L::TMEM_COLS);
     if (tid == 0) {
         for (int s = 0; s < NSX; ++s) {
-            tc::mbar_init(&xf_bar[s], 32);
+            tc::mbar_init(&xf_bar[s], SWX ? 1 : 32 * WG_LOADERS);
             tc::mbar_init(&xe_bar[s], 1);
         }
         for (int s = 0; s < NSG; ++s) {
-            tc::mbar_init(&gf_bar[s], 32);
+            tc::mbar_init(&gf_bar[s], SWG ? 1 : 32 * WG_LOADERS);
             tc::mbar_init(&ge_bar[s], 1 + WG_SUM_WARPS);
         }
         tc::mbar_init(&done_bar, 1);
@@ -831,7 +858,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
     tc::fence_after_sync();
     const uint32_t tmem = tmem_base_s;
 
-    if (warp == CONV_LOAD_WARP) {
+    if (warp == CONV_LOAD_WARP || (!(SWX && SWG) && warp >= WG_SUM_WARPS && warp < CONV_EPI_WARPS)) {
+        const bool tma = warp == CONV_LOAD_WARP && lane == 0;
+        const int loader = 32 * (warp == CONV_LOAD_WARP ? 0 : warp - WG_SUM_WARPS + 1) + lane;
         const __nv_bfloat16 *xg = static_cast<const __nv_bfloat16 *>(a.x);
         const __nv_bfloat16 *gg = static_cast<const __nv_bfloat16 *>(a.g);
         long long gx = 0, gn = 0;
@@ -841,28 +870,53 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
             if (gx >= NSX && !tc::mbar_wait(&xe_bar[slot], uint32_t((gx / NSX - 1) & 1), CONV_WAIT_TRIES)) return false;
             int yy = (sg.y_s - 1 + j) % H;
             yy = yy < 0 ? yy + H : yy;
-            const __nv_bfloat16 *row = xg + ((size_t)sg.img * H + yy) * W * CS;
-            for (int i = lane; i < CCS * HP; i += 32) {
-                const int c = i % CCS, px = i / CCS;
-                int xx = sg.x0 + px - 1;
-                xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
-                const __nv_bfloat16 *src = row + (size_t)xx * CS + 8 * c;
-                cp_async16(Xs + ((slot * 8 + c) * HP + px) * 16, src);
-                if (slot == 0) cp_async16(Xs + ((NSX * 8 + c) * HP + px) * 16, src);
+            const int row = sg.img * H + yy;
+            if constexpr (SWX) {
+                if (tma) {
+                    const uint32_t dst = tc::smem_addr(Xs) + uint32_t(slot * L::XSLOT);
+                    tc::mbar_arrive_expect_tx(&xf_bar[slot], (slot == 0 ? 2 : 1) * L::XSLOT);
+                    conv_tma(dst, &maps.x128, sg.x0, row, &xf_bar[slot]);
+                    if (slot == 0) conv_tma(dst + NSX * L::XSLOT, &maps.x128, sg.x0, row, &xf_bar[slot]);
+                }
+                __syncwarp();
+            } else {
+                const __nv_bfloat16 *src = xg + ((size_t)row * W + sg.x0) * CS;
+                for (int i = loader; i < CCS * 128; i += 32 * WG_LOADERS) {
+                    const int c = i % XB + i / (XB * 128) * XB, px = i / XB % 128;
+                    cp_async16(Xs + ((slot * 8 + c) * 128 + px) * 16, src + px * CS + 8 * c);
+                    if (slot == 0) cp_async16(Xs + ((NSX * 8 + c) * 128 + px) * 16, src + px * CS + 8 * c);
+                }
+                cp_async_arrive_noinc(&xf_bar[slot]);
             }
-            cp_async_arrive_noinc(&xf_bar[slot]);
             ++gx;
             return true;
         };
         auto load_g = [&](const ConvSeg &sg, int i) -> bool {
             const int slot = int(gn % NSG);
             if (gn >= NSG && !tc::mbar_wait(&ge_bar[slot], uint32_t((gn / NSG - 1) & 1), CONV_WAIT_TRIES)) return false;
-            const __nv_bfloat16 *row = gg + (((size_t)sg.img * H + sg.y_s + i) * W + sg.x0) * NT;
-            for (int k = lane; k < (NT / 8) * 128; k += 32) {
-                const int c = k % (NT / 8), px = k / (NT / 8);
-                cp_async16(Gs + slot * L::GSLOT + (c * 128 + px) * 16, row + (size_t)px * NT + 8 * c);
+            const int row = sg.img * H + sg.y_s + i;
+            if constexpr (SWG) {
+                if (tma) {
+                    const uint32_t dst = tc::smem_addr(Gs) + uint32_t(slot * L::GSLOT);
+                    tc::mbar_arrive_expect_tx(&gf_bar[slot], L::GSLOT);
+                    conv_tma(dst, &maps.g1, sg.x0 == 0 ? W - 1 : sg.x0 - 1, row, &gf_bar[slot]);
+                    conv_tma(dst + 128, &maps.g128, sg.x0, row, &gf_bar[slot]);
+                    conv_tma(dst + 129 * 128, &maps.g1, sg.x0 + 128 == W ? 0 : sg.x0 + 128, row, &gf_bar[slot]);
+                }
+                __syncwarp();
+            } else {
+                const __nv_bfloat16 *src = gg + (size_t)row * W * NT;
+                for (int k = loader; k < CCT * 128; k += 32 * WG_LOADERS) {
+                    const int c = k % GB + k / (GB * 128) * GB, px = k / GB % 128;
+#pragma unroll
+                    for (int s = 0; s < 3; ++s) {
+                        int xx = sg.x0 + px - 1 + s;
+                        xx = xx < 0 ? xx + W : (xx >= W ? xx - W : xx);
+                        cp_async16(Gs + slot * L::GSLOT + ((s * CCT + c) * 128 + px) * 16, src + (size_t)xx * NT + 8 * c);
+                    }
+                }
+                cp_async_arrive_noinc(&gf_bar[slot]);
             }
-            cp_async_arrive_noinc(&gf_bar[slot]);
             ++gn;
             return true;
         };
@@ -873,16 +927,25 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
             u0 += sg.len;
         }
         cp_async_wait_0();
+        // no copy outlives the CTA, also when a role gave up
+        if constexpr (SWX)
+            for (long long r = gx > NSX ? gx - NSX : 0; r < gx; ++r)
+                if (!tc::mbar_wait(&xf_bar[r % NSX], uint32_t((r / NSX) & 1), CONV_WAIT_TRIES)) ok = false;
+        if constexpr (SWG)
+            for (long long r = gn > NSG ? gn - NSG : 0; r < gn; ++r)
+                if (!tc::mbar_wait(&gf_bar[r % NSG], uint32_t((r / NSG) & 1), CONV_WAIT_TRIES)) ok = false;
         if (!ok && lane == 0) atomicExch(a.error, 1);
     } else if (warp == CONV_MMA_WARP) {
-        constexpr uint32_t IDESC = tc::make_idesc_bf16(128, NT) | (1u << 15) | (1u << 16);  // A, B MN-major
+        constexpr uint32_t IDESC = tc::make_idesc_bf16(128, 3 * NT) | (1u << 15) | (1u << 16);  // A, B MN-major
         const uint32_t x_base = tc::smem_addr(Xs), g_base = tc::smem_addr(Gs);
-        // MN-major, no swizzle: a core matrix is 8 k-rows x 16 B (8 channels);
-        // the leading byte offset steps along K (128 B: the next 8 pixels), the
-        // stride byte offset along M/N (the next 8-channel chunk).
-        constexpr uint32_t A_LBO = 128, A_SBO = HP * 16;
-        constexpr uint32_t B_LBO = 128, B_SBO = 128 * 16;
-        const uint64_t ad0 = tc::make_desc(x_base, A_LBO, A_SBO), bd0 = tc::make_desc(g_base, B_LBO, B_SBO);
+        // MN-major, swizzled: an atom is 8 pixels (lines) x 64 channels; the leading
+        // byte offset steps along M/N (the next row of x; the g shifted by one
+        // pixel more: the next line), the stride byte offset along K (the next 8
+        // lines). Without swizzle a core matrix is 8 pixels x 8 channels; the
+        // leading byte offset steps along K, the stride byte offset along M/N.
+        const uint64_t ad0 = SWX ? tc::make_desc_sw128(x_base, 1024, L::XSLOT) : tc::make_desc(x_base, 128, 128 * 16);
+        const uint64_t bd0 = SWG ? tc::make_desc_sw128(g_base, 1024, 128) : tc::make_desc(g_base, 128, 128 * 16);
+        constexpr uint32_t A_K = SWX ? 128 : 16, B_K = SWG ? 128 : 16;  // 16 pixels on, in 16 bytes
         const uint32_t a_lo0 = uint32_t(ad0), a_hi = uint32_t(ad0 >> 32);
         const uint32_t b_lo0 = uint32_t(bd0), b_hi = uint32_t(bd0 >> 32);
         const uint32_t leader = tc::elect_one();
@@ -900,18 +963,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
                 tc::fence_after_sync();
                 const uint32_t s0 = uint32_t((gx + i) % NSX), s2 = uint32_t((gx + i + 2) % NSX);
                 const uint32_t g_lo = b_lo0 + uint32_t(gn % NSG) * (L::GSLOT >> 4);
-                const uint32_t a0_lo = a_lo0 + s0 * 8 * HP, a1_lo = a_lo0 + s2 * 8 * HP;
+                const uint32_t a0_lo = a_lo0 + s0 * (L::XSLOT >> 4), a1_lo = a_lo0 + s2 * (L::XSLOT >> 4);
                 const uint32_t acc0 = first ? 0u : 1u;
 #pragma unroll
                 for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-                    for (int kx = 0; kx < 3; ++kx) {
-                        const uint32_t acc = kk == 0 ? acc0 : 1u;
-                        tc::mma_bf16_leader(leader, tmem + kx * NT, a0_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk, b_hi,
-                                            IDESC, acc);
-                        tc::mma_bf16_leader(leader, tmem + (3 + kx) * NT, a1_lo + kx + 16 * kk, a_hi, g_lo + 16 * kk,
-                                            b_hi, IDESC, acc);
-                    }
+                    const uint32_t acc = kk == 0 ? acc0 : 1u;
+                    tc::mma_bf16_leader(leader, tmem, a0_lo + A_K * kk, a_hi, g_lo + B_K * kk, b_hi, IDESC, acc);
+                    tc::mma_bf16_leader(leader, tmem + 3 * NT, a1_lo + A_K * kk, a_hi, g_lo + B_K * kk, b_hi, IDESC, acc);
                 }
                 tc::mma_commit_leader(leader, &ge_bar[gn % NSG]);
                 tc::mma_commit_leader(leader, &xe_bar[(gx + i) % NSX]);
@@ -942,10 +1000,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
                 ok = false;
                 break;
             }
-            const uint4 *const row = reinterpret_cast<const uint4 *>(Gs + slot * L::GSLOT) + 32 * warp + lane;
+            const int px = 32 * warp + lane;
+            const uint8_t *const line = Gs + slot * L::GSLOT + (px + 1) * 128;
+            const uint32_t swz = (tc::smem_addr(line) >> 7) & 7;
 #pragma unroll
             for (int c = 0; c < NT / 8; ++c) {
-                const uint4 v = row[c * 128];
+                const uint4 v = *reinterpret_cast<const uint4 *>(
+                    SWG ? line + ((c ^ swz) << 4) : Gs + slot * L::GSLOT + ((CCT + c) * 128 + px) * 16);
                 const uint32_t vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
@@ -982,14 +1043,14 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
                     if (NT == 64) {
                         tc::tmem_ld32(tmem + (pr * 3 + kx) * NT + 32 * half + (uint32_t(32 * q) << 16), v);
                         if (ky <= 2) {
-                            float *o = part + ((size_t)(ky * 3 + kx) * NT + 32 * half) * 64 + c;
+                            float *o = part + ((size_t)(ky * 3 + 2 - kx) * NT + 32 * half) * 64 + c;
 #pragma unroll
                             for (int k = 0; k < 32; ++k) o[k * 64] = v[k];
                         }
                     } else {
                         tc::tmem_ld32(tmem + (pr * 3 + kx) * NT + (uint32_t(32 * q) << 16), v);  // 16 used
                         if (ky <= 2) {
-                            float *o = part + ((size_t)(ky * 3 + kx) * NT) * 64 + c;
+                            float *o = part + ((size_t)(ky * 3 + 2 - kx) * NT) * 64 + c;
 #pragma unroll
                             for (int k = 0; k < 16; ++k) o[k * 64] = v[k];
                         }
@@ -1011,11 +1072,17 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
 
 template <int CS, int NT>
 cudaError_t launch_wgrad_t(const WgradArgs &a, int grid, cudaStream_t st) {
-    using L = WgradLayout<NT>;
+    using L = WgradLayout<CS, NT>;
     cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel<CS, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          L::SMEM);
     if (e != cudaSuccess) return e;
-    wgrad_tc_kernel<CS, NT><<<grid, CONV_THREADS, L::SMEM, st>>>(a);
+    WgradMaps maps;
+    memset(&maps, 0, sizeof(maps));
+    const long long rows = (long long)a.nimg * a.H;
+    if (L::SWX && (e = pixel_map(&maps.x128, a.x, a.W, rows, 128)) != cudaSuccess) return e;
+    if (L::SWG && (e = pixel_map(&maps.g128, a.g, a.W, rows, 128)) != cudaSuccess) return e;
+    if (L::SWG && (e = pixel_map(&maps.g1, a.g, a.W, rows, 1)) != cudaSuccess) return e;
+    wgrad_tc_kernel<CS, NT><<<grid, CONV_THREADS, L::SMEM, st>>>(a, maps);
     return cudaGetLastError();
 }
 

@@ -36,9 +36,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
 // values), 16-byte chunk c of the row at absolute 128-byte line l stored at
 // chunk c ^ (l & 7); sbo_bytes between groups of eight rows. The start address
 // may lie on any 128-byte line (the swizzle goes by absolute address), plus 32
-// bytes per 16-value step along K.
-__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr, uint32_t sbo_bytes) {
-    return make_desc(saddr, 16, sbo_bytes) | uint64_t(2) << 61;
+// bytes per 16-value step along K. MN-major operands take the same lines, one per
+// value of K: lbo_bytes between atoms of 64 M or N, sbo_bytes between groups of
+// eight K.
+__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr, uint32_t sbo_bytes, uint32_t lbo_bytes = 16) {
+    return make_desc(saddr, lbo_bytes, sbo_bytes) | uint64_t(2) << 61;
 }
 
 // Instruction descriptor for kind::f16 with BF16 A and B, FP32 accumulator,
