@@ -138,7 +138,8 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
             int x = (strip * g.w_valid - g.halo + c) % g.Nx;
             x = x < 0 ? x + g.Nx : x;
             const size_t i = size_t(y) * g.Nx + x;
-            T *const d = rec + (size_t(strip) * rows + r) * MARCH_FIELDS * g.W + c;
+            T *const d = rec + (size_t(strip) * rows + r) * MARCH_FIELDS * g.W +
+                         march_column(c, int(sizeof(T)));
             make_pair_of<T>(delta / (4.0 * ncx[i]), ck, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
             if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), ck, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
             for (int axis = 0; axis < 2; ++axis) {

@@ -28,7 +28,7 @@ struct CoefView {
         const int y = int(i / g.Nx), x = int(i - (long long)y * g.Nx), strip = x / g.w_valid;
         const T *r = rec[plane >= P_TE_VX] +
                      ((size_t(strip) * (MARCH_ABOVE + g.Ny + MARCH_BELOW) + MARCH_ABOVE + y) * MARCH_FIELDS +
-                      fields[plane]) * g.W + (x - strip * g.w_valid + g.halo);
+                      fields[plane]) * g.W + march_column(x - strip * g.w_valid + g.halo, int(sizeof(T)));
         typename Ar<T>::T2 v;
         v.x = r[0];
         v.y = r[g.W];

@@ -235,10 +235,15 @@ int sweep_occupancy_f64(int K, int interleaved);
 // ---------------------------------------------------------------------------
 // Records of a family: [strips][MARCH_ABOVE + Ny + MARCH_BELOW] rows of fields
 // x, y of C_X, C_Y, V_X, V_Y (see CoefPair; TM: C_Y unused, its C_X serves
-// both), each W values: the strip's columns with their halo. Rows repeat
+// both), each W values: the strip's columns with their halo, column c at place
+// march_column(c, es). Rows repeat
 // periodically above row 0 and below row Ny - 1, as far as the shares at either
 // end copy. Flags of a family: [strips][Ny] bytes, see launch_march_records.
 constexpr int MARCH_FIELDS = 8;
+// FP32 lanes hold columns (0, 2) and (1, 3) of their four in a vector each.
+constexpr __host__ __device__ int march_column(int c, int es) {
+    return es == 4 ? (c & ~3) | (c & 1) << 1 | (c >> 1 & 1) : c;
+}
 constexpr int F_CX = 0, F_CY = 2, F_VX = 4, F_VY = 6;
 constexpr int MARCH_ABOVE = 20, MARCH_BELOW = 24;
 constexpr int MARCH_GROUP = 4;  // rows covered by a flag

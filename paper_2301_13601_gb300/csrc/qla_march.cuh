@@ -184,17 +184,22 @@ __device__ __forceinline__ void march_vop(V &h, V &p, V s, V c) {
     }
 }
 
+// A lane's vectors. FP64: its columns in order. FP32: columns (0, 2) and (1, 3) of
+// its four (march_column), so that a shift by one column is a rename, one shuffle
+// and one register move: of pairs (0, 1), (2, 3) it takes three moves (2048^2 39.8
+// -> 38.5 us per step, unitary 1536 x 1000 18.7 -> 17.2). Records hold the columns
+// in that order; state rows are regrouped where a lane reads and writes them.
+//
 // a(x) <- a(x-1), a(x) <- a(x+1) across the warp's 32 C columns
 template <typename T, int NV, typename V = typename MarchVec<T>::V>
 __device__ __forceinline__ void march_from_left(V (&a)[NV]) {
     if constexpr (MarchVec<T>::N == 2) {
-        float x[NV], y[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(a[k], x[k], y[k]);
-        const float e = __shfl_up_sync(0xffffffffu, y[NV - 1], 1);
-        a[0] = MarchVec<T>::pack(e, x[0]);
-#pragma unroll
-        for (int k = 1; k < NV; ++k) a[k] = MarchVec<T>::pack(y[k - 1], x[k]);
+        static_assert(NV == 2, "four columns");
+        float x1, x3;
+        MarchVec<T>::unpack(a[1], x1, x3);
+        const float e = __shfl_up_sync(0xffffffffu, x3, 1);
+        a[1] = a[0];
+        a[0] = MarchVec<T>::pack(e, x1);
     } else {
         const V e = __shfl_up_sync(0xffffffffu, a[NV - 1], 1);
 #pragma unroll
@@ -205,13 +210,12 @@ __device__ __forceinline__ void march_from_left(V (&a)[NV]) {
 template <typename T, int NV, typename V = typename MarchVec<T>::V>
 __device__ __forceinline__ void march_from_right(V (&a)[NV]) {
     if constexpr (MarchVec<T>::N == 2) {
-        float x[NV], y[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(a[k], x[k], y[k]);
-        const float e = __shfl_down_sync(0xffffffffu, x[0], 1);
-#pragma unroll
-        for (int k = 0; k + 1 < NV; ++k) a[k] = MarchVec<T>::pack(y[k], x[k + 1]);
-        a[NV - 1] = MarchVec<T>::pack(y[NV - 1], e);
+        static_assert(NV == 2, "four columns");
+        float x0, x2;
+        MarchVec<T>::unpack(a[0], x0, x2);
+        const float e = __shfl_down_sync(0xffffffffu, x0, 1);
+        a[0] = a[1];
+        a[1] = MarchVec<T>::pack(x2, e);
     } else {
         const V e = __shfl_down_sync(0xffffffffu, a[0], 1);
 #pragma unroll
@@ -220,39 +224,48 @@ __device__ __forceinline__ void march_from_right(V (&a)[NV]) {
     }
 }
 
-// The lane's NV vectors of a staged row (p: its first byte), and their store.
+// The lane's NV vectors of a staged record row, whose values lie in the order of
+// the vectors (p: its first byte); of a staged state row; and their store.
 template <typename T, int NV, typename V = typename MarchVec<T>::V>
 __device__ __forceinline__ void march_lds(V (&v)[NV], const unsigned char *p) {
-    if constexpr (sizeof(V) * NV == 16) {
-        const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(p);
-        memcpy(&v[0], &a.x, 8);
-        memcpy(&v[1], &a.y, 8);
-    } else {
-        static_assert(sizeof(V) * NV == 8, "8 or 16 bytes per lane");
-        v[0] = *reinterpret_cast<const V *>(p);
-    }
+    static_assert(sizeof(V) * NV == 16, "16 bytes per lane");
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(p);
+    memcpy(&v[0], &a.x, 8);
+    memcpy(&v[1], &a.y, 8);
 }
 template <typename T, int NV, typename V = typename MarchVec<T>::V>
-__device__ __forceinline__ void march_stg(T *dst, const V (&v)[NV]) {
-    if constexpr (sizeof(V) * NV == 16) {
-        ulonglong2 a;
-        memcpy(&a.x, &v[0], 8);
-        memcpy(&a.y, &v[1], 8);
-        *reinterpret_cast<ulonglong2 *>(dst) = a;
+__device__ __forceinline__ void march_lds_state(V (&v)[NV], const unsigned char *p) {
+    if constexpr (MarchVec<T>::N == 2) {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        v[0] = MarchVec<T>::pack(a.x, a.z);
+        v[1] = MarchVec<T>::pack(a.y, a.w);
     } else {
-        *reinterpret_cast<V *>(dst) = v[0];
+        march_lds<T, NV>(v, p);
     }
 }
 template <typename T, int C, int NV, typename V = typename MarchVec<T>::V>
-__device__ __forceinline__ void march_stg_some(T *dst, const V (&v)[NV], const bool (&ok)[C]) {
-    T x[C];
+__device__ __forceinline__ void march_columns(T (&x)[C], const V (&v)[NV]) {
     if constexpr (MarchVec<T>::N == 2) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) MarchVec<T>::unpack(v[k], x[2 * k], x[2 * k + 1]);
+        MarchVec<T>::unpack(v[0], x[0], x[2]);
+        MarchVec<T>::unpack(v[1], x[1], x[3]);
     } else {
 #pragma unroll
         for (int k = 0; k < C; ++k) x[k] = v[k];
     }
+}
+template <typename T, int C, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_stg(T *dst, const V (&v)[NV]) {
+    T x[C];
+    march_columns<T, C, NV>(x, v);
+    if constexpr (C == 4)
+        *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+    else
+        *reinterpret_cast<double2 *>(dst) = make_double2(x[0], x[1]);
+}
+template <typename T, int C, int NV, typename V = typename MarchVec<T>::V>
+__device__ __forceinline__ void march_stg_some(T *dst, const V (&v)[NV], const bool (&ok)[C]) {
+    T x[C];
+    march_columns<T, C, NV>(x, v);
 #pragma unroll
     for (int k = 0; k < C; ++k)
         if (ok[k]) dst[k] = x[k];
@@ -571,9 +584,9 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
                 const unsigned char *cb = sm + L::C_OFF + ((j - 1) * 2 + (i & 1)) * L::CREC;
                 if (j == 0) {
                     const unsigned char *rec = sm + rd_off;
-                    march_lds<T, NV>(hh[0], rec);
-                    march_lds<T, NV>(hx[0], rec + RB);
-                    march_lds<T, NV>(hp[0], rec + 2 * RB);
+                    march_lds_state<T, NV>(hh[0], rec);
+                    march_lds_state<T, NV>(hx[0], rec + RB);
+                    march_lds_state<T, NV>(hp[0], rec + 2 * RB);
 #pragma unroll
                     for (int c = 0; c < NV; ++c) hh[0][c] = MV::flip(hh[0][c], hsign);
                     cb = rec + 3 * RB;
@@ -602,9 +615,9 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
                          *const oy = reinterpret_cast<T *>(F.opy + out_off);
                 if constexpr (VEC) {
                     if (ok[0]) {
-                        march_stg<T, NV>(oh, h);
-                        march_stg<T, NV>(ox, hx[K - 1]);
-                        march_stg<T, NV>(oy, hp[K - 1]);
+                        march_stg<T, C, NV>(oh, h);
+                        march_stg<T, C, NV>(ox, hx[K - 1]);
+                        march_stg<T, C, NV>(oy, hp[K - 1]);
                     }
                 } else {
                     march_stg_some<T, C, NV>(oh, h, ok);
