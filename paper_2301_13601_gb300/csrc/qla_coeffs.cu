@@ -8,54 +8,20 @@ namespace qla {
 
 namespace {
 
-// FP32 rotation pair (t, s) for the three-shear collision of the sweep:
-// t = tan(a / 2) rounded to FP32, and s the FP32 value nearest to
-// 2t / (1 + t^2), the sine of the angle 2 atan(t) that t represents exactly.
-// The three shears (determinant exactly 1) are then a rotation to within one
-// rounding of s, and the angle differs from a by at most half an ulp of t.
-__device__ void shear_pair_f32(double ang, float &tf, float &sf) {
+// FP32 rotation pair (t, s): t = tan(a / 2) rounded to FP32, and s the FP32 value
+// nearest to 2t / (1 + t^2), the sine of the angle 2 atan(t) that t represents
+// exactly. The three shears and the four-operation form of the sweep (determinant
+// exactly 1) are then a rotation to within one rounding of s, and the angle
+// differs from a by at most half an ulp of t.
+__device__ void rotation_pair_f32(double ang, float &tf, float &sf) {
     tf = (float)tan(0.5 * ang);
     const double t = (double)tf;
     sf = (float)(2.0 * t / (1.0 + t * t));
 }
 
-// FP32 pair (t, s) near (tan(a / 2), sin(a)) for the four-FMA rotation of the
-// sweep, whose matrix is [1 - s t, s; -s, 1 - s t]: among FP32 values next to the
-// correctly rounded ones, the pair that brings
-// (1 - s t)^2 + s^2 - 1 = s (s (1 + t^2) - 2 t) (evaluated in FP64) closest to
-// zero, so that each rotation keeps the energy (Eq. 27) to ~1e-12.
-__device__ void tuned_pair_f32(double ang, float &tf, float &sf) {
-    const float t0 = (float)tan(0.5 * ang), s0 = (float)sin(ang);
-    if (!(fabsf(t0) >= 1e-30f) || !(fabsf(s0) >= 1e-30f)) {  // zero or denormal: keep the rounded values
-        tf = t0;
-        sf = s0;
-        return;
-    }
-    // for each t the best s is the FP32 value nearest to 2 t / (1 + t^2); t moves
-    // by one ulp at most (four brought the norm no closer than the arithmetic's own
-    // rounding and put 1e-7 of angle error, 4% in a 48-step run, in its place)
-    double best = 1e300;
-    tf = t0;
-    sf = s0;
-    for (int dt = -1; dt <= 1; ++dt) {
-        const float tc = __int_as_float(__float_as_int(t0) + dt);
-        const double t = (double)tc, q = 1.0 + t * t;
-        const float sc = (float)(2.0 * t / q);
-        const double s = (double)sc;
-        const double e = fabs(s * (s * q - 2.0 * t));
-        if (e < best) {
-            best = e;
-            tf = tc;
-            sf = sc;
-        }
-    }
-}
-
-// How a pair is stored (see CoefPair and rot in the sweep): a collision of the
-// three-shear form (FP32 with the printed potentials), a rotation of the
-// four-FMA form (FP32: tuned for orthogonality), both (tan(a/2), sin a), or a
-// printed potential row (cos a - 1, sin a).
-enum PairKind { PK_SHEAR, PK_ROTATION, PK_PRINTED_V };
+// How a pair is stored (see CoefPair and rot in the sweep): a rotation
+// (tan(a/2), sin a) or a printed potential row (cos a - 1, sin a).
+enum PairKind { PK_ROTATION, PK_PRINTED_V };
 
 template <typename T>
 __device__ void make_pair_of(double ang, PairKind kind, T &x, T &y) {
@@ -64,8 +30,7 @@ __device__ void make_pair_of(double ang, PairKind kind, T &x, T &y) {
         x = (T)(-2.0 * sh * sh);  // cos(ang) - 1 without cancellation
         y = (T)sin(ang);
     } else if constexpr (sizeof(T) == 4) {
-        if (kind == PK_SHEAR) shear_pair_f32(ang, x, y);
-        else tuned_pair_f32(ang, x, y);
+        rotation_pair_f32(ang, x, y);
     } else {
         x = tan(0.5 * ang);
         y = sin(ang);
@@ -108,11 +73,10 @@ __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, 
         const double b1 = potential_angle(nx, x, y, Nx, Ny, 1, delta);
         const double b2 = potential_angle(nz, x, y, Nx, Ny, 0, delta);
         const double b3 = potential_angle(nz, x, y, Nx, Ny, 1, delta);
-        const PairKind ck = unitary ? PK_ROTATION : PK_SHEAR;
         const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
-        store_pair<T>(coef, P, P_TM_C, i, th2, ck);
-        store_pair<T>(coef, P, P_TE_CX, i, th1, ck);
-        store_pair<T>(coef, P, P_TE_CY, i, th0, ck);
+        store_pair<T>(coef, P, P_TM_C, i, th2, PK_ROTATION);
+        store_pair<T>(coef, P, P_TE_CX, i, th1, PK_ROTATION);
+        store_pair<T>(coef, P, P_TE_CY, i, th0, PK_ROTATION);
         store_pair<T>(coef, P, P_TM_VX, i, b2 * vscale, vk);
         store_pair<T>(coef, P, P_TM_VY, i, b3 * vscale, vk);
         store_pair<T>(coef, P, P_TE_VX, i, b0 * vscale, vk);
@@ -128,7 +92,6 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
     const double *nx = n, *ny = n + P, *nz = n + 2 * P;
     const double *ncx = fam ? ny : nz, *ncy = fam ? nx : nz;  // indices of C_X and V_X, of C_Y and V_Y
     const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
-    const PairKind ck = unitary ? PK_ROTATION : PK_SHEAR;
     const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW, strip = blockIdx.x;
     for (int r = blockIdx.y; r < rows; r += gridDim.y) {
@@ -140,8 +103,8 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
             const size_t i = size_t(y) * g.Nx + x;
             T *const d = rec + (size_t(strip) * rows + r) * MARCH_FIELDS * g.W +
                          march_column(c, int(sizeof(T)));
-            make_pair_of<T>(delta / (4.0 * ncx[i]), ck, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
-            if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), ck, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
+            make_pair_of<T>(delta / (4.0 * ncx[i]), PK_ROTATION, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
+            if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), PK_ROTATION, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
             for (int axis = 0; axis < 2; ++axis) {
                 const double b = potential_angle(axis ? ncy : ncx, x, y, g.Nx, g.Ny, axis, delta) * vscale;
                 T *const v = d + (axis ? F_VY : F_VX) * g.W;

@@ -14,9 +14,8 @@ namespace qla {
 // 1/2 again for the unitary potentials).
 // A collision pair, and a potential pair of the unitary potentials, is
 // (x = tan(a/2), y = sin(a)); a printed potential pair is (cos(b) - 1, sin(b)).
-// FP32 pairs of the three-shear collisions (printed potentials) take y nearest
-// to 2x / (1 + x^2), the others are tuned for orthogonality. Signs of the
-// operators are applied by the kernels.
+// FP32 rotation pairs take y nearest to 2x / (1 + x^2). Signs of the operators are
+// applied by the kernels.
 // The order puts the two planes that the sweep copies together next to each
 // other: (V_X, C_X) for the x-pass and (C_Y, V_Y) for the y-pass of a family.
 enum CoefPair {

@@ -165,10 +165,16 @@ __device__ __forceinline__ void march_rot(V &h, V &p, V m, V s) {
         p = A::fma(pos ? A::neg(s) : s, h, p);
         h = A::fma(pos ? m : A::neg(m), p, h);
     } else {
-        const V u = A::fma(pos ? A::neg(m) : m, h, p);
-        const V v = A::fma(pos ? m : A::neg(m), p, h);
-        h = A::fma(pos ? s : A::neg(s), u, h);
-        p = A::fma(pos ? A::neg(s) : s, v, p);
+        const V t = pos ? A::neg(m) : m, u = A::fma(t, h, p);
+        if constexpr (sizeof(T) == 4) {
+            const V h0 = h;
+            h = A::fma(pos ? s : A::neg(s), u, h);
+            p = A::fma(t, A::add(h0, h), p);
+        } else {
+            const V v = A::fma(A::neg(t), p, h);
+            h = A::fma(pos ? s : A::neg(s), u, h);
+            p = A::fma(pos ? A::neg(s) : s, v, p);
+        }
     }
 }
 template <int TAU, bool HUB, bool UNIT, typename T, typename V = typename MarchVec<T>::V>

@@ -36,9 +36,8 @@
 //  * In FP32 with the printed potentials a collision is three shears
 //    (h += t p, p -= s h, h += t p with t = tan(theta/2): three FMAs, the
 //    determinant exactly 1); otherwise each output is its input plus sin(theta)
-//    times a combination formed first, one rounding at the scale of the output,
-//    with FP32 pairs tuned at creation for orthogonality. Coefficients are stored
-//    as pairs of the form the kernel uses (see rot).
+//    times a combination formed first, one rounding at the scale of the output.
+//    Coefficients are stored as pairs of the form the kernel uses (see rot).
 #pragma once
 
 #include <cuda.h>
@@ -168,13 +167,18 @@ struct Fam<1> {
 // Collision C (DAG = false) or its transpose (DAG = true) on (h, p) with
 // orientation SG: the rotation h' = c h + SG s p, p' = -SG s h + c p by the
 // angle theta (c = cos theta, s = sin theta).
-//  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t,
-//    so
-//      h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p)
-//    (four FMAs; one rounding at the scale of each output, those of the inner
-//    combinations enter scaled by s). The form h' = h + (m h + s p) with m =
-//    cos theta - 1 took six operations for the same errors: FP64 256^2, whose
-//    pipe is the bound, 64 -> 43 us per step.
+//  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t.
+//    Both forms take four operations and round once at the scale of each output
+//    (the inner combinations enter scaled by s or t). h' = h + (m h + s p) with
+//    m = cos theta - 1 took six for the same errors: FP64 256^2, whose pipe is
+//    the bound, 64 -> 43 us per step.
+//    FP64: h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p).
+//    FP32: h' = h + SG s (p - SG t h),   p' = p - SG t (h + h'),
+//    the same rotation, whose matrix has determinant 1 and the transpose as its
+//    exact inverse whatever the rounding of t and s. The FP64 form scales h^2 + p^2
+//    by s (s (1 + t^2) - 2 t), in FP32 up to 1e-10 each time and no pair of nearby
+//    FP32 values much closer (s and 2 t round alike): 1.7e-6 of energy in 1e4 steps
+//    at 2048^2 against 5.8e-7. (In FP64 its two independent chains are 4% faster.)
 //  * SHEAR = true (FP32 with the printed potentials): pair (t, s) with
 //    t = tan(theta / 2), as three shears
 //      h1 = h + SG t p,  p' = p - SG s h1,  h' = h1 + SG t p'
@@ -196,16 +200,22 @@ __device__ __forceinline__ void rot(T &h, T &p, T m, T s) {
     } else {
         const T t = m;
         const T u = A::fma(pos ? -t : t, h, p);
-        const T v = A::fma(pos ? t : -t, p, h);
-        h = A::fma(pos ? s : -s, u, h);
-        p = A::fma(pos ? -s : s, v, p);
+        if constexpr (sizeof(T) == 4) {
+            const T h0 = h;
+            h = A::fma(pos ? s : -s, u, h);
+            p = A::fma(pos ? -t : t, A::add(h0, h), p);
+        } else {
+            const T v = A::fma(pos ? t : -t, p, h);
+            h = A::fma(pos ? s : -s, u, h);
+            p = A::fma(pos ? -s : s, v, p);
+        }
     }
 }
 
 // Collision form of a configuration: three shears in FP32 with the printed
-// potentials; the four-FMA form in FP64, and in FP32 with the unitary
-// potentials, where every operator is an exact rotation and the tuned pairs
-// keep the energy (Eq. 27) to FP32 rounding over 1e4 steps.
+// potentials; the four-operation forms in FP64, and in FP32 with the unitary
+// potentials, where every operator is an exact rotation and the energy (Eq. 27)
+// is kept to FP32 rounding over 1e4 steps.
 template <typename T, bool UNIT>
 constexpr bool shear_collisions() {
     return std::is_same<T, float>::value && !UNIT;
