@@ -32,11 +32,10 @@ sys.path.insert(0, ROOT)
 
 # DRAM bytes per sweep launch (dram__bytes_read.sum + dram__bytes_write.sum) from an ncu capture
 # (one pass) of two sweep launches of this benchmark's own command on the 8192^2 workload (its
-# summary sits in profiles/ beside the launch list), valid while the sweep's code (comment lines
-# excluded), the workload, the steps per pass and the launch form (balanced split, one launch per
-# pass or all passes of a bench step in one persistent launch) match.
-MEASURED_TRAFFIC = {"sweep_sha256_prefix": "677c90822e6ffdd2", "workload": "cylinders8192_fp32",
-                    "steps_per_pass": 2, "chunk_rows": 0, "launch": "per_pass", "bytes_per_launch": 7.77284e9}
+# summary sits in profiles/), valid while the sweep's code (comment lines excluded), the workload,
+# the steps per pass and the launch form match.
+MEASURED_TRAFFIC = {"sweep_sha256_prefix": "f6fc4bb6a851c9e3", "workload": "cylinders8192_fp32",
+                    "steps_per_pass": 2, "chunk_rows": 0, "launch": "per_pass", "bytes_per_launch": 3.50679e9}
 
 L2_BYTES = 129e6  # GB300 L2
 METRIC = "site-updates/s per QLA step"
@@ -116,12 +115,12 @@ class ClockSampler:
 
 def sweep_code_hash() -> str:
     """sha256 prefix of the per-pass sweep kernel's sources (the kernel, its
-    instantiations and launch split, the shared declarations) with their
+    instantiation and launch, the shared declarations) with their
     comment lines removed."""
     import hashlib
 
     code = []
-    for name in ("qla_sweep.cuh", "qla_sweep_f32.cu", "qla_internal.h"):
+    for name in ("qla_sweep.cuh", "qla_march.cuh", "qla_march.cu", "qla_march_f32_k2.cu", "qla_internal.h"):
         with open(os.path.join(ROOT, "paper_2301_13601_gb300", "csrc", name)) as f:
             code += [l for l in f.read().splitlines() if not l.lstrip().startswith("//")]
     return hashlib.sha256("\n".join(code).encode()).hexdigest()[:16]
@@ -272,7 +271,7 @@ def run_ours(args):
         dist.barrier()
     # one launch per pass, or every pass of a bench step in one persistent launch
     launch_form = sim.launch
-    launches_per_step = 1 if launch_form == "persistent" else math.ceil(S / sim.steps_per_pass)
+    launches_per_step = 1 if launch_form == "persistent" else math.ceil(S / min(sim.steps_per_pass, 2))
     # e2e through the public API with host buffers: pinned H2D state copy,
     # qla_step, diagnostics, D2H state copy, every bench step. Serial: one
     # context, each step's copies between its compute. Pipelined (the reported
@@ -364,13 +363,13 @@ def run_ours(args):
                    "qla_steps_per_bench_step": S, "steps_per_pass": k, "chunk_rows": sim.chunk_rows,
                    "launch": launch_form,
                    "precision": "fp32", "sequence": "interleaved", "potential": "paper",
-                   "l2": (f"inputs {'larger' if 80 * sites > L2_BYTES else 'smaller'} than L2 (state "
-                          f"{24 * sites / 1e9:.2f} GB + coefficients {56 * sites / 1e9:.2f} GB read per pass)"),
+                   "l2": (f"inputs {'larger' if 48 * sites > L2_BYTES else 'smaller'} than L2 (state "
+                          f"{24 * sites / 1e9:.2f} GB read and written per pass, and its coefficients)"),
                    "parallelism": f"replicas x{world}"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                      "kernel": (f"sweep_persistent_kernel<float,{k}> ({S // k} passes per launch)"
-                                if launch_form == "persistent" else f"sweep_kernel<float,{k}>"),
+                                if launch_form == "persistent" else f"march_kernel<float,{min(k, 2)}>"),
                      "bytes_per_site_update": BYTES_PER_SITE_UPDATE,
                      "note": "algorithmic bytes of the unfused step x steps per launch"},
         "cpu_baseline": cb,

@@ -16,7 +16,7 @@
 //    through shared memory and no block barrier is needed.
 //  * The strip carries a halo of at least 4K columns on each side; the columns
 //    between are written. A share of rows [y0, y1) is fed from y0 - 4K.
-//  * FP32 arithmetic is packed: two adjacent columns per fma.rn.f32x2 (the
+//  * FP32 arithmetic is packed: two of a lane's columns per fma.rn.f32x2 (the
 //    same roundings as two scalar FMAs). Measured on GB300 with independent
 //    rotations in registers: 28 T FMA/s scalar, 36 packed, in half the issue
 //    slots.
@@ -37,16 +37,17 @@
 // strip's 32 C columns (halo included), periodic rows repeated above and below,
 // so that every coefficient copy of an iteration, whatever its level and lag, is
 // one address register plus a constant, aligned for any Nx.
-// Measured on GB300 against the shared-memory sweep (us per step, both
-// families, three-cylinder-like media): 8192^2 874 -> 538 (124.7 G site-updates/s,
-// 5.6 TB/s of HBM traffic), 4096^2 240 -> 155, 2048^2 83 -> 52, 1024^2 43.6 ->
-// 21.7, 256^2 29 -> 10. That sweep was bound by instruction issue (half of its
-// instructions index and control work) and its two block barriers per row
-// block; this one by the fixed latencies of its chains with the 8 warps per SM
-// that 255 registers leave (two steps; issue slots 47% busy, FMA pipe 38%) and,
-// on the largest lattices, by HBM. On the way there (8192^2): one body per family
-// and with and without potentials, scalar FMAs 925 us (instruction cache); one
-// body for both families 731; packed FMAs 628; planes by 32-bit offsets 591.
+// Measured on GB300 against the shared-memory sweep (us per step, both families,
+// interleaved with other contexts' calls): 8192^2 810 -> 480 (140 G site-updates/s,
+// 3.5 TB/s of HBM traffic), 2048^2 78 -> 39, 1024^2 44 -> 13, 256^2 26 -> 4; 4096^2,
+// one family, 106 -> 65; 256^2 FP64 330 -> 62. That sweep was bound by instruction
+// issue (half of its instructions index and control work) and its two block
+// barriers per row block; this one by the fixed latencies of its chains with the 8
+// warps per SM that 247 registers leave (two steps; issue slots 41% busy, FMA pipe
+// 38%), on the smallest lattices by the latency of a pass. On the way there
+// (8192^2): one body per family and with and without potentials, scalar FMAs 925 us
+// (instruction cache); one body for both families 731; packed FMAs 628; planes by
+// 32-bit offsets 591; coefficient records 538; row ranges by measured costs 505.
 #pragma once
 
 #include "qla_sweep.cuh"

@@ -170,8 +170,8 @@ struct Fam<1> {
 //  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t.
 //    Both forms take four operations and round once at the scale of each output
 //    (the inner combinations enter scaled by s or t). h' = h + (m h + s p) with
-//    m = cos theta - 1 took six for the same errors: FP64 256^2, whose pipe is
-//    the bound, 64 -> 43 us per step.
+//    m = cos theta - 1 took six for the same errors (a third more of the FP64
+//    pipe, which bounds FP64 steps).
 //    FP64: h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p).
 //    FP32: h' = h + SG s (p - SG t h),   p' = p - SG t (h + h'),
 //    the same rotation, whose matrix has determinant 1 and the transpose as its
