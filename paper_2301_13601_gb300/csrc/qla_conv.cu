@@ -42,13 +42,6 @@ __device__ __forceinline__ float tanh_fast(float x) {
     return y;
 }
 
-__device__ __forceinline__ float gelu_f(float x) {
-    const float k0 = 0.7978845608028654f, k1 = 0.7978845608028654f * 0.044715f;  // sqrt(2/pi), sqrt(2/pi) 0.044715
-    const float t = tanh_fast(x * fmaf(k1, x * x, k0));
-    const float hx = 0.5f * x;
-    return fmaf(hx, t, hx);
-}
-
 __device__ __forceinline__ float gelu_grad(float x) {
     const float k0 = 0.7978845608028654f, k1 = 0.7978845608028654f * 0.044715f;
     const float x2 = x * x;
@@ -61,7 +54,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tc::smem_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Two channels per operation (the same roundings as one by one): the epilogues
@@ -92,7 +84,7 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
-__device__ __forceinline__ F2 gelu_f2(F2 x) {  // gelu_f of both
+__device__ __forceinline__ F2 gelu_f2(F2 x) {  // GELU, tanh form; k0 = sqrt(2/pi), k1 = 0.044715 k0
     const float k0 = 0.7978845608028654f, k1 = 0.7978845608028654f * 0.044715f;
     const F2 arg = f2_mul(x, f2_fma(f2(k1, k1), f2_mul(x, x), f2(k0, k0)));
     float a, b;

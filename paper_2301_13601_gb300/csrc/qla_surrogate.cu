@@ -39,9 +39,6 @@ constexpr int NOUTP[NL] = {64, 64, 64, 64, 64, 16};
 constexpr int X0C = 16;                              // x0 channels: Q hi (6), Q lo (6), n (3), 0
 constexpr int RED_BLOCKS = 512;                      // partial sums of the loss reductions
 
-__device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
-
 __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t *>(&h);

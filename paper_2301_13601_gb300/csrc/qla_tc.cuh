@@ -141,32 +141,6 @@ __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 
-// D[tmem] (+)= A * B^T, one 128 x N x 16 step; issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same with the descriptors given as 32-bit halves: a descriptor for
-// start + off is the base descriptor plus (off >> 4) in its low word, so a
-// loop over operand offsets costs one integer add per operand.
-__device__ __forceinline__ void mma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                              uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n.reg .b64 ad, bd;\n"
-        "mov.b64 ad, {%1, %2};\n"
-        "mov.b64 bd, {%3, %4};\n"
-        "setp.ne.b32 p, %6, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, p;\n}\n" ::"r"(d_tmem),
-        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // True in one lane of a converged warp.
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t p;
@@ -174,12 +148,14 @@ __device__ __forceinline__ uint32_t elect_one() {
     return p;
 }
 
-// The same issued by the lane whose `leader` is set, with the whole warp in
-// uniform control flow: the operands are then computed in uniform registers,
-// where the instruction takes them, instead of being moved there one by one in
-// a branch that one lane takes. That branch cost 190 cycles per MMA whatever its
-// width: 1024^2 hidden layer without its epilogue 78 -> 56 us, last layer with it
-// 72 -> 42 us.
+// D[tmem] (+)= A * B^T, one 128 x N x 16 step, the descriptors given as 32-bit
+// halves: a descriptor for start + off is the base descriptor plus (off >> 4) in
+// its low word, so a loop over operand offsets costs one integer add per operand.
+// Issued by the lane whose `leader` is set, with the whole warp in uniform
+// control flow: the operands are then computed in uniform registers, where the
+// instruction takes them, instead of being moved there one by one in a branch that
+// one lane takes. That branch cost 190 cycles per MMA whatever its width: 1024^2
+// hidden layer without its epilogue 78 -> 56 us, last layer with it 72 -> 42 us.
 __device__ __forceinline__ void mma_bf16_leader(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
                                                 uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -192,19 +168,13 @@ __device__ __forceinline__ void mma_bf16_leader(uint32_t leader, uint32_t d_tmem
         "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(leader)
         : "memory");
 }
+// Arrive on an mbarrier when all MMAs that the leader issued before are done.
 __device__ __forceinline__ void mma_commit_leader(uint32_t leader, uint64_t *bar) {
     asm volatile(
         "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_addr(bar)),
         "r"(leader)
         : "memory");
-}
-
-// Arrive on an mbarrier when all previously issued MMAs of this thread are done.
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                     smem_addr(bar))
-                 : "memory");
 }
 
 // Each thread of a warp reads 32 consecutive FP32 columns of its TMEM lane.
