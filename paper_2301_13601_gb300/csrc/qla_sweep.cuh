@@ -174,9 +174,9 @@ struct Fam<1> {
 //    pipe, which bounds FP64 steps).
 //    FP64: h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p).
 //    FP32: h' = h + SG s (p - SG t h),   p' = p - SG t (h + h'),
-//    the same rotation, whose matrix has determinant 1 and the transpose as its
-//    exact inverse whatever the rounding of t and s. The FP64 form scales h^2 + p^2
-//    by s (s (1 + t^2) - 2 t), in FP32 up to 1e-10 each time and no pair of nearby
+//    the same rotation, whose matrix has determinant 1, and whose inverse is the
+//    form with both signs flipped, whatever the rounding of t and s. The FP64 form
+//    scales h^2 + p^2 by s (s (1 + t^2) - 2 t), in FP32 up to 1e-10 each time and no pair of nearby
 //    FP32 values much closer (s and 2 t round alike): 1.7e-6 of energy in 1e4 steps
 //    at 2048^2 against 5.8e-7. (In FP64 its two independent chains are 4% faster.)
 //  * SHEAR = true (FP32 with the printed potentials): pair (t, s) with
