@@ -170,15 +170,16 @@ struct Fam<1> {
 //  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t.
 //    Both forms take four operations and round once at the scale of each output
 //    (the inner combinations enter scaled by s or t). h' = h + (m h + s p) with
-//    m = cos theta - 1 took six for the same errors (a third more of the FP64
-//    pipe, which bounds FP64 steps).
+//    m = cos theta - 1 took six for the same errors (half more of the FP64 pipe,
+//    which bounds FP64 steps).
 //    FP64: h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p).
 //    FP32: h' = h + SG s (p - SG t h),   p' = p - SG t (h + h'),
 //    the same rotation, whose matrix has determinant 1, and whose inverse is the
 //    form with both signs flipped, whatever the rounding of t and s. The FP64 form
-//    scales h^2 + p^2 by s (s (1 + t^2) - 2 t), in FP32 up to 1e-10 each time and no pair of nearby
-//    FP32 values much closer (s and 2 t round alike): 1.7e-6 of energy in 1e4 steps
-//    at 2048^2 against 5.8e-7. (In FP64 its two independent chains are 4% faster.)
+//    scales h^2 + p^2 by s (s (1 + t^2) - 2 t), in FP32 up to 1e-10 each time, and
+//    no pair of nearby FP32 values is much closer (s and 2 t round alike): 1.7e-6
+//    of energy in 1e4 steps at 2048^2 against 5.8e-7. (In FP64 its two independent
+//    chains are 4% faster.)
 //  * SHEAR = true (FP32 with the printed potentials): pair (t, s) with
 //    t = tan(theta / 2), as three shears
 //      h1 = h + SG t p,  p' = p - SG s h1,  h' = h1 + SG t p'
