@@ -438,6 +438,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) conv3x3_tc_kernel(const ConvA
             if (ok && conv_row_acc_wait(j, sg.len, on, NB, &par) && !tc::mbar_wait(&acce_bar[b0], par, CONV_WAIT_TRIES))
                 ok = false;
             if (!ok) return false;
+            // Rows copied by cp.async are generic-proxy writes; the barrier orders
+            // them before this thread, the fence before the tensor cores' reads.
+            if constexpr (!L::SWZ) tc::fence_proxy_async();
             tc::fence_after_sync();
             {
                 // (slot * HP * line bytes) >> 4
@@ -952,6 +955,8 @@ __global__ void __launch_bounds__(CONV_THREADS, 1) wgrad_tc_kernel(const WgradAr
                 }
                 if (!tc::mbar_wait(&gf_bar[gn % NSG], uint32_t((gn / NSG) & 1), CONV_WAIT_TRIES)) ok = false;
                 if (!ok) break;
+                // as in conv3x3_tc_kernel: rows copied by cp.async, before the tensor cores read them
+                if constexpr (!(SWX && SWG)) tc::fence_proxy_async();
                 tc::fence_after_sync();
                 const uint32_t s0 = uint32_t((gx + i) % NSX), s2 = uint32_t((gx + i + 2) % NSX);
                 const uint32_t g_lo = b_lo0 + uint32_t(gn % NSG) * (L::GSLOT >> 4);
