@@ -44,6 +44,7 @@ struct qla_ctx {
     bool march = false;             // the marching form (launch_march) serves the context's passes
     qla::MarchGeo geo{};
     int nfam = 2, fam0 = 0;         // families advanced (TM = 0, TE = 1)
+    int mode = 0;                   // SweepMode
     bool persistent = false;        // passes of K steps in one cooperative launch per qla_step (QLA_LAUNCH_*)
     unsigned *pass_done = nullptr;  // device [2][kPersistMaxCtas]: passes completed per share (persistent form)
     unsigned pass_epoch = 0;        // passes the persistent launches have completed (the counters' base)
@@ -135,11 +136,12 @@ int balanced_ctas(int Nx, int Ny, int K, int prec, int interleaved, int sms) {
 
 // Whether the context's passes of K steps can take the persistent launch form:
 // FP32, the balanced split, K instantiated for it, the seam layout (Nx a
-// multiple of 8, at least 256 columns) and at most kPersistMaxCtas shares.
+// multiple of 8, at least 256 columns), at most kPersistMaxCtas shares and
+// rotations in the half-angle form.
 bool persistent_applies(const qla_ctx *c) {
-    return !c->march && c->opt.precision == QLA_FP32 && c->chunk == 0 && qla::sweep_persistent_supported(0, c->K) &&
-           c->Nx % 8 == 0 && c->Nx >= qla::sweep_strip_width() && c->ctas[c->K] >= 1 &&
-           c->ctas[c->K] <= qla::kPersistMaxCtas;
+    return !c->march && !(c->mode & qla::MODE_WIDE) && c->opt.precision == QLA_FP32 && c->chunk == 0 &&
+           qla::sweep_persistent_supported(0, c->K) && c->Nx % 8 == 0 && c->Nx >= qla::sweep_strip_width() &&
+           c->ctas[c->K] >= 1 && c->ctas[c->K] <= qla::kPersistMaxCtas;
 }
 
 // Whether the marching form serves a context: unless the persistent launch form
@@ -179,8 +181,7 @@ qla_status launch_pass(qla_ctx *c, int K, bool chained) {
         for (int k = 0; k < K; k += per) {
             const cudaError_t e = qla::launch_march(
                 c->geo, per, c->state[c->cur], c->state[c->cur ^ 1], c->coef, c->nfam, c->fam0,
-                c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, c->opt.potential == QLA_POT_UNITARY ? 1 : 0,
-                chained, c->stream);
+                c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, c->mode, chained, c->stream);
             chained = true;
             if (e != cudaSuccess) return fail(c, QLA_ECUDA, "sweep launch (K=%d): %s", K, cudaGetErrorString(e));
             c->cur ^= 1;
@@ -198,7 +199,7 @@ qla_status launch_pass(qla_ctx *c, int K, bool chained) {
     a.ctas = c->ctas[K];
     a.order = c->share_order;
     a.interleaved = c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0;
-    a.unitary = c->opt.potential == QLA_POT_UNITARY ? 1 : 0;
+    a.mode = c->mode;
     a.vec = (c->Nx % int(16 / c->esize)) == 0 ? 1 : 0;
     // one CTA grid layer per advanced family (TM = family 0, TE = family 1);
     // the planes of a family that is not advanced stay zero in both buffers
@@ -229,7 +230,7 @@ qla_status launch_persistent(qla_ctx *c, int passes, bool *refused) {
     a.ctas = c->ctas[K];
     a.order = nullptr;
     a.interleaved = c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0;
-    a.unitary = c->opt.potential == QLA_POT_UNITARY ? 1 : 0;
+    a.mode = c->mode;
     a.vec = (c->Nx % int(16 / c->esize)) == 0 ? 1 : 0;
     const int nfam = c->opt.families == QLA_FAMILIES_BOTH ? 2 : 1;
     a.fam0 = c->opt.families == QLA_FAMILY_TE ? 1 : 0;
@@ -323,9 +324,9 @@ qla_status qla_create(int Nx, int Ny, const double *n_x, const double *n_y, cons
     if (o.steps_per_pass > 0 && !qla::sweep_supported(o.precision, o.steps_per_pass)) return QLA_EUNSUPPORTED;
     const size_t P = size_t(Nx) * size_t(Ny);
     const double *nn[3] = {n_x, n_y, n_z};
+    bool ordinary = true;
     for (int k = 0; k < 3; ++k)
-        for (size_t i = 0; i < P; ++i)
-            if (!(nn[k][i] > 0.0) || !std::isfinite(nn[k][i])) return QLA_EINVAL;
+        if (!qla::index_valid(nn[k], P, &ordinary)) return QLA_EINVAL;
 
     qla_ctx *c = new qla_ctx();
     c->Nx = Nx;
@@ -393,10 +394,12 @@ qla_status qla_create(int Nx, int Ny, const double *n_x, const double *n_y, cons
     c->march = march_applies(o, Nx, Ny, &c->geo);
     c->nfam = o.families == QLA_FAMILIES_BOTH ? 2 : 1;
     c->fam0 = o.families == QLA_FAMILY_TE ? 1 : 0;
-    const int inter = o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, unit = o.potential == QLA_POT_UNITARY ? 1 : 0;
+    const int inter = o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0;
+    c->mode = qla::rotation_mode(nn, ordinary, Nx, Ny, delta, o.precision == QLA_FP64 ? 1 : 0, inter,
+                                 o.potential == QLA_POT_UNITARY ? 1 : 0);
     if ((c->march ? qla::launch_march_records(c->geo, c->index, c->coef, c->nfam, c->fam0, delta,
-                                              o.precision == QLA_FP64 ? 1 : 0, inter, unit, c->stream)
-                  : qla::launch_coefficients(c->index, c->coef, Nx, Ny, delta, o.precision, inter, unit, c->stream)) !=
+                                              o.precision == QLA_FP64 ? 1 : 0, inter, c->mode, c->stream)
+                  : qla::launch_coefficients(c->index, c->coef, Nx, Ny, delta, o.precision, inter, c->mode, c->stream)) !=
         cudaSuccess)
         return bail(QLA_ECUDA);
     if (cudaMemsetAsync(c->state[0], 0, bs.state_bytes, c->stream) != cudaSuccess ||
@@ -512,7 +515,8 @@ qla_status qla_step(qla_ctx *c, long long nsteps) {
     }
     while (left > 0) {
         int k = c->K;
-        while (k > 1 && (k > left || !qla::sweep_supported(c->opt.precision, k))) --k;
+        while (k > 1 && (k > left || !qla::sweep_supported(c->opt.precision, k) ||
+                         (!c->march && (c->mode & qla::MODE_WIDE)))) --k;
         s = launch_pass(c, k, left < nsteps);
         if (s != QLA_OK) return s;
         left -= k;
@@ -613,7 +617,7 @@ qla_status qla_debug_apply(qla_ctx *c, int op, int count) {
     for (int k = 0; k < count; ++k) {
         bool swapped = false;
         const cudaError_t e = qla::debug_apply(op, c->opt.precision, c->state[c->cur], c->state[c->cur ^ 1], c->coef,
-                                               c->march ? &c->geo : nullptr, c->nfam, c->fam0, c->Nx, c->Ny, c->opt.potential == QLA_POT_UNITARY ? 1 : 0, c->stream,
+                                               c->march ? &c->geo : nullptr, c->nfam, c->fam0, c->Nx, c->Ny, c->mode, c->stream,
                                                &swapped);
         if (e != cudaSuccess) return fail(c, QLA_ECUDA, "qla_debug_apply: %s", cudaGetErrorString(e));
         if (swapped) c->cur ^= 1;

@@ -35,6 +35,7 @@ struct BatchInst {
     int Nx, Ny, w_valid, halo, strips, chunks;
     int tiles;                      // per pass and family
     int passes;                     // of kBatchSteps steps
+    int wide;                       // its rotations take the form for any angle (MODE_WIDE)
 };
 
 struct BatchSched {
@@ -71,12 +72,14 @@ __device__ __forceinline__ int warp_search(const long long *a, int n, long long 
     return lo;
 }
 
-template <bool INTER, bool UNIT, bool VEC>
+// MODE with MODE_WIDE: some lattice of the batch (BatchInst::wide) rotates in that
+// form, the others as without it.
+template <bool INTER, int MODE, bool VEC>
 __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSched S) {
     using L = MarchLayout<float, BC, kBatchSteps, BD, INTER>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ MarchArgs args;  // the item's lattice and family (entry 0)
-    __shared__ int item[4];     // stop, instance, family, tile
+    __shared__ int item[5];     // stop, instance, family, tile, wide
     const int lane = threadIdx.x & 31;
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0);
     for (;;) {
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSche
             if (lane == 0) g = atomicAdd(S.next, 1ull);
             g = __shfl_sync(0xffffffffu, g, 0);
             int stop = g >= (unsigned long long)S.pass_start[S.maxpass] || *(volatile int *)S.error ? 1 : 0;
-            int inst = 0, fam = 0, tile = 0;
+            int inst = 0, fam = 0, tile = 0, wide = 0;
             if (!stop) {
                 const int pass = warp_search(S.pass_start, S.maxpass, (long long)g, lane);
                 const long long r = (long long)g - S.pass_start[pass];
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSche
                 const BatchInst &I = S.inst[inst];
                 const int rr = int(r - S.tile_prefix[inst]);
                 const int tiles = I.tiles;
+                if constexpr (MODE & MODE_WIDE) wide = I.wide;
                 fam = rr / tiles;
                 tile = rr % tiles;
                 if (lane == 0) {
@@ -128,6 +132,7 @@ __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSche
                 item[1] = inst;
                 item[2] = fam;
                 item[3] = tile;
+                item[4] = wide;
             }
         }
         __syncthreads();
@@ -137,8 +142,13 @@ __global__ void __launch_bounds__(32 * BWPC, BMINB) batch_kernel(const BatchSche
             const int strip = w % args.strips, chunk = w / args.strips;
             const int y0 = int((long long)args.Ny * chunk / args.chunks);
             const int y1 = int((long long)args.Ny * (chunk + 1) / args.chunks);
-            march_share<float, BC, kBatchSteps, BD, BU, INTER, UNIT, VEC, false>(args, args.fam[0], strip, y0, y1,
-                                                                           smem_raw + warp * L::WARP, lane);
+            constexpr int NARROW = MODE & ~MODE_WIDE;
+            if ((MODE & MODE_WIDE) && item[4])
+                march_share<float, BC, kBatchSteps, BD, BU, INTER, MODE, VEC, false>(args, args.fam[0], strip, y0, y1,
+                                                                                   smem_raw + warp * L::WARP, lane);
+            else
+                march_share<float, BC, kBatchSteps, BD, BU, INTER, NARROW, VEC, false>(args, args.fam[0], strip, y0, y1,
+                                                                                     smem_raw + warp * L::WARP, lane);
         }
         __threadfence();
         __syncthreads();
@@ -158,11 +168,11 @@ __global__ void batch_flip(const BatchInst *inst, int *cur, int n) {
 
 // Sets the shared-memory attribute and returns the persistent grid size (SMs x
 // resident CTAs); called before stream capture. With S: launches *grid CTAs.
-template <bool INTER, bool UNIT, bool VEC>
+template <bool INTER, int MODE, bool VEC>
 cudaError_t batch_t(int sms, int *grid, const BatchSched *S, cudaStream_t st) {
     using L = MarchLayout<float, BC, kBatchSteps, BD, INTER>;
     constexpr int smem = L::WARP * BWPC;
-    auto kern = batch_kernel<INTER, UNIT, VEC>;
+    auto kern = batch_kernel<INTER, MODE, VEC>;
     if (S == nullptr) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -178,13 +188,18 @@ cudaError_t batch_t(int sms, int *grid, const BatchSched *S, cudaStream_t st) {
 
 // S == nullptr: prepare (attribute + grid size); otherwise launch with *grid CTAs.
 // vec: every lattice's rows copy in vectors (march_vectors).
-template <bool VEC>
-cudaError_t batch_modes(bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
-    if (inter) return unit ? batch_t<true, true, VEC>(sms, grid, S, st) : batch_t<true, false, VEC>(sms, grid, S, st);
-    return unit ? batch_t<false, true, VEC>(sms, grid, S, st) : batch_t<false, false, VEC>(sms, grid, S, st);
+template <bool INTER, bool VEC>
+cudaError_t batch_mode(int mode, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
+    switch (mode) {
+        case 0: return batch_t<INTER, 0, VEC>(sms, grid, S, st);
+        case MODE_UNITARY: return batch_t<INTER, MODE_UNITARY, VEC>(sms, grid, S, st);
+        case MODE_UNITARY | MODE_WIDE: return batch_t<INTER, MODE_UNITARY | MODE_WIDE, VEC>(sms, grid, S, st);
+    }
+    return cudaErrorInvalidValue;
 }
-cudaError_t batch_dispatch(bool vec, bool inter, bool unit, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
-    return vec ? batch_modes<true>(inter, unit, sms, grid, S, st) : batch_modes<false>(inter, unit, sms, grid, S, st);
+cudaError_t batch_dispatch(bool vec, bool inter, int mode, int sms, int *grid, const BatchSched *S, cudaStream_t st) {
+    if (vec) return inter ? batch_mode<true, true>(mode, sms, grid, S, st) : batch_mode<false, true>(mode, sms, grid, S, st);
+    return inter ? batch_mode<true, false>(mode, sms, grid, S, st) : batch_mode<false, false>(mode, sms, grid, S, st);
 }
 
 }  // namespace qla
@@ -198,7 +213,8 @@ struct qla_batch {
     int K = 4;
     int dev = 0;
     int sms = 152;
-    bool inter = true, unit = false, vec = true;
+    bool inter = true, vec = true;
+    int mode = 0;  // SweepMode: MODE_WIDE if any lattice's
     cudaStream_t stream = nullptr;
     std::vector<qla::BatchInst> inst;  // sorted order
     std::vector<int> order;            // order[k] = user index of sorted instance k
@@ -264,6 +280,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     if (o.precision != QLA_FP32 || o.families != QLA_FAMILIES_BOTH) return QLA_EUNSUPPORTED;
     const int K = o.steps_per_pass > 0 ? o.steps_per_pass : 4;
     if (K != 2 && K != 4) return QLA_EUNSUPPORTED;
+    std::vector<int> modes(count);
     for (int i = 0; i < count; ++i) {
         const qla_instance_desc &d = descs[i];
         if (d.Nx < 4 || d.Ny < 1 || d.Nx % 4 != 0 || (long long)d.Nx * d.Ny > 2147483647LL) return QLA_EINVAL;
@@ -271,9 +288,11 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         if (d.nsteps < 0 || d.nsteps % K != 0) return QLA_EINVAL;
         const size_t P = size_t(d.Nx) * d.Ny;
         const double *nn[3] = {d.n_x, d.n_y, d.n_z};
+        bool ordinary = true;
         for (int k = 0; k < 3; ++k)
-            for (size_t s = 0; s < P; ++s)
-                if (!(nn[k][s] > 0.0) || !std::isfinite(nn[k][s])) return QLA_EINVAL;
+            if (!qla::index_valid(nn[k], P, &ordinary)) return QLA_EINVAL;
+        modes[i] = qla::rotation_mode(nn, ordinary, d.Nx, d.Ny, d.delta, 0, o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0,
+                                      o.potential == QLA_POT_UNITARY ? 1 : 0);
     }
     qla_batch *b = new qla_batch();
     auto bail = [&](qla_status s) {
@@ -283,7 +302,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     b->n = count;
     b->K = K;
     b->inter = o.sequence == QLA_SEQ_INTERLEAVED;
-    b->unit = o.potential == QLA_POT_UNITARY;
+    for (const int m : modes) b->mode |= m;
     if (o.device >= 0) {
         if (cudaSetDevice(o.device) != cudaSuccess) return bail(QLA_ECUDA);
         b->dev = o.device;
@@ -324,6 +343,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         I.chunks = (d.Ny + ch - 1) / ch;
         I.tiles = (I.strips * I.chunks + qla::BWPC - 1) / qla::BWPC;
         I.passes = int(d.nsteps / qla::kBatchSteps);
+        I.wide = modes[b->order[k]] & qla::MODE_WIDE ? 1 : 0;
         float *q0, *q1;
         char *mem;
         double *idx;
@@ -342,7 +362,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         for (int c = 0; c < 3; ++c)
             if (cudaMemcpyAsync(idx + c * P, nn[c], P * 8, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
                 return bail(QLA_ECUDA);
-        if (qla::launch_march_records(g, idx, mem, 2, 0, d.delta, 0, b->inter ? 1 : 0, b->unit ? 1 : 0, b->stream) !=
+        if (qla::launch_march_records(g, idx, mem, 2, 0, d.delta, 0, b->inter ? 1 : 0, modes[b->order[k]], b->stream) !=
             cudaSuccess)
             return bail(QLA_ECUDA);
         if (cudaMemsetAsync(q0, 0, 6 * P * 4, b->stream) != cudaSuccess ||
@@ -392,7 +412,7 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(b->d_cur, 0, sizeof(int) * count) != cudaSuccess)
         return bail(QLA_ECUDA);
-    if (qla::batch_dispatch(b->vec, b->inter, b->unit, b->sms, &b->grid, nullptr, nullptr) != cudaSuccess)
+    if (qla::batch_dispatch(b->vec, b->inter, b->mode, b->sms, &b->grid, nullptr, nullptr) != cudaSuccess)
         return bail(QLA_ECUDA);
     *out = b;
     return QLA_OK;
@@ -420,7 +440,7 @@ qla_status qla_batch_run(qla_batch *b) {
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned) * 2 * b->n, b->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_error, 0, 64, b->stream);
         if (e == cudaSuccess && b->maxpass > 0)
-            e = qla::batch_dispatch(b->vec, b->inter, b->unit, b->sms, &b->grid, &S, b->stream);
+            e = qla::batch_dispatch(b->vec, b->inter, b->mode, b->sms, &b->grid, &S, b->stream);
         if (e == cudaSuccess) {
             qla::batch_flip<<<(b->n + 127) / 128, 128, 0, b->stream>>>(b->d_inst, b->d_cur, b->n);
             e = cudaGetLastError();

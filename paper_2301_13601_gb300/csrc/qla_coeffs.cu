@@ -2,6 +2,9 @@
 // initial condition and precision conversions.
 #include <math.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "qla_internal.h"
 
 namespace qla {
@@ -19,13 +22,48 @@ __device__ void rotation_pair_f32(double ang, float &tf, float &sf) {
     sf = (float)(2.0 * t / (1.0 + t * t));
 }
 
+// FP32 (cos(a) - 1, sin(a)) pair chosen among FP32 values within a few ulps of
+// the correctly rounded ones so that (1 + m)^2 + s^2 - 1 (evaluated exactly in
+// FP64: every term is a product of two FP32 values) is as small as possible:
+// each rotation then keeps the energy (Eq. 27) closely, with the angle changed
+// by a few ulps of m and s at most.
+__device__ void wide_pair_f32(double ang, float &mf, float &sf) {
+    const double sh = sin(0.5 * ang);
+    mf = (float)(-2.0 * sh * sh);  // cos(ang) - 1 without cancellation
+    sf = (float)sin(ang);
+    if (!(fabsf(mf) >= 1e-30f) || !(fabsf(sf) >= 1e-30f)) return;  // zero or nearly: the rounded values
+    const int mi = __float_as_int(mf), si = __float_as_int(sf);
+    double best = 1e300;
+    int bdm = 0, bds = 0;
+    for (int dm = -4; dm <= 4; ++dm) {
+        for (int ds = -2; ds <= 2; ++ds) {
+            const double m = (double)__int_as_float(mi + dm), s = (double)__int_as_float(si + ds);
+            const double e = fabs(2.0 * m + m * m + s * s);
+            if (e < best || (e == best && abs(dm) + abs(ds) < abs(bdm) + abs(bds))) {
+                best = e;
+                bdm = dm;
+                bds = ds;
+            }
+        }
+    }
+    mf = __int_as_float(mi + bdm);
+    sf = __int_as_float(si + bds);
+}
+
 // How a pair is stored (see CoefPair and rot in the sweep): a rotation
-// (tan(a/2), sin a) or a printed potential row (cos a - 1, sin a).
-enum PairKind { PK_ROTATION, PK_PRINTED_V };
+// (tan(a/2), sin a), one in the form for any angle (cos a - 1, sin a), or a
+// printed potential row (cos a - 1, sin a).
+enum PairKind { PK_ROTATION, PK_WIDE, PK_PRINTED_V };
+__device__ __forceinline__ PairKind rotation_kind(int mode) { return mode & MODE_WIDE ? PK_WIDE : PK_ROTATION; }
 
 template <typename T>
 __device__ void make_pair_of(double ang, PairKind kind, T &x, T &y) {
-    if (kind == PK_PRINTED_V) {
+    if (sizeof(T) == 4 && kind == PK_WIDE) {
+        float m, sn;
+        wide_pair_f32(ang, m, sn);
+        x = m;
+        y = sn;
+    } else if (kind != PK_ROTATION) {
         const double sh = sin(0.5 * ang);
         x = (T)(-2.0 * sh * sh);  // cos(ang) - 1 without cancellation
         y = (T)sin(ang);
@@ -59,12 +97,12 @@ __device__ __forceinline__ double potential_angle(const double *__restrict__ n, 
 // One thread per site. n: [3][Ny][Nx] double (n_x, n_y, n_z).
 template <typename T>
 __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, int Nx, int Ny, double delta,
-                            int interleaved, int unitary) {
+                            int interleaved, int mode) {
     const size_t P = size_t(Nx) * size_t(Ny);
     const double *nx = n, *ny = n + P, *nz = n + 2 * P;
     // effective potential angle: halved when interleaved (Eq. 28), halved
     // again for the unitary pair rotation
-    const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
+    const double vscale = (interleaved ? 0.5 : 1.0) * (mode & MODE_UNITARY ? 0.5 : 1.0);
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < P; i += size_t(gridDim.x) * blockDim.x) {
         const int y = int(i / Nx), x = int(i % Nx);
         // Eq. 24
@@ -73,10 +111,10 @@ __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, 
         const double b1 = potential_angle(nx, x, y, Nx, Ny, 1, delta);
         const double b2 = potential_angle(nz, x, y, Nx, Ny, 0, delta);
         const double b3 = potential_angle(nz, x, y, Nx, Ny, 1, delta);
-        const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
-        store_pair<T>(coef, P, P_TM_C, i, th2, PK_ROTATION);
-        store_pair<T>(coef, P, P_TE_CX, i, th1, PK_ROTATION);
-        store_pair<T>(coef, P, P_TE_CY, i, th0, PK_ROTATION);
+        const PairKind ck = rotation_kind(mode), vk = mode & MODE_UNITARY ? ck : PK_PRINTED_V;
+        store_pair<T>(coef, P, P_TM_C, i, th2, ck);
+        store_pair<T>(coef, P, P_TE_CX, i, th1, ck);
+        store_pair<T>(coef, P, P_TE_CY, i, th0, ck);
         store_pair<T>(coef, P, P_TM_VX, i, b2 * vscale, vk);
         store_pair<T>(coef, P, P_TM_VY, i, b3 * vscale, vk);
         store_pair<T>(coef, P, P_TE_VX, i, b0 * vscale, vk);
@@ -87,12 +125,12 @@ __global__ void coef_kernel(const double *__restrict__ n, T *__restrict__ coef, 
 // The same pairs as the marching form's records (one block per row of a strip).
 template <typename T>
 __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict__ rec, int fam, MarchGeo g,
-                                     double delta, int interleaved, int unitary) {
+                                     double delta, int interleaved, int mode) {
     const size_t P = size_t(g.Nx) * size_t(g.Ny);
     const double *nx = n, *ny = n + P, *nz = n + 2 * P;
     const double *ncx = fam ? ny : nz, *ncy = fam ? nx : nz;  // indices of C_X and V_X, of C_Y and V_Y
-    const double vscale = (interleaved ? 0.5 : 1.0) * (unitary ? 0.5 : 1.0);
-    const PairKind vk = unitary ? PK_ROTATION : PK_PRINTED_V;
+    const double vscale = (interleaved ? 0.5 : 1.0) * (mode & MODE_UNITARY ? 0.5 : 1.0);
+    const PairKind ck = rotation_kind(mode), vk = mode & MODE_UNITARY ? ck : PK_PRINTED_V;
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW, strip = blockIdx.x;
     for (int r = blockIdx.y; r < rows; r += gridDim.y) {
         int y = (r - MARCH_ABOVE) % g.Ny;
@@ -103,8 +141,8 @@ __global__ void march_records_kernel(const double *__restrict__ n, T *__restrict
             const size_t i = size_t(y) * g.Nx + x;
             T *const d = rec + (size_t(strip) * rows + r) * MARCH_FIELDS * g.W +
                          march_column(c, int(sizeof(T)));
-            make_pair_of<T>(delta / (4.0 * ncx[i]), PK_ROTATION, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
-            if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), PK_ROTATION, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
+            make_pair_of<T>(delta / (4.0 * ncx[i]), ck, d[F_CX * g.W], d[(F_CX + 1) * g.W]);
+            if (fam) make_pair_of<T>(delta / (4.0 * ncy[i]), ck, d[F_CY * g.W], d[(F_CY + 1) * g.W]);
             for (int axis = 0; axis < 2; ++axis) {
                 const double b = potential_angle(axis ? ncy : ncx, x, y, g.Nx, g.Ny, axis, delta) * vscale;
                 T *const v = d + (axis ? F_VY : F_VX) * g.W;
@@ -196,21 +234,81 @@ int grid_for(size_t n, int block) {
 
 }  // namespace
 
+namespace {
+// Smallest and largest value of a plane (16 independent chains; one alone is bound
+// by the latency of its comparisons).
+void plane_range(const double *n, size_t P, double range[2]) {
+    constexpr int L = 16;
+    double lo[L], hi[L];
+    for (int k = 0; k < L; ++k) lo[k] = hi[k] = n[0];
+    auto take = [&](int k, double v) {
+        lo[k] = v < lo[k] ? v : lo[k];
+        hi[k] = v > hi[k] ? v : hi[k];
+    };
+    size_t i = 0;
+    for (; i + L <= P; i += L)
+        for (int k = 0; k < L; ++k) take(k, n[i + k]);
+    for (; i < P; ++i) take(0, n[i]);
+    range[0] = *std::min_element(lo, lo + L);
+    range[1] = *std::max_element(hi, hi + L);
+}
+}  // namespace
+
+bool index_valid(const double *n, size_t P, bool *ordinary) {
+    for (size_t i = 0; i < P; ++i) {
+        const double v = n[i];
+        if (v >= kOrdinaryIndex[0] && v <= kOrdinaryIndex[1]) continue;
+        *ordinary = false;
+        if (!(v > 0.0) || !std::isfinite(v)) return false;
+    }
+    return true;
+}
+
+int rotation_mode(const double *const n[3], bool ordinary, int Nx, int Ny, double delta, int precision, int interleaved,
+                  int unitary) {
+    const int mode = unitary ? MODE_UNITARY : 0;
+    if (ordinary) return mode;
+    if (precision == 0 && !unitary) return mode;  // collisions are shears, potential rows no rotations
+    double range[3][2];
+    for (int k = 0; k < 3; ++k) {
+        plane_range(n[k], size_t(Nx) * Ny, range[k]);
+        if (delta / (4.0 * range[k][0]) > kHalfAngleLimit) return mode | MODE_WIDE;  // Eq. 24
+    }
+    if (!unitary) return mode;
+    // Eq. 25: n_y along x, n_x along y, n_z along both. Sites are looked at only if
+    // the planes' ranges leave the possibility.
+    const double scale = 0.5 * delta * (interleaved ? 0.5 : 1.0) * 0.5;
+    for (int k = 0; k < 3; ++k) {
+        if (scale * (range[k][1] - range[k][0]) / (range[k][0] * range[k][0]) <= kHalfAngleLimit) continue;
+        const double *const p = n[k];
+        for (int y = 0; y < Ny; ++y) {
+            const double *const r = p + size_t(y) * Nx;
+            const double *const up = p + size_t(y + 1 == Ny ? 0 : y + 1) * Nx, *const dn = p + size_t(y ? y - 1 : Ny - 1) * Nx;
+            for (int x = 0; x < Nx; ++x) {
+                const double dx = r[x + 1 == Nx ? 0 : x + 1] - r[x ? x - 1 : Nx - 1], dy = up[x] - dn[x];
+                const double d = fmax(k != 0 ? fabs(dx) : 0.0, k != 1 ? fabs(dy) : 0.0);
+                if (!(scale * d / (r[x] * r[x]) <= kHalfAngleLimit)) return mode | MODE_WIDE;
+            }
+        }
+    }
+    return mode;
+}
+
 cudaError_t launch_coefficients(const double *n, void *coef, int Nx, int Ny, double delta, int precision,
-                                int interleaved, int unitary, cudaStream_t st) {
+                                int interleaved, int mode, cudaStream_t st) {
     const size_t P = size_t(Nx) * size_t(Ny);
     const int B = 256;
     if (precision == 0)
         coef_kernel<float><<<grid_for(P, B), B, 0, st>>>(n, static_cast<float *>(coef), Nx, Ny, delta,
-                                                          interleaved, unitary);
+                                                          interleaved, mode);
     else
         coef_kernel<double><<<grid_for(P, B), B, 0, st>>>(n, static_cast<double *>(coef), Nx, Ny, delta,
-                                                           interleaved, unitary);
+                                                           interleaved, mode);
     return cudaGetLastError();
 }
 
 cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, int nfam, int fam0, double delta,
-                                 int precision, int interleaved, int unitary, cudaStream_t st) {
+                                 int precision, int interleaved, int mode, cudaStream_t st) {
     char *m = static_cast<char *>(mem);
     const int rows = MARCH_ABOVE + g.Ny + MARCH_BELOW;
     const int fblocks = (g.Ny + FLAG_ROWS - 1) / FLAG_ROWS;
@@ -221,11 +319,11 @@ cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, 
         unsigned char *flags = reinterpret_cast<unsigned char *>(m + nfam * g.record_bytes + z * g.flag_bytes);
         if (precision == 0) {
             march_records_kernel<float><<<grid, g.W, 0, st>>>(n, static_cast<float *>(rec), fam0 + z, g, delta,
-                                                              interleaved, unitary);
+                                                              interleaved, mode);
             march_flags_kernel<float><<<fgrid, 256, 0, st>>>(static_cast<const float *>(rec), flags, fam0 + z, g);
         } else {
             march_records_kernel<double><<<grid, g.W, 0, st>>>(n, static_cast<double *>(rec), fam0 + z, g, delta,
-                                                               interleaved, unitary);
+                                                               interleaved, mode);
             march_flags_kernel<double><<<fgrid, 256, 0, st>>>(static_cast<const double *>(rec), flags, fam0 + z, g);
         }
         const cudaError_t e = cudaGetLastError();

@@ -36,53 +36,53 @@ struct CoefView {
     }
 };
 
-template <bool DAG, int SG, bool SHR, typename T>
+template <bool DAG, int SG, RotForm FORM, typename T>
 __device__ __forceinline__ void rot_pair(T *q, const CoefView<T> &cp, long long P, long long i, int hub,
                                          int partner, int plane) {
     if (!cp.has(plane)) return;
     const typename Ar<T>::T2 c = cp.at(plane, P, i);
     T h = q[hub * P + i], p = q[partner * P + i];
-    rot<DAG, SG, SHR>(h, p, c.x, c.y);
+    rot<DAG, SG, FORM>(h, p, c.x, c.y);
     q[hub * P + i] = h;
     q[partner * P + i] = p;
 }
 
 // C_X (axis 0) or C_Y (axis 1) on both families, or their transposes.
-template <int AXIS, bool DAG, bool SHR, typename T>
+template <int AXIS, bool DAG, RotForm FORM, typename T>
 __global__ void __launch_bounds__(DBG_THREADS) collide_kernel(T *q, const CoefView<T> cp, long long P) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
         if (AXIS == 0) {
-            rot_pair<DAG, Fam<0>::SGX, SHR>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::CX);
-            rot_pair<DAG, Fam<1>::SGX, SHR>(q, cp, P, i, Fam<1>::H, Fam<1>::PX, Fam<1>::CX);
+            rot_pair<DAG, Fam<0>::SGX, FORM>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::CX);
+            rot_pair<DAG, Fam<1>::SGX, FORM>(q, cp, P, i, Fam<1>::H, Fam<1>::PX, Fam<1>::CX);
         } else {
-            rot_pair<DAG, Fam<0>::SGY, SHR>(q, cp, P, i, Fam<0>::H, Fam<0>::PY, Fam<0>::CY);
-            rot_pair<DAG, Fam<1>::SGY, SHR>(q, cp, P, i, Fam<1>::H, Fam<1>::PY, Fam<1>::CY);
+            rot_pair<DAG, Fam<0>::SGY, FORM>(q, cp, P, i, Fam<0>::H, Fam<0>::PY, Fam<0>::CY);
+            rot_pair<DAG, Fam<1>::SGY, FORM>(q, cp, P, i, Fam<1>::H, Fam<1>::PY, Fam<1>::CY);
         }
     }
 }
 
-template <int TAU, bool HUB, bool UNIT, typename T>
+template <int TAU, bool HUB, int MODE, typename T>
 __device__ __forceinline__ void pot_pair(T *q, const CoefView<T> &cp, long long P, long long i, int hub,
                                          int partner, int plane) {
     if (!cp.has(plane)) return;
     const typename Ar<T>::T2 c = cp.at(plane, P, i);  // (cos b - 1, sin b)
     T h = q[hub * P + i], p = q[partner * P + i];
-    vop_pair<TAU, HUB, UNIT>(h, p, c.y, c.x);
+    vop_pair<TAU, HUB, MODE>(h, p, c.y, c.x);
     q[hub * P + i] = h;
     q[partner * P + i] = p;
 }
 
 // V_X (axis 0) or V_Y (axis 1) on both families, as one application in the
 // context's step (its pair planes hold that application's angles).
-template <int AXIS, bool UNIT, typename T>
+template <int AXIS, int MODE, typename T>
 __global__ void __launch_bounds__(DBG_THREADS) potential_kernel(T *q, const CoefView<T> cp, long long P) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
         if (AXIS == 0) {
-            pot_pair<Fam<0>::TX, Fam<0>::VX_HUB, UNIT>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::VX);
-            pot_pair<Fam<1>::TX, Fam<1>::VX_HUB, UNIT>(q, cp, P, i, Fam<1>::H, Fam<1>::PX, Fam<1>::VX);
+            pot_pair<Fam<0>::TX, Fam<0>::VX_HUB, MODE>(q, cp, P, i, Fam<0>::H, Fam<0>::PX, Fam<0>::VX);
+            pot_pair<Fam<1>::TX, Fam<1>::VX_HUB, MODE>(q, cp, P, i, Fam<1>::H, Fam<1>::PX, Fam<1>::VX);
         } else {
-            pot_pair<Fam<0>::TY, Fam<0>::VY_HUB, UNIT>(q, cp, P, i, Fam<0>::H, Fam<0>::PY, Fam<0>::VY);
-            pot_pair<Fam<1>::TY, Fam<1>::VY_HUB, UNIT>(q, cp, P, i, Fam<1>::H, Fam<1>::PY, Fam<1>::VY);
+            pot_pair<Fam<0>::TY, Fam<0>::VY_HUB, MODE>(q, cp, P, i, Fam<0>::H, Fam<0>::PY, Fam<0>::VY);
+            pot_pair<Fam<1>::TY, Fam<1>::VY_HUB, MODE>(q, cp, P, i, Fam<1>::H, Fam<1>::PY, Fam<1>::VY);
         }
     }
 }
@@ -107,9 +107,29 @@ __global__ void __launch_bounds__(DBG_THREADS) stream_kernel(const T *__restrict
     }
 }
 
+template <typename T, RotForm FORM>
+void collide(int op, T *q, const CoefView<T> &cp, long long P, int blocks, cudaStream_t st) {
+    switch (op) {
+        case QLA_OP_CX: collide_kernel<0, false, FORM><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
+        case QLA_OP_CX_T: collide_kernel<0, true, FORM><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
+        case QLA_OP_CY: collide_kernel<1, false, FORM><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
+        default: collide_kernel<1, true, FORM><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
+    }
+}
+
+template <typename T, int AXIS>
+void potential(int mode, T *q, const CoefView<T> &cp, long long P, int blocks, cudaStream_t st) {
+    if (!(mode & MODE_UNITARY))
+        potential_kernel<AXIS, 0><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
+    else if (mode & MODE_WIDE)
+        potential_kernel<AXIS, MODE_UNITARY | MODE_WIDE><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
+    else
+        potential_kernel<AXIS, MODE_UNITARY><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
+}
+
 template <typename T>
 cudaError_t apply_t(int op, void *state, void *spare, const void *coef, const MarchGeo *geo, int nfam, int fam0, int Nx,
-                    int Ny, int unitary, cudaStream_t st, bool *swapped) {
+                    int Ny, int mode, cudaStream_t st, bool *swapped) {
     T *q = static_cast<T *>(state);
     CoefView<T> cp{};
     if (geo) {
@@ -126,29 +146,17 @@ cudaError_t apply_t(int op, void *state, void *spare, const void *coef, const Ma
         case QLA_OP_CX:
         case QLA_OP_CX_T:
         case QLA_OP_CY:
-        case QLA_OP_CY_T: {
+        case QLA_OP_CY_T:
             // the collision form of the context's configuration (see rot)
-            const bool shear = shear_collisions<T, false>() && !unitary;
-            const int k = (op == QLA_OP_CX ? 0 : op == QLA_OP_CX_T ? 1 : op == QLA_OP_CY ? 2 : 3) + (shear ? 4 : 0);
-            switch (k) {
-                case 0: collide_kernel<0, false, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 1: collide_kernel<0, true, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 2: collide_kernel<1, false, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 3: collide_kernel<1, true, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 4: collide_kernel<0, false, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 5: collide_kernel<0, true, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                case 6: collide_kernel<1, false, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-                default: collide_kernel<1, true, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P); break;
-            }
+            if (rot_form<T, 0>() == ROT_SHEAR && !(mode & MODE_UNITARY)) collide<T, ROT_SHEAR>(op, q, cp, P, blocks, st);
+            else if (mode & MODE_WIDE) collide<T, ROT_WIDE>(op, q, cp, P, blocks, st);
+            else collide<T, ROT_HALF>(op, q, cp, P, blocks, st);
             break;
-        }
         case QLA_OP_VX:
-            if (unitary) potential_kernel<0, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
-            else potential_kernel<0, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
+            potential<T, 0>(mode, q, cp, P, blocks, st);
             break;
         case QLA_OP_VY:
-            if (unitary) potential_kernel<1, true><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
-            else potential_kernel<1, false><<<blocks, DBG_THREADS, 0, st>>>(q, cp, P);
+            potential<T, 1>(mode, q, cp, P, blocks, st);
             break;
         default: {
             // streaming ops QLA_OP_S14_XP .. QLA_OP_S25_YM: (components, axis, direction)
@@ -166,10 +174,10 @@ cudaError_t apply_t(int op, void *state, void *spare, const void *coef, const Ma
 }  // namespace
 
 cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, const MarchGeo *geo,
-                        int nfam, int fam0, int Nx, int Ny, int unitary, cudaStream_t st, bool *swapped) {
+                        int nfam, int fam0, int Nx, int Ny, int mode, cudaStream_t st, bool *swapped) {
     return precision == QLA_FP64
-               ? apply_t<double>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, unitary, st, swapped)
-               : apply_t<float>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, unitary, st, swapped);
+               ? apply_t<double>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, mode, st, swapped)
+               : apply_t<float>(op, state, spare, coef, geo, nfam, fam0, Nx, Ny, mode, st, swapped);
 }
 
 }  // namespace qla

@@ -8,14 +8,21 @@
 
 namespace qla {
 
+// Kernel variant of a context (template parameter MODE of the sweeps, a sum of):
+// unitary potentials; rotations in the form for any angle (rot in
+// qla_sweep.cuh), chosen by rotation_mode where the half-angle form loses
+// accuracy.
+enum SweepMode { MODE_UNITARY = 1, MODE_WIDE = 2 };
+
 // Coefficient pair planes: NPAIR planes of [Ny][Nx] pairs, element type =
 // state precision. The angle a is a collision angle (Eq. 24) or an effective
 // potential angle b (Eq. 25, scaled by 1/2 when interleaved (Eq. 28) and by
 // 1/2 again for the unitary potentials).
 // A collision pair, and a potential pair of the unitary potentials, is
-// (x = tan(a/2), y = sin(a)); a printed potential pair is (cos(b) - 1, sin(b)).
-// FP32 rotation pairs take y nearest to 2x / (1 + x^2). Signs of the operators are
-// applied by the kernels.
+// (x = tan(a/2), y = sin(a)), or with MODE_WIDE (cos(a) - 1, sin(a)); a printed
+// potential pair is (cos(b) - 1, sin(b)). FP32 rotation pairs take y nearest to
+// 2x / (1 + x^2), with MODE_WIDE the nearby pair closest to orthogonality. Signs of
+// the operators are applied by the kernels.
 // The order puts the two planes that the sweep copies together next to each
 // other: (V_X, C_X) for the x-pass and (C_Y, V_Y) for the y-pass of a family.
 enum CoefPair {
@@ -204,7 +211,7 @@ struct SweepArgs {
     // order they start; null: share = blockIdx.x.
     unsigned *order;
     int interleaved;    // 1: Eq. 28, 0: Eq. 23
-    int unitary;        // 1: unitary potentials
+    int mode;           // SweepMode
     int vec;            // 1: 16-byte vector access is legal (Nx multiple of 16/sizeof(T))
     int fam0;           // first family index handled by blockIdx.z = 0 (0 = TM, 1 = TE)
     int *error;         // device flag set when a bounded wait of the TMA copy path runs out (null: no TMA)
@@ -214,6 +221,9 @@ struct SweepArgs {
 // Returns cudaSuccess or the launch error.
 cudaError_t launch_sweep_f32(int K, const SweepArgs &a, int nfam, cudaStream_t st);
 cudaError_t launch_sweep_f64(int K, const SweepArgs &a, int nfam, cudaStream_t st);
+// MODE_WIDE, K = 1 only (launch_sweep_f32 and _f64 go there by themselves).
+cudaError_t launch_sweep_wide_f32(int K, const SweepArgs &a, int nfam, cudaStream_t st);
+cudaError_t launch_sweep_wide_f64(int K, const SweepArgs &a, int nfam, cudaStream_t st);
 bool sweep_supported(int precision, int K);
 // Persistent form of the balanced split (qla_sweep_persist.cu): `passes`
 // passes of K steps in one cooperative launch of a.ctas CTAs (at most
@@ -277,14 +287,26 @@ void march_plan(MarchGeo *g, int nfam, int chunk, int sms);
 // the last launch on the stream was such a pass, over the same records.
 size_t march_bytes(const MarchGeo &g, int nfam);
 cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out, const void *mem, int nfam, int fam0,
-                         int interleaved, int unitary, bool chained, cudaStream_t st);
+                         int interleaved, int mode, bool chained, cudaStream_t st);
 // Records and flags from the device index planes n[3][Ny][Nx] (double).
 cudaError_t launch_march_records(const MarchGeo &g, const double *n, void *mem, int nfam, int fam0, double delta,
-                                 int precision, int interleaved, int unitary, cudaStream_t st);
+                                 int precision, int interleaved, int mode, cudaStream_t st);
+
+// Whether every value of an index plane is positive and finite; *ordinary is cleared
+// if one lies outside kOrdinaryIndex, the range in which no angle passes
+// kHalfAngleLimit whatever delta (<= 0.5) and the medium: a collision stays below
+// 0.5 / (4 0.9), a potential rotation below 0.5 (4 - 0.9) / (4 0.9^2) = 0.48.
+constexpr double kOrdinaryIndex[2] = {0.9, 4.0};
+bool index_valid(const double *n, size_t P, bool *ordinary);
+// SweepMode of a medium (n: host planes n_x, n_y, n_z, index_valid): MODE_WIDE if a rotation by more than kHalfAngleLimit occurs, in any
+// family, so that a family alone is advanced as beside the other.
+constexpr double kHalfAngleLimit = 0.5;
+int rotation_mode(const double *const n[3], bool ordinary, int Nx, int Ny, double delta, int precision, int interleaved,
+                  int unitary);
 
 // Coefficients (Eq. 24-25) from the device index planes n[3][Ny][Nx] (double).
 cudaError_t launch_coefficients(const double *n, void *coef, int Nx, int Ny, double delta,
-                                int precision, int interleaved, int unitary, cudaStream_t st);
+                                int precision, int interleaved, int mode, cudaStream_t st);
 // Pulse initial condition into state (precision-typed) [6][Ny][Nx].
 cudaError_t launch_init_pulse(void *q, int Nx, int Ny, int precision, int pol, double x0,
                               double sigma, double amp, cudaStream_t st);
@@ -367,7 +389,7 @@ cudaError_t launch_pack_weights(const float *w, int nout, int cin, int nout_pad,
 // records of families fam0 .. fam0 + nfam - 1 (a family without records is zero
 // and stays so).
 cudaError_t debug_apply(int op, int precision, void *state, void *spare, const void *coef, const MarchGeo *geo,
-                        int nfam, int fam0, int Nx, int Ny, int unitary, cudaStream_t st, bool *swapped);
+                        int nfam, int fam0, int Nx, int Ny, int mode, cudaStream_t st, bool *swapped);
 
 }  // namespace qla
 

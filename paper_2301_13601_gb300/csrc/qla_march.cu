@@ -78,7 +78,7 @@ void march_plan(MarchGeo *g, int nfam, int chunk, int sms) {
 }
 
 cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out, const void *mem, int nfam, int fam0,
-                         int interleaved, int unitary, bool chained, cudaStream_t st) {
+                         int interleaved, int mode, bool chained, cudaStream_t st) {
     const bool f64 = g.es == 8;
     if (!(K == 1 || (K == 2 && !f64))) return cudaErrorInvalidValue;
     MarchArgs a;
@@ -99,12 +99,12 @@ cudaError_t launch_march(const MarchGeo &g, int K, const void *q_in, void *q_out
     a.chained = chained ? 1 : 0;
     a.chunks = g.chunks[K];
     const bool vec = march_vectors(g);
-    if (f64) return vec ? launch_march_f64_k1(a, nfam, interleaved, unitary, st)
-                        : launch_march_f64_k1_any(a, nfam, interleaved, unitary, st);
-    if (K == 2) return vec ? launch_march_f32_k2(a, nfam, interleaved, unitary, st)
-                           : launch_march_f32_k2_any(a, nfam, interleaved, unitary, st);
-    return vec ? launch_march_f32_k1(a, nfam, interleaved, unitary, st)
-               : launch_march_f32_k1_any(a, nfam, interleaved, unitary, st);
+    if (f64) return vec ? launch_march_f64_k1(a, nfam, interleaved, mode, st)
+                        : launch_march_f64_k1_any(a, nfam, interleaved, mode, st);
+    if (K == 2) return vec ? launch_march_f32_k2(a, nfam, interleaved, mode, st)
+                           : launch_march_f32_k2_any(a, nfam, interleaved, mode, st);
+    return vec ? launch_march_f32_k1(a, nfam, interleaved, mode, st)
+               : launch_march_f32_k1_any(a, nfam, interleaved, mode, st);
 }
 
 }  // namespace qla

@@ -157,14 +157,19 @@ struct MarchVec<double> {
 };
 
 // rot and vop_pair of qla_sweep.cuh on vectors.
-template <bool DAG, int SG, bool SHEAR, typename T, typename V = typename MarchVec<T>::V>
+template <bool DAG, int SG, RotForm FORM, typename T, typename V = typename MarchVec<T>::V>
 __device__ __forceinline__ void march_rot(V &h, V &p, V m, V s) {
     using A = MarchVec<T>;
     constexpr bool pos = (SG > 0) != DAG;
-    if constexpr (SHEAR) {
+    if constexpr (FORM == ROT_SHEAR) {
         h = A::fma(pos ? m : A::neg(m), p, h);
         p = A::fma(pos ? A::neg(s) : s, h, p);
         h = A::fma(pos ? m : A::neg(m), p, h);
+    } else if constexpr (FORM == ROT_WIDE) {
+        const V sp = A::mul(s, p), sh = A::mul(s, h);
+        const V u = A::fma(m, h, pos ? sp : A::neg(sp)), v = A::fma(m, p, pos ? A::neg(sh) : sh);
+        h = A::add(h, u);
+        p = A::add(p, v);
     } else {
         const V t = pos ? A::neg(m) : m, u = A::fma(t, h, p);
         if constexpr (sizeof(T) == 4) {
@@ -178,13 +183,13 @@ __device__ __forceinline__ void march_rot(V &h, V &p, V m, V s) {
         }
     }
 }
-template <int TAU, bool HUB, bool UNIT, typename T, typename V = typename MarchVec<T>::V>
+template <int TAU, bool HUB, int MODE, typename T, typename V = typename MarchVec<T>::V>
 __device__ __forceinline__ void march_vop(V &h, V &p, V s, V c) {
     using A = MarchVec<T>;
     V &t = HUB ? h : p;
     V &src = HUB ? p : h;
-    if constexpr (UNIT) {
-        march_rot<false, TAU, false, T>(t, src, c, s);
+    if constexpr (MODE & MODE_UNITARY) {
+        march_rot<false, TAU, rot_form<T, MODE>(), T>(t, src, c, s);
     } else {
         const V ss = A::mul(s, src);
         t = A::add(t, A::fma(c, t, TAU > 0 ? ss : A::neg(ss)));
@@ -301,7 +306,7 @@ static_assert(Fam<1>::SGX == -Fam<0>::SGX && Fam<1>::SGY == -Fam<0>::SGY && Fam<
 static_assert(!Fam<0>::VX_HUB && !Fam<0>::VY_HUB && Fam<1>::VX_HUB && Fam<1>::VY_HUB, "potential targets");
 
 // V' on the lane's columns of all levels (ld loads level j's coefficients).
-template <int TAU, bool UNIT, typename T, int K, int NV, typename V, class LD>
+template <int TAU, int MODE, typename T, int K, int NV, typename V, class LD>
 __device__ __forceinline__ void march_v(bool te, V (&h)[K][NV], V (&p)[K][NV], LD &&ld) {
 #pragma unroll
     for (int j = 0; j < K; ++j) {
@@ -309,10 +314,10 @@ __device__ __forceinline__ void march_v(bool te, V (&h)[K][NV], V (&p)[K][NV], L
         ld(j, m, s);
         if (te) {
 #pragma unroll
-            for (int c = 0; c < NV; ++c) march_vop<TAU, true, UNIT, T>(h[j][c], p[j][c], s[c], m[c]);
+            for (int c = 0; c < NV; ++c) march_vop<TAU, true, MODE, T>(h[j][c], p[j][c], s[c], m[c]);
         } else {
 #pragma unroll
-            for (int c = 0; c < NV; ++c) march_vop<TAU, false, UNIT, T>(h[j][c], p[j][c], s[c], m[c]);
+            for (int c = 0; c < NV; ++c) march_vop<TAU, false, MODE, T>(h[j][c], p[j][c], s[c], m[c]);
         }
     }
 }
@@ -321,12 +326,12 @@ __device__ __forceinline__ void march_v(bool te, V (&h)[K][NV], V (&p)[K][NV], L
 // row R_j of its input and leave as row R_j - 4 of its output. vx, vy2, vy4
 // load the V coefficients (V_X of row R, or of R - 4 with Eq. 23; V_Y of rows
 // R - 2 and R - 4).
-template <bool INTER, bool UNIT, typename T, int K, int NV, typename V, class VX, class VY2, class VY4>
+template <bool INTER, int MODE, typename T, int K, int NV, typename V, class VX, class VY2, class VY4>
 __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][NV], V (&p)[K][NV], V (&px)[K][NV],
                                            const V (&cxm)[K][NV], const V (&cxs)[K][NV], const V (&cym)[K][NV],
                                            const V (&cys)[K][NV], bool von, bool te, VX &&vx, VY2 &&vy2, VY4 &&vy4) {
     using Fm = Fam<0>;
-    constexpr bool SHR = shear_collisions<T, UNIT>();
+    constexpr RotForm SHR = rot_form<T, MODE>();
     constexpr int SX = Fm::SGX, SY = Fm::SGY;
 #define MARCH_ALL(expr)               \
     _Pragma("unroll") for (int j = 0; j < K; ++j) { expr; }
@@ -344,7 +349,7 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
     MARCH_X(false)
     MARCH_ALL((march_from_left<T, NV>(h[j])))
     if constexpr (INTER) {
-        if (von) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);
+        if (von) march_v<Fm::TX, MODE, T, K, NV, V>(te, h, px, vx);
     }
     MARCH_X(false)
     MARCH_ALL((march_from_right<T, NV>(px[j])))
@@ -355,7 +360,7 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
     MARCH_X(true)
     MARCH_ALL((march_from_right<T, NV>(h[j])))
     if constexpr (INTER) {
-        if (von) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);
+        if (von) march_v<Fm::TX, MODE, T, K, NV, V>(te, h, px, vx);
     }
     auto swap = [&](V (&a)[NV], V (&b)[NV]) {
 #pragma unroll
@@ -374,7 +379,7 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
     MARCH_Y(false, Y[j].m[1], Y[j].s[1])  // C    (row R-2)
     MARCH_ALL(swap(Y[j].S[3], h[j]))      // h <- h(r-1)
     if constexpr (INTER) {
-        if (von) march_v<Fm::TY, UNIT, T, K, NV, V>(te, h, p, vy2);  // V_Y' (row R-2)
+        if (von) march_v<Fm::TY, MODE, T, K, NV, V>(te, h, p, vy2);  // V_Y' (row R-2)
     }
     MARCH_Y(false, Y[j].m[1], Y[j].s[1])  // C    (row R-2)
     MARCH_ALL(swap(Y[j].S[4], h[j]))      // p <- p(r+1): now row R-3
@@ -402,8 +407,8 @@ __device__ __forceinline__ void march_rows(MarchPipe<V, NV> (&Y)[K], V (&h)[K][N
             Y[j].s[0][c] = cys[j][c];
         }
     if (von) {
-        if constexpr (!INTER) march_v<Fm::TX, UNIT, T, K, NV, V>(te, h, px, vx);  // V_X (row R-4)
-        march_v<Fm::TY, UNIT, T, K, NV, V>(te, h, p, vy4);                        // V_Y (row R-4)
+        if constexpr (!INTER) march_v<Fm::TX, MODE, T, K, NV, V>(te, h, px, vx);  // V_X (row R-4)
+        march_v<Fm::TY, MODE, T, K, NV, V>(te, h, p, vy4);                        // V_Y (row R-4)
     }
 #undef MARCH_ALL
 #undef MARCH_ROT
@@ -427,7 +432,7 @@ constexpr bool march_chains(int K) {
     return sizeof(T) == 4 && K == 1;
 }
 
-template <typename T, int C, int K, int D, int U, bool INTER, bool UNIT, bool VEC, bool CHAIN>
+template <typename T, int C, int K, int D, int U, bool INTER, int MODE, bool VEC, bool CHAIN>
 __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &F, int strip, int y0, int y1, unsigned char *sm,
                                             int lane) {
     using L = MarchLayout<T, C, K, D, INTER>;
@@ -611,7 +616,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
                     march_lds<T, NV>(s, vb + RB);
                 };
             };
-            march_rows<INTER, UNIT, T, K, NV, V>(pipe, hh, hp, hx, cxm, cxs, cym, cys, on, te, vrow(i & 1),
+            march_rows<INTER, MODE, T, K, NV, V>(pipe, hh, hp, hx, cxm, cxs, cym, cys, on, te, vrow(i & 1),
                                                  vrow(2 + ((i + 2) & 3)), vrow(INTER ? 2 + (i & 3) : 2 + (i & 1)));
             const int ro = it0 + u - march_delay(K);
             if (ro >= 0 && ro < n_out) {
@@ -650,7 +655,7 @@ __device__ __forceinline__ void march_share(const MarchArgs &A, const MarchFam &
     cp_async_wait_all();
 }
 
-template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, bool UNIT, bool VEC>
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, int MODE, bool VEC>
 __global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_constant__ MarchArgs A) {
     using L = MarchLayout<T, C, K, D, INTER>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -662,7 +667,7 @@ __global__ void __launch_bounds__(32 * WPC, MINB) march_kernel(const __grid_cons
     const int strip = w % A.strips, chunk = w / A.strips;
     const int y0 = int((long long)A.Ny * chunk / A.chunks);
     const int y1 = int((long long)A.Ny * (chunk + 1) / A.chunks);
-    march_share<T, C, K, D, U, INTER, UNIT, VEC, march_chains<T>(K)>(A, A.fam[layer], strip, y0, y1,
+    march_share<T, C, K, D, U, INTER, MODE, VEC, march_chains<T>(K)>(A, A.fam[layer], strip, y0, y1,
                                                                      smem_raw + warp * L::WARP, lane);
 }
 
@@ -688,10 +693,10 @@ __host__ __device__ MarchFam march_fam(const void *q_in, void *q_out, const void
     return f;
 }
 
-template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, bool UNIT, bool VEC>
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool INTER, int MODE, bool VEC>
 cudaError_t launch_march_t(const MarchArgs &a, int nfam, cudaStream_t st) {
     using L = MarchLayout<T, C, K, D, INTER>;
-    auto kern = march_kernel<T, C, K, D, U, WPC, MINB, INTER, UNIT, VEC>;
+    auto kern = march_kernel<T, C, K, D, U, WPC, MINB, INTER, MODE, VEC>;
     // set on every launch: the attribute belongs to the device, a process may use several
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::WARP * WPC);
     if (e != cudaSuccess) return e;
@@ -710,21 +715,31 @@ cudaError_t launch_march_t(const MarchArgs &a, int nfam, cudaStream_t st) {
     cudaLaunchKernelEx(&cfg, kern, m);
     return cudaGetLastError();
 }
+template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool VEC, bool INTER>
+cudaError_t launch_march_mode(const MarchArgs &a, int nfam, int mode, cudaStream_t st) {
+    constexpr int UW = MODE_UNITARY | MODE_WIDE;
+    switch (mode) {
+        case 0: return launch_march_t<T, C, K, D, U, WPC, MINB, INTER, 0, VEC>(a, nfam, st);
+        case MODE_UNITARY: return launch_march_t<T, C, K, D, U, WPC, MINB, INTER, MODE_UNITARY, VEC>(a, nfam, st);
+        case UW: return launch_march_t<T, C, K, D, U, WPC, MINB, INTER, UW, VEC>(a, nfam, st);
+        case MODE_WIDE:  // FP32 collisions are shears then (rotation_mode)
+            if constexpr (sizeof(T) == 8)
+                return launch_march_t<T, C, K, D, U, WPC, MINB, INTER, MODE_WIDE, VEC>(a, nfam, st);
+    }
+    return cudaErrorInvalidValue;
+}
 template <typename T, int C, int K, int D, int U, int WPC, int MINB, bool VEC>
-cudaError_t launch_march_modes(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st) {
-    if (interleaved)
-        return unitary ? launch_march_t<T, C, K, D, U, WPC, MINB, true, true, VEC>(a, nfam, st)
-                       : launch_march_t<T, C, K, D, U, WPC, MINB, true, false, VEC>(a, nfam, st);
-    return unitary ? launch_march_t<T, C, K, D, U, WPC, MINB, false, true, VEC>(a, nfam, st)
-                   : launch_march_t<T, C, K, D, U, WPC, MINB, false, false, VEC>(a, nfam, st);
+cudaError_t launch_march_modes(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st) {
+    return interleaved ? launch_march_mode<T, C, K, D, U, WPC, MINB, VEC, true>(a, nfam, mode, st)
+                       : launch_march_mode<T, C, K, D, U, WPC, MINB, VEC, false>(a, nfam, mode, st);
 }
 
 // The instantiated forms, one translation unit each (qla_march_*.cu).
-cudaError_t launch_march_f32_k1(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
-cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
-cudaError_t launch_march_f32_k2(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
-cudaError_t launch_march_f32_k2_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
-cudaError_t launch_march_f64_k1(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
-cudaError_t launch_march_f64_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st);
+cudaError_t launch_march_f32_k1(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
+cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
+cudaError_t launch_march_f32_k2(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
+cudaError_t launch_march_f32_k2_any(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
+cudaError_t launch_march_f64_k1(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
+cudaError_t launch_march_f64_k1_any(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st);
 
 }  // namespace qla

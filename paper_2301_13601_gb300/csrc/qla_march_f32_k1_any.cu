@@ -2,7 +2,7 @@
 #include "qla_march.cuh"
 
 namespace qla {
-cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int unitary, cudaStream_t st) {
-    return launch_march_modes<float, 4, 1, 2, 2, 4, 3, false>(a, nfam, interleaved, unitary, st);
+cudaError_t launch_march_f32_k1_any(const MarchArgs &a, int nfam, int interleaved, int mode, cudaStream_t st) {
+    return launch_march_modes<float, 4, 1, 2, 2, 4, 3, false>(a, nfam, interleaved, mode, st);
 }
 }  // namespace qla

@@ -35,8 +35,8 @@
 //    not used.)
 //  * In FP32 with the printed potentials a collision is three shears
 //    (h += t p, p -= s h, h += t p with t = tan(theta/2): three FMAs, the
-//    determinant exactly 1); otherwise each output is its input plus sin(theta)
-//    times a combination formed first, one rounding at the scale of the output.
+//    determinant exactly 1); otherwise each output is its input plus a combination
+//    formed first, one rounding at the scale of the output.
 //    Coefficients are stored as pairs of the form the kernel uses (see rot).
 #pragma once
 
@@ -167,11 +167,10 @@ struct Fam<1> {
 // Collision C (DAG = false) or its transpose (DAG = true) on (h, p) with
 // orientation SG: the rotation h' = c h + SG s p, p' = -SG s h + c p by the
 // angle theta (c = cos theta, s = sin theta).
-//  * SHEAR = false: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t.
+//  * ROT_HALF: pair (t, s) with t = tan(theta / 2); cos theta - 1 = -s t.
 //    Both forms take four operations and round once at the scale of each output
-//    (the inner combinations enter scaled by s or t). h' = h + (m h + s p) with
-//    m = cos theta - 1 took six for the same errors (half more of the FP64 pipe,
-//    which bounds FP64 steps).
+//    (the inner combinations enter scaled by s or t), where ROT_WIDE takes six
+//    (half more of the FP64 pipe, which bounds FP64 steps).
 //    FP64: h' = h + SG s (p - SG t h),   p' = p - SG s (h + SG t p).
 //    FP32: h' = h + SG s (p - SG t h),   p' = p - SG t (h + h'),
 //    the same rotation, whose matrix has determinant 1, and whose inverse is the
@@ -180,7 +179,15 @@ struct Fam<1> {
 //    no pair of nearby FP32 values is much closer (s and 2 t round alike): 1.7e-6
 //    of energy in 1e4 steps at 2048^2 against 5.8e-7. (In FP64 its two independent
 //    chains are 4% faster.)
-//  * SHEAR = true (FP32 with the printed potentials): pair (t, s) with
+//    For |theta| <= 1/2 only (rotation_mode): p' takes the roundings of h + h' times
+//    t, which is without bound towards theta = pi. Relative error of a rotation of
+//    random pairs, FP32, this form / ROT_WIDE: angle 0.125 2.6e-8 / 2.8e-8, 0.5
+//    3.3e-8 / 3.9e-8, 1 5.1e-8 / 7.9e-8, 3 6.2e-7 / 5.6e-8, 3.1415 1e-3 / 5e-8; the
+//    FP64 form at 3 2.3e-16 / 1.1e-16.
+//  * ROT_WIDE: pair (m, s) with m = cos(theta) - 1, any angle:
+//      h' = h + (m h + SG s p),   p' = p + (m p - SG s h)
+//    (one rounding at the scale of each output; six operations).
+//  * ROT_SHEAR (FP32 with the printed potentials): pair (t, s) with
 //    t = tan(theta / 2), as three shears
 //      h1 = h + SG t p,  p' = p - SG s h1,  h' = h1 + SG t p'
 //    (three FMAs). Each shear has determinant exactly 1 whatever the rounding
@@ -189,15 +196,21 @@ struct Fam<1> {
 //    shears a rotation to within one rounding of s, and the small remaining
 //    asymmetry biases the energy with opposite signs in C and its transpose,
 //    which alternate in Eq. 18 and Eq. 20.
-template <bool DAG, int SG, bool SHEAR, typename T>
+enum RotForm { ROT_SHEAR, ROT_HALF, ROT_WIDE };
+template <bool DAG, int SG, RotForm FORM, typename T>
 __device__ __forceinline__ void rot(T &h, T &p, T m, T s) {
     using A = Ar<T>;
     constexpr bool pos = (SG > 0) != DAG;
-    if constexpr (SHEAR) {
+    if constexpr (FORM == ROT_SHEAR) {
         const T t = m;
         h = pos ? A::fma(t, p, h) : A::fma(-t, p, h);
         p = pos ? A::fma(-s, h, p) : A::fma(s, h, p);
         h = pos ? A::fma(t, p, h) : A::fma(-t, p, h);
+    } else if constexpr (FORM == ROT_WIDE) {
+        const T sp = A::mul(s, p), sh = A::mul(s, h);
+        const T u = A::fma(m, h, pos ? sp : -sp), v = A::fma(m, p, pos ? -sh : sh);
+        h = A::add(h, u);
+        p = A::add(p, v);
     } else {
         const T t = m;
         const T u = A::fma(pos ? -t : t, h, p);
@@ -213,23 +226,24 @@ __device__ __forceinline__ void rot(T &h, T &p, T m, T s) {
     }
 }
 
-// Collision form of a configuration: three shears in FP32 with the printed
-// potentials; the four-operation forms in FP64, and in FP32 with the unitary
-// potentials, where every operator is an exact rotation and the energy (Eq. 27)
-// is kept to FP32 rounding over 1e4 steps.
-template <typename T, bool UNIT>
-constexpr bool shear_collisions() {
-    return std::is_same<T, float>::value && !UNIT;
+// Form of a configuration's rotations (potentials: rotations with MODE_UNITARY
+// only): three shears in FP32 with the printed potentials; the other forms in
+// FP64, and in FP32 with the unitary potentials, where every operator is an exact
+// rotation and the energy (Eq. 27) is kept to FP32 rounding over 1e4 steps.
+template <typename T, int MODE>
+constexpr RotForm rot_form() {
+    if (std::is_same<T, float>::value && !(MODE & MODE_UNITARY)) return ROT_SHEAR;
+    return MODE & MODE_WIDE ? ROT_WIDE : ROT_HALF;
 }
 
 // Potential row as printed: target' = target + (c target + TAU s source),
 // c = cos(b) - 1, s = sin(b). The unitary variant rotates the pair (target,
-// source) by b with orientation TAU (rot, pair (tan(b / 2), sin(b))).
-template <int TAU, bool UNIT, typename T>
+// source) by b with orientation TAU (rot).
+template <int TAU, int MODE, typename T>
 __device__ __forceinline__ void vop(T &target, T &source, T s, T c) {
     using A = Ar<T>;
-    if constexpr (UNIT) {
-        rot<false, TAU, false>(target, source, c, s);
+    if constexpr (MODE & MODE_UNITARY) {
+        rot<false, TAU, rot_form<T, MODE>()>(target, source, c, s);
         return;
     }
     const T ss = A::mul(s, source);
@@ -237,10 +251,10 @@ __device__ __forceinline__ void vop(T &target, T &source, T s, T c) {
     target = t2;
 }
 
-template <int TAU, bool HUB, bool UNIT, typename T>
+template <int TAU, bool HUB, int MODE, typename T>
 __device__ __forceinline__ void vop_pair(T &h, T &p, T s, T c) {
-    if (HUB) vop<TAU, UNIT>(h, p, s, c);
-    else vop<TAU, UNIT>(p, h, s, c);
+    if (HUB) vop<TAU, MODE>(h, p, s, c);
+    else vop<TAU, MODE>(p, h, s, c);
 }
 
 // Magnitude bits of a coefficient (zero for +0 and -0 only).
@@ -457,7 +471,7 @@ struct YPipe {
 // TMA_ONLY: the caller guarantees TMA copies for every strip (the seam
 // layout); the per-lane copy path is compiled out, and a strip that could not
 // copy with TMA sets the error flag instead.
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT, int FAM, bool TMA_ONLY = false>
+template <typename T, int K, int R, int NY, bool INTER, int MODE, int FAM, bool TMA_ONLY = false>
 __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb, int ye, unsigned char *smem_raw,
                                            const SweepMaps *M = nullptr, bool merged = false,
                                            bool swap = false) {
@@ -468,7 +482,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
     constexpr int NT = Cfg::NT;
     constexpr int NWARP = Cfg::NWARP;
     constexpr int NYS = L::NYS, NXS = L::NXS;
-    constexpr bool SHR = shear_collisions<T, UNIT>();
+    constexpr RotForm SHR = rot_form<T, MODE>();
     // coefficient stash slots, in the order of the pair planes (so that a
     // group's planes arrive in one TMA box): x-pass (Eq. 28) V_X then C_X,
     // (Eq. 23) C_X; y-pass C_Y, V_Y (+ V_X for Eq. 23)
@@ -786,7 +800,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
                 if (vx_on) {
 #pragma unroll
                     for (int c = 0; c < LANE_COLS; ++c)
-                        vop_pair<Fm::TX, Fm::VX_HUB, UNIT>(h[c], p[c], vs[c], vc[c]);
+                        vop_pair<Fm::TX, Fm::VX_HUB, MODE>(h[c], p[c], vs[c], vc[c]);
                 }
             }
             // ops 9-16
@@ -806,7 +820,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
                 if (vx_on) {
 #pragma unroll
                     for (int c = 0; c < LANE_COLS; ++c)
-                        vop_pair<Fm::TX, Fm::VX_HUB, UNIT>(h[c], p[c], vs[c], vc[c]);
+                        vop_pair<Fm::TX, Fm::VX_HUB, MODE>(h[c], p[c], vs[c], vc[c]);
                 }
             }
             sstore8(rh, sl, h);
@@ -890,7 +904,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
                     rot<false, SG, SHR>(h, p, Y.m2, Y.s2);           // op 7  C    (row R-2)
                     { const T t = Y.S8; Y.S8 = h; h = t; }      // op 8  h <- h(r-1)
                     if constexpr (INTER && VON)
-                        vop_pair<Fm::TY, Fm::VY_HUB, UNIT>(h, p, Y.vs2, Y.vc2);  // V_Y' (row R-2)
+                        vop_pair<Fm::TY, Fm::VY_HUB, MODE>(h, p, Y.vs2, Y.vc2);  // V_Y' (row R-2)
                     rot<false, SG, SHR>(h, p, Y.m2, Y.s2);           // op 9  C    (row R-2)
                     { const T t = Y.S10; Y.S10 = h; h = t; }    // op 10 p <- p(r+1): now row R-3
                     rot<true, SG, SHR>(h, p, Y.m3, Y.s3);            // op 11 C+   (row R-3)
@@ -902,10 +916,10 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
                     T px = Y.d3;
                     Y.d3 = Y.d2; Y.d2 = Y.d1; Y.d1 = Y.d0; Y.d0 = px0;
                     if constexpr (INTER) {
-                        if constexpr (VON) vop_pair<Fm::TY, Fm::VY_HUB, UNIT>(h, p, Y.vs4, Y.vc4);  // V_Y' (row R-4)
+                        if constexpr (VON) vop_pair<Fm::TY, Fm::VY_HUB, MODE>(h, p, Y.vs4, Y.vc4);  // V_Y' (row R-4)
                     } else {
-                        vop_pair<Fm::TX, Fm::VX_HUB, UNIT>(h, px, Y.ws4, Y.wc4);  // V_X  (row R-4)
-                        vop_pair<Fm::TY, Fm::VY_HUB, UNIT>(h, p, Y.vs4, Y.vc4);   // V_Y  (row R-4)
+                        vop_pair<Fm::TX, Fm::VX_HUB, MODE>(h, px, Y.ws4, Y.wc4);  // V_X  (row R-4)
+                        vop_pair<Fm::TY, Fm::VY_HUB, MODE>(h, p, Y.vs4, Y.vc4);   // V_Y  (row R-4)
                         const T2 vx = ys[2 * YSLOT + ir * W_IN];
                         Y.wc4 = Y.wc3; Y.ws4 = Y.ws3; Y.wc3 = Y.wc2; Y.ws3 = Y.ws2;
                         Y.wc2 = Y.wc1; Y.ws2 = Y.ws1; Y.wc1 = vx.x; Y.ws1 = vx.y;
@@ -962,7 +976,7 @@ __device__ __forceinline__ bool sweep_body(const SweepArgs &A, int strip, int yb
     return failed;
 }
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
+template <typename T, int K, int R, int NY, bool INTER, int MODE>
 __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, NY>::MINB)
     sweep_kernel(const __grid_constant__ SweepParams prm) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -996,8 +1010,8 @@ __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, N
         const int y1 = min(Ny, y0 + (u1 - u));
         const bool failed =
             prm.a.fam0 + int(blockIdx.z) != 0
-                ? sweep_body<T, K, R, NY, INTER, UNIT, 1>(prm.a, s, y0, y1, smem_raw, maps, prm.merged != 0)
-                : sweep_body<T, K, R, NY, INTER, UNIT, 0>(prm.a, s, y0, y1, smem_raw, maps, prm.merged != 0);
+                ? sweep_body<T, K, R, NY, INTER, MODE, 1>(prm.a, s, y0, y1, smem_raw, maps, prm.merged != 0)
+                : sweep_body<T, K, R, NY, INTER, MODE, 0>(prm.a, s, y0, y1, smem_raw, maps, prm.merged != 0);
         if (failed) break;
         u += y1 - y0;
     }
@@ -1071,21 +1085,21 @@ inline bool make_sweep_maps(const SweepArgs &a, int K, int R, SweepMaps &m, int 
     return true;
 }
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
+template <typename T, int K, int R, int NY, bool INTER, int MODE>
 int occupancy_t() {
     using Cfg = SweepCfg<T, K, R, NY>;
     using L = SweepLayout<T, K, R, INTER>;
-    cudaFuncSetAttribute(sweep_kernel<T, K, R, NY, INTER, UNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(sweep_kernel<T, K, R, NY, INTER, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          int(L::SMEM));
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, K, R, NY, INTER, UNIT>, Cfg::NT,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_kernel<T, K, R, NY, INTER, MODE>, Cfg::NT,
                                                       L::SMEM) != cudaSuccess)
         n = 1;
     cudaGetLastError();
     return n < 1 ? 1 : n;
 }
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
+template <typename T, int K, int R, int NY, bool INTER, int MODE>
 cudaError_t launch_sweep_t(const SweepArgs &a, int nfam, cudaStream_t st) {
     using Cfg = SweepCfg<T, K, R, NY>;
     using L = SweepLayout<T, K, R, INTER>;
@@ -1094,7 +1108,7 @@ cudaError_t launch_sweep_t(const SweepArgs &a, int nfam, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured_dev != dev) {
-        e = cudaFuncSetAttribute(sweep_kernel<T, K, R, NY, INTER, UNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(sweep_kernel<T, K, R, NY, INTER, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(L::SMEM));
         if (e != cudaSuccess) return e;
         configured_dev = dev;
@@ -1119,7 +1133,7 @@ cudaError_t launch_sweep_t(const SweepArgs &a, int nfam, cudaStream_t st) {
         // equal share of its family's rows: no tail wave, and the warm-up
         // rows once per share and strip instead of once per tile
         if (a.ctas < 1) return cudaErrorInvalidValue;
-        sweep_kernel<T, K, R, NY, INTER, UNIT><<<dim3(unsigned(a.ctas), 1, nfam), Cfg::NT, L::SMEM, st>>>(prm);
+        sweep_kernel<T, K, R, NY, INTER, MODE><<<dim3(unsigned(a.ctas), 1, nfam), Cfg::NT, L::SMEM, st>>>(prm);
         return cudaGetLastError();
     }
     const int ncy = (a.Ny + a.chunk - 1) / a.chunk;
@@ -1131,24 +1145,26 @@ cudaError_t launch_sweep_t(const SweepArgs &a, int nfam, cudaStream_t st) {
     // code) ran 13% slower.
     prm.tiles_fastest = K >= 4 ? 1 : 0;
     const dim3 grid = prm.tiles_fastest ? dim3(ncy, nsx, nfam) : dim3(nsx, ncy, nfam);
-    sweep_kernel<T, K, R, NY, INTER, UNIT><<<grid, Cfg::NT, L::SMEM, st>>>(prm);
+    sweep_kernel<T, K, R, NY, INTER, MODE><<<grid, Cfg::NT, L::SMEM, st>>>(prm);
     return cudaGetLastError();
 }
 
-// Dispatch on the step order and the potential variant.
-template <typename T, int K, int R, int NY>
+// Dispatch on the step order and the variant, with or without MODE_WIDE.
+template <typename T, int K, int R, int NY, int WIDE = 0>
 cudaError_t launch_sweep_modes(const SweepArgs &a, int nfam, cudaStream_t st) {
+    constexpr int PAPER = WIDE, UNITARY = MODE_UNITARY | WIDE;
+    if ((a.mode & MODE_WIDE) != WIDE) return cudaErrorInvalidValue;
     if (a.interleaved) {
-        return a.unitary ? launch_sweep_t<T, K, R, NY, true, true>(a, nfam, st)
-                         : launch_sweep_t<T, K, R, NY, true, false>(a, nfam, st);
+        return a.mode & MODE_UNITARY ? launch_sweep_t<T, K, R, NY, true, UNITARY>(a, nfam, st)
+                                     : launch_sweep_t<T, K, R, NY, true, PAPER>(a, nfam, st);
     }
-    return a.unitary ? launch_sweep_t<T, K, R, NY, false, true>(a, nfam, st)
-                     : launch_sweep_t<T, K, R, NY, false, false>(a, nfam, st);
+    return a.mode & MODE_UNITARY ? launch_sweep_t<T, K, R, NY, false, UNITARY>(a, nfam, st)
+                                 : launch_sweep_t<T, K, R, NY, false, PAPER>(a, nfam, st);
 }
 
 template <typename T, int K, int R, int NY>
 int occupancy_modes(int interleaved) {
-    return interleaved ? occupancy_t<T, K, R, NY, true, false>() : occupancy_t<T, K, R, NY, false, false>();
+    return interleaved ? occupancy_t<T, K, R, NY, true, 0>() : occupancy_t<T, K, R, NY, false, 0>();
 }
 
 }  // namespace qla

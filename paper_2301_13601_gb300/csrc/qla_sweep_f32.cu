@@ -1,4 +1,5 @@
-// FP32 instantiations of the fused sweep (K = 1, 2, 4 steps per HBM pass).
+// FP32 instantiations of the fused sweep (K = 1, 2, 4 steps per HBM pass; with
+// MODE_WIDE one step, qla_sweep_wide.cu).
 #include "qla_sweep.cuh"
 
 namespace qla {
@@ -6,6 +7,7 @@ namespace qla {
 // (K, rows per iteration R, column pipelines per thread NY): shared memory is
 // 112 KB for K = 1, 2 (two CTAs per SM) and 224 KB for K = 4.
 cudaError_t launch_sweep_f32(int K, const SweepArgs &a, int nfam, cudaStream_t st) {
+    if (a.mode & MODE_WIDE) return launch_sweep_wide_f32(K, a, nfam, st);
     switch (K) {
         case 1: return launch_sweep_modes<float, 1, 8, 1>(a, nfam, st);
         case 2: return launch_sweep_modes<float, 2, 4, 2>(a, nfam, st);

@@ -39,7 +39,7 @@ constexpr int kPersistDeps = 64;
 constexpr size_t kPersistSmemExtra = 2 * kPersistDeps * sizeof(unsigned short) + 2 * sizeof(int);
 constexpr unsigned long long kPersistWaitNs = 2000000000ull;  // default wait limit
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
+template <typename T, int K, int R, int NY, bool INTER, int MODE>
 __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, NY>::MINB)
     sweep_persistent_kernel(const __grid_constant__ SweepPersistParams pp) {
     using Cfg = SweepCfg<T, K, R, NY>;
@@ -113,9 +113,9 @@ __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, N
                 const int y1 = min(Ny, y0 + (u1 - u));
                 const bool failed =
                     prm.a.fam0 + f != 0
-                        ? sweep_body<T, K, R, NY, INTER, UNIT, 1, true>(prm.a, s, y0, y1, smem_raw, maps,
+                        ? sweep_body<T, K, R, NY, INTER, MODE, 1, true>(prm.a, s, y0, y1, smem_raw, maps,
                                                                         prm.merged != 0, odd)
-                        : sweep_body<T, K, R, NY, INTER, UNIT, 0, true>(prm.a, s, y0, y1, smem_raw, maps,
+                        : sweep_body<T, K, R, NY, INTER, MODE, 0, true>(prm.a, s, y0, y1, smem_raw, maps,
                                                                         prm.merged != 0, odd);
                 if (failed) return;  // the error flag is set: the other CTAs stop at their next wait
                 u += y1 - y0;
@@ -130,12 +130,12 @@ __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, N
     }
 }
 
-template <typename T, int K, int R, int NY, bool INTER, bool UNIT>
+template <typename T, int K, int R, int NY, bool INTER, int MODE>
 cudaError_t launch_persistent_t(const SweepArgs &a, int nfam, int passes, unsigned base, unsigned *done,
                                 unsigned withhold, unsigned long long wait_ns, cudaStream_t st) {
     using Cfg = SweepCfg<T, K, R, NY>;
     using L = SweepLayout<T, K, R, INTER>;
-    auto kern = sweep_persistent_kernel<T, K, R, NY, INTER, UNIT>;
+    auto kern = sweep_persistent_kernel<T, K, R, NY, INTER, MODE>;
     static int configured_dev = -1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -188,16 +188,16 @@ cudaError_t launch_persistent_t(const SweepArgs &a, int nfam, int passes, unsign
 cudaError_t launch_sweep_persistent_hooked_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
                                                unsigned *done, unsigned withhold, unsigned long long wait_ns,
                                                cudaStream_t st) {
-    if (K != 2) return cudaErrorNotSupported;
+    if (K != 2 || (a.mode & MODE_WIDE)) return cudaErrorNotSupported;
     if (a.interleaved) {
-        return a.unitary
-                   ? launch_persistent_t<float, 2, 4, 2, true, true>(a, nfam, passes, base, done, withhold, wait_ns, st)
-                   : launch_persistent_t<float, 2, 4, 2, true, false>(a, nfam, passes, base, done, withhold, wait_ns,
+        return a.mode & MODE_UNITARY
+                   ? launch_persistent_t<float, 2, 4, 2, true, MODE_UNITARY>(a, nfam, passes, base, done, withhold, wait_ns, st)
+                   : launch_persistent_t<float, 2, 4, 2, true, 0>(a, nfam, passes, base, done, withhold, wait_ns,
                                                                       st);
     }
-    return a.unitary
-               ? launch_persistent_t<float, 2, 4, 2, false, true>(a, nfam, passes, base, done, withhold, wait_ns, st)
-               : launch_persistent_t<float, 2, 4, 2, false, false>(a, nfam, passes, base, done, withhold, wait_ns, st);
+    return a.mode & MODE_UNITARY
+               ? launch_persistent_t<float, 2, 4, 2, false, MODE_UNITARY>(a, nfam, passes, base, done, withhold, wait_ns, st)
+               : launch_persistent_t<float, 2, 4, 2, false, 0>(a, nfam, passes, base, done, withhold, wait_ns, st);
 }
 
 cudaError_t launch_sweep_persistent_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
