@@ -255,11 +255,16 @@ void plane_range(const double *n, size_t P, double range[2]) {
 }  // namespace
 
 bool index_valid(const double *n, size_t P, bool *ordinary) {
-    for (size_t i = 0; i < P; ++i) {
-        const double v = n[i];
-        if (v >= kOrdinaryIndex[0] && v <= kOrdinaryIndex[1]) continue;
+    constexpr size_t BLOCK = 1024;  // without a branch per value
+    for (size_t i0 = 0; i0 < P; i0 += BLOCK) {
+        const size_t i1 = std::min(P, i0 + BLOCK);
+        unsigned long long outside = 0;
+        for (size_t i = i0; i < i1; ++i)
+            outside += 1ull - (unsigned long long)((n[i] >= kOrdinaryIndex[0]) & (n[i] <= kOrdinaryIndex[1]));
+        if (outside == 0) continue;
         *ordinary = false;
-        if (!(v > 0.0) || !std::isfinite(v)) return false;
+        for (size_t i = i0; i < i1; ++i)
+            if (!(n[i] > 0.0) || !std::isfinite(n[i])) return false;
     }
     return true;
 }
