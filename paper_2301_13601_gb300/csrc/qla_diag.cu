@@ -373,6 +373,7 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) divD_partial(const T *__restr
             const double dnz = nz[i];
             const float fx = narrow_for_screen(dx, &ok), fy = narrow_for_screen(here, &ok);
             const float fz = narrow_for_screen(dnz, &ok) * narrow_for_screen(widen(v2), &ok);
+            ok = ok && (is_zero(fz) || pair_range(fz));  // D_z itself, as D_x and D_y are products above
             const float f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
             if (mine) {
                 if (!ok) {
