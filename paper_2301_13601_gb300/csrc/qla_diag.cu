@@ -159,20 +159,44 @@ __device__ __forceinline__ bool pair_range(float v) {
 }
 __device__ __forceinline__ bool is_zero(float v) { return (__float_as_uint(v) << 1) == 0u; }
 
+// div B of a site, times 2: (r - l) + (u - d) as the FP64 operations give it (each
+// is exact, or rounds once). The differences, their sum and all of their errors are
+// formed in FP32 (TwoSum); where the errors add up exactly (values within about 2^23
+// of each other) the sum of the two parts is the only FP64 operation, and there is
+// none where the FP32 sum is exact.
+__device__ __forceinline__ double divergence(float r, float l, float u, float d) {
+    const float h1 = __fsub_rn(r, l), b1 = __fsub_rn(h1, r);
+    const float e1 = __fsub_rn(__fsub_rn(r, __fsub_rn(h1, b1)), __fadd_rn(l, b1));
+    const float h2 = __fsub_rn(u, d), b2 = __fsub_rn(h2, u);
+    const float e2 = __fsub_rn(__fsub_rn(u, __fsub_rn(h2, b2)), __fadd_rn(d, b2));
+    const float s = __fadd_rn(h1, h2), bs = __fsub_rn(s, h1);
+    const float t = __fadd_rn(__fsub_rn(h1, __fsub_rn(s, bs)), __fsub_rn(h2, bs));
+    const float te = __fadd_rn(t, e2), lo = __fadd_rn(te, e1);
+    // both sums exact (so their TwoSum errors vanish), and no overflow, infinity or NaN
+    if (fabsf(s) < 0x1p120f && __fsub_rn(te, t) == e2 && __fsub_rn(te, e2) == t && __fsub_rn(lo, te) == e1 &&
+        __fsub_rn(lo, e1) == te) {
+        const double v = f2d_exact(s);
+        return lo == 0.0f ? v : v + f2d_exact(lo);
+    }
+    return (f2d_exact(r) - f2d_exact(l)) + (f2d_exact(u) - f2d_exact(d));
+}
+
 // FP32 state. GB300's FP64 pipe takes a warp instruction in 64 cycles of a
 // scheduler (the generic kernel below is bound by it, and so was this one with
-// six FP64 operations per site: 305 us at 4096^2), so a site costs none:
-//  * its sum of squares and its squared divergence are FP32 pairs (products
-//    with their FMA errors, sums by TwoSum), added to pairs that enter the FP64
-//    sums after PAIR_SITES sites: relative error about 2^-46 of such a partial
-//    sum, unbiased, over many of them below FP64's own rounding;
-//  * the divergence (q3(x+1) - q3(x-1)) + (q4(y+1) - q4(y-1)) is formed as a pair
-//    from exact differences; the factors 1/2 and 1/4 are applied to the reduced
-//    max and sum;
-//  * the maxima are screened in FP32 (Screen below); max |div| is kept as the bit
+// six FP64 operations per site: 305 us at 4096^2), so a site costs few:
+//  * its sum of squares is an FP32 pair (products with their FMA errors, sums by
+//    TwoSum), added to a pair that enters the FP64 sum after PAIR_SITES sites:
+//    relative error about 2^-46 of such a partial sum, over many of them below that
+//    of the squares' own low parts (2^-50, all of one sign: the low bits of a square
+//    are not uniform);
+//  * the divergence (see above) enters the FP64 sum by one FMA, two operations at
+//    most (as a pair squared in FP32 the sum was off by 5 to 8 units of 2^-53, in
+//    FP64 by less than one); the factors 1/2 and 1/4 are applied to the reduced max
+//    and sum;
+//  * max |B| is screened in FP32 (Screen below); max |div| is kept as the bit
 //    pattern of a non-negative double (integer order = numeric order; NaN
 //    excluded, as fmax would).
-// Sites with values outside [2^-50, 2^60) take FP64 throughout.
+// Sites with values outside [2^-50, 2^60) take FP64 for their squares.
 constexpr int PAIR_SITES = 32;
 // (four blocks per SM: all of the grid's 608 resident at once)
 __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float *__restrict__ q, int Nx, int Ny,
@@ -182,21 +206,16 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
     CSum e{0.0, 0.0}, d{0.0, 0.0};
     unsigned long long dmax_bits = 0;
     double b2max = 0.0;
-    Screen sb, sd;
-    float pb[3] = {0.0f, 0.0f, 0.0f}, pd[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // the pending sites' values
+    Screen sb;
+    float pb[3] = {0.0f, 0.0f, 0.0f};  // the pending site's values
     auto exact_b2 = [&](float v3, float v4, float v5) {
         const double d3 = f2d_exact(v3), d4 = f2d_exact(v4), d5 = f2d_exact(v5);
         const double b2 = (d3 * d3 + d4 * d4) + d5 * d5;
         if (b2 > b2max) b2max = b2;
     };
-    auto exact_div = [&](float rr, float l, float up, float dn) {
-        const double dv = (f2d_exact(rr) - f2d_exact(l)) + (f2d_exact(up) - f2d_exact(dn));
-        const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) & 0x7fffffffffffffffull;
-        if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
-        return dv;
-    };
     unsigned long long nf = 0;
-    FPair ep{0.0f, 0.0f}, dp{0.0f, 0.0f};
+    FPair ep{0.0f, 0.0f};
+    double d64 = 0.0;
     int pending = 0;
     const unsigned W = unsigned(Nx);
     for (int y = blockIdx.x; y < Ny; y += gridDim.x) {
@@ -205,7 +224,7 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
 #pragma unroll
         for (int c = 0; c < 6; ++c) row[c] = q + c * P + size_t(y) * W;
         const float *const q4p = q4 + size_t(yp) * W, *const q4m = q4 + size_t(ym) * W;
-        double e64 = 0.0, d64 = 0.0;  // sites outside the pair range
+        double e64 = 0.0;  // sites outside the pair range
         for (unsigned x = threadIdx.x; x < W; x += DIAG_THREADS) {
             const unsigned xp = x + 1 == W ? 0 : x + 1, xm = x == 0 ? W - 1 : x - 1;
             float v[6];
@@ -246,47 +265,24 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
             } else if (sb.close(b2f) && !(v[3] == pb[0] && v[4] == pb[1] && v[5] == pb[2])) {
                 exact_b2(v[3], v[4], v[5]);
             }
-            // the divergence as a pair: exact differences, their sum by TwoSum
-            FPair g{__fsub_rn(rr, l), 0.0f};
-            {
-                const float bb = __fsub_rn(g.hi, rr);
-                g.lo = __fsub_rn(__fsub_rn(rr, __fsub_rn(g.hi, bb)), __fadd_rn(l, bb));
-                const float s2 = __fsub_rn(up, dn);
-                const float b2 = __fsub_rn(s2, up);
-                g.add(s2, __fsub_rn(__fsub_rn(up, __fsub_rn(s2, b2)), __fadd_rn(dn, b2)));
-                const float h = __fadd_rn(g.hi, g.lo);  // renormalised
-                g.lo = __fsub_rn(g.lo, __fsub_rn(h, g.hi));
-                g.hi = h;
-            }
-            const float ga = fabsf(g.hi);
-            if (pair_range(g.hi)) {
-                const float p = __fmul_rn(g.hi, g.hi);
-                dp.add(p, __fmaf_rn(2.0f * g.hi, g.lo, __fmaf_rn(g.hi, g.hi, -p)));
-                if (sd.replaces(ga)) {
-                    sd.best = ga;
-                    pd[0] = rr; pd[1] = l; pd[2] = up; pd[3] = dn;
-                } else if (sd.close(ga) && !(rr == pd[0] && l == pd[1] && up == pd[2] && dn == pd[3])) {
-                    exact_div(rr, l, up, dn);
-                }
-            } else if (!is_zero(g.hi)) {
-                const double dv = exact_div(rr, l, up, dn);
-                d64 = fma(dv, dv, d64);
-            }
+            // the divergence: in FP32 where its parts add up exactly, otherwise in FP64
+            const double dv = divergence(rr, l, up, dn);
+            d64 = fma(dv, dv, d64);
+            const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) & 0x7fffffffffffffffull;
+            if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
             if (++pending == PAIR_SITES) {
                 e.add(ep.value());
-                d.add(0.25 * dp.value());
+                d.add(0.25 * d64);
                 ep = FPair{0.0f, 0.0f};
-                dp = FPair{0.0f, 0.0f};
+                d64 = 0.0;
                 pending = 0;
             }
         }
         if (e64 != 0.0) e.add(e64);  // (a NaN is not zero)
-        if (d64 != 0.0) d.add(0.25 * d64);
     }
     e.add(ep.value());
-    d.add(0.25 * dp.value());
+    d.add(0.25 * d64);
     exact_b2(pb[0], pb[1], pb[2]);
-    exact_div(pd[0], pd[1], pd[2], pd[3]);
     const double dmax = 0.5 * __longlong_as_double(static_cast<long long>(dmax_bits));
     block_reduce_write(Partial{e.s, e.c, d.s, d.c, dmax, sqrt(b2max), nf, 0ull}, part);
 }

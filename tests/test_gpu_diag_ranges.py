@@ -26,3 +26,28 @@ def test_divD_maximum_of_one_component(index, field, precision):
     assert div == 0.0 and dmax == 0.0
     ref = oracle.divD(q, *n)[2]
     assert abs(largest - ref) <= 1e-14 * ref
+
+
+@pytest.mark.parametrize("Nx, Ny", [(200, 300), (513, 129)])
+@pytest.mark.parametrize("kind", ["noise", "waves"])
+def test_squared_divergence_to_the_last_bits(Nx, Ny, kind):
+    """FP32 states, against exact integer arithmetic. A site's divergence and square round
+    a few times in FP64 (unbiased, at most 3 units of 2^-53), and sums of at most 32
+    sites round at most 32 times: over more than 6e4 sites both average to less than
+    0.1 unit of the sum, whose compensated end rounds once or twice by half a unit."""
+    rng = np.random.default_rng(8)
+    if kind == "noise":
+        q = rng.standard_normal((6, Ny, Nx))
+    else:
+        y, x = np.mgrid[0:Ny, 0:Nx]
+        q = np.stack([0.2 * np.cos(2 * np.pi * ((k + 1) * x / Nx + 2 * y / Ny) + k) +
+                      np.exp(-((x - Nx / 2) / (0.05 * Nx)) ** 2) for k in range(6)])
+    q = q.astype(np.float32).astype(np.float64)
+    with Simulation(*np.ones((3, Ny, Nx)), 0.1) as sim:
+        sim.set_fields(q)
+        got = sim.diagnostics()["div_l2_sq"]
+    scaled = [int(v * 2.0 ** 64) for v in q[3:5].ravel()]
+    bx, by = np.array(scaled[:Nx * Ny], dtype=object).reshape(Ny, Nx), np.array(scaled[Nx * Ny:], dtype=object).reshape(Ny, Nx)
+    div = np.roll(bx, -1, 1) - np.roll(bx, 1, 1) + np.roll(by, -1, 0) - np.roll(by, 1, 0)
+    ref = int((div * div).sum())  # times 4 * 2^128
+    assert abs(int(got * 2.0 ** 130) - ref) <= 2 * ref >> 53
