@@ -159,6 +159,20 @@ __device__ __forceinline__ bool pair_range(float v) {
 }
 __device__ __forceinline__ bool is_zero(float v) { return (__float_as_uint(v) << 1) == 0u; }
 
+// Sum of squares of six values below 2^60, the largest zero or at least 2^-44
+// (a square of less than 2^-100 has an error term off by 2^-149 at most).
+__device__ __forceinline__ FPair sum_of_squares(const float (&v)[6]) {
+    FPair s;
+    s.hi = __fmul_rn(v[0], v[0]);
+    s.lo = __fmaf_rn(v[0], v[0], -s.hi);
+#pragma unroll
+    for (int c = 1; c < 6; ++c) {
+        const float p = __fmul_rn(v[c], v[c]);
+        s.add(p, __fmaf_rn(v[c], v[c], -p));
+    }
+    return s;
+}
+
 // div B of a site, times 2: (r - l) + (u - d) as the FP64 operations give it (each
 // is exact, or rounds once). The differences, their sum and all of their errors are
 // formed in FP32 (TwoSum); where the errors add up exactly (values within about 2^23
@@ -196,7 +210,9 @@ __device__ __forceinline__ double divergence(float r, float l, float u, float d)
 //  * max |B| is screened in FP32 (Screen below); max |div| is kept as the bit
 //    pattern of a non-negative double (integer order = numeric order; NaN
 //    excluded, as fmax would).
-// Sites with values outside [2^-50, 2^60) take FP64 for their squares.
+// Sites with a value outside [2^-60, 2^60) take FP64 for their squares, those with no
+// value of 2^-44 or more (squares near FP32's smallest) a pair of scaled values that
+// enters the FP64 sum at once.
 constexpr int PAIR_SITES = 32;
 // (four blocks per SM: all of the grid's 608 resident at once)
 __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float *__restrict__ q, int Nx, int Ny,
@@ -206,7 +222,8 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
     CSum e{0.0, 0.0}, d{0.0, 0.0};
     unsigned long long dmax_bits = 0;
     double b2max = 0.0;
-    Screen sb;
+    Screen sb, st;  // st: sites with |B|^2 < 2^-116, values scaled by 2^90
+    bool tiny_pending = false;
     float pb[3] = {0.0f, 0.0f, 0.0f};  // the pending site's values
     auto exact_b2 = [&](float v3, float v4, float v5) {
         const double d3 = f2d_exact(v3), d4 = f2d_exact(v4), d5 = f2d_exact(v5);
@@ -215,7 +232,7 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
     };
     unsigned long long nf = 0;
     FPair ep{0.0f, 0.0f};
-    double d64 = 0.0;
+    double e64 = 0.0, d64 = 0.0;  // plain sums of the pending sites
     int pending = 0;
     const unsigned W = unsigned(Nx);
     for (int y = blockIdx.x; y < Ny; y += gridDim.x) {
@@ -224,30 +241,31 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
 #pragma unroll
         for (int c = 0; c < 6; ++c) row[c] = q + c * P + size_t(y) * W;
         const float *const q4p = q4 + size_t(yp) * W, *const q4m = q4 + size_t(ym) * W;
-        double e64 = 0.0;  // sites outside the pair range
         for (unsigned x = threadIdx.x; x < W; x += DIAG_THREADS) {
             const unsigned xp = x + 1 == W ? 0 : x + 1, xm = x == 0 ? W - 1 : x - 1;
             float v[6];
-            unsigned big = 0u, small = 0xffffffffu;
+            unsigned big[2] = {0u, 0u}, small = 0xffffffffu;  // big: of Q0-Q2, of B
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 v[c] = row[c][x];
                 const unsigned ua = __float_as_uint(v[c]) & 0x7fffffffu;
-                big = max(big, ua);
+                big[c / 3] = max(big[c / 3], ua);
                 small = min(small, ua - 1u);  // zero counts as large
             }
-            const bool ff = big < 0x5d800000u && small >= 0x267fffffu;  // every |v| zero or in [2^-50, 2^60)
+            const unsigned bigq = max(big[0], big[1]);
             const float l = row[3][xm], rr = row[3][xp], dn = q4m[x], up = q4p[x];
-            if (ff) {
-                FPair s;
-                s.hi = __fmul_rn(v[0], v[0]);
-                s.lo = __fmaf_rn(v[0], v[0], -s.hi);
+            if (bigq < 0x5d800000u && small >= 0x217fffffu) {  // every |v| zero or in [2^-60, 2^60)
+                if (bigq - 1u >= 0x297fffffu) {  // the largest zero or at least 2^-44
+                    const FPair s = sum_of_squares(v);
+                    ep.add(s.hi, s.lo);
+                } else {
+                    float w[6];
 #pragma unroll
-                for (int c = 1; c < 6; ++c) {
-                    const float p = __fmul_rn(v[c], v[c]);
-                    s.add(p, __fmaf_rn(v[c], v[c], -p));
+                    for (int c = 0; c < 6; ++c) w[c] = v[c] * 0x1p64f;
+                    const FPair s = sum_of_squares(w);
+                    e64 = fma(f2d_exact(s.hi), 0x1p-128, e64);
+                    e64 = fma(f2d_exact(s.lo), 0x1p-128, e64);
                 }
-                ep.add(s.hi, s.lo);
             } else {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) {
@@ -256,14 +274,31 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
                     e64 = fma(dv, dv, e64);
                 }
             }
+            // max |B|: the pending site is one of tiny values only while no other was met
             const float b2f = fmaf(v[3], v[3], fmaf(v[4], v[4], v[5] * v[5]));
-            if (!ff) {
+            if (big[1] >= 0x5d800000u) {
                 exact_b2(v[3], v[4], v[5]);
-            } else if (sb.replaces(b2f)) {
-                sb.best = b2f;
-                pb[0] = v[3]; pb[1] = v[4]; pb[2] = v[5];
-            } else if (sb.close(b2f) && !(v[3] == pb[0] && v[4] == pb[1] && v[5] == pb[2])) {
-                exact_b2(v[3], v[4], v[5]);
+            } else if (b2f >= 0x1p-116f) {
+                if (sb.replaces(b2f)) {
+                    if (tiny_pending && b2f < 0x1p-115f) exact_b2(pb[0], pb[1], pb[2]);
+                    tiny_pending = false;
+                    sb.best = b2f;
+                    pb[0] = v[3]; pb[1] = v[4]; pb[2] = v[5];
+                } else if (sb.close(b2f) && !(v[3] == pb[0] && v[4] == pb[1] && v[5] == pb[2])) {
+                    exact_b2(v[3], v[4], v[5]);
+                }
+            } else if (big[1] != 0u && sb.best < 0x1p-115f) {
+                const float w3 = v[3] * 0x1p90f, w4 = v[4] * 0x1p90f, w5 = v[5] * 0x1p90f;
+                const float t2f = fmaf(w3, w3, fmaf(w4, w4, w5 * w5));
+                if (sb.best > 0.0f) {
+                    exact_b2(v[3], v[4], v[5]);
+                } else if (st.replaces(t2f)) {
+                    tiny_pending = true;
+                    st.best = t2f;
+                    pb[0] = v[3]; pb[1] = v[4]; pb[2] = v[5];
+                } else if (st.close(t2f) && !(v[3] == pb[0] && v[4] == pb[1] && v[5] == pb[2])) {
+                    exact_b2(v[3], v[4], v[5]);
+                }
             }
             // the divergence: in FP32 where its parts add up exactly, otherwise in FP64
             const double dv = divergence(rr, l, up, dn);
@@ -271,16 +306,15 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
             const unsigned long long ab = static_cast<unsigned long long>(__double_as_longlong(dv)) & 0x7fffffffffffffffull;
             if (ab <= 0x7ff0000000000000ull && ab > dmax_bits) dmax_bits = ab;
             if (++pending == PAIR_SITES) {
-                e.add(ep.value());
+                e.add(ep.value() + e64);
                 d.add(0.25 * d64);
                 ep = FPair{0.0f, 0.0f};
-                d64 = 0.0;
+                e64 = d64 = 0.0;
                 pending = 0;
             }
         }
-        if (e64 != 0.0) e.add(e64);  // (a NaN is not zero)
     }
-    e.add(ep.value());
+    e.add(ep.value() + e64);
     d.add(0.25 * d64);
     exact_b2(pb[0], pb[1], pb[2]);
     const double dmax = 0.5 * __longlong_as_double(static_cast<long long>(dmax_bits));

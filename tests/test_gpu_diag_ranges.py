@@ -51,3 +51,37 @@ def test_squared_divergence_to_the_last_bits(Nx, Ny, kind):
     div = np.roll(bx, -1, 1) - np.roll(bx, 1, 1) + np.roll(by, -1, 0) - np.roll(by, 1, 0)
     ref = int((div * div).sum())  # times 4 * 2^128
     assert abs(int(got * 2.0 ** 130) - ref) <= 2 * ref >> 53
+
+
+def field_of(kind, shape, rng):
+    """States with small values: sites of one scale, of scales mixed site by site or within
+    a site, and the tails of a pulse."""
+    v = rng.standard_normal((6,) + shape)
+    if kind == "edge -44" or kind == "edge -58" or kind == "edge -60":
+        return v * 2.0 ** int(kind.split()[1])
+    if kind == "subnormal":
+        return v * 2.0 ** -140
+    if kind == "mixed sites":
+        return v * 2.0 ** rng.integers(-80, 3, shape)
+    if kind == "mixed components":
+        return v * 2.0 ** rng.integers(-80, 3, v.shape)
+    x = np.arange(shape[1])
+    g = np.exp(-(x - shape[1] / 8) ** 2 / (2 * (shape[1] / 40) ** 2))
+    return np.stack([0 * v[0], 0 * v[0], g + 0 * v[0], 0 * v[0], -g + 0 * v[0], 0 * v[0]])
+
+
+@pytest.mark.parametrize("Nx, Ny", [(1, 9), (300, 40), (1030, 300)])
+@pytest.mark.parametrize("kind", ["edge -44", "edge -58", "edge -60", "subnormal", "mixed sites", "mixed components",
+                                  "pulse"])
+def test_small_values_fp32(Nx, Ny, kind):
+    """A site's sum of squares is an FP32 pair (2^-46 of it, low parts rounded) or FP64:
+    1e-14, as the other tests of the sums."""
+    q = field_of(kind, (Ny, Nx), np.random.default_rng(Nx)).astype(np.float32).astype(np.float64)
+    with Simulation(*np.ones((3, Ny, Nx)), 0.1) as sim:
+        sim.set_fields(q)
+        d = sim.diagnostics()
+    s, m, b = oracle.divB(q)
+    assert d["nonfinite"] == 0
+    for got, ref, tol in ((d["energy"], oracle.energy(q), 1e-14), (d["div_l2_sq"], s, 1e-13), (d["div_max"], m, 1e-14),
+                          (d["b_max"], b, 1e-14)):
+        assert abs(got - ref) <= tol * abs(ref)
