@@ -85,9 +85,10 @@ typedef struct {
     int potential;       /* QLA_POT_PAPER (default) or QLA_POT_UNITARY */
     int steps_per_pass;  /* full time steps fused per HBM pass: 0 = automatic (2; FP32 with chunk_rows
                             set: 2 from 2^25 sites up, else 4), else 1, 2 or 4 */
-    int chunk_rows;      /* rows swept by one warp of a strip (0 = automatic); with the shared-memory
-                            sweep (the persistent launch form, planes of 2^32 bytes or more), rows of
-                            one tile, 0 = the balanced split (see qla_sweep_split) */
+    int chunk_rows;      /* most rows of a strip swept by one warp (0 = no limit: as many as are
+                            fastest); where the shared-memory sweep serves the context (coefficients
+                            in pair planes, see qla_buffer_sizes), rows of one of its tiles, 0 = the
+                            balanced split (see qla_sweep_split). Results do not depend on it */
     int device;          /* CUDA device ordinal; -1 = the calling thread's current device */
     void *stream;        /* cudaStream_t to run on; NULL = a non-blocking stream owned by the context */
     int families;        /* QLA_FAMILIES_BOTH (default), or QLA_FAMILY_TM / QLA_FAMILY_TE: only that
@@ -364,7 +365,7 @@ typedef struct {
     long long nsteps;                /* steps per qla_batch_run; a multiple of steps_per_pass */
     int pulse_polarization;          /* QLA_POL_EZ or QLA_POL_EY: initial pulse as qla_init_pulse; -1: zero state */
     double pulse_x0, pulse_sigma, pulse_amplitude;
-    int chunk_rows;                  /* rows swept by one warp of a strip; 0 = automatic */
+    int chunk_rows;                  /* most rows of a strip swept by one warp; 0 = no limit */
 } qla_instance_desc;
 
 /* Create a batch of `count` lattices (descs copied; the host arrays are only

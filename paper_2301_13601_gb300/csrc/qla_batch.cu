@@ -255,7 +255,7 @@ cudaError_t dalloc(qla_batch *b, P **p, size_t bytes) {
     return e;
 }
 
-// Rows per share of the lattices that set none: as many as let the batch's
+// Rows per share, at most: as many as let the batch's
 // warps fill the GPU's slots (8 per SM) a little more than once (a lattice's
 // pass ends with its last tile; more, lower shares pay the march_delay(2) = 17
 // warm-up rows more often), and at least 8. Ten lattices of sides 256 to 1024,
@@ -339,7 +339,10 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         I.w_valid = g.w_valid;
         I.halo = g.halo;
         I.strips = g.strips;
-        const int ch = std::min(d.chunk_rows > 0 ? d.chunk_rows : rows, d.Ny);
+        // (a lattice's chunk_rows: at most, see march_plan; ten lattices of sides 256 to
+        // 1024, 100 steps, 768 rows: 30 ms in tiles of the shared-memory sweep, 32 with
+        // as many rows per warp, 5.8 now)
+        const int ch = std::min(d.chunk_rows > 0 ? std::min(d.chunk_rows, rows) : rows, d.Ny);
         I.chunks = (d.Ny + ch - 1) / ch;
         I.tiles = (I.strips * I.chunks + qla::BWPC - 1) / qla::BWPC;
         I.passes = int(d.nsteps / qla::kBatchSteps);

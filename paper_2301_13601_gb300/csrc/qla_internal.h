@@ -280,7 +280,7 @@ bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g);
 // Whether its state rows are copied in 16-byte vectors at 32-bit offsets.
 bool march_vectors(const MarchGeo &g);
 // Chooses the row ranges of a pass over nfam families on a device of sms SMs.
-// chunk: rows per range (0: automatic).
+// chunk: at most so many rows per range (0: as many as are best).
 void march_plan(MarchGeo *g, int nfam, int chunk, int sms);
 // One pass of K steps (FP32: 1, 2; FP64: 1) over the families f0 .. f0 + nfam - 1.
 // mem: the advanced families' records, then their flags (march_bytes). chained:

@@ -72,8 +72,15 @@ int march_chunks(const MarchGeo &g, int nfam, int K, int sms) {
 }  // namespace
 
 void march_plan(MarchGeo *g, int nfam, int chunk, int sms) {
-    for (int K = 1; K <= 2; ++K)
-        g->chunks[K] = chunk > 0 ? (g->Ny + chunk - 1) / chunk : march_chunks(*g, nfam, K, sms);
+    for (int K = 1; K <= 2; ++K) {
+        g->chunks[K] = march_chunks(*g, nfam, K, sms);
+        // A caller's rows are those of a tile, which a CTA of the shared-memory sweep
+        // took (and whose best heights were 64 to 1024): a warp alone that swept as
+        // many would leave the GPU to few warps (us per step, shared-memory sweep /
+        // that many rows per warp / this: 256^2 256 rows 101 / 134 / 9, 1024^2 256
+        // rows 97 / 111 / 24, 4096^2 1024 rows 343 / 380 / 157).
+        if (chunk > 0) g->chunks[K] = std::max(g->chunks[K], (g->Ny + chunk - 1) / chunk);
+    }
     g->chunks[0] = 0;
 }
 
