@@ -271,7 +271,9 @@ def run_ours(args):
         dist.barrier()
     # one launch per pass, or every pass of a bench step in one persistent launch
     launch_form = sim.launch
-    launches_per_step = 1 if launch_form == "persistent" else math.ceil(S / min(sim.steps_per_pass, 2))
+    # (small lattices run one step per pass unless told otherwise)
+    per_pass = 1 if args.steps_per_pass == 0 and sites <= 1 << 19 else min(sim.steps_per_pass, 2)
+    launches_per_step = 1 if launch_form == "persistent" else math.ceil(S / per_pass)
     # e2e through the public API with host buffers: pinned H2D state copy,
     # qla_step, diagnostics, D2H state copy, every bench step. Serial: one
     # context, each step's copies between its compute. Pipelined (the reported
@@ -453,7 +455,7 @@ def batch_instances(args):
 
 def batch_report(args, peak, peak_kind, steps: int = 3):
     """The batched workload in one persistent CUDA-graph launch per bench step,
-    with the steps per pass and rows per tile chosen by the autotuner (timed
+    with the steps per pass and most rows per warp chosen by the autotuner (timed
     candidates, cached per GPU, kernel version and batch shape)."""
     import torch
 
@@ -655,7 +657,7 @@ def run_batch(args):
 
     _build.build()
     ws, inst = batch_instances(args)
-    # --steps-per-pass 0 (the default): the autotuner chooses steps per pass and tile rows
+    # --steps-per-pass 0 (the default): the autotuner chooses steps per pass and rows per warp
     with Batch(inst, steps_per_pass=args.steps_per_pass) as b:
         info = b.info()
         K = info["steps_per_pass"]

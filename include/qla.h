@@ -370,7 +370,7 @@ typedef struct {
 
 /* Create a batch of `count` lattices (descs copied; the host arrays are only
  * read during the call). opt: precision must be QLA_FP32; steps_per_pass 2 or 4
- * (0 = 4); sequence and potential apply to every lattice; opt->stream is
+ * (0 = 4): every nsteps is a multiple of it; sequence and potential apply to every lattice; opt->stream is
  * ignored (the batch owns a stream). Errors: QLA_EINVAL (bad descriptor),
  * QLA_EUNSUPPORTED (precision, steps_per_pass, or opt->families other than
  * QLA_FAMILIES_BOTH), QLA_ENOMEM, QLA_ECUDA. */
@@ -387,7 +387,8 @@ qla_status qla_batch_get_fields_f32(qla_batch *b, int i, float *q);
 /* Diagnostics of lattice i (as qla_diagnostics). */
 qla_status qla_batch_diagnostics(qla_batch *b, int i, qla_diag *out);
 
-/* Work items per run, steps per pass, and site-updates per run. */
+/* Work items per run, steps_per_pass as given at creation (the passes take two
+ * steps either way), and site-updates per run. */
 qla_status qla_batch_info(const qla_batch *b, long long *total_items, int *steps_per_pass, long long *site_updates);
 
 /* Test hook: limit of each dependency wait in nanoseconds (default 4 s), and a

@@ -1,4 +1,4 @@
-"""Autotuner for the fused sweep: steps per HBM pass and rows per tile.
+"""Autotuner for the fused sweep: steps per HBM pass and most rows per warp.
 
 For a lattice (single context) or a set of lattices (batch), every candidate
 configuration is timed on the GPU with CUDA events after warm-up, and the
@@ -38,15 +38,18 @@ def save_cache(cache: dict, path: Optional[str] = None) -> None:
     os.replace(tmp, p)
 
 
-def kernel_version() -> str:
-    """sha256 prefix of the sweep kernels' sources: cached choices of an older
-    kernel are not reused."""
+def kernel_version(csrc: Optional[str] = None) -> str:
+    """sha256 prefix of the library's sources (the kernels, and the rules that choose
+    their row ranges and passes): cached choices of an older build are not reused."""
+    import glob
     import hashlib
 
+    csrc = csrc or os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
     h = hashlib.sha256()
     try:
-        for name in ("qla_sweep.cuh", "qla_march.cuh"):
-            with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", name), "rb") as f:
+        for path in sorted(p for ext in ("cu", "cuh", "h") for p in glob.glob(os.path.join(csrc, f"*.{ext}"))):
+            h.update(os.path.basename(path).encode())
+            with open(path, "rb") as f:
                 h.update(f.read())
     except OSError:
         return "unknown"
@@ -58,11 +61,11 @@ def single_key(Nx: int, Ny: int, precision: str, sequence: str, potential: str, 
 
 
 def chunk_candidates(Ny: int, K: int) -> List[int]:
-    """Rows per tile to try: 0 (the balanced split: one equal-cost share of
-    each family's rows per resident CTA) and a few fixed tile heights between
-    16 K (warm-up at most a third) and the whole lattice."""
+    """Limits of the rows per warp to try: 0 (none: the rows that the sweep's own cost
+    model chooses), a few between 16 K (warm-up at most a third) and the heights
+    that it chooses on the largest lattices, and the whole lattice."""
     out = {0}
-    for h in (128, 192, 256, 320, 384, 512, 768, 1024, 2048, 4096):
+    for h in (16, 32, 48, 64, 96, 128, 192, 256):
         if 16 * K <= h < Ny:
             out.add(h)
     out.add(Ny)
@@ -81,9 +84,10 @@ def pick_best(results: Iterable[Tuple[dict, float]]) -> Tuple[dict, float]:
 
 
 def tune_single(n_x, n_y, n_z, delta: float, precision: str = "fp32", sequence: str = "interleaved",
-                potential: str = "paper", ks: Sequence[int] = (1, 2, 4), steps: int = 16, repeats: int = 3,
+                potential: str = "paper", ks: Sequence[int] = (1, 2), steps: int = 16, repeats: int = 3,
                 use_cache: bool = True, timer: Optional[Callable] = None) -> dict:
-    """Time qla_step(steps) for each (steps per pass, rows per tile) candidate."""
+    """Time qla_step(steps) for each (steps per pass, limit of rows per warp) candidate
+    (4 steps per pass run as two passes of 2)."""
     import torch
 
     from .qla import QLAError, Simulation
@@ -124,11 +128,12 @@ def tune_single(n_x, n_y, n_z, delta: float, precision: str = "fp32", sequence: 
     return entry
 
 
-def tune_batch(instances: List[dict], ks: Sequence[int] = (2, 4), chunks: Sequence[int] = (0, 32, 64, 128, 256),
+def tune_batch(instances: List[dict], ks: Sequence[int] = (2,), chunks: Sequence[int] = (0, 16, 32, 64, 128),
                step_scale: int = 8, use_cache: bool = True, sequence: str = "interleaved",
                potential: str = "paper") -> dict:
-    """Pick steps per pass and one rows-per-tile value for a batch by timing a
-    shortened copy of it (every lattice run for nsteps/step_scale steps)."""
+    """Pick steps per pass (the batch's passes take two whatever is asked for) and one
+    limit of the rows per warp for a batch by timing a shortened copy of it (every
+    lattice run for nsteps/step_scale steps)."""
     import torch
 
     from .qla import Batch

@@ -447,7 +447,7 @@ class Batch:
     nsteps, and optionally pulse=(polarization 'Ez'/'Ey', x0, sigma, amplitude)
     and chunk_rows.
     steps_per_pass = 0 lets the autotuner (autotune.tune_batch, cached per GPU
-    and batch shape) choose the steps per pass and the rows per tile of the
+    and batch shape) choose the steps per pass and the most rows per warp of the
     instances that do not set chunk_rows; the choice is kept in self.tuned.
     """
 
