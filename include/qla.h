@@ -101,11 +101,14 @@ typedef struct {
 /* Fill *opt with the defaults listed above. */
 void qla_default_options(qla_options *opt);
 
-/* Device memory one context needs (bytes; each buffer 256-byte aligned). */
+/* Device memory one context needs (bytes; each buffer 256-byte aligned). The sizes
+ * depend on Nx, Ny and the precision only. */
 typedef struct {
     size_t state_bytes;    /* one state buffer (6 planes); two are needed (ping-pong) */
-    size_t coeff_bytes;    /* rotation and potential coefficients, in the layout of the sweep that the
-                              options select (query with the options given to qla_create) */
+    size_t coeff_bytes;    /* rotation and potential coefficients: strip records of the marching sweep,
+                              or the pair planes of the shared-memory sweep (the persistent launch form;
+                              lattices much narrower than a strip and very tall, or too large for the
+                              device with records). The larger of the two where both are possible */
     size_t index_bytes;    /* n_x, n_y, n_z (double) */
     size_t scratch_bytes;  /* reduction scratch for the diagnostics */
 } qla_buffer_sizes;

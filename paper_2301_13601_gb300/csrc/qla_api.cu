@@ -144,14 +144,36 @@ bool persistent_applies(const qla_ctx *c) {
            c->ctas[c->K] >= 1 && c->ctas[c->K] <= qla::kPersistMaxCtas;
 }
 
-// Whether the marching form serves a context: unless the persistent launch form
-// (on the shared-memory sweep and its pair planes) was asked for and applies,
-// every lattice but a tall one much narrower than a strip, whose records (a
-// whole strip wide) would take many times the memory of the pair planes.
+// What a context may take of a GB300's 298 GB for the marching form's sake; the
+// rest is left to the CUDA context and the caller's allocator.
+constexpr size_t kDeviceBytes = 285000000000ull;
+
+size_t pair_plane_bytes(int precision, int Nx, int Ny) {
+    return size_t(qla::NCOEF) * size_t(Nx) * size_t(Ny) * (precision == QLA_FP64 ? 8 : 4);
+}
+size_t scratch_bytes(int Nx, int Ny) {
+    return round_up(qla::diag_scratch_bytes(Nx, Ny), kAlign) + round_up(sizeof(qla::DiagResult), kAlign) +
+           kAlign +            // sweep error flag, share-order counter
+           kPassCounterBytes;  // per-share pass counters of the persistent launch form
+}
+
+// Whether the memory of the marching form's records allows it, whatever the other
+// options: not for a tall lattice much narrower than a strip (records are a whole
+// strip wide, many times the pair planes), nor for one that fits the device with
+// pair planes only (145 against 128 bytes per FP32 site in all: above 1.96e9
+// sites, which the shared-memory sweep then serves as before).
+bool march_fits(int precision, int Nx, int Ny, qla::MarchGeo *g) {
+    if (!qla::march_geometry(precision == QLA_FP64 ? 1 : 0, Nx, Ny, g)) return false;
+    const size_t P = size_t(Nx) * size_t(Ny), records = qla::march_bytes(*g, 2);
+    if (records > std::max(size_t(1) << 30, 4 * pair_plane_bytes(precision, Nx, Ny))) return false;
+    return 2 * 6 * P * g->es + records + 3 * P * sizeof(double) + scratch_bytes(Nx, Ny) <= kDeviceBytes;
+}
+
+// Whether the marching form serves a context: where it fits, unless the persistent
+// launch form (on the shared-memory sweep and its pair planes) was asked for and
+// applies.
 bool march_applies(const qla_options &o, int Nx, int Ny, qla::MarchGeo *g) {
-    if (!qla::march_geometry(o.precision == QLA_FP64 ? 1 : 0, Nx, Ny, g)) return false;
-    const size_t pairs = size_t(qla::NCOEF) * size_t(Nx) * Ny * g->es;
-    if (qla::march_bytes(*g, 2) > std::max(size_t(1) << 30, 4 * pairs)) return false;
+    if (!march_fits(o.precision, Nx, Ny, g)) return false;
     const int K = o.steps_per_pass > 0 ? o.steps_per_pass
                                        : default_steps_per_pass(o.precision, Nx, Ny, o.chunk_rows);
     return !(o.launch == QLA_LAUNCH_PERSISTENT && o.precision == QLA_FP32 && o.chunk_rows == 0 &&
@@ -294,14 +316,14 @@ qla_status qla_query_buffer_sizes(int Nx, int Ny, const qla_options *opt, qla_bu
     const size_t P = size_t(Nx) * size_t(Ny);
     const size_t es = elem_size(o);
     out->state_bytes = round_up(6 * P * es, kAlign);
+    // The larger of the two layouts, for both families: the size depends on the lattice
+    // and the precision only, so that buffers serve a context of any other options.
     qla::MarchGeo g;
-    const int nfam = o.families == QLA_FAMILIES_BOTH ? 2 : 1;
-    out->coeff_bytes = round_up(march_applies(o, Nx, Ny, &g) ? qla::march_bytes(g, nfam)
-                                                             : size_t(qla::NCOEF) * P * es, kAlign);
+    const size_t pairs = pair_plane_bytes(o.precision, Nx, Ny);
+    out->coeff_bytes =
+        round_up(march_fits(o.precision, Nx, Ny, &g) ? std::max(pairs, qla::march_bytes(g, 2)) : pairs, kAlign);
     out->index_bytes = round_up(3 * P * sizeof(double), kAlign);
-    out->scratch_bytes = round_up(qla::diag_scratch_bytes(Nx, Ny), kAlign) + round_up(sizeof(qla::DiagResult), kAlign) +
-                         kAlign +  // sweep error flag, share-order counter
-                         kPassCounterBytes;  // per-share pass counters of the persistent launch form
+    out->scratch_bytes = scratch_bytes(Nx, Ny);
     return QLA_OK;
 }
 
