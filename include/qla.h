@@ -288,6 +288,11 @@ qla_status qla_get_launch(const qla_ctx *ctx, int *launch);
  * <= 0 or a negative withhold. */
 qla_status qla_set_wait_limit(qla_ctx *ctx, long long timeout_ns, int withhold);
 
+/* Test hook: from here on the context is served by the shared-memory sweep, its
+ * coefficients in pair planes, as where strip records do not fit (see
+ * qla_buffer_sizes). The results do not change. */
+qla_status qla_use_pair_planes(qla_ctx *ctx);
+
 /* The balanced split of one fused pass of steps_per_pass steps (the sweep of
  * Eq. 28 / Eq. 23 over the lattice, one CTA grid layer per family). The
  * lattice is cut into strips of 256 - 8K output columns (K = steps_per_pass;

@@ -731,6 +731,16 @@ qla_status qla_set_wait_limit(qla_ctx *c, long long timeout_ns, int withhold) {
     return QLA_OK;
 }
 
+qla_status qla_use_pair_planes(qla_ctx *c) {
+    qla_status s = enter(c);
+    if (s != QLA_OK) return s;
+    if (!c->march) return QLA_OK;
+    QLA_CUDA(c, qla::launch_coefficients(c->index, c->coef, c->Nx, c->Ny, c->delta, c->opt.precision,
+                                         c->opt.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0, c->mode, c->stream));
+    c->march = false;
+    return QLA_OK;
+}
+
 qla_status qla_get_launch(const qla_ctx *c, int *launch) {
     if (!c || !launch) return QLA_EINVAL;
     *launch = c->persistent ? QLA_LAUNCH_PERSISTENT : QLA_LAUNCH_PER_PASS;

@@ -40,6 +40,7 @@ EXPORTS = [
     "qla_get_fields_f32", "qla_state_device_ptr", "qla_synchronize", "qla_step_count", "qla_get_config",
     "qla_last_error", "qla_status_string", "qla_destroy", "qla_diagnostics_noalloc", "qla_sweep_split",
     "qla_get_sweep_split", "qla_sweep_dependencies", "qla_get_launch", "qla_set_wait_limit",
+    "qla_use_pair_planes",
     "qla_batch_create", "qla_batch_run", "qla_batch_get_fields_f32", "qla_batch_diagnostics", "qla_batch_info",
     "qla_batch_set_wait_limit", "qla_batch_last_error", "qla_batch_destroy",
 ]
@@ -139,6 +140,8 @@ def load_library(path: str = LIB_PATH):
     L.qla_get_launch.restype = st
     L.qla_set_wait_limit.argtypes = [v, ctypes.c_longlong, i]
     L.qla_set_wait_limit.restype = st
+    L.qla_use_pair_planes.argtypes = [v]
+    L.qla_use_pair_planes.restype = st
     _lib = L
     return L
 
@@ -265,6 +268,10 @@ class Simulation:
     def set_wait_limit(self, timeout_ns: int, withhold: int = 0):
         """Test hook of the persistent form's waits (qla_set_wait_limit)."""
         self._check(self._L.qla_set_wait_limit(self._ctx, int(timeout_ns), int(withhold)), "qla_set_wait_limit")
+
+    def use_pair_planes(self):
+        """Test hook: the shared-memory sweep serves the context (qla_use_pair_planes)."""
+        self._check(self._L.qla_use_pair_planes(self._ctx), "qla_use_pair_planes")
 
     @property
     def launch(self) -> str:
