@@ -144,10 +144,6 @@ bool persistent_applies(const qla_ctx *c) {
            c->ctas[c->K] >= 1 && c->ctas[c->K] <= qla::kPersistMaxCtas;
 }
 
-// What a context may take of a GB300's 298 GB for the marching form's sake; the
-// rest is left to the CUDA context and the caller's allocator.
-constexpr size_t kDeviceBytes = 285000000000ull;
-
 size_t pair_plane_bytes(int precision, int Nx, int Ny) {
     return size_t(qla::NCOEF) * size_t(Nx) * size_t(Ny) * (precision == QLA_FP64 ? 8 : 4);
 }
@@ -158,15 +154,15 @@ size_t scratch_bytes(int Nx, int Ny) {
 }
 
 // Whether the memory of the marching form's records allows it, whatever the other
-// options: not for a tall lattice much narrower than a strip (records are a whole
-// strip wide, many times the pair planes), nor for one that fits the device with
-// pair planes only (145 against 128 bytes per FP32 site in all: above 1.96e9
+// options: not where they are not worth it (march_worth), nor for a lattice that
+// fits the device with pair planes only (145 against 128 bytes per FP32 site in all: above 1.96e9
 // sites, which the shared-memory sweep then serves as before).
 bool march_fits(int precision, int Nx, int Ny, qla::MarchGeo *g) {
     if (!qla::march_geometry(precision == QLA_FP64 ? 1 : 0, Nx, Ny, g)) return false;
-    const size_t P = size_t(Nx) * size_t(Ny), records = qla::march_bytes(*g, 2);
-    if (records > std::max(size_t(1) << 30, 4 * pair_plane_bytes(precision, Nx, Ny))) return false;
-    return 2 * 6 * P * g->es + records + 3 * P * sizeof(double) + scratch_bytes(Nx, Ny) <= kDeviceBytes;
+    if (!qla::march_worth(*g, pair_plane_bytes(precision, Nx, Ny))) return false;
+    const size_t P = size_t(Nx) * size_t(Ny);
+    return 2 * 6 * P * g->es + qla::march_bytes(*g, 2) + 3 * P * sizeof(double) + scratch_bytes(Nx, Ny) <=
+           qla::kDeviceBytes;
 }
 
 // Whether the marching form serves a context: where it fits, unless the persistent

@@ -38,6 +38,18 @@ struct BatchInst {
     int wide;                       // its rotations take the form for any angle (MODE_WIDE)
 };
 
+// A lattice whose records are not worth their memory, or do not fit: coefficients in
+// pair planes, advanced by the shared-memory sweep, whose passes follow the batch
+// kernel in the graph. Its state returns to q[0] after every run.
+struct BatchPlanes {
+    void *q[2];
+    const void *coef;
+    int Nx, Ny, chunk, mode;
+    int K;                          // steps per pass
+    int ctas;                       // balanced split (chunk = 0)
+    long long passes;
+};
+
 struct BatchSched {
     const BatchInst *inst;           // sorted by passes, descending
     int ninst;
@@ -166,6 +178,28 @@ __global__ void batch_flip(const BatchInst *inst, int *cur, int n) {
     if (i < n) cur[i] ^= (inst[i].passes & 1);
 }
 
+cudaError_t launch_planes(const BatchPlanes &p, bool inter, int *error, cudaStream_t st) {
+    SweepArgs a{};
+    a.coef = p.coef;
+    a.Nx = p.Nx;
+    a.Ny = p.Ny;
+    a.w_valid = sweep_strip_width() - 8 * p.K;
+    a.chunk = p.chunk;
+    a.ctas = p.ctas;
+    a.interleaved = inter ? 1 : 0;
+    a.mode = p.mode;
+    a.vec = 1;  // Nx is a multiple of 4
+    a.error = error;
+    for (long long i = 0; i < p.passes; ++i) {
+        a.q_in = p.q[i & 1];
+        a.q_out = p.q[(i + 1) & 1];
+        const cudaError_t e = launch_sweep_f32(p.K, a, 2, st);
+        if (e != cudaSuccess) return e;
+    }
+    return p.passes & 1 ? cudaMemcpyAsync(p.q[0], p.q[1], 24ull * p.Nx * p.Ny, cudaMemcpyDeviceToDevice, st)
+                        : cudaSuccess;
+}
+
 // Sets the shared-memory attribute and returns the persistent grid size (SMs x
 // resident CTAs); called before stream capture. With S: launches *grid CTAs.
 template <bool INTER, int MODE, bool VEC>
@@ -217,6 +251,7 @@ struct qla_batch {
     int mode = 0;  // SweepMode: MODE_WIDE if any lattice's
     cudaStream_t stream = nullptr;
     std::vector<qla::BatchInst> inst;  // sorted order
+    std::vector<qla::BatchPlanes> planes;
     std::vector<int> order;            // order[k] = user index of sorted instance k
     std::vector<int> slot;             // slot[user index] = sorted position
     std::vector<int> cur;              // host copy of the parities
@@ -255,10 +290,9 @@ cudaError_t dalloc(qla_batch *b, P **p, size_t bytes) {
     return e;
 }
 
-// Rows per share, at most: as many as let the batch's
-// warps fill the GPU's slots (8 per SM) a little more than once (a lattice's
-// pass ends with its last tile; more, lower shares pay the march_delay(2) = 17
-// warm-up rows more often), and at least 8. Ten lattices of sides 256 to 1024,
+// Rows per share, at most: as many as let the batch's warps fill the GPU's slots (8
+// per SM) a little more than once (a lattice's pass ends with its last tile; more,
+// lower shares pay the march_delay(2) = 17 warm-up rows more often), and at least 8. Ten lattices of sides 256 to 1024,
 // 400 steps: 16 rows 34.8 ms, 28 (filled twice) 23.9, 48 21.2, 64 22.2, 96 28.5;
 // the three largest of them: 15 rows 16.5 ms, 32 14.1, 64 20.4.
 int batch_rows(const std::vector<qla::MarchGeo> &geo, int sms) {
@@ -281,6 +315,9 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     const int K = o.steps_per_pass > 0 ? o.steps_per_pass : 4;
     if (K != 2 && K != 4) return QLA_EUNSUPPORTED;
     std::vector<int> modes(count);
+    std::vector<char> planes(count);  // on pair planes (BatchPlanes)
+    std::vector<qla::MarchGeo> geo_of(count);
+    size_t bytes = 0, index_bytes = 0;
     for (int i = 0; i < count; ++i) {
         const qla_instance_desc &d = descs[i];
         if (d.Nx < 4 || d.Ny < 1 || d.Nx % 4 != 0 || (long long)d.Nx * d.Ny > 2147483647LL) return QLA_EINVAL;
@@ -293,7 +330,12 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
             if (!qla::index_valid(nn[k], P, &ordinary)) return QLA_EINVAL;
         modes[i] = qla::rotation_mode(nn, ordinary, d.Nx, d.Ny, d.delta, 0, o.sequence == QLA_SEQ_INTERLEAVED ? 1 : 0,
                                       o.potential == QLA_POT_UNITARY ? 1 : 0);
+        const size_t pairs = size_t(qla::NCOEF) * P * 4;
+        planes[i] = !qla::march_geometry(0, d.Nx, d.Ny, &geo_of[i]) || !qla::march_worth(geo_of[i], pairs);
+        bytes += 48 * P + (planes[i] ? pairs : qla::march_bytes(geo_of[i], 2));
+        index_bytes = std::max(index_bytes, 24 * P);
     }
+    if (bytes + index_bytes > qla::kDeviceBytes) planes.assign(count, 1);
     qla_batch *b = new qla_batch();
     auto bail = [&](qla_status s) {
         qla_batch_destroy(b);
@@ -312,27 +354,31 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->dev);
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) return bail(QLA_ECUDA);
 
-    // sort by number of passes, descending (active instances of a pass are a prefix)
+    // sort by number of passes, descending (active instances of a pass are a prefix;
+    // lattices on pair planes take no part: the last)
+    auto steps = [&](int i) { return planes[i] ? 0LL : descs[i].nsteps; };
     b->order.resize(count);
     std::iota(b->order.begin(), b->order.end(), 0);
     std::stable_sort(b->order.begin(), b->order.end(),
-                     [&](int a, int c) { return descs[a].nsteps > descs[c].nsteps; });
+                     [&](int a, int c) { return steps(a) > steps(c); });
     b->slot.resize(count);
     for (int k = 0; k < count; ++k) b->slot[b->order[k]] = k;
     b->inst.resize(count);
     b->cur.assign(count, 0);
     size_t scratch_max = 0;
-    std::vector<qla::MarchGeo> geo(count);
-    for (int k = 0; k < count; ++k) {
-        const qla_instance_desc &d = descs[b->order[k]];
-        if (!qla::march_geometry(0, d.Nx, d.Ny, &geo[k])) return bail(QLA_EUNSUPPORTED);
-        b->vec = b->vec && qla::march_vectors(geo[k]);
+    std::vector<qla::MarchGeo> marching;
+    for (int i = 0; i < count; ++i) {
+        if (planes[i]) continue;
+        marching.push_back(geo_of[i]);
+        b->vec = b->vec && qla::march_vectors(geo_of[i]);
     }
-    const int rows = batch_rows(geo, b->sms);
+    const int rows = batch_rows(marching, b->sms);
     for (int k = 0; k < count; ++k) {
         const qla_instance_desc &d = descs[b->order[k]];
         qla::BatchInst &I = b->inst[k];
-        const qla::MarchGeo &g = geo[k];
+        const qla::MarchGeo &g = geo_of[b->order[k]];
+        const bool planar = planes[b->order[k]] != 0;
+        const int mode = modes[b->order[k]];
         const size_t P = size_t(d.Nx) * d.Ny;
         I.Nx = d.Nx;
         I.Ny = d.Ny;
@@ -346,18 +392,25 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         I.chunks = (d.Ny + ch - 1) / ch;
         I.tiles = (I.strips * I.chunks + qla::BWPC - 1) / qla::BWPC;
         I.passes = int(d.nsteps / qla::kBatchSteps);
-        I.wide = modes[b->order[k]] & qla::MODE_WIDE ? 1 : 0;
+        I.wide = mode & qla::MODE_WIDE ? 1 : 0;
+        if (planar) I.passes = I.tiles = 0;
         float *q0, *q1;
         char *mem;
         double *idx;
         if (dalloc(b, &q0, 6 * P * 4) != cudaSuccess || dalloc(b, &q1, 6 * P * 4) != cudaSuccess ||
-            dalloc(b, &mem, qla::march_bytes(g, 2)) != cudaSuccess || dalloc(b, &idx, 3 * P * 8) != cudaSuccess) {
+            dalloc(b, &mem, planar ? size_t(qla::NCOEF) * P * 4 : qla::march_bytes(g, 2)) != cudaSuccess ||
+            dalloc(b, &idx, 3 * P * 8) != cudaSuccess) {
             cudaGetLastError();
             return bail(QLA_ENOMEM);
         }
         I.q[0] = reinterpret_cast<char *>(q0);
         I.q[1] = reinterpret_cast<char *>(q1);
         for (int f = 0; f < 2; ++f) {
+            if (planar) {
+                I.rec[f] = nullptr;
+                I.flags[f] = nullptr;
+                continue;
+            }
             I.rec[f] = mem + f * g.record_bytes;
             I.flags[f] = reinterpret_cast<const unsigned char *>(mem + 2 * g.record_bytes + f * g.flag_bytes);
         }
@@ -365,9 +418,25 @@ qla_status qla_batch_create(int count, const qla_instance_desc *descs, const qla
         for (int c = 0; c < 3; ++c)
             if (cudaMemcpyAsync(idx + c * P, nn[c], P * 8, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
                 return bail(QLA_ECUDA);
-        if (qla::launch_march_records(g, idx, mem, 2, 0, d.delta, 0, b->inter ? 1 : 0, modes[b->order[k]], b->stream) !=
-            cudaSuccess)
+        const int inter = b->inter ? 1 : 0;
+        if ((planar ? qla::launch_coefficients(idx, mem, d.Nx, d.Ny, d.delta, 0, inter, mode, b->stream)
+                    : qla::launch_march_records(g, idx, mem, 2, 0, d.delta, 0, inter, mode, b->stream)) != cudaSuccess)
             return bail(QLA_ECUDA);
+        if (planar) {
+            qla::BatchPlanes p;
+            p.q[0] = q0;
+            p.q[1] = q1;
+            p.coef = mem;
+            p.Nx = d.Nx;
+            p.Ny = d.Ny;
+            p.chunk = d.chunk_rows > 0 ? std::min(d.chunk_rows, d.Ny) : 0;
+            p.mode = mode;
+            p.K = mode & qla::MODE_WIDE ? 1 : 2;
+            const qla::SweepSplit sp = qla::make_sweep_split(d.Nx, d.Ny, p.K, qla::sweep_block_rows(0, p.K), 1);
+            p.ctas = int(std::min((long long)b->sms * qla::sweep_occupancy_f32(p.K, inter), (long long)sp.nsx * d.Ny));
+            p.passes = d.nsteps / p.K;
+            b->planes.push_back(p);
+        }
         if (cudaMemsetAsync(q0, 0, 6 * P * 4, b->stream) != cudaSuccess ||
             cudaMemsetAsync(q1, 0, 6 * P * 4, b->stream) != cudaSuccess)
             return bail(QLA_ECUDA);
@@ -444,6 +513,8 @@ qla_status qla_batch_run(qla_batch *b) {
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_error, 0, 64, b->stream);
         if (e == cudaSuccess && b->maxpass > 0)
             e = qla::batch_dispatch(b->vec, b->inter, b->mode, b->sms, &b->grid, &S, b->stream);
+        for (const qla::BatchPlanes &p : b->planes)
+            if (e == cudaSuccess) e = qla::launch_planes(p, b->inter, b->d_error, b->stream);
         if (e == cudaSuccess) {
             qla::batch_flip<<<(b->n + 127) / 128, 128, 0, b->stream>>>(b->d_inst, b->d_cur, b->n);
             e = cudaGetLastError();
@@ -468,7 +539,7 @@ qla_status qla_batch_run(qla_batch *b) {
         return QLA_ECUDA;
     for (int k = 0; k < b->n; ++k) b->cur[k] ^= (b->inst[k].passes & 1);
     if (err) {
-        b->msg = "a dependency wait timed out";
+        b->msg = "a dependency wait or a wait for row copies timed out";
         return QLA_ETIMEOUT;
     }
     return QLA_OK;
@@ -511,6 +582,7 @@ qla_status qla_batch_info(const qla_batch *b, long long *total_items, int *steps
     if (site_updates) {
         long long s = 0;
         for (const auto &I : b->inst) s += (long long)I.Nx * I.Ny * I.passes * qla::kBatchSteps;
+        for (const auto &p : b->planes) s += (long long)p.Nx * p.Ny * p.passes * p.K;
         *site_updates = s;
     }
     return QLA_OK;

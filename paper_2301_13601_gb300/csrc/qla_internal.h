@@ -277,6 +277,13 @@ struct MarchGeo {
 // Whether the marching form serves the lattice, and its geometry: FP32 128
 // columns with a halo of 8 (two steps), FP64 64 with 4 (one).
 bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g);
+// Whether the records (of both families) are worth their memory beside pair planes of
+// `pairs` bytes: not for a tall lattice much narrower than a strip, whose records
+// are a whole strip wide.
+bool march_worth(const MarchGeo &g, size_t pairs);
+// What a context or batch may take of a GB300's 298 GB for the records' sake; the rest
+// is left to the CUDA context and the caller's allocator.
+constexpr size_t kDeviceBytes = 285000000000ull;
 // Whether its state rows are copied in 16-byte vectors at 32-bit offsets.
 bool march_vectors(const MarchGeo &g);
 // Chooses the row ranges of a pass over nfam families on a device of sms SMs.

@@ -19,6 +19,10 @@ bool march_geometry(int precision, int Nx, int Ny, MarchGeo *g) {
     return (long long)g->strips * Ny < (1LL << 30);  // shares, at most
 }
 
+bool march_worth(const MarchGeo &g, size_t pairs) {
+    return march_bytes(g, 2) <= std::max(size_t(1) << 30, 4 * pairs);
+}
+
 bool march_vectors(const MarchGeo &g) {
     return g.Nx % (16 / g.es) == 0 && (unsigned long long)g.Nx * g.Ny * g.es < (1ull << 32);
 }
