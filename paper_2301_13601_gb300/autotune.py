@@ -128,7 +128,7 @@ def tune_single(n_x, n_y, n_z, delta: float, precision: str = "fp32", sequence: 
     return entry
 
 
-def tune_batch(instances: List[dict], ks: Sequence[int] = (2,), chunks: Sequence[int] = (0, 16, 32, 64, 128),
+def tune_batch(instances: List[dict], ks: Sequence[int] = (2,), chunks: Sequence[int] = (0, 32, 64, 128, 256),
                step_scale: int = 8, use_cache: bool = True, sequence: str = "interleaved",
                potential: str = "paper") -> dict:
     """Pick steps per pass (the batch's passes take two whatever is asked for) and one
