@@ -12,13 +12,6 @@
 #include "../../include/qla.h"
 #include "qla_internal.h"
 
-namespace qla {
-// The persistent launch with the test hook of its waits (qla_sweep_persist.cu).
-cudaError_t launch_sweep_persistent_hooked_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
-                                               unsigned *done, unsigned withhold, unsigned long long wait_ns,
-                                               cudaStream_t st);
-}  // namespace qla
-
 struct qla_ctx {
     int Nx = 0, Ny = 0;
     double delta = 0.0;

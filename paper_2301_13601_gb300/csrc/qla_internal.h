@@ -42,14 +42,8 @@ constexpr int NCOEF = 2 * NPAIR;  // scalars per site
 //   TM: hub q2, x-partner q4, y-partner q3   (E_z polarisation)
 //   TE: hub q5, x-partner q1, y-partner q0   (E_y polarisation)
 // In both families the first streaming group (S_14 along x, S_03 along y)
-// moves the partner and the second (S_25) moves the hub.
-struct Family {
-    int h, px, py;            // state planes
-    int cx, cy, vx, vy;       // coefficient pair planes
-    float sgx, sgy;           // collision orientation: C is h' = h + (m h + sg sin p)
-    float tx, ty;             // potential orientation: target' = ... + t sin source
-    int vx_hub, vy_hub;       // 1 if the potential row targets the hub, 0 if the partner
-};
+// moves the partner and the second (S_25) moves the hub (Fam in
+// qla_sweep.cuh).
 
 // Strips and balanced split of a pass. The row units u = strip * Ny + y of
 // a family (nsx strips, Ny rows each) are shared among the G CTAs of the
@@ -232,8 +226,11 @@ bool sweep_supported(int precision, int K);
 // values before the launch all <= base). FP32 with tensor maps and the seam
 // layout only: cudaErrorNotSupported otherwise.
 constexpr int kPersistMaxCtas = 4096;
-cudaError_t launch_sweep_persistent_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
-                                        unsigned *done, cudaStream_t st);
+// Every wait demands `withhold` passes more (0 but for the test hook) and is limited to
+// wait_ns.
+cudaError_t launch_sweep_persistent_hooked_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
+                                               unsigned *done, unsigned withhold, unsigned long long wait_ns,
+                                               cudaStream_t st);
 bool sweep_persistent_supported(int precision, int K);
 int sweep_strip_width();  // input columns per strip (halo included)
 int sweep_occupancy_f32(int K, int interleaved);  // resident CTAs per SM

@@ -37,7 +37,6 @@ struct SweepPersistParams {
 // for every share of the family).
 constexpr int kPersistDeps = 64;
 constexpr size_t kPersistSmemExtra = 2 * kPersistDeps * sizeof(unsigned short) + 2 * sizeof(int);
-constexpr unsigned long long kPersistWaitNs = 2000000000ull;  // default wait limit
 
 template <typename T, int K, int R, int NY, bool INTER, int MODE>
 __global__ void __launch_bounds__(SweepCfg<T, K, R, NY>::NT, SweepCfg<T, K, R, NY>::MINB)
@@ -198,11 +197,6 @@ cudaError_t launch_sweep_persistent_hooked_f32(int K, const SweepArgs &a, int nf
     return a.mode & MODE_UNITARY
                ? launch_persistent_t<float, 2, 4, 2, false, MODE_UNITARY>(a, nfam, passes, base, done, withhold, wait_ns, st)
                : launch_persistent_t<float, 2, 4, 2, false, 0>(a, nfam, passes, base, done, withhold, wait_ns, st);
-}
-
-cudaError_t launch_sweep_persistent_f32(int K, const SweepArgs &a, int nfam, int passes, unsigned base,
-                                        unsigned *done, cudaStream_t st) {
-    return launch_sweep_persistent_hooked_f32(K, a, nfam, passes, base, done, 0u, kPersistWaitNs, st);
 }
 
 bool sweep_persistent_supported(int precision, int K) { return precision == 0 && K == 2; }
