@@ -68,8 +68,10 @@ enum { QLA_FAMILIES_BOTH = 0, QLA_FAMILY_TM = 1, QLA_FAMILY_TE = 2 };
  *   whose previous pass wrote what it reads or read what it overwrites (see
  *   qla_sweep_dependencies), not for the whole lattice. Bit-identical results.
  *   Applies to FP32 contexts with the balanced split (chunk_rows = 0), 2 steps
- *   per pass, Nx a multiple of 8 and at least 256; other contexts, and a launch
- *   the device refuses, use one launch per pass.
+ *   per pass, Nx a multiple of 8 and at least 256, and with the unitary
+ *   potentials to media whose rotations stay below 0.5 rad (Eq. 24-25; any
+ *   medium of indices 0.9 to 4); other contexts, and a launch the device
+ *   refuses, use one launch per pass.
  * QLA_LAUNCH_AUTO: one launch per pass (the faster form where measured). */
 enum { QLA_LAUNCH_AUTO = 0, QLA_LAUNCH_PER_PASS = 1, QLA_LAUNCH_PERSISTENT = 2 };
 
@@ -83,8 +85,12 @@ typedef struct {
     int precision;       /* QLA_FP32 (default) or QLA_FP64 (correctness mode) */
     int sequence;        /* QLA_SEQ_INTERLEAVED (default, Eq. 28) or QLA_SEQ_PLAIN (Eq. 23) */
     int potential;       /* QLA_POT_PAPER (default) or QLA_POT_UNITARY */
-    int steps_per_pass;  /* full time steps fused per HBM pass: 0 = automatic (2; FP32 with chunk_rows
-                            set: 2 from 2^25 sites up, else 4), else 1, 2 or 4 */
+    int steps_per_pass;  /* full time steps fused per HBM pass: 0 = automatic, else 1, 2 or 4 (FP64: 1,
+                            2). The marching sweep runs 4 as two passes of 2, FP64 in passes of 1 and,
+                            automatically, FP32 lattices of at most 2^19 sites in passes of 1, larger
+                            ones of 2; the shared-memory sweep takes 2 (FP32 with chunk_rows set: 2 from
+                            2^25 sites up, else 4). qla_get_config reports the shared-memory sweep's
+                            number. Results do not depend on it */
     int chunk_rows;      /* most rows of a strip swept by one warp (0 = no limit: as many as are
                             fastest); where the shared-memory sweep serves the context (coefficients
                             in pair planes, see qla_buffer_sizes), rows of one of its tiles, 0 = the
@@ -269,7 +275,7 @@ qla_status qla_synchronize(qla_ctx *ctx);
 /* Steps taken since the last state reset; -1 for a NULL context. */
 long long qla_step_count(const qla_ctx *ctx);
 
-/* Resolved configuration: steps per pass and rows per tile used by qla_step
+/* Resolved configuration: steps per pass and chunk_rows (see qla_options) of qla_step
  * (0: the balanced split), and the precision. Any pointer may be NULL. */
 qla_status qla_get_config(const qla_ctx *ctx, int *steps_per_pass, int *chunk_rows, int *precision);
 

@@ -328,9 +328,11 @@ __global__ void __launch_bounds__(DIAG_THREADS, 4) diag_partial_f32(const float 
 //
 // The FP64 pipe is the bound, so each product is formed once: a warp covers 30
 // columns with one more on either side (D_x of the neighbours by shuffle) and
-// walks down a tile's rows (D_y of the rows above and below in registers); six
-// FP64 operations per site, where a thread per site that formed its four
-// neighbours' products and |D|^2 itself took about thirty (4096^2: 760 us).
+// walks down a tile's rows (D_y of the rows above and below in registers): six
+// FP64 operations per site and those of the tiles' halo rows, shared columns and
+// maxima, 8.6 by the pipe's time (4096^2: 298 us, pipe 82% busy), where a thread per
+// site that formed its four neighbours' products and |D|^2 itself took about thirty
+// (760 us).
 // max |D|^2 is screened in FP32 (Screen), FP32 states are widened
 // on the integer pipe, and the factors 1/2 and 1/4 are applied to the reduced
 // values.
